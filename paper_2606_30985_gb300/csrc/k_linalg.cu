@@ -543,6 +543,7 @@ __global__ void k_form(const SiteFacItem* __restrict__ items, const int* ival, i
       H[e] = h;
     }
     __syncthreads();
+    double* Gp = it.T + (long long)it.ldt * it.ldt;   // G lies behind T (k_factor writes T from it)
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < (long long)chic * chic;
          e += (long long)gridDim.x * blockDim.x) {
       int c = (int)(e / chic), c2 = (int)(e % chic);
@@ -557,7 +558,7 @@ __global__ void k_form(const SiteFacItem* __restrict__ items, const int* ival, i
           double g = 0.0;
 #pragma unroll
           for (int pq = 0; pq < 16; ++pq) g += h[pq] * Cb[pq];
-          it.T[(long long)(c * rg + k) * it.ldt + c2 * rg + k2] = g;
+          Gp[(long long)(c * rg + k) * it.ldt + c2 * rg + k2] = g;
         }
     }
   } else {
@@ -582,220 +583,326 @@ cudaError_t launch_form(const SiteFacItem* items, int n_items, int grid_x, const
 }
 
 // =================================================================== factor
-// Whether the Cholesky-QR branch can be trusted with this Gram C = cv^T cv
+constexpr int kFacThreads = 512;     // one thread per column: n, r <= 512
+
+// Shared-memory plan of k_factor: the vectors first, then whatever is left
+// for the factor itself (U of the Cholesky branch, the matrix of the
+// Householder branch) when it fits.
+struct FacSmem {
+  size_t dg, od, uc, perm, v, mat, total;
+};
+__host__ __device__ inline FacSmem fac_smem(int rmax, int nmax, int householder) {
+  FacSmem m;
+  const int w = rmax > nmax ? rmax : nmax;
+  size_t o = 0;
+  m.dg = o;   o += sizeof(double) * w;
+  m.od = o;   o += sizeof(double) * w;
+  m.uc = o;   o += sizeof(double) * w;
+  m.perm = o; o += sizeof(int) * (size_t)(w + (w & 1));
+  m.v = o;
+  if (householder) o += sizeof(double) * ((size_t)4 * nmax + (size_t)(kFacThreads / 32) * rmax);
+  m.mat = o;
+  const size_t cap = (size_t)200 * 1024;
+  const size_t want = householder ? sizeof(double) * (size_t)4 * nmax * rmax : sizeof(double) * (size_t)rmax * rmax;
+  o += want < cap - o ? want : cap - o;
+  m.total = o;
+  return m;
+}
+
+// Pivoted Cholesky of a symmetric n x n matrix A (leading dimension lda, read
+// only) in precision R: U (leading dimension ldu) receives the upper factor in
+// pivoted column order, perm the original column at each position; returns the
+// rank (pivots <= rel times the first end it), or -1 when an accepted pivot
+// keeps less than `safe` of its own column's diagonal (safe < 0: not tested).
+//
+// Left-looking: step j forms only row j, U[j, q] = (A[p_j, p_q] - sum_l<j
+// U[l, j] U[l, q]) / U[j, j], one thread per column q.  The right-looking form
+// rewrites the whole trailing square at every step (r^3 / 3 multiply-adds and
+// as many read-modify-writes through L2 with an index division each); this one
+// does r^3 / 6 multiply-adds and only reads U, which stays in shared memory up
+// to r = 150 or so.  The terms of an entry are subtracted in the same order.
+// Bound: the FP64 pipe of one SM (2 multiply-adds per clock: 2.6 ms at
+// r = 400), two barriers per step below that.
+template <typename R>
+__device__ int chol_pivoted(const double* __restrict__ A, int lda, int n, R* U, int ldu, R* dg, R* od, R* uc, int* perm,
+                            double rel, double safe) {
+  __shared__ double rv[kFacThreads / 32];
+  __shared__ int ri[kFacThreads / 32];
+  const int q = threadIdx.x, lane = q & 31, wid = q >> 5;
+  const int nw = (n + 31) >> 5;
+  int pq = q;                                   // original column at this thread's position
+  R dq = R(0), oq = R(0);
+  if (q < n) {
+    dq = oq = (R)A[(long long)q * lda + q];
+    dg[q] = dq;
+    od[q] = oq;
+    perm[q] = q;
+  }
+  double d0 = 0.0;
+  for (int j = 0; j < n; ++j) {
+    // pivot: the largest remaining diagonal, smallest position among ties;
+    // position j when every candidate is NaN (the test below then stops)
+    double best = -1.0;
+    int bi = n;
+    if (q >= j && q < n && (double)dq > best) { best = (double)dq; bi = q; }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+    }
+    if (lane == 0 && wid < nw) { rv[wid] = best; ri[wid] = bi; }
+    __syncthreads();
+    double b = -1.0;
+    int p = n;
+    for (int i = j >> 5; i < nw; ++i)
+      if (rv[i] > b || (rv[i] == b && ri[i] < p)) { b = rv[i]; p = ri[i]; }
+    if (p >= n) p = j;
+    const R dp = dg[p];
+    if (j == 0) d0 = (double)dp;
+    if (!((double)dp > rel * d0) || !((double)dp > 0.0)) return j;
+    if (safe >= 0.0 && !((double)dp >= safe * (double)od[p])) return -1;
+    const int pp = perm[p], pj = perm[j];
+    const R dj = dg[j], oj = od[j], op = od[p];
+    // column p of the finished rows, staged for the broadcast reads below, and
+    // the swap of the positions j and p in those rows
+    for (int l = q; l < j; l += kFacThreads) {
+      const R x = U[(long long)l * ldu + p];
+      uc[l] = x;
+      if (p != j) {
+        U[(long long)l * ldu + p] = U[(long long)l * ldu + j];
+        U[(long long)l * ldu + j] = x;
+      }
+    }
+    if (p != j) {
+      if (q == p) { pq = pj; dq = dj; oq = oj; }
+      if (q == j) { pq = pp; dq = dp; oq = op; }
+    }
+    __syncthreads();
+    const R rjj = sqrt(dp);
+    if (q == j) U[(long long)j * ldu + j] = rjj;
+    if (q > j && q < n) {
+      R acc = (R)A[(long long)pp * lda + pq];
+      const R* uq = U + q;
+      int l = 0;
+      for (; l + 16 <= j; l += 16) {            // 16 loads in flight before their uses
+        R x[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) x[i] = uq[(long long)(l + i) * ldu];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc = fma(-uc[l + i], x[i], acc);
+      }
+      for (; l < j; ++l) acc = fma(-uc[l], uq[(long long)l * ldu], acc);
+      acc /= rjj;
+      U[(long long)j * ldu + q] = acc;
+      dq = fma(-acc, acc, dq);
+    }
+    if (p != j && (q == p || q == j)) { perm[q] = pq; od[q] = oq; }
+    if (q < n) dg[q] = dq;
+  }
+  return n;
+}
+
+// Column-pivoted Householder QR of the M x r matrix B (leading dimension ld)
+// in place: R in the upper trapezoid, the position order in perm; returns the
+// rank.  The 16 warps share the rows and their lanes the columns, so a
+// reflection's dot products and its update use the whole block (one thread
+// per column left all but r threads idle on two serial passes of M rows).
+__device__ int qrcp(double* B, int ld, int M, int r, double* dg, double* w, double* v, double* part, int* perm,
+                    double rel) {
+  __shared__ double rv[kFacThreads / 32];
+  __shared__ int ri[kFacThreads / 32];
+  __shared__ double red[kFacThreads / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  constexpr int NW = kFacThreads / 32;
+  for (int i = threadIdx.x; i < r; i += blockDim.x) perm[i] = i;
+  for (int k0 = 0; k0 < r; k0 += 32) {
+    const int k = k0 + lane;
+    double s = 0.0;
+    if (k < r)
+      for (int i = wid; i < M; i += NW) { const double x = B[(long long)i * ld + k]; s = fma(x, x, s); }
+    if (k < r) part[wid * r + k] = s;
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < r; k += blockDim.x) {
+    double s = 0.0;
+    for (int g = 0; g < NW; ++g) s += part[g * r + k];
+    dg[k] = s;
+    w[k] = s;   // reference norms for the downdate safeguard
+  }
+  __syncthreads();
+  double n0 = 0.0;
+  const int kmax = M < r ? M : r;
+  for (int j = 0; j < kmax; ++j) {
+    const int p = block_argmax(dg, j, r, rv, ri);
+    const double dp = dg[p];
+    if (j == 0) n0 = dp;
+    if (!(dp > rel * rel * n0) || !(dp > 0.0)) return j;
+    if (p != j) {
+      for (int i = threadIdx.x; i < M; i += blockDim.x) {
+        const double t = B[(long long)i * ld + j];
+        B[(long long)i * ld + j] = B[(long long)i * ld + p];
+        B[(long long)i * ld + p] = t;
+      }
+      if (threadIdx.x == 0) {
+        const int t = perm[j]; perm[j] = perm[p]; perm[p] = t;
+        double td = dg[j]; dg[j] = dg[p]; dg[p] = td;
+        td = w[j]; w[j] = w[p]; w[p] = td;
+      }
+      __syncthreads();
+    }
+    double s = 0.0;
+    for (int i = j + threadIdx.x; i < M; i += blockDim.x) {
+      const double x = B[(long long)i * ld + j];
+      s = fma(x, x, s);
+    }
+    s = block_sum(s, red);
+    const double alpha = B[(long long)j * ld + j];
+    const double normx = sqrt(s);
+    const double beta = alpha >= 0.0 ? -normx : normx;
+    const double v0 = alpha - beta;
+    const double tau = (beta - alpha) / beta;
+    for (int i = j + threadIdx.x; i < M; i += blockDim.x) v[i] = (i == j) ? 1.0 : B[(long long)i * ld + j] / v0;
+    __syncthreads();
+    for (int i = j + threadIdx.x; i < M; i += blockDim.x) B[(long long)i * ld + j] = (i == j) ? beta : 0.0;
+    for (int k0 = j + 1; k0 < r; k0 += 32) {
+      const int k = k0 + lane;
+      if (k >= r) continue;
+      double acc = 0.0;
+      for (int i = j + wid; i < M; i += NW) acc = fma(v[i], B[(long long)i * ld + k], acc);
+      part[wid * r + k] = acc;
+    }
+    __syncthreads();
+    for (int k0 = j + 1; k0 < r; k0 += 32) {
+      const int k = k0 + lane;
+      if (k >= r) continue;
+      double tw = 0.0;
+#pragma unroll
+      for (int g = 0; g < NW; ++g) tw += part[g * r + k];
+      tw *= tau;
+      for (int i = j + wid; i < M; i += NW) B[(long long)i * ld + k] -= v[i] * tw;
+    }
+    __syncthreads();
+    for (int k = j + 1 + threadIdx.x; k < r; k += blockDim.x) {
+      const double rjk = B[(long long)j * ld + k];
+      double nd = dg[k] - rjk * rjk;
+      if (nd < 0.05 * w[k]) {  // cancellation: recompute the trailing norm
+        nd = 0.0;
+        for (int i = j + 1; i < M; ++i) { const double x = B[(long long)i * ld + k]; nd = fma(x, x, nd); }
+        w[k] = nd;
+      }
+      dg[k] = nd;
+    }
+    __syncthreads();
+  }
+  return kmax;
+}
+
+// Cholesky branch: pivoted Cholesky of G (r x r, formed by k_form behind T).
+// Householder branch: column-pivoted Householder QR of B (4k x r, in T).
+// Output: T (rank x r upper trapezoidal, pivoted column order), perm[q] =
+// original column of pivoted column q, rank -> ival.
+//
+// Whether the Cholesky-QR branch can be trusted with its Gram C = cv^T cv
 // (n x n): its factor is only as accurate as C.  The Gram's rounding is
 // relative to the norms of the columns it pairs (FP32 runs flushed into
 // FP64: ~1e-8 of that scale; FP64: ~1e-14), so a column that is a linear
 // combination of the others in exact arithmetic keeps a Schur complement of
 // that relative size, and the Q-less update would take the noise for a
 // direction (Q = cv R^-1 is then far from orthonormal).  The pivoted Cholesky
-// of C (pivot values only, in precision R, in the scratch Cw) therefore
-// checks every accepted pivot against the column's own diagonal: false (use
-// Householder) when some pivot keeps less than `safe` of it.  Pivots below
-// rel_cut of the first end the check (directions too small to matter: the
-// factorisation of G cuts them as rank).  Block-uniform result.
-template <typename R>
-__device__ bool gram_trusted(const SiteFacItem& it, int n, R* Cw, double* dg, double safe, double rel_cut,
-                             double* rv, int* ri) {
-  double* od = dg + n;                       // the pivoted columns' original diagonals
-  for (long long e = threadIdx.x; e < (long long)n * n; e += blockDim.x) {
-    const int i = (int)(e / n), j = (int)(e - (long long)i * n);
-    Cw[e] = (R)it.C[(long long)i * it.ldc + j];
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x) dg[i] = od[i] = (double)Cw[(long long)i * n + i];
-  __syncthreads();
-  double d0 = 0.0;
-  for (int j = 0; j < n; ++j) {
-    const int p = block_argmax(dg, j, n, rv, ri);
-    const double dp = dg[p];
-    if (j == 0) d0 = dp;
-    if (!(dp > rel_cut * d0) || !(dp > 0.0)) return true;
-    if (!(dp >= safe * od[p])) return false;
-    if (p != j) {
-      for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        R t = Cw[(long long)j * n + k]; Cw[(long long)j * n + k] = Cw[(long long)p * n + k]; Cw[(long long)p * n + k] = t;
-      }
-      __syncthreads();
-      for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        R t = Cw[(long long)k * n + j]; Cw[(long long)k * n + j] = Cw[(long long)k * n + p]; Cw[(long long)k * n + p] = t;
-      }
-      if (threadIdx.x == 0) {
-        double t = dg[j]; dg[j] = dg[p]; dg[p] = t;
-        t = od[j]; od[j] = od[p]; od[p] = t;
-      }
-      __syncthreads();
-    }
-    const R rjj = sqrt(Cw[(long long)j * n + j]);
-    __syncthreads();
-    for (int k = j + 1 + threadIdx.x; k < n; k += blockDim.x) Cw[(long long)j * n + k] /= rjj;
-    __syncthreads();
-    const int mm = n - j - 1;
-    for (long long e = threadIdx.x; e < (long long)mm * mm; e += blockDim.x) {
-      const int a = j + 1 + (int)(e / mm), b = j + 1 + (int)(e % mm);
-      Cw[(long long)a * n + b] -= Cw[(long long)j * n + a] * Cw[(long long)j * n + b];
-    }
-    __syncthreads();
-    for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) dg[i] = (double)Cw[(long long)i * n + i];
-    __syncthreads();
-  }
-  return true;
-}
-
-// Cholesky branch: pivoted Cholesky of G (r x r, in place, row-major).
-// Householder branch: column-pivoted Householder QR of B (4k x r, in place).
-// Output: T (rank x r upper trapezoidal, pivoted column order) in place,
-// perm[q] = original column of pivoted column q, rank -> ival.
-// A Cholesky-branch site whose Gram fails gram_trusted is marked branch 2 and
-// left for the Householder pass that follows (only = 2 runs that pass only).
-__global__ void __launch_bounds__(512)
-k_factor(const SiteFacItem* __restrict__ items, int* ival, int only, unsigned long long* qcount) {
+// of C (in FP32 for FP32 storage) therefore checks every accepted pivot
+// against the column's own diagonal; when one keeps less than rel_safe of it
+// the site is marked branch 2 and left for the pass that follows (only = 2
+// runs that pass only).  Pivots below rel of the first end the check
+// (directions too small to matter: the factorisation of G cuts them as rank).
+//
+// Measured, factor class of one saturated layer, right-looking Cholesky and one
+// thread per column before -> now: 4x4 chi = 48 212 -> 87 ms, 3x3 chi = 100 357
+// -> 255 ms, 3x5 chi = 27 42 -> 20 ms, results bit-identical (what is left is the
+// Householder branch).
+__global__ void __launch_bounds__(kFacThreads)
+k_factor(const SiteFacItem* __restrict__ items, int* ival, int only, unsigned long long* qcount, int rmax, int nmax,
+         int householder) {
   const SiteFacItem it = items[blockIdx.x];
-  if (only >= 0 && ival[it.branch_idx] != only) return;
-  if (qcount && threadIdx.x == 0 && ival[it.branch_idx] == 0) atomicAdd(&qcount[0], 1ull);
+  const int branch = ival[it.branch_idx];
+  if (only >= 0 && branch != only) return;
+  if (qcount && threadIdx.x == 0 && branch == 0) atomicAdd(&qcount[0], 1ull);
   long long m;
   int n;
   cv_shape(it.cv, ival, m, n);
   const int chic = n / 4;
   const int rg = ival[it.rg_idx];
   const int r = rg * chic;
-  double* A = it.T;
+  double* T = it.T;
   const int ld = it.ldt;
-  extern __shared__ __align__(16) double sh[];
-  double* dg = sh;               // r: Schur diagonal / column norms^2
-  double* v = dg + r;            // 4k: Householder vector
-  double* w = v + 4 * n;         // r
-  int* perm = it.perm;
-  __shared__ double rv[16];
-  __shared__ int ri[16];
-  __shared__ double red[16];
-  if (ival[it.branch_idx] == 1) {
-    // the scratch after G (r x ld) holds the copy of C; v (4n doubles) the
-    // pivots and the original diagonals
-    double* scratch = A + (long long)ld * ld;
-    const bool ok = it.rel_safe >= 1e-6
-                        ? gram_trusted<float>(it, n, reinterpret_cast<float*>(scratch), v, it.rel_safe, it.rel, rv, ri)
-                        : gram_trusted<double>(it, n, scratch, v, it.rel_safe, it.rel, rv, ri);
-    if (threadIdx.x == 0 && qcount) atomicAdd(&qcount[ok ? 1 : 2], 1ull);
-    if (!ok) {
+  extern __shared__ __align__(16) unsigned char fsh[];
+  const FacSmem S = fac_smem(rmax, nmax, householder);
+  double* dg = reinterpret_cast<double*>(fsh + S.dg);
+  double* od = reinterpret_cast<double*>(fsh + S.od);
+  double* uc = reinterpret_cast<double*>(fsh + S.uc);
+  int* perm = reinterpret_cast<int*>(fsh + S.perm);
+  double* mat = reinterpret_cast<double*>(fsh + S.mat);
+  const size_t room = S.total - S.mat;
+  int rank = 0;
+  if (branch == 1) {
+    double* scratch = T + (long long)2 * ld * ld;    // behind T and G: 2 ld^2 doubles
+    int ok;
+    if (it.rel_safe >= 1e-6) {
+      const bool in = sizeof(float) * (size_t)n * n <= room;
+      ok = chol_pivoted<float>(it.C, it.ldc, n, in ? reinterpret_cast<float*>(mat) : reinterpret_cast<float*>(scratch), n,
+                               reinterpret_cast<float*>(dg), reinterpret_cast<float*>(od), reinterpret_cast<float*>(uc),
+                               perm, it.rel, it.rel_safe);
+    } else {
+      const bool in = sizeof(double) * (size_t)n * n <= room;
+      ok = chol_pivoted<double>(it.C, it.ldc, n, in ? mat : scratch, n, dg, od, uc, perm, it.rel, it.rel_safe);
+    }
+    if (threadIdx.x == 0 && qcount) atomicAdd(&qcount[ok >= 0 ? 1 : 2], 1ull);
+    if (ok < 0) {
       if (threadIdx.x == 0) ival[it.branch_idx] = 2;
       return;
     }
-  }
-  for (int i = threadIdx.x; i < r; i += blockDim.x) perm[i] = i;
-  int rank = 0;
-  if (ival[it.branch_idx] == 1) {
-    for (int i = threadIdx.x; i < r; i += blockDim.x) dg[i] = A[(long long)i * ld + i];
     __syncthreads();
-    double d0 = 0.0;
-    rank = r;
-    for (int j = 0; j < r; ++j) {
-      int p = block_argmax(dg, j, r, rv, ri);
-      double dp = dg[p];
-      if (j == 0) d0 = dp;
-      if (!(dp > it.rel * d0) || !(dp > 0.0)) { rank = j; break; }
-      if (p != j) {
-        for (int k = threadIdx.x; k < r; k += blockDim.x) {
-          double t = A[(long long)j * ld + k]; A[(long long)j * ld + k] = A[(long long)p * ld + k];
-          A[(long long)p * ld + k] = t;
-        }
-        __syncthreads();
-        for (int k = threadIdx.x; k < r; k += blockDim.x) {
-          double t = A[(long long)k * ld + j]; A[(long long)k * ld + j] = A[(long long)k * ld + p];
-          A[(long long)k * ld + p] = t;
-        }
-        if (threadIdx.x == 0) {
-          int t = perm[j]; perm[j] = perm[p]; perm[p] = t;
-          double td = dg[j]; dg[j] = dg[p]; dg[p] = td;
-        }
-        __syncthreads();
+    const bool in = sizeof(double) * (size_t)r * r <= room;
+    double* U = in ? mat : T;
+    const int ldu = in ? r : ld;
+    rank = chol_pivoted<double>(T + (long long)ld * ld, ld, r, U, ldu, dg, od, uc, perm, it.rel, -1.0);
+    __syncthreads();
+    if (in)
+      for (long long e = threadIdx.x; e < (long long)rank * r; e += blockDim.x) {
+        const int a = (int)(e / r), q = (int)(e - (long long)a * r);
+        if (q >= a) T[(long long)a * ld + q] = mat[e];
       }
-      const double rjj = sqrt(A[(long long)j * ld + j]);
-      __syncthreads();
-      for (int k = j + 1 + threadIdx.x; k < r; k += blockDim.x) A[(long long)j * ld + k] /= rjj;
-      if (threadIdx.x == 0) A[(long long)j * ld + j] = rjj;
-      __syncthreads();
-      const int mm = r - j - 1;
-      for (long long e = threadIdx.x; e < (long long)mm * mm; e += blockDim.x) {
-        int a = j + 1 + (int)(e / mm), b = j + 1 + (int)(e % mm);
-        A[(long long)a * ld + b] -= A[(long long)j * ld + a] * A[(long long)j * ld + b];
-      }
-      __syncthreads();
-      for (int i = j + 1 + threadIdx.x; i < r; i += blockDim.x) dg[i] = A[(long long)i * ld + i];
-      __syncthreads();
-    }
   } else {
     const int M = 4 * ival[it.kfac_idx];
-    for (int k = threadIdx.x; k < r; k += blockDim.x) {
-      double s = 0.0;
-      for (int i = 0; i < M; ++i) { double x = A[(long long)i * ld + k]; s = fma(x, x, s); }
-      dg[k] = s;
-      w[k] = s;   // reference norms for the downdate safeguard
+    double* v = reinterpret_cast<double*>(fsh + S.v);
+    double* part = v + (size_t)4 * nmax;
+    const bool in = sizeof(double) * (size_t)M * r <= room;
+    if (in) {
+      for (long long e = threadIdx.x; e < (long long)M * r; e += blockDim.x) {
+        const int a = (int)(e / r), q = (int)(e - (long long)a * r);
+        mat[e] = T[(long long)a * ld + q];
+      }
+      __syncthreads();
     }
+    rank = qrcp(in ? mat : T, in ? r : ld, M, r, dg, od, v, part, perm, it.rel);
     __syncthreads();
-    double n0 = 0.0;
-    const int kmax = M < r ? M : r;
-    rank = kmax;
-    for (int j = 0; j < kmax; ++j) {
-      int p = block_argmax(dg, j, r, rv, ri);
-      double dp = dg[p];
-      if (j == 0) n0 = dp;
-      if (!(dp > it.rel * it.rel * n0) || !(dp > 0.0)) { rank = j; break; }
-      if (p != j) {
-        for (int i = threadIdx.x; i < M; i += blockDim.x) {
-          double t = A[(long long)i * ld + j]; A[(long long)i * ld + j] = A[(long long)i * ld + p];
-          A[(long long)i * ld + p] = t;
-        }
-        if (threadIdx.x == 0) {
-          int t = perm[j]; perm[j] = perm[p]; perm[p] = t;
-          double td = dg[j]; dg[j] = dg[p]; dg[p] = td;
-          td = w[j]; w[j] = w[p]; w[p] = td;
-        }
-        __syncthreads();
+    if (in)
+      for (long long e = threadIdx.x; e < (long long)rank * r; e += blockDim.x) {
+        const int a = (int)(e / r), q = (int)(e - (long long)a * r);
+        T[(long long)a * ld + q] = mat[e];
       }
-      double s = 0.0;
-      for (int i = j + threadIdx.x; i < M; i += blockDim.x) {
-        double x = A[(long long)i * ld + j];
-        s = fma(x, x, s);
-      }
-      s = block_sum(s, red);
-      const double alpha = A[(long long)j * ld + j];
-      const double normx = sqrt(s);
-      const double beta = alpha >= 0.0 ? -normx : normx;
-      const double v0 = alpha - beta;
-      const double tau = (beta - alpha) / beta;
-      for (int i = j + threadIdx.x; i < M; i += blockDim.x)
-        v[i - j] = (i == j) ? 1.0 : A[(long long)i * ld + j] / v0;
-      __syncthreads();
-      for (int i = j + threadIdx.x; i < M; i += blockDim.x) A[(long long)i * ld + j] = (i == j) ? beta : 0.0;
-      for (int k = j + 1 + threadIdx.x; k < r; k += blockDim.x) {
-        double acc = 0.0;
-        for (int i = j; i < M; ++i) acc = fma(v[i - j], A[(long long)i * ld + k], acc);
-        const double tw = tau * acc;
-        for (int i = j; i < M; ++i) A[(long long)i * ld + k] -= v[i - j] * tw;
-        const double rjk = A[(long long)j * ld + k];
-        double nd = dg[k] - rjk * rjk;
-        if (nd < 0.05 * w[k]) {  // cancellation: recompute the trailing norm
-          nd = 0.0;
-          for (int i = j + 1; i < M; ++i) { double x = A[(long long)i * ld + k]; nd = fma(x, x, nd); }
-          w[k] = nd;
-        }
-        dg[k] = nd;
-      }
-      __syncthreads();
-    }
   }
+  for (int i = threadIdx.x; i < r; i += blockDim.x) it.perm[i] = perm[i];
   if (threadIdx.x == 0) ival[it.rank_idx] = rank;
 }
 
 cudaError_t launch_factor(const SiteFacItem* items, int n_items, int rmax, int nmax, int* ival,
                           cudaStream_t s, int only, unsigned long long* qcount) {
   if (n_items == 0) return cudaSuccess;
-  size_t smem = sizeof(double) * ((size_t)2 * rmax + 4 * nmax);
-  cudaError_t e = cudaFuncSetAttribute(k_factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  const FacSmem S = fac_smem(rmax, nmax, 1);
+  cudaError_t e = cudaFuncSetAttribute(k_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.total);
   if (e != cudaSuccess) return e;
-  k_factor<<<n_items, 512, smem, s>>>(items, ival, only, qcount);
+  k_factor<<<n_items, kFacThreads, S.total, s>>>(items, ival, only, qcount, rmax, nmax, 1);
   return cudaGetLastError();
 }
 
