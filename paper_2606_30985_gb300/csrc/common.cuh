@@ -54,6 +54,7 @@ struct GramRowsItem {
   double* partial;         // [splits][Fmax * Fmax]
   double* out;             // F x F, leading dimension ldo
   int ldo;
+  unsigned* colmax;        // Fmax: largest magnitude per column (float bits; exact Gram)
 };
 
 // Free-leg contraction: out[i, i'] = sum_{o,q} X[o, i, q] Y[o, i', q], free leg

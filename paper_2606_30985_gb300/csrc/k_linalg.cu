@@ -6,10 +6,10 @@
 //                  Gram, so no eigensolver is needed.
 //   k_branch       Eq. 10 branch rule: Cholesky-QR when n > n_thr and
 //                  m / n > ratio_thr, Householder otherwise (Sec. 4.2).
-//   k_hh_level     Householder QR (TSQR tree, R only) of cv in its storage
-//                  precision with FP64 reductions (Sec. 4.2 Householder-QR);
-//                  each tree block factored in panels (compact WY).
-//   k_formG / k_formB   fold the gate's operator-Schmidt factors into the
+//   k_hh_level     FP64 storage: Householder QR (TSQR tree, R only) of cv
+//                  (Sec. 4.2 Householder-QR); each tree block factored in panels
+//                  (compact WY).
+//   k_form         fold the gate's operator-Schmidt factors into the
 //                  R-factor: X = (F_kappa (x) 1) cv, G = X^T X or B = R-side of X.
 //   k_factor       rank-revealing factor T of X: pivoted Cholesky of G
 //                  (Cholesky-QR branch) or column-pivoted Householder of B.
@@ -173,9 +173,7 @@ __host__ __device__ inline long long hh_leaf_rows(int n) { return n * 4 > 256 ? 
 constexpr int kHhThreads = 512;   // threads of a TSQR block
 
 // Panel width of the blocked QR: the panel (L x NB) lives in shared memory.
-template <typename T> struct HhPanel;
-template <> struct HhPanel<float> { static constexpr int NB = 16; };
-template <> struct HhPanel<double> { static constexpr int NB = 8; };
+constexpr int kHhPanel = 8;
 
 // Shared-memory plan of one TSQR block (leaf rows L): panel V (column-major,
 // leading dimension L + 1 so that consecutive rows of a column and the rows
@@ -188,7 +186,7 @@ struct HhSmem {
 };
 template <typename T>
 __host__ __device__ inline HhSmem hh_smem(long long L) {
-  constexpr int NB = HhPanel<T>::NB;
+  constexpr int NB = kHhPanel;
   HhSmem m;
   m.lp = (int)L + 1;
   size_t o = 0;
@@ -206,13 +204,6 @@ __host__ __device__ inline HhSmem hh_smem(long long L) {
   return m;
 }
 
-__device__ inline void ld4(const float* p, float (&x)[4]) {
-  const float4 v = *reinterpret_cast<const float4*>(p);
-  x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
-}
-__device__ inline void st4(float* p, const float (&x)[4]) {
-  *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
-}
 __device__ inline void ld4(const double* p, double (&x)[4]) {
   const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
   x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
@@ -227,12 +218,11 @@ __device__ inline void st4(double* p, const double (&x)[4]) {
 // Blocked by panels of NB columns in the compact WY form H_1 ... H_nb =
 // I - V T V^T: the panel is factored in shared memory, then the trailing
 // columns take all nb reflections in one pass, A <- A - V (T^T (V^T A)),
-// instead of one pass per reflection.  Arithmetic in T's precision (FP32
-// storage: FP32 reflections, backward stable to the data's own precision),
-// norms, cross-warp sums and the T factor in FP64.  512 threads.
+// instead of one pass per reflection.  512 threads.  FP64 storage only: FP32
+// storage factors the exact Gram of its data instead (k_gram_exact).
 template <typename T>
 __device__ void hh_block_qr(T* A, long long rows, int n, unsigned char* smem, const HhSmem& S) {
-  constexpr int NB = HhPanel<T>::NB;
+  constexpr int NB = kHhPanel;
   T* P = reinterpret_cast<T*>(smem + S.p);
   T* red = reinterpret_cast<T*>(smem + S.red);
   double* Wd = reinterpret_cast<double*>(smem + S.wd);
@@ -519,9 +509,9 @@ cudaError_t launch_hh_extract(const SiteFacItem* items, int n_items, void* const
 }
 
 // ============================================================ formG / formB
-// Cholesky branch: G[(c,k),(c',k')] = sum_{p,q} (F_k^T F_k')[p,q] C[(c,p),(c',q)].
-// Householder branch: B[(a,p'),(c,k)] = sum_p F_k[p',p] R[a,(c,p)].
-__global__ void k_form(const SiteFacItem* __restrict__ items, const int* ival, int only) {
+// From a Gram: G[(c,k),(c',k')] = sum_{p,q} (F_k^T F_k')[p,q] C[(c,p),(c',q)].
+// From a Householder R: B[(a,p'),(c,k)] = sum_p F_k[p',p] R[a,(c,p)].
+__global__ void k_form(const SiteFacItem* __restrict__ items, const int* ival, int only, int householder) {
   const SiteFacItem it = items[blockIdx.y];
   if (only >= 0 && ival[it.branch_idx] != only) return;
   long long m;
@@ -534,7 +524,7 @@ __global__ void k_form(const SiteFacItem* __restrict__ items, const int* ival, i
   __shared__ double H[PEPO_RG * PEPO_RG * 16];
   for (int e = threadIdx.x; e < rg * 16; e += blockDim.x) F[e] = it.F[e];
   __syncthreads();
-  if (ival[it.branch_idx] == 1) {
+  if (ival[it.branch_idx] == 1 || !householder) {
     for (int e = threadIdx.x; e < rg * rg * 16; e += blockDim.x) {
       int k = e / (rg * 16), rest = e % (rg * 16);
       int k2 = rest / 16, pq = rest % 16, p = pq / 4, q = pq % 4;
@@ -576,9 +566,9 @@ __global__ void k_form(const SiteFacItem* __restrict__ items, const int* ival, i
 }
 
 cudaError_t launch_form(const SiteFacItem* items, int n_items, int grid_x, const int* ival,
-                        cudaStream_t s, int only) {
+                        cudaStream_t s, int only, int householder) {
   if (n_items == 0) return cudaSuccess;
-  k_form<<<dim3(grid_x, n_items), 256, 0, s>>>(items, ival, only);
+  k_form<<<dim3(grid_x, n_items), 256, 0, s>>>(items, ival, only, householder);
   return cudaGetLastError();
 }
 
@@ -798,8 +788,9 @@ __device__ int qrcp(double* B, int ld, int M, int r, double* dg, double* w, doub
   return kmax;
 }
 
-// Cholesky branch: pivoted Cholesky of G (r x r, formed by k_form behind T).
-// Householder branch: column-pivoted Householder QR of B (4k x r, in T).
+// From a Gram (the Cholesky-QR branch; FP32 storage: every site): pivoted
+// Cholesky of G (r x r, formed by k_form behind T).
+// From a Householder R (FP64 storage): column-pivoted Householder QR of B (4k x r, in T).
 // Output: T (rank x r upper trapezoidal, pivoted column order), perm[q] =
 // original column of pivoted column q, rank -> ival.
 //
@@ -862,6 +853,8 @@ k_factor(const SiteFacItem* __restrict__ items, int* ival, int only, unsigned lo
       return;
     }
     __syncthreads();
+  }
+  if (branch == 1 || !householder) {
     const bool in = sizeof(double) * (size_t)r * r <= room;
     double* U = in ? mat : T;
     const int ldu = in ? r : ld;
@@ -897,12 +890,12 @@ k_factor(const SiteFacItem* __restrict__ items, int* ival, int only, unsigned lo
 }
 
 cudaError_t launch_factor(const SiteFacItem* items, int n_items, int rmax, int nmax, int* ival,
-                          cudaStream_t s, int only, unsigned long long* qcount) {
+                          cudaStream_t s, int only, int householder, unsigned long long* qcount) {
   if (n_items == 0) return cudaSuccess;
-  const FacSmem S = fac_smem(rmax, nmax, 1);
+  const FacSmem S = fac_smem(rmax, nmax, householder);
   cudaError_t e = cudaFuncSetAttribute(k_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.total);
   if (e != cudaSuccess) return e;
-  k_factor<<<n_items, kFacThreads, S.total, s>>>(items, ival, only, qcount, rmax, nmax, 1);
+  k_factor<<<n_items, kFacThreads, S.total, s>>>(items, ival, only, qcount, rmax, nmax, householder);
   return cudaGetLastError();
 }
 
@@ -1322,12 +1315,8 @@ cudaError_t launch_core(const CoreItem* items, int n_items, int* ival, int* flag
   return cudaGetLastError();
 }
 
-template cudaError_t launch_hh_level<float>(const SiteFacItem*, int, int, int, int, void* const*,
-                                            const int*, cudaStream_t, int);
 template cudaError_t launch_hh_level<double>(const SiteFacItem*, int, int, int, int, void* const*,
                                              const int*, cudaStream_t, int);
-template cudaError_t launch_hh_extract<float>(const SiteFacItem*, int, void* const*, int*,
-                                              cudaStream_t, int, double*);
 template cudaError_t launch_hh_extract<double>(const SiteFacItem*, int, void* const*, int*,
                                                cudaStream_t, int, double*);
 

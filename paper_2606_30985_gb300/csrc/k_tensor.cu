@@ -186,6 +186,260 @@ cudaError_t launch_gram_rows_reduce(const GramRowsItem* items, int n_items, int 
 }
 
 
+// ======================================================= exact Gram (rows)
+// C = cv^T cv of FP32 data to about 47 bits, for the sites the branch rule of
+// Eq. 10 sends to Householder and for those whose FP32-run Gram failed the
+// trust test.  A pivoted Cholesky of this C is as good a factor of cv as a
+// Householder QR in FP32: QR perturbs a column by ~6e-8 of its norm, this
+// Gram's ~1e-14 moves a direction that keeps a share e of it by 1e-14 / e,
+// which is smaller for every direction the rank cut leaves (e > 3e-7).
+//
+// Sum: an accumulator s starts at the anchor 3 P_i P_j, P the next power of two
+// above the run's column norm, so by Cauchy-Schwarz s stays in one binade and
+// every addition rounds to the same grid: with s' = fma(a, b, s), h = s' - s is
+// exact and fma(a, b, -h) is what the rounding left over.  Four FP32
+// operations a term instead of one FP64 multiply-add, which takes 64 issue
+// slots here; a double-float sum takes ten.  Runs of 64 rows go into a
+// two-float sum (S, C), the splits into FP64.  Columns are scaled to a largest
+// magnitude in [1/2, 1) first (k_col_scale), so tiny tensors do not underflow.
+//
+// 64 x 64 tiles, 4 x 4 entries a thread (64 FP32 operations per two 16-byte
+// shared loads: ALU-bound), 16-byte asynchronous copies one run ahead.
+// K splits: rows per split ~512, at most kExactSplits.
+constexpr int GX_T = 64;
+constexpr int GX_RUN = 64;
+constexpr int kExactSplits = 60;
+
+__device__ inline float pow2f(int e) { return __int_as_float((min(max(e, -126), 127) + 127) << 23); }
+
+// largest magnitude per column -> colmax (float bits, zeroed by the caller)
+__global__ void __launch_bounds__(256)
+k_col_scale(const GramRowsItem* __restrict__ items, int pass, int step, void* const* ptrs, const int* __restrict__ ival) {
+  const GramRowsItem it = items[blockIdx.y];
+  if (ival[it.active] != pass) return;
+  int d[PEPO_MAXLEG];
+  load_dims(it.x, ival, d);
+  const int nl = it.x.nlegs;
+  const int quads = nl > 0 ? d[nl - 1] : 1;            // F / 4
+  const int F = 4 * quads;
+  unsigned* cm = it.colmax;
+  if (step == 0) {
+    for (int c = threadIdx.x; c < F; c += blockDim.x) cm[c] = 0u;
+    return;
+  }
+  long long K = 1;
+  for (int i = 0; i + 1 < nl; ++i) K *= d[i];
+  __shared__ unsigned sm[4 * 128];
+  for (int c = threadIdx.x; c < F; c += blockDim.x) sm[c] = 0u;
+  __syncthreads();
+  const int rpb = 256 / quads;
+  const int rr = threadIdx.x / quads, qd = threadIdx.x - rr * quads;
+  if (rr < rpb) {
+    const float* X = static_cast<const float*>(ptrs[it.x.ref]);
+    unsigned m[4] = {0u, 0u, 0u, 0u};
+    for (long long r = (long long)blockIdx.x * rpb + rr; r < K; r += (long long)gridDim.x * rpb) {
+      const float4 v = *reinterpret_cast<const float4*>(X + r * F + 4 * qd);
+      m[0] = max(m[0], __float_as_uint(fabsf(v.x)));
+      m[1] = max(m[1], __float_as_uint(fabsf(v.y)));
+      m[2] = max(m[2], __float_as_uint(fabsf(v.z)));
+      m[3] = max(m[3], __float_as_uint(fabsf(v.w)));
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (m[i]) atomicMax(&sm[4 * qd + i], m[i]);
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < F; c += blockDim.x)
+    if (sm[c]) atomicMax(&cm[c], sm[c]);
+}
+
+// exponent e with the column's largest magnitude in [2^(e-1), 2^e)
+__device__ inline int col_exp(unsigned bits) { return (int)(bits >> 23) - 126; }
+
+__device__ inline void gx_copy16(void* dst, const void* src, bool live) {
+  const int n = live ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(n)
+               : "memory");
+}
+
+__global__ void __launch_bounds__(256, 2)
+k_gram_exact(const GramRowsItem* __restrict__ items, int pass, void* const* ptrs, const int* __restrict__ ival) {
+  const GramRowsItem it = items[blockIdx.z];
+  if (ival[it.active] != pass) return;
+  int d[PEPO_MAXLEG];
+  load_dims(it.x, ival, d);
+  const int nl = it.x.nlegs;
+  const int F = 4 * (nl > 0 ? d[nl - 1] : 1);
+  long long K = 1;
+  for (int i = 0; i + 1 < nl; ++i) K *= d[i];
+  const int S = gram_rows_splits(K, kExactSplits);
+  const int sp = blockIdx.x % kExactSplits;
+  const int nt = ceil_div(F, GX_T);
+  if (sp >= S || (int)(blockIdx.x / kExactSplits) >= nt * (nt + 1) / 2) return;
+  int ti, tj;
+  tile_of(blockIdx.x / kExactSplits, nt, 1, ti, tj);
+  const bool diag = ti == tj;
+  const long long k0 = K * sp / S, k1 = K * (sp + 1) / S;
+  const float* __restrict__ X = static_cast<const float*>(ptrs[it.x.ref]);
+  extern __shared__ __align__(16) float gx_sh[];      // 2 buffers of [X tile | Y tile], 64 rows x 64 columns each
+  __shared__ float nrm[2][2 * GX_T];                   // half sums of squares per column
+  __shared__ float pw[2 * GX_T];                       // P per column
+  __shared__ float sc[2 * GX_T];                       // column pre-scale 2^-e
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  if (tid < 2 * GX_T) {
+    const int c = (tid < GX_T ? ti : tj) * GX_T + (tid & (GX_T - 1));
+    sc[tid] = c < F ? pow2f(-col_exp(it.colmax[c])) : 0.f;
+  }
+  auto load = [&](int buf, long long kb) {
+    float* xs = gx_sh + buf * (2 * GX_RUN * GX_T);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = tid + 256 * u;                     // 64 rows x 16 quads
+      const int row = e >> 4, qd = e & 15;
+      const long long k = kb + row;
+      const int ci = ti * GX_T + 4 * qd, cj = tj * GX_T + 4 * qd;
+      const bool okk = k < k1;
+      gx_copy16(xs + row * GX_T + 4 * qd, okk && ci < F ? X + k * F + ci : X, okk && ci < F);
+      if (!diag) gx_copy16(xs + (GX_RUN + row) * GX_T + 4 * qd, okk && cj < F ? X + k * F + cj : X, okk && cj < F);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float Sh[4][4], Cl[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) Sh[a][b] = Cl[a][b] = 0.f;
+  load(0, k0);
+  int buf = 0;
+  for (long long kb = k0; kb < k1; kb += GX_RUN, buf ^= 1) {
+    if (kb + GX_RUN < k1) {
+      load(buf ^ 1, kb + GX_RUN);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    float* xs = gx_sh + buf * (2 * GX_RUN * GX_T);
+    float* ys = diag ? xs : xs + GX_RUN * GX_T;
+    {   // scale the columns in place and sum their squares, half a column a thread
+      const int c = tid & (GX_T - 1), half = (tid >> 6) & 1, isy = tid >> 7;
+      if (!(isy && diag)) {
+        float* col = (isy ? ys : xs) + c + half * (GX_RUN / 2) * GX_T;
+        const float f = sc[isy * GX_T + c];
+        float q = 0.f;
+#pragma unroll 8
+        for (int i = 0; i < GX_RUN / 2; ++i) {
+          const float x = col[i * GX_T] * f;
+          col[i * GX_T] = x;
+          q = fmaf(x, x, q);
+        }
+        nrm[half][isy * GX_T + c] = q;
+      }
+    }
+    __syncthreads();
+    if (tid < 2 * GX_T) {
+      const int c = diag ? (tid & (GX_T - 1)) : tid;
+      const float q = (nrm[0][c] + nrm[1][c]) * 1.01f;
+      const int e = (int)(__float_as_uint(q) >> 23) - 127;     // q < 2^(e + 1)
+      pw[tid] = pow2f(max((e + 2) >> 1, -50));                 // P^2 > q
+    }
+    __syncthreads();
+    float P[4], Q[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) { P[a] = pw[ty * 4 + a]; Q[a] = pw[GX_T + tx * 4 + a]; }
+    float s[4][4], c[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) { s[a][b] = 3.f * (P[a] * Q[b]); c[a][b] = 0.f; }
+#pragma unroll 8
+    for (int kk = 0; kk < GX_RUN; ++kk) {
+      const float4 xa = *reinterpret_cast<const float4*>(xs + kk * GX_T + ty * 4);
+      const float4 yb = *reinterpret_cast<const float4*>(ys + kk * GX_T + tx * 4);
+      const float a4[4] = {xa.x, xa.y, xa.z, xa.w}, b4[4] = {yb.x, yb.y, yb.z, yb.w};
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const float t = fmaf(a4[a], b4[b], s[a][b]);
+          const float h = t - s[a][b];
+          c[a][b] += fmaf(a4[a], b4[b], -h);
+          s[a][b] = t;
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const float v = s[a][b] - 3.f * (P[a] * Q[b]);          // exact
+        const float t = Sh[a][b] + v, bb = t - Sh[a][b];
+        Cl[a][b] += ((Sh[a][b] - (t - bb)) + (v - bb)) + c[a][b];
+        Sh[a][b] = t;
+      }
+    __syncthreads();                                           // the buffer is refilled next
+  }
+  double* Pt = it.partial + (long long)sp * F * F;
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const int fi = ti * GX_T + ty * 4 + a;
+    if (fi >= F) continue;
+    const int ei = col_exp(it.colmax[fi]);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int fj = tj * GX_T + tx * 4 + b;
+      if (fj < F) {
+        const double v = (double)Sh[a][b] + (double)Cl[a][b];
+        Pt[(long long)fi * F + fj] = scalbn(v, ei + col_exp(it.colmax[fj]));
+      }
+    }
+  }
+}
+
+// Sum of the splits, mirrored into the lower triangle; acct (2 doubles, may be
+// null) accumulates the FLOPs (one multiply-add per entry of the triangle and
+// row) and bytes (one read of the matrix), which only the device knows.
+__global__ void k_gram_exact_reduce(const GramRowsItem* __restrict__ items, int pass, const int* __restrict__ ival,
+                                    double* acct) {
+  const GramRowsItem it = items[blockIdx.y];
+  if (ival[it.active] != pass) return;
+  int d[PEPO_MAXLEG];
+  load_dims(it.x, ival, d);
+  const int nl = it.x.nlegs;
+  const int F = 4 * (nl > 0 ? d[nl - 1] : 1);
+  long long K = 1;
+  for (int i = 0; i + 1 < nl; ++i) K *= d[i];
+  const int S = gram_rows_splits(K, kExactSplits);
+  if (acct && blockIdx.x == 0 && threadIdx.x == 0) {
+    atomicAdd(&acct[0], (double)K * F * (F + 1.0));
+    atomicAdd(&acct[1], (double)K * F * sizeof(float));
+  }
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < F * F; e += gridDim.x * blockDim.x) {
+    const int fi = e / F, fj = e - fi * F;
+    if (fi > fj) continue;
+    double sum = 0.0;
+    for (int s = 0; s < S; ++s) sum += it.partial[(long long)s * F * F + e];
+    it.out[(long long)fi * it.ldo + fj] = sum;
+    it.out[(long long)fj * it.ldo + fi] = sum;
+  }
+}
+
+cudaError_t launch_gram_exact(const GramRowsItem* items, int n_items, int fmax, int pass, void* const* ptrs,
+                              const int* ival, double* acct, cudaStream_t s) {
+  if (n_items == 0) return cudaSuccess;
+  k_col_scale<<<dim3(1, n_items), 256, 0, s>>>(items, pass, 0, ptrs, ival);
+  k_col_scale<<<dim3(64, n_items), 256, 0, s>>>(items, pass, 1, ptrs, ival);
+  const size_t smem = sizeof(float) * 4 * GX_RUN * GX_T;
+  cudaError_t e = cudaFuncSetAttribute(k_gram_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int nt = ceil_div(fmax, GX_T);
+  k_gram_exact<<<dim3(nt * (nt + 1) / 2 * kExactSplits, 1, n_items), 256, smem, s>>>(items, pass, ptrs, ival);
+  int gx = ceil_div(fmax * fmax, 256);
+  if (gx > 256) gx = 256;
+  k_gram_exact_reduce<<<dim3(gx, n_items), 256, 0, s>>>(items, pass, ival, acct);
+  return cudaGetLastError();
+}
+
 // ================================================================ reconstruct
 // out[r, (c', p')] = sum_{(c,p)} in[r, (c,p)] W[(c,p), (c',p')], stored in the
 // permuted output layout.  64 x 64 output tiles, K streamed 16 at a time.

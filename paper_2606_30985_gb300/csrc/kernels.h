@@ -16,6 +16,11 @@ cudaError_t launch_gram_rows(const GramRowsItem* items, int n_items, int tiles_m
                              int sym, void* const* ptrs, const int* ival, cudaStream_t s);
 cudaError_t launch_gram_rows_reduce(const GramRowsItem* items, int n_items, int fmax,
                                     int splits_max, int sym, const int* ival, cudaStream_t s);
+// exact FP32 Gram of the items whose branch value is `pass` (FP32 storage):
+// four launches; acct as in launch_hh_extract
+constexpr int kGramExactLaunches = 4;
+cudaError_t launch_gram_exact(const GramRowsItem* items, int n_items, int fmax, int pass, void* const* ptrs,
+                              const int* ival, double* acct, cudaStream_t s);
 template <typename T>
 cudaError_t launch_gram_leg(const GramLegItem* items, int n_items, int splits_max, int chimax,
                             void* const* ptrs, const int* ival, cudaStream_t s);

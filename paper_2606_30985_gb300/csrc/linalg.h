@@ -15,12 +15,14 @@ cudaError_t launch_hh_level(const SiteFacItem* items, int n_items, int level, in
 template <typename T>
 cudaError_t launch_hh_extract(const SiteFacItem* items, int n_items, void* const* ptrs, int* ival,
                               cudaStream_t s, int pass, double* acct);
+// householder = 1 (FP64 storage): the sites of the Householder passes hold an
+// R-factor (launch_hh_extract); 0 (FP32 storage): every site holds a Gram
 cudaError_t launch_form(const SiteFacItem* items, int n_items, int grid_x, const int* ival,
-                        cudaStream_t s, int only);
+                        cudaStream_t s, int only, int householder);
 // qcount (3 counters, may be null): sites per outcome of this pass, indexed
 // by the final branch value (0 Householder, 1 Cholesky-QR, 2 handed back)
 cudaError_t launch_factor(const SiteFacItem* items, int n_items, int rmax, int nmax, int* ival,
-                          cudaStream_t s, int only, unsigned long long* qcount);
+                          cudaStream_t s, int only, int householder, unsigned long long* qcount);
 cudaError_t launch_core(const CoreItem* items, int n_items, int* ival, int* flags_base, cudaStream_t s);
 }  // namespace pepo
 

@@ -358,6 +358,7 @@ struct SlotWS {              // per in-flight site slot (gate update)
   double* T;
   int* perm;
   double* partial;
+  unsigned* colmax;
   double* W;
 };
 
@@ -447,6 +448,7 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
     size_t pg = (size_t)kGramSplitsMax * nmax * nmax;
     size_t pl = (size_t)PEPO_MAXLEG * kLegSplitsMax * cm2;
     w.partial = cv.take<double>(std::max(pg, pl));
+    w.colmax = cv.take<unsigned>(nmax);
     w.W = cv.take<double>((size_t)nmax * nmax);
   }
   size_t maxcol = 0;
@@ -633,6 +635,7 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
           g.partial = W.partial;
           g.out = sws[v].C;
           g.ldo = nmax;
+          g.colmax = W.colmax;
           gram.push_back(g);
           // reconstruct: input = site tensor (layout lay), output layout nlay
           ReconItem rc;
@@ -1321,9 +1324,22 @@ pepo_status run_gate_wave(pepo_ctx* c, Inst& I, GateWave& w) {
                                c->d_ival, s));
     LAUNCH_T(K_GRAM_ROWS_RED, nullptr, w.gram.n, launch_gram_rows_reduce(w.gram.d, w.gram.n, nmax, c->tune.gram_rows_splits, 1, c->d_ival, s));
   }
-  // Householder TSQR of the sites with branch value `pass` (0: the Householder
-  // branch; 2: the Cholesky-branch sites whose Gram was too ill-conditioned)
-  auto tsqr = [&](int pass) -> pepo_status {
+  // R-factor of the sites with branch value `pass` (0: the Householder branch of
+  // Eq. 10; 2: the Cholesky-branch sites whose Gram was too ill-conditioned).
+  // FP64 storage: Householder TSQR.  FP32 storage: the exact Gram of the FP32
+  // data, whose Cholesky factor carries no more error than FP32 reflections
+  // (k_gram_exact).  Both sides, TSQR and its column-pivoted factor against exact
+  // Gram and Cholesky, per saturated layer: 4x4 chi = 64 229 -> 34 ms, 4x4 chi = 48
+  // 155 -> 16 ms, 3x5 chi = 27 50 -> 4 ms; 3x3 chi = 100 (two interior and eight
+  // corner factors) 443 -> 86 ms.
+  const int householder = sizeof(T) == 8 ? 1 : 0;
+  auto factor_rows = [&](int pass) -> pepo_status {
+    if (!householder) {
+      LAUNCH_T(K_HH, nullptr, w.gram.n, launch_gram_exact(w.gram.d, w.gram.n, nmax, pass, c->d_ptrs, c->d_ival,
+                                                          c->d_hh_acct, s));
+      if (w.gram.n > 0) c->launches += kGramExactLaunches - 1;
+      return PEPO_OK;
+    }
     const long long mmax = (long long)pow_sz(chimax, 3);
     const long long L0 = 256;
     long long nb0 = (mmax + L0 - 1) / L0;
@@ -1332,23 +1348,23 @@ pepo_status run_gate_wave(pepo_ctx* c, Inst& I, GateWave& w) {
     while (nb > 1) { nb = (nb + 3) / 4; ++levels; }
     long long g = nb0;
     for (int l = 0; l < levels; ++l) {
-      LAUNCH_T(K_HH, nullptr, w.fac.n, launch_hh_level<T>(w.fac.d, w.fac.n, l, (int)std::max<long long>(g, 1), nmax, c->d_ptrs,
+      LAUNCH_T(K_HH, nullptr, w.fac.n, launch_hh_level<double>(w.fac.d, w.fac.n, l, (int)std::max<long long>(g, 1), nmax, c->d_ptrs,
                                 c->d_ival, s, pass));
       g = (g + 3) / 4;
     }
-    LAUNCH_T(K_HH, nullptr, w.fac.n, launch_hh_extract<T>(w.fac.d, w.fac.n, c->d_ptrs, c->d_ival, s, pass, c->d_hh_acct));
+    LAUNCH_T(K_HH, nullptr, w.fac.n, launch_hh_extract<double>(w.fac.d, w.fac.n, c->d_ptrs, c->d_ival, s, pass, c->d_hh_acct));
     return PEPO_OK;
   };
-  pepo_status st = tsqr(0);
+  pepo_status st = factor_rows(0);
   if (st != PEPO_OK) return st;
-  LAUNCH_T(K_FACTOR, nullptr, w.fac.n, launch_form(w.fac.d, w.fac.n, 16, c->d_ival, s, -1));
-  LAUNCH_T(K_FACTOR, nullptr, w.fac.n, launch_factor(w.fac.d, w.fac.n, rmax, nmax, c->d_ival, s, -1, c->d_qr_count));
-  // the sites k_factor handed back (branch 2): Householder on the same absorbed
-  // tensor, which the Gram only read
-  st = tsqr(2);
+  LAUNCH_T(K_FACTOR, nullptr, w.fac.n, launch_form(w.fac.d, w.fac.n, 16, c->d_ival, s, -1, householder));
+  LAUNCH_T(K_FACTOR, nullptr, w.fac.n, launch_factor(w.fac.d, w.fac.n, rmax, nmax, c->d_ival, s, -1, householder, c->d_qr_count));
+  // the sites k_factor handed back (branch 2): from the same absorbed tensor,
+  // which the Gram only read
+  st = factor_rows(2);
   if (st != PEPO_OK) return st;
-  LAUNCH_T(K_FACTOR, nullptr, w.fac.n, launch_form(w.fac.d, w.fac.n, 16, c->d_ival, s, 2));
-  LAUNCH_T(K_FACTOR, nullptr, w.fac.n, launch_factor(w.fac.d, w.fac.n, rmax, nmax, c->d_ival, s, 2, nullptr));
+  LAUNCH_T(K_FACTOR, nullptr, w.fac.n, launch_form(w.fac.d, w.fac.n, 16, c->d_ival, s, 2, householder));
+  LAUNCH_T(K_FACTOR, nullptr, w.fac.n, launch_factor(w.fac.d, w.fac.n, rmax, nmax, c->d_ival, s, 2, householder, nullptr));
   return PEPO_OK;
 }
 
