@@ -1252,9 +1252,11 @@ void timing_harvest(pepo_ctx* c) {
 
 // A tensor-core kernel's error word was set: report it once and clear it, so
 // that the context stays usable (its state is undefined until restored or
-// re-uploaded).
+// re-uploaded).  The flags that the kernels behind the aborted one raised on
+// its unwritten results (a rank-0 bond core, a zero trace) go with it.
 pepo_status kernel_error(pepo_ctx* c, int kerr) {
   cudaMemsetAsync(c->d_kerr, 0, sizeof(int), c->stream);
+  cudaMemsetAsync(c->d_flags, 0, sizeof(int) * c->n_inst, c->stream);
   cudaStreamSynchronize(c->stream);
   return fail(c, PEPO_E_CUDA,
               "tensor-core kernel error word %d (bit 0: a pipeline wait ran longer than the wait limit, "
