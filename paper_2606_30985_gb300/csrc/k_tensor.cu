@@ -310,7 +310,7 @@ k_gram_exact(const GramRowsItem* __restrict__ items, int pass, void* const* ptrs
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) Sh[a][b] = Cl[a][b] = 0.f;
-  load(0, k0);
+  if (k0 < k1) load(0, k0);
   int buf = 0;
   for (long long kb = k0; kb < k1; kb += GX_RUN, buf ^= 1) {
     if (kb + GX_RUN < k1) {

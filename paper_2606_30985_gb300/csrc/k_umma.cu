@@ -275,7 +275,8 @@ __device__ inline void leg_dims(const LegItem& it, void* const* ptrs, const int*
   L.R = L.O * L.Q;
   L.tiles = (L.R + kM - 1) / kM;
   L.K8 = round_up(L.J, 8);
-  L.N16 = round_up(L.Jout, 16);
+  // N >= 16: a factor of rank 0 (a message that is not finite) still issues MMAs
+  L.N16 = round_up(L.Jout > 0 ? L.Jout : 1, 16);
   L.in = static_cast<const float*>(ptrs[it.in.ref]);
   L.out = static_cast<float*>(ptrs[it.out_ref]);
   L.A = it.A;
