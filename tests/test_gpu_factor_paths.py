@@ -44,3 +44,21 @@ def test_fp32_factor_paths_match_fp64(Lx, Ly, chi, n_thresh):
         k = min(len(a), len(b))
         assert np.max(np.abs(a[:k] - b[:k])) < 1e-5
         assert max(np.max(a[k:], initial=0.0), np.max(b[k:], initial=0.0)) < 1e-5
+
+
+def test_nan_site_in_a_tensor_core_step_is_flagged():
+    # a NaN coefficient makes its bonds' messages NaN, whose factors have rank 0: the
+    # later colours' contractions then have an output leg of size 0
+    cfg = pkg.Config(Lx=3, Ly=3, J=1.0, h=2.0, dt=0.05, order=2, obs=(1, 1), chi_max=8, precision="tf32x3")
+    eng = pkg.Engine(cfg)
+    try:
+        eng.trotter_step(2)
+        t, _ = eng.site(0, 4)
+        t.reshape(-1)[0] = np.nan
+        eng.set_site(0, 4, t)
+        eng.trotter_step(2)
+        eng.bp_converge()
+        _, D = eng.correlator()
+        assert D[0]["flags"] & 2
+    finally:
+        eng.close()
