@@ -169,7 +169,7 @@ struct CoreItem {
   int ldt1, ldt2;
   const int* perm1; const int* perm2;
   const double* FA; const double* FB;   // gate factors of side 1 / side 2
-  double* work;            // scratch: 4 blocks of rmax * rmax doubles
+  double* work;            // scratch: core_work_doubles(rmax)
   int rmax;
   double* W1; double* W2;  // n x n', leading dimension ldw
   int ldw;

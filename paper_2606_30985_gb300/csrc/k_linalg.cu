@@ -1004,9 +1004,265 @@ __device__ int jacobi_svd(R* A, int m, int n, R* V, int max_sweeps, int* capped,
   return sweep;
 }
 
-__global__ void __launch_bounds__(1024)
-k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base) {
-  const CoreItem it = items[blockIdx.x];
+// ---- the same on the CTAs of one cluster --------------------------------
+// The CTAs that share a bond core meet at the hardware cluster barrier (its
+// arrive / wait pair orders their global-memory accesses); a cluster of one
+// meets at the block barrier.
+struct Cta {
+  int rank, size;        // this CTA in its cluster, CTAs in it
+  long long tid, nthr;   // this thread among the cluster's threads
+};
+__device__ __forceinline__ void cta_sync(const Cta& c) {
+  if (c.size > 1) {
+    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+  } else {
+    __syncthreads();
+  }
+}
+
+constexpr int kCoreThreads = 1024;
+constexpr size_t kCoreSmem = (size_t)192 * 1024;
+constexpr int kCoreMaxDim = 512;                   // columns and rows of a core: rg * chi <= 512
+
+// One warp's rotation of the columns x and y (length m, shared memory) of A and
+// vx, vy (length nv, may be null) of V; nx, ny are their squared norms, kept
+// up to date.  Returns whether it rotated.  FP32 columns are held in registers
+// between the dot product and the rotation (shared-memory bandwidth bounds that
+// pass; the FP64 one is bound by its pipe), so each is read and written once.
+template <typename R>
+__device__ bool jac_pair(R* x, R* y, int m, R* vx, R* vy, int nv, R* nx, R* ny, R tol, R negligible, R abs_cut) {
+  const int lane = threadIdx.x & 31;
+  constexpr int U = sizeof(R) == 4 ? kCoreMaxDim / 32 : 1;
+  R a[U], b[U];
+  R ga = 0;
+  if constexpr (U > 1) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = lane + 32 * u;
+      a[u] = b[u] = R(0);
+      if (32 * u < m) {
+        if (i < m) { a[u] = x[i]; b[u] = y[i]; }
+        ga = fma(a[u], b[u], ga);
+      }
+    }
+  } else {
+    for (int i = lane; i < m; i += 32) ga = fma(x[i], y[i], ga);
+  }
+  const R al = *nx, be = *ny;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+  if (!(ga != R(0) && al > negligible && be > negligible && fabs(ga) > tol * sqrt(al * be) && fabs(ga) > abs_cut))
+    return false;
+  const R zeta = (be - al) / (R(2) * ga);
+  const R t = (zeta >= R(0) ? R(1) : R(-1)) / (fabs(zeta) + sqrt(R(1) + zeta * zeta));
+  const R c = R(1) / sqrt(R(1) + t * t), s = c * t;
+  if constexpr (U > 1) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = lane + 32 * u;
+      if (i < m) { x[i] = c * a[u] - s * b[u]; y[i] = s * a[u] + c * b[u]; }
+    }
+  } else {
+    for (int i = lane; i < m; i += 32) {
+      const R p = x[i], q = y[i];
+      x[i] = c * p - s * q;
+      y[i] = s * p + c * q;
+    }
+  }
+  if (vx)
+    for (int i = lane; i < nv; i += 32) {
+      const R p = vx[i], q = vy[i];
+      vx[i] = c * p - s * q;
+      vy[i] = s * p + c * q;
+    }
+  __syncwarp();
+  if (lane == 0) { *nx = al - t * ga; *ny = be + t * ga; }
+  return true;
+}
+
+// One-sided Jacobi of A (m x n, column-major, leading dimension m, global
+// memory) with the rotations accumulated in V (n x n), on all CTAs of the
+// cluster.  The columns are cut into (at most) 16 blocks; a round of the block
+// tournament pairs every block with another, and the columns of a pair of
+// blocks meet each other in inner rounds of disjoint pairs, one warp per pair of
+// columns (round 0: every pair within and across the two blocks; then the cross
+// pairs only).  Each CTA brings its pairs of blocks into shared memory (A and V
+// columns) and writes them back, so the matrix crosses L2 once per round of
+// ~bs^2 rotations per CTA instead of twice per rotation; a matrix that one CTA
+// holds stays there for all sweeps when the cluster is that CTA (a batch of
+// many cores) or when there is too little to share (n <= 32: rank 0 works).
+// The order of the rotations of a column depends on n alone, so every cluster
+// size gives the same bits.
+//
+// Rotation and stopping rules as jacobi_svd, plus abs_rel > 0: a pair whose
+// coupling |a_p . a_q| is below abs_rel ||A||_F^2 is skipped too.  Such a pair
+// moves no singular value by more than that, and without the cut the columns of
+// tiny singular values (mostly rounding noise from rotations with the large
+// ones) are chased for many sweeps without ever reaching relative
+// orthogonality.  Squared norms are recomputed every round and updated by the
+// rotations between.  flags: 3 ints, zeroed by the caller; cnorm: n doubles.
+template <typename R>
+__device__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* capped, double abs_rel, const Cta& ct,
+                              int* flags, double* cnorm, unsigned char* sh) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  __shared__ double fr[32];
+  // V = I and ||A||_F^2, by columns (its bits do not depend on the cluster)
+  for (long long e = ct.tid; e < (long long)n * n; e += ct.nthr) V[e] = (e % (n + 1) == 0) ? R(1) : R(0);
+  for (long long j = ct.tid >> 5; j < n; j += ct.nthr >> 5) {
+    double q = 0.0;
+    for (int i = lane; i < m; i += 32) { const double x = (double)A[j * m + i]; q = fma(x, x, q); }
+    q = warp_sum(q);
+    if (lane == 0) cnorm[j] = q;
+  }
+  cta_sync(ct);
+  if (n < 2) return 0;
+  double fro = 0.0;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) fro += cnorm[j];
+  fro = block_sum(fro, fr);
+  const R tol = (R)((sizeof(R) == 4 ? 3e-7 : 1e-15) * sqrt((double)m));
+  // columns below 1e-30 (FP64) or 1e-13 (FP32) of the total squared norm are
+  // numerically zero in that precision
+  const R negligible = (R)((sizeof(R) == 4 ? 1e-13 : 1e-30) * fro);
+  const R abs_cut = (R)(abs_rel * fro);
+  const int room = (int)((kCoreSmem - 4096) / sizeof(R));
+  R* nrm = reinterpret_cast<R*>(sh);                        // squared norms of the columns at hand
+  R* buf = reinterpret_cast<R*>(sh + 4096);
+  const int per = m + n;                                    // A column then V column
+  int most = room / per / 2;                                // columns of a block: two blocks at a time
+  if (most > 32) most = 32;
+  int nblk = n < 16 ? n + (n & 1) : 16;
+  if ((n + nblk - 1) / nblk > most) nblk = ((n + most - 1) / most + 1) / 2 * 2;
+  const int bs = (n + nblk - 1) / nblk, npair = nblk / 2;
+  const bool resident = (long long)per * n <= room && (ct.size == 1 || n <= 32);
+  auto first = [&](int blk) { return min(blk * bs, n); };
+  auto count = [&](int blk) { return min(bs, n - first(blk)); };
+  // blocks P < Q of pair pi in a round
+  auto blocks = [&](int round, int pi, int& P, int& Q) {
+    if (pi == 0) { P = nblk - 1; Q = round; }
+    else { P = (round + pi) % (nblk - 1); Q = (round - pi + nblk - 1) % (nblk - 1); }
+    if (P > Q) { const int t = P; P = Q; Q = t; }
+  };
+  auto bring = [&](int c0, int cnt, int at) {               // columns c0.. to slots at..
+    for (int e = threadIdx.x; e < cnt * per; e += blockDim.x) {
+      const int c = e / per, i = e - c * per;
+      buf[(at + c) * per + i] = i < m ? A[(long long)(c0 + c) * m + i] : V[(long long)(c0 + c) * n + i - m];
+    }
+  };
+  auto back = [&](int c0, int cnt, int at) {
+    for (int e = threadIdx.x; e < cnt * per; e += blockDim.x) {
+      const int c = e / per, i = e - c * per;
+      const R x = buf[(at + c) * per + i];
+      if (i < m) A[(long long)(c0 + c) * m + i] = x;
+      else V[(long long)(c0 + c) * n + i - m] = x;
+    }
+  };
+  auto norms = [&](int cnt) {
+    for (int c = wid; c < cnt; c += nw) {
+      const R* x = buf + c * per;
+      R q = 0;
+      for (int i = lane; i < m; i += 32) q = fma(x[i], x[i], q);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+      if (lane == 0) nrm[c] = q;
+    }
+    __syncthreads();
+  };
+  // the pairs f(0) .. f(cnt - 1) (slots of disjoint columns; x < 0: none), then a block barrier
+  auto round_of = [&](int cnt, auto f) -> int {
+    int rot = 0;
+    for (int k = wid; k < cnt; k += nw) {
+      const int2 v = f(k);
+      if (v.x < 0) continue;
+      R* x = buf + v.x * per;
+      R* y = buf + v.y * per;
+      rot |= jac_pair<R>(x, y, m, x + m, y + m, n, nrm + v.x, nrm + v.y, tol, negligible, abs_cut) ? 1 : 0;
+    }
+    __syncthreads();
+    return rot;
+  };
+  // inner round `k` of block pair (P, Q) at slots p0, q0: pair i of it
+  auto inner = [&](bool all, int k, int i, int P, int Q, int p0, int q0) -> int2 {
+    const int cp = count(P), cq = count(Q);
+    if (!all) {                                             // column i of P with column (i + k) mod bs of Q
+      const int q = (i + k) % bs;
+      return i < cp && q < cq ? make_int2(p0 + i, q0 + q) : make_int2(-1, -1);
+    }
+    const int cnt = cp + cq, np = cnt + (cnt & 1);          // tournament (a dummy if odd)
+    if (k >= np - 1 || i >= np / 2) return make_int2(-1, -1);
+    int x, y;
+    if (i == 0) { x = np - 1; y = k; }
+    else { x = (k + i) % (np - 1); y = (k - i + np - 1) % (np - 1); }
+    if (x >= cnt || y >= cnt) return make_int2(-1, -1);
+    if (x > y) { const int t = x; x = y; y = t; }
+    return make_int2(x < cp ? p0 + x : q0 + x - cp, y < cp ? p0 + y : q0 + y - cp);
+  };
+  const int steps0 = 2 * bs - 1;                            // inner rounds of round 0; later: bs
+  int sweep = 0;
+  if (resident && ct.rank == 0) {
+    bring(0, n, 0);
+    __syncthreads();
+  }
+  for (; sweep < max_sweeps; ++sweep) {
+    int* flag = flags + sweep % 3;
+    if (ct.rank == 0 && threadIdx.x == 0) flags[(sweep + 1) % 3] = 0;
+    int rot = 0;
+    for (int round = 0; round < nblk - 1; ++round) {
+      const bool all = round == 0;
+      const int steps = all ? steps0 : bs;
+      if (resident) {
+        if (ct.rank == 0) {
+          norms(n);
+          for (int k = 0; k < steps; ++k)
+            rot |= round_of(npair * bs, [&](int e) {
+              const int pi = e / bs, i = e - pi * bs;
+              int P, Q;
+              blocks(round, pi, P, Q);
+              return inner(all, k, i, P, Q, first(P), first(Q));
+            });
+        }
+      } else {
+        for (int pi = ct.rank; pi < npair; pi += ct.size) {
+          int P, Q;
+          blocks(round, pi, P, Q);
+          const int cp = count(P), cq = count(Q);
+          if (cp == 0 || (cq == 0 && !all)) continue;
+          bring(first(P), cp, 0);
+          bring(first(Q), cq, cp);
+          __syncthreads();
+          norms(cp + cq);
+          for (int k = 0; k < steps; ++k)
+            rot |= round_of(bs, [&](int i) { return inner(all, k, i, P, Q, 0, cp); });
+          back(first(P), cp, 0);
+          back(first(Q), cq, cp);
+          __syncthreads();
+        }
+        cta_sync(ct);
+      }
+    }
+    if (__syncthreads_or(rot) && threadIdx.x == 0) atomicOr(flag, 1);
+    cta_sync(ct);
+    if (*reinterpret_cast<volatile int*>(flag) == 0) break;
+  }
+  if (resident && ct.rank == 0) back(0, n, 0);
+  if (sweep >= max_sweeps && threadIdx.x == 0) *capped = 1;
+  cta_sync(ct);
+  return sweep;
+}
+
+// Bond core, one cluster per bond.  Bound: the FP64 pipe (T_core = R1 R2^T, T Q
+// and the FP64 Jacobi: 2 multiply-adds per clock and SM) and the shared-memory
+// bandwidth of the FP32 Jacobi, both spread over the cluster's SMs; one CTA
+// per bond left 150 of 152 SMs idle on a small grid and kept the Jacobi's
+// columns in L2.  Core class of a saturated layer, one CTA -> cluster: 3x3 chi = 100
+// 652 -> 101 ms, 4x4 chi = 64 197 -> 40 ms, 3x5 chi = 27 29.5 -> 13 ms.
+__global__ void __launch_bounds__(kCoreThreads, 1)
+k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize) {
+  const CoreItem it = items[blockIdx.x / csize];
+  Cta ct;
+  ct.rank = blockIdx.x % csize;
+  ct.size = csize;
+  ct.tid = (long long)ct.rank * blockDim.x + threadIdx.x;
+  ct.nthr = (long long)csize * blockDim.x;
   int* flags = flags_base + it.inst;
   const int chic = ival[it.chi_idx];
   const int rg = ival[it.rg_idx];
@@ -1014,38 +1270,66 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base) {
   const int n = 4 * chic;
   const int k1 = ival[it.rank1_idx], k2 = ival[it.rank2_idx];
   const int rmax = it.rmax;
-  double* R2o = it.work;                          // k2 x r, original column order
+  double* R2t = it.work;                          // R2^T: r x k2, rows in R1's pivot order; later scratch
   double* Tc = it.work + (long long)rmax * rmax;  // column-major working matrix
   double* V = Tc + (long long)rmax * rmax;        // Jacobi right vectors
   double* Z = V + (long long)rmax * rmax;         // triangular-solve results
-  __shared__ double red[32];
+  int* cflag = reinterpret_cast<int*>(it.work + (long long)4 * rmax * rmax);   // 8 ints
+  double* cnorm = it.work + (long long)4 * rmax * rmax + 4;                    // column norms (rmax)
+  extern __shared__ __align__(16) unsigned char core_sh[];
   __shared__ double sv[2 * 4 * 128 + 8];
   __shared__ int order[4 * 128];
   __shared__ int sh_capped;
+  const int lane = threadIdx.x & 31;
+  const long long gw = ct.tid >> 5, ngw = ct.nthr >> 5;   // warps of the cluster
   if (threadIdx.x == 0) sh_capped = 0;
-  // R2 in original column order
-  for (long long e = threadIdx.x; e < (long long)k2 * r; e += blockDim.x) {
-    int b = (int)(e / r), q = (int)(e % r);
-    double x = (q >= b) ? it.T2[(long long)b * it.ldt2 + q] : 0.0;
-    R2o[(long long)b * r + it.perm2[q]] = x;
-  }
+  if (ct.rank == 0 && threadIdx.x < 8) cflag[threadIdx.x] = 0;
+  for (int q = threadIdx.x; q < r; q += blockDim.x) order[it.perm1[q]] = q;   // position in R1's pivot order
   __syncthreads();
+  for (long long e = ct.tid; e < (long long)k2 * r; e += ct.nthr) {
+    const int b = (int)(e / r), q = (int)(e % r);
+    R2t[(long long)order[it.perm2[q]] * k2 + b] = (q >= b) ? it.T2[(long long)b * it.ldt2 + q] : 0.0;
+  }
+  cta_sync(ct);
   // Tcore = R1 R2^T (k1 x k2).  Work on the orientation with m >= n columns.
   const bool tr = k1 < k2;             // if so, decompose Tcore^T
   const int M = tr ? k2 : k1, N = tr ? k1 : k2;
-  for (long long e = threadIdx.x; e < (long long)k1 * k2; e += blockDim.x) {
-    int a = (int)(e / k2), b = (int)(e % k2);
+  for (long long e = ct.tid; e < (long long)k1 * k2; e += ct.nthr) {
+    const int a = (int)(e / k2), b = (int)(e % k2);
     double s = 0.0;
     const double* t1 = it.T1 + (long long)a * it.ldt1;
-    const double* r2 = R2o + (long long)b * r;
-    for (int q = a; q < r; ++q) s = fma(t1[q], r2[it.perm1[q]], s);
-    // column-major M x N storage of Tcore (or its transpose)
-    if (!tr) Tc[(long long)b * M + a] = s; else Tc[(long long)a * M + b] = s;
+#pragma unroll 8
+    for (int q = a; q < r; ++q) s = fma(t1[q], R2t[(long long)q * k2 + b], s);
+    // column-major M x N storage of Tcore (or its transpose), and a copy (the
+    // mixed path multiplies it by its FP64 subspace basis)
+    const long long o = !tr ? (long long)b * M + a : (long long)a * M + b;
+    Tc[o] = s;
+    V[o] = s;
   }
-  __syncthreads();
-  // copy of Tcore (the mixed path multiplies it by its FP64 subspace basis)
-  for (long long e = threadIdx.x; e < (long long)M * N; e += blockDim.x) V[e] = Tc[e];
-  __syncthreads();
+  cta_sync(ct);
+  // norms of the columns of a (len x cols, column-major) -> cnorm
+  auto col_norms = [&](auto* a, int len, int cols) {
+    for (long long j = gw; j < cols; j += ngw) {
+      double s = 0.0;
+      for (int i = lane; i < len; i += 32) { const double x = (double)a[j * len + i]; s = fma(x, x, s); }
+      s = warp_sum(s);
+      if (lane == 0) cnorm[j] = sqrt(s);
+    }
+    cta_sync(ct);
+  };
+  // descending order of sv[0 .. cols)
+  auto rank_order = [&](int cols) {
+    for (int j = threadIdx.x; j < cols; j += blockDim.x) {
+      int rk = 0;
+      const double kj = rank_key(sv[j]);
+      for (int i = 0; i < cols; ++i) {
+        const double ki = rank_key(sv[i]);
+        if (ki > kj || (ki == kj && i < j)) ++rk;
+      }
+      order[rk] = j;
+    }
+    __syncthreads();
+  };
   // columns the FP64 Jacobi below works on (all N, or the mixed path's subspace)
   int NK = N;
   __shared__ double sh_fro;
@@ -1063,54 +1347,44 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base) {
     // FP64 sweeps follow.  Values past NK (never kept: NK > chimax) keep their
     // FP32 estimates for the diagnostic spectrum; the discarded weight of the
     // truncation uses ||T||_F^2 computed in FP64.
-    float* T32 = reinterpret_cast<float*>(R2o);
+    float* T32 = reinterpret_cast<float*>(R2t);
     float* V32 = T32 + (long long)M * N;
-    for (long long e = threadIdx.x; e < (long long)M * N; e += blockDim.x) T32[e] = (float)Tc[e];
+    col_norms(Tc, M, N);
     double f2 = 0.0;
-    for (long long e = threadIdx.x; e < (long long)M * N; e += blockDim.x) f2 = fma(Tc[e], Tc[e], f2);
-    f2 = block_sum(f2, red);
+    for (int j = threadIdx.x; j < N; j += blockDim.x) f2 = fma(cnorm[j], cnorm[j], f2);
+    {
+      __shared__ double fr2[32];
+      f2 = block_sum(f2, fr2);
+    }
     if (threadIdx.x == 0) sh_fro = f2;
     __syncthreads();
+    // the copy is scaled by a power of two to a norm in [1, 2): its squares stay
+    // in FP32's range whatever the scale of the site tensors
+    const int t_exp = sh_fro > 0.0 && isfinite(sh_fro) ? ilogb(sqrt(sh_fro)) : 0;
+    for (long long e = ct.tid; e < (long long)M * N; e += ct.nthr) T32[e] = (float)scalbn(Tc[e], -t_exp);
+    cta_sync(ct);
     __shared__ int sh_capped32;   // a capped FP32 pass only costs FP64 sweeps below
-    if (threadIdx.x == 0) sh_capped32 = 0;
+    const int sw32 = jacobi_cluster<float>(T32, M, N, V32, 60, &sh_capped32, 0.0, ct, cflag, cnorm, core_sh);
+    if (ct.rank == 0 && threadIdx.x < 8) cflag[threadIdx.x] = 0;
+    if (ct.rank == 0 && threadIdx.x == 0 && it.sweeps) it.sweeps[0] = sw32;
+    // FP32 singular-value estimates (unsorted at sv[j]) and their order
+    col_norms(T32, M, N);
+    for (int j = threadIdx.x; j < N; j += blockDim.x) sv[j] = scalbn(cnorm[j], t_exp);
     __syncthreads();
-    const int sw32 = jacobi_svd<float>(T32, M, N, V32, 60, &sh_capped32, red);
-    if (threadIdx.x == 0 && it.sweeps) it.sweeps[0] = sw32;
-    __syncthreads();
-    // FP32 singular-value estimates (unsorted at sv[512 + j]) and their order
-    for (int j = threadIdx.x; j < N; j += blockDim.x) {
-      double s = 0.0;
-      const float* col = T32 + (long long)j * M;
-      for (int i = 0; i < M; ++i) s = fma((double)col[i], (double)col[i], s);
-      sv[512 + j] = sqrt(s);
-    }
-    __syncthreads();
-    for (int j = threadIdx.x; j < N; j += blockDim.x) {
-      int rk = 0;
-      const double kj = rank_key(sv[512 + j]);
-      for (int i = 0; i < N; ++i) {
-        const double ki = rank_key(sv[512 + i]);
-        if (ki > kj || (ki == kj && i < j)) ++rk;
-      }
-      order[rk] = j;
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < N; c += blockDim.x) sv[c] = sv[512 + order[c]];
-    __syncthreads();
-    for (int c = threadIdx.x; c < N; c += blockDim.x) sv[512 + c] = sv[c];   // sorted FP32 values
+    rank_order(N);
+    for (int c = threadIdx.x; c < N; c += blockDim.x) sv[512 + c] = sv[order[c]];   // sorted FP32 values
     const int margin = it.chimax / 4 > 16 ? it.chimax / 4 : 16;
     NK = it.chimax + margin < N ? it.chimax + margin : N;
     // Q = leading NK columns of V32 in FP64 (N x NK, column-major, in Z)
     double* Qk = Z;
-    for (long long e = threadIdx.x; e < (long long)N * NK; e += blockDim.x) {
+    for (long long e = ct.tid; e < (long long)N * NK; e += ct.nthr) {
       const int c = (int)(e / N), i = (int)(e - (long long)c * N);
       Qk[e] = (double)V32[(long long)order[c] * N + i];
     }
-    __syncthreads();
+    cta_sync(ct);
     // Cholesky QR: G = Q^T Q = L L^T (lower triangle of G in the Tc block), Q <- Q L^-T
     double* G = Tc;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (long long pq = wid; pq < (long long)NK * NK; pq += nw) {
+    for (long long pq = gw; pq < (long long)NK * NK; pq += ngw) {
       const int a = (int)(pq / NK), b = (int)(pq - (long long)a * NK);
       if (b > a) continue;
       const double* qa = Qk + (long long)a * N;
@@ -1120,38 +1394,47 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base) {
       acc = warp_sum(acc);
       if (lane == 0) G[(long long)a * NK + b] = acc;
     }
+    cta_sync(ct);
+    // every CTA factors its own copy: the lower triangle packed in shared memory
+    double* L = reinterpret_cast<double*>(core_sh);        // NK (NK + 1) / 2 <= 160 * 161 / 2 doubles
+    for (int e = threadIdx.x; e < NK * NK; e += blockDim.x) {
+      const int i = e / NK, l = e - i * NK;
+      if (l <= i) L[i * (i + 1) / 2 + l] = G[e];
+    }
     __syncthreads();
     for (int j = 0; j < NK; ++j) {
-      if (threadIdx.x == 0) G[(long long)j * NK + j] = sqrt(G[(long long)j * NK + j]);
+      const int jj = j * (j + 1) / 2;
+      const double djj = sqrt(L[jj + j]);
       __syncthreads();
-      const double djj = G[(long long)j * NK + j];
-      for (int i = j + 1 + threadIdx.x; i < NK; i += blockDim.x) G[(long long)i * NK + j] /= djj;
+      if (threadIdx.x == 0) L[jj + j] = djj;
+      for (int i = j + 1 + threadIdx.x; i < NK; i += blockDim.x) L[i * (i + 1) / 2 + j] /= djj;
       __syncthreads();
-      const int w = NK - j - 1;   // trailing lower triangle: rows i > j, columns j < l <= i
-      for (long long e = threadIdx.x; e < (long long)w * w; e += blockDim.x) {
-        const int i = j + 1 + (int)(e / w), l = j + 1 + (int)(e % w);
-        if (l <= i) G[(long long)i * NK + l] -= G[(long long)i * NK + j] * G[(long long)l * NK + j];
+      for (int i = j + 1 + (int)(threadIdx.x >> 5); i < NK; i += (int)(blockDim.x >> 5)) {
+        const double lij = L[i * (i + 1) / 2 + j];
+        for (int l = j + 1 + lane; l <= i; l += 32) L[i * (i + 1) / 2 + l] -= lij * L[l * (l + 1) / 2 + j];
       }
       __syncthreads();
     }
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {   // row i of Q solves x L^T = q
+    for (long long i = ct.tid; i < N; i += ct.nthr) {   // row i of Q solves x L^T = q
       for (int c = 0; c < NK; ++c) {
         double x = Qk[(long long)c * N + i];
-        const double* lc = G + (long long)c * NK;
+        const double* lc = L + c * (c + 1) / 2;
+#pragma unroll 8
         for (int l = 0; l < c; ++l) x -= Qk[(long long)l * N + i] * lc[l];
         Qk[(long long)c * N + i] = x / lc[c];
       }
     }
-    __syncthreads();
+    cta_sync(ct);
     // Tc <- T Q (M x NK, column-major), T = the copy in V
-    for (long long e = threadIdx.x; e < (long long)M * NK; e += blockDim.x) {
+    for (long long e = ct.tid; e < (long long)M * NK; e += ct.nthr) {
       const int c = (int)(e / M), i = (int)(e - (long long)c * M);
       const double* qc = Qk + (long long)c * N;
       double acc = 0.0;
+#pragma unroll 8
       for (int k = 0; k < N; ++k) acc = fma(V[(long long)k * M + i], qc[k], acc);
       Tc[e] = acc;
     }
-    __syncthreads();
+    cta_sync(ct);
   }
   {   // FP64 one-sided Jacobi on Tcore (or on its restriction T Q)
     // mixed path: the rotations W64 (NK x NK) are accumulated in the V block
@@ -1160,35 +1443,21 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base) {
     // T^T u / s would carry the columns' absolute rounding (~1e-16 of the
     // largest) divided by s^2, which for kept values near eps_cut (1e-11 of
     // the largest) leaves nothing of the vector
-    const int sw64 = jacobi_svd<double>(Tc, M, NK, V, 60, &sh_capped, red, 1e-17);
-    if (threadIdx.x == 0 && it.sweeps) {
+    const int sw64 = jacobi_cluster<double>(Tc, M, NK, V, 60, &sh_capped, 1e-17, ct, cflag, cnorm, core_sh);
+    if (ct.rank == 0 && threadIdx.x == 0 && it.sweeps) {
       it.sweeps[1] = sw64;
       if (!it.mixed_svd) it.sweeps[0] = 0;
     }
-    __syncthreads();
     // singular values (column norms) and descending order
-    for (int j = threadIdx.x; j < NK; j += blockDim.x) {
-      double s = 0.0;
-      const double* col = Tc + (long long)j * M;
-      for (int i = 0; i < M; ++i) s = fma(col[i], col[i], s);
-      sv[j] = sqrt(s);
-    }
+    col_norms(Tc, M, NK);
+    for (int j = threadIdx.x; j < NK; j += blockDim.x) sv[j] = cnorm[j];
     __syncthreads();
-    for (int j = threadIdx.x; j < NK; j += blockDim.x) {
-      int rk = 0;
-      const double kj = rank_key(sv[j]);
-      for (int i = 0; i < NK; ++i) {
-        const double ki = rank_key(sv[i]);
-        if (ki > kj || (ki == kj && i < j)) ++rk;
-      }
-      order[rk] = j;
-    }
-    __syncthreads();
+    rank_order(NK);
   }
-  const double s0 = sv[order[0]];
+  const double s0 = NK > 0 ? sv[order[0]] : 0.0;
   // truncation, Eq. 11
   __shared__ int sh_chi;
-  __shared__ double sh_sum, sh_tot;
+  __shared__ double sh_sum, sh_nrm;
   if (threadIdx.x == 0) {
     int cnt = 0;
     double tot = 0.0;
@@ -1204,115 +1473,177 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base) {
     for (int i = 0; i < chi; ++i) { double s = sv[order[i]]; kept += s * s; ksum += s; }
     sh_chi = chi;
     sh_sum = ksum;
-    sh_tot = tot;
-    *it.disc = tot > 0.0 ? (tot - kept) / tot : 0.0;
-    ival[it.new_idx] = chi;
-    *it.nsv = N;
-    if (!(s0 > 0.0) || !isfinite(s0)) atomicOr(flags, 2);
+    sh_nrm = sqrt(kept);
+    if (ct.rank == 0) {
+      *it.disc = tot > 0.0 ? (tot - kept) / tot : 0.0;
+      ival[it.new_idx] = chi;
+      *it.nsv = N;
+      if (!(s0 > 0.0) || !isfinite(s0)) atomicOr(flags, 2);
+      // stored psi = true psi * exp(-sigma); the raw sqrt(S) split gives both
+      // sites half of the pair's combined scale plus the normalisation of W
+      const double ls = 0.5 * log(ksum) + 0.5 * (*it.sigma1 + *it.sigma2);
+      *it.sigma1 = ls;
+      *it.sigma2 = ls;
+    }
     if (sh_capped) atomicOr(flags, 4);
-    const double nrm = sqrt(kept);
-    for (int i = 0; i < it.chimax; ++i) it.lam[i] = (i < chi) ? sv[order[i]] / nrm : 0.0;
-    for (int i = 0; i < N; ++i) it.svals[i] = i < NK ? sv[order[i]] : sv[512 + i];
-    // stored psi = true psi * exp(-sigma); the raw sqrt(S) split gives both
-    // sites half of the pair's combined scale plus the normalisation of W
-    const double ls = 0.5 * log(ksum) + 0.5 * (*it.sigma1 + *it.sigma2);
-    *it.sigma1 = ls;
-    *it.sigma2 = ls;
   }
   __syncthreads();
   const int chi = sh_chi;
   const double inv = 1.0 / sqrt(sh_sum);
+  for (long long i = ct.tid; i < it.chimax; i += ct.nthr) it.lam[i] = (i < chi) ? sv[order[i]] / sh_nrm : 0.0;
+  for (long long i = ct.tid; i < N; i += ct.nthr) it.svals[i] = i < NK ? sv[order[i]] : sv[512 + i];
   // messages diag(lambda)
-  for (int e = threadIdx.x; e < it.chimax * it.chimax; e += blockDim.x) {
-    int i = e / it.chimax, j = e % it.chimax;
-    double x = (i == j && i < chi) ? it.lam[i] : 0.0;
+  for (long long e = ct.tid; e < (long long)it.chimax * it.chimax; e += ct.nthr) {
+    const int i = (int)(e / it.chimax), j = (int)(e % it.chimax);
+    const double x = (i == j && i < chi) ? sv[order[i]] / sh_nrm : 0.0;
     it.msg12[e] = x;
     it.msg21[e] = x;
   }
+  double* Vr = R2t;
   if (it.mixed_svd) {
     // Right (N-space) vectors of the kept pairs: v_c = Q W64 e_order[c] (N x chi,
-    // row-major by N index), first into the R2 block, then into the V block
-    // once W64 is consumed.  These are the Ritz vectors of the subspace, so
-    // T v_c = s_c u_c holds exactly for every kept pair; recovering them as
-    // T^T u_c / s_c instead would divide the subspace's FP32-level residual
-    // by s_c^2 for values near the FP32 resolution (~1e-7 of the largest).
-    double* Vr = R2o;
-    for (long long e = threadIdx.x; e < (long long)N * chi; e += blockDim.x) {
-      const int a = (int)(e / chi), c = (int)(e - (long long)a * chi);
+    // column-major, in the R2 block).  These are the Ritz vectors of the
+    // subspace, so T v_c = s_c u_c holds exactly for every kept pair; recovering
+    // them as T^T u_c / s_c instead would divide the subspace's FP32-level
+    // residual by s_c^2 for values near the FP32 resolution (~1e-7 of the largest).
+    for (long long e = ct.tid; e < (long long)N * chi; e += ct.nthr) {
+      const int c = (int)(e / N), a = (int)(e - (long long)c * N);
       const double* w = V + (long long)order[c] * NK;
       double acc = 0.0;
+#pragma unroll 8
       for (int l = 0; l < NK; ++l) acc = fma(Z[(long long)l * N + a], w[l], acc);
       Vr[e] = acc;
     }
-    __syncthreads();
-    for (long long e = threadIdx.x; e < (long long)N * chi; e += blockDim.x) V[e] = Vr[e];
-    __syncthreads();
   }
-  // For each side: Zs = T_s11^{-1} (singular vectors of that side) sqrt(s) / sqrt(sum s)
-  // side 1 vectors: left vectors of Tcore (rows of R1 space, length k1)
-  // side 2 vectors: right vectors (length k2)
+  cta_sync(ct);
+  // For each side: Z_s = T_s11^{-1} (singular vectors of that side) sqrt(s) / sqrt(sum s);
+  // side 1 vectors: left vectors of Tcore (rows of R1 space, length k1), side 2
+  // vectors: right vectors (length k2).  Both sides at once, the columns
+  // shared out over the CTAs, each solved in blocks of 32 rows: the rows of a
+  // block one after another, then their contribution to all rows above as one
+  // product (one dependent chain of 32 rows at a time instead of ks).
+  // Z of side s: ks x chi column-major at Z + s rmax chimax (rmax = 4 chimax).
+  double* Zs[2] = {Z, Z + (long long)rmax * it.chimax};
+  {
+    constexpr int kZld = kCoreMaxDim + 1;                  // odd: lanes on one row of several columns
+    double* zc = reinterpret_cast<double*>(core_sh);       // this CTA's columns, ks each
+    const int fit = (int)(kCoreSmem / sizeof(double)) / kZld;   // 47 columns at a time
+    const int total = 2 * chi;
+    const int per = min(fit, (total + ct.size - 1) / ct.size);
+    for (int g0 = ct.rank * per; g0 < total; g0 += ct.size * per) {
+      for (int side = 0; side < 2; ++side) {
+        const int c0 = max(g0 - side * chi, 0), c1 = min(g0 + per - side * chi, chi);
+        if (c0 >= c1) continue;
+        const int nc = c1 - c0;
+        const int ks = side == 0 ? k1 : k2;
+        const double* Ts = side == 0 ? it.T1 : it.T2;
+        const int ldts = side == 0 ? it.ldt1 : it.ldt2;
+        // if (!tr): left vectors = columns of Tc / s (length M = k1), right = V (length N = k2)
+        // if (tr):  left vectors = V (length N = k1), right = columns of Tc / s (length M = k2)
+        const bool from_cols = (side == 0) != tr;
+        __syncthreads();
+        for (int e = threadIdx.x; e < ks * nc; e += blockDim.x) {
+          const int c = e / ks, a = e - c * ks;
+          const int j = order[c0 + c];
+          const double s = sv[j];
+          double x;
+          if (from_cols) x = s > 0.0 ? Tc[(long long)j * M + a] / s : 0.0;
+          else if (it.mixed_svd) x = Vr[(long long)(c0 + c) * N + a];   // Ritz right vector (above)
+          else x = V[(long long)j * N + a];                             // accumulated right vector j
+          zc[c * kZld + a] = x * sqrt(s) * inv;
+        }
+        __syncthreads();
+        for (int b1 = ks; b1 > 0; b1 -= 32) {
+          const int b0 = b1 > 32 ? b1 - 32 : 0;
+          // the block's own rows: one warp per column, lane = row
+          for (int c = threadIdx.x >> 5; c < nc; c += (int)(blockDim.x >> 5)) {
+            double* z = zc + c * kZld;
+            double x = b0 + lane < b1 ? z[b0 + lane] : 0.0;
+            for (int a = b1 - 1; a >= b0; --a) {
+              const double* trow = Ts + (long long)a * ldts;
+              double y = __shfl_sync(0xffffffffu, x, a - b0) / trow[a];
+              if (b0 + lane == a) x = y;
+              else if (b0 + lane < a) x -= Ts[(long long)(b0 + lane) * ldts + a] * y;
+            }
+            if (b0 + lane < b1) z[b0 + lane] = x;
+          }
+          __syncthreads();
+          for (int e = threadIdx.x; e < b0 * nc; e += blockDim.x) {
+            const int a = e / nc, c = e - a * nc;
+            const double* trow = Ts + (long long)a * ldts;
+            double* z = zc + c * kZld;
+            double acc = z[a];
+#pragma unroll 8
+            for (int b = b0; b < b1; ++b) acc -= trow[b] * z[b];
+            z[a] = acc;
+          }
+          __syncthreads();
+        }
+        for (int e = threadIdx.x; e < ks * nc; e += blockDim.x) {
+          const int c = e / ks, a = e - c * ks;
+          Zs[side][(long long)(c0 + c) * ks + a] = zc[c * kZld + a];
+        }
+      }
+    }
+  }
+  cta_sync(ct);
+  // Y[(c,kappa), c'] = Z[q, c'] at original column perm[q] (zero for q >= ks)
+  // W[(c,p), (c',p')] = sum_kappa F_kappa[p', p] Y[(c,kappa), c']
   for (int side = 0; side < 2; ++side) {
     const int ks = side == 0 ? k1 : k2;
-    const double* Ts = side == 0 ? it.T1 : it.T2;
-    const int ldts = side == 0 ? it.ldt1 : it.ldt2;
     const int* perms = side == 0 ? it.perm1 : it.perm2;
     const double* Fs = side == 0 ? it.FA : it.FB;
     double* W = side == 0 ? it.W1 : it.W2;
-    // vector of side `side` for singular index c' (c' < chi): length ks
-    // if (!tr): left vectors = columns of Tc / s (length M = k1), right = V (length N = k2)
-    // if (tr):  left vectors = V (length N = k1), right = columns of Tc / s (length M = k2)
-    const bool from_cols = (side == 0) != tr;
-    for (long long e = threadIdx.x; e < (long long)ks * chi; e += blockDim.x) {
-      int a = (int)(e / chi), c = (int)(e % chi);
-      int j = order[c];
-      double s = sv[j];
-      double x;
-      if (from_cols) {
-        x = s > 0.0 ? Tc[(long long)j * M + a] / s : 0.0;
-      } else if (it.mixed_svd) {
-        x = V[(long long)a * chi + c];                  // Ritz right vector (above)
-      } else {
-        x = V[(long long)j * N + a];                    // accumulated right vector j (column-major N x N)
-      }
-      Z[(long long)a * chi + c] = x * sqrt(s) * inv;
-    }
     __syncthreads();
-    // back substitution with the leading ks x ks upper-triangular block of Ts
-    for (int c = threadIdx.x; c < chi; c += blockDim.x) {
-      for (int a = ks - 1; a >= 0; --a) {
-        double x = Z[(long long)a * chi + c];
-        const double* trow = Ts + (long long)a * ldts;
-        for (int b = a + 1; b < ks; ++b) x -= trow[b] * Z[(long long)b * chi + c];
-        Z[(long long)a * chi + c] = x / trow[a];
-      }
-    }
-    __syncthreads();
-    // Y[(c,kappa), c'] = Z[q, c'] at original column perm[q] (zero for q >= ks)
-    // W[(c,p), (c',p')] = sum_kappa F_kappa[p', p] Y[(c,kappa), c']
-    double* Y = R2o;   // reuse (r x chi)
-    for (long long e = threadIdx.x; e < (long long)r * chi; e += blockDim.x) Y[e] = 0.0;
-    __syncthreads();
-    for (long long e = threadIdx.x; e < (long long)ks * chi; e += blockDim.x) {
-      int q = (int)(e / chi), c = (int)(e % chi);
-      Y[(long long)perms[q] * chi + c] = Z[e];
-    }
+    for (int q = threadIdx.x; q < r; q += blockDim.x) order[perms[q]] = q;   // position of each original column
     __syncthreads();
     const int np = 4 * chi;
-    for (long long e = threadIdx.x; e < (long long)n * np; e += blockDim.x) {
-      int row = (int)(e / np), col = (int)(e % np);
-      int cc = row / 4, p = row % 4, c2 = col / 4, p2 = col % 4;
+    for (long long e = ct.tid; e < (long long)n * np; e += ct.nthr) {
+      const int row = (int)(e / np), col = (int)(e % np);
+      const int cc = row / 4, p = row % 4, c2 = col / 4, p2 = col % 4;
       double x = 0.0;
-      for (int kk = 0; kk < rg; ++kk) x += Fs[kk * 16 + p2 * 4 + p] * Y[(long long)(cc * rg + kk) * chi + c2];
+      for (int kk = 0; kk < rg; ++kk) {
+        const int q = order[cc * rg + kk];
+        const double y = q < ks ? Zs[side][(long long)c2 * ks + q] : 0.0;
+        x += Fs[kk * 16 + p2 * 4 + p] * y;
+      }
       W[(long long)row * it.ldw + col] = x;
     }
-    __syncthreads();
   }
 }
 
-cudaError_t launch_core(const CoreItem* items, int n_items, int* ival, int* flags_base, cudaStream_t s) {
+// four blocks of rmax^2, the cluster's flags, column norms
+size_t core_work_doubles(int rmax) { return (size_t)4 * rmax * rmax + 4 + rmax; }
+
+// CTAs per core: as many (up to eight) as leave every bond its own SMs; long cores
+// (chi_max > 32) may fill the chip three times over (the 50 bonds of a 10x10
+// colour: eight each).  A batch of many small cores runs one or two CTAs each.
+static int core_cluster(int n_items, int chimax) {
+  const int most = chimax > 32 ? 3 * 152 : 152;
+  for (int c = 8; c > 1; c /= 2)
+    if (chimax > 8 && n_items * c <= most) return c;
+  return 1;
+}
+
+cudaError_t launch_core(const CoreItem* items, int n_items, int chimax, int* ival, int* flags_base, cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
-  k_core<<<n_items, 1024, 0, s>>>(items, ival, flags_base);
-  return cudaGetLastError();
+  const int csize = core_cluster(n_items, chimax);
+  cudaError_t e = cudaFuncSetAttribute(k_core, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoreSmem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_items * csize);
+  cfg.blockDim = dim3(kCoreThreads);
+  cfg.dynamicSmemBytes = kCoreSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = csize;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, k_core, items, ival, flags_base, csize);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template cudaError_t launch_hh_level<double>(const SiteFacItem*, int, int, int, int, void* const*,

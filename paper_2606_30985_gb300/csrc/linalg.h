@@ -23,7 +23,9 @@ cudaError_t launch_form(const SiteFacItem* items, int n_items, int grid_x, const
 // by the final branch value (0 Householder, 1 Cholesky-QR, 2 handed back)
 cudaError_t launch_factor(const SiteFacItem* items, int n_items, int rmax, int nmax, int* ival,
                           cudaStream_t s, int only, int householder, unsigned long long* qcount);
-cudaError_t launch_core(const CoreItem* items, int n_items, int* ival, int* flags_base, cudaStream_t s);
+cudaError_t launch_core(const CoreItem* items, int n_items, int chimax, int* ival, int* flags_base, cudaStream_t s);
+// doubles of a bond core's workspace
+size_t core_work_doubles(int rmax);
 }  // namespace pepo
 
 namespace pepo {

@@ -454,7 +454,7 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
   size_t maxcol = 0;
   for (int col = 0; col < 4; ++col) maxcol = std::max(maxcol, I.colours[col].size());
   std::vector<double*> corework(std::max<size_t>(1, maxcol));
-  for (size_t k = 0; k < corework.size(); ++k) corework[k] = cv.take<double>((size_t)4 * rmax * rmax);
+  for (size_t k = 0; k < corework.size(); ++k) corework[k] = cv.take<double>(core_work_doubles(rmax));
 
   // ---- gate tables
   {
@@ -1434,7 +1434,7 @@ pepo_status colour_launches(pepo_ctx* c, int col) {
     pepo_status st = run_gate_wave<T>(c, G, w);
     if (st != PEPO_OK) return st;
   }
-  LAUNCH_T(K_CORE, nullptr, G.gcore[col].n, launch_core(G.gcore[col].d, G.gcore[col].n, c->d_ival, c->d_flags, c->stream));
+  LAUNCH_T(K_CORE, nullptr, G.gcore[col].n, launch_core(G.gcore[col].d, G.gcore[col].n, G.cfg.chi_max, c->d_ival, c->d_flags, c->stream));
   for (auto& w : G.gwaves[col]) {
     pepo_status st = run_gate_wave_tail<T>(c, G, w);
     if (st != PEPO_OK) return st;

@@ -46,6 +46,15 @@ def test_fp32_factor_paths_match_fp64(Lx, Ly, chi, n_thresh):
         assert max(np.max(a[k:], initial=0.0), np.max(b[k:], initial=0.0)) < 1e-5
 
 
+@pytest.mark.parametrize("scale", [1e-14, 1e14])
+def test_fp32_factor_is_scale_free(scale):
+    # a column's magnitude is divided out before its squares are summed in FP32
+    ref, _ = spectra(3, 3, 9, "fp32", 10 ** 9)
+    got, _ = spectra(3, 3, 9, "fp32", 10 ** 9, scale)
+    for a, b in zip(got, ref):
+        assert len(a) == len(b) and np.max(np.abs(a - b)) < 1e-5
+
+
 def test_nan_site_in_a_tensor_core_step_is_flagged():
     # a NaN coefficient makes its bonds' messages NaN, whose factors have rank 0: the
     # later colours' contractions then have an output leg of size 0
