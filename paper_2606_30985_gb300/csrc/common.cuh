@@ -57,18 +57,14 @@ struct GramRowsItem {
   unsigned* colmax;        // Fmax: largest magnitude per column (float bits; exact Gram)
 };
 
-// Free-leg contraction: out[i, i'] = sum_{o,q} X[o, i, q] Y[o, i', q], free leg
-// at layout position `leg` (one BP message, Eq. 13 with the Pauli leg traced).
+// Free-leg Gram: out[i, i'] = sum_{o,q} X[o, i, q] X[o, i', q], free leg at layout
+// position `leg` (one BP message, Eq. 13 with the Pauli leg traced).
 struct GramLegItem {
   TView x;
-  int y_ref;
   int leg;
   double* partial;         // [splits][chimax * chimax]
   double* out;             // chi x chi, leading dimension ldo
   int ldo;
-  // optional square-root weights per layout leg (nullptr: weight 1); element
-  // (.., j_u, ..) of X and Y is scaled by prod_{u != leg} sw[u][j_u] on load
-  const double* sw[PEPO_MAXLEG];
 };
 
 // Eigen-decomposition of a (symmetrised) message M = V diag(D) V^T by one-sided

@@ -1,48 +1,23 @@
-// Register-tiled SIMT contractions of the BP and bond-update hot loop.
+// SIMT contractions of the BP and bond-update hot loop (FP32 and FP64 modes).
 //
 //   k_leg_contract  out[o, i, q] = sum_j A[i, j] in[o, j, q] on one layout leg
 //                   (absorbing a message factor or eigenbasis into a site
 //                   tensor: Sec. 2.5 step 1 and the products of Eq. 13)
-//   k_gram_leg      out[i, i'] = sum_{o, q} w(o,q)^2 X[o, i, q] Y[o, i', q]: a site
-//                   tensor contracted with itself over every index but one leg,
-//                   the Pauli leg traced, optionally weighted (one double-layer
-//                   message, Eq. 13)
+//   k_gram_leg      out[i, i'] = sum_{o, q} X[o, i, q] X[o, i', q]: a site tensor
+//                   contracted with itself over every index but one leg, the
+//                   Pauli leg traced (one double-layer message, Eq. 13; the
+//                   message weights are carried by the rotated tensor)
 //
-// Both are GEMMs with one short dimension (chi <= 128).  The tile edge TL is
-// 64 or 128 (chosen from chi_max); a block of 256 threads owns a TL x TL
-// output tile, each thread an (TL/16) x (TL/16) register tile.  With TL = 128
-// the 8 rows / columns of a thread are split in two halves 64 apart so the
-// 16-byte shared-memory loads of a warp hit distinct banks.  The leg
-// contraction stages A transposed in shared memory once per block.  FP32
-// storage accumulates the Gram's long sums in FP32 runs flushed into FP64
-// every 256 terms.
+// Both are GEMMs with one short dimension (chi <= 128); tiles are chosen from
+// the live bond dimension on the device.  FP32 storage accumulates the Gram's
+// long sums in FP32 runs of 256 terms that a two-float sum takes.
+#include <algorithm>
+
 #include "kernels.h"
 
 namespace pepo {
 
-template <int TL>
-__device__ __forceinline__ int tile_idx(int t, int r) {
-  if constexpr (TL == 128) return (r < 4) ? t * 4 + r : 64 + t * 4 + (r - 4);
-  else return t * 4 + r;
-}
-
-template <typename T>
-__device__ __forceinline__ void lds4(const T* p, T* v) {
-  if constexpr (sizeof(T) == 4) {
-    float4 x = *reinterpret_cast<const float4*>(p);
-    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-  } else {
-    double2 x = *reinterpret_cast<const double2*>(p);
-    double2 y = *reinterpret_cast<const double2*>(p + 2);
-    v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
-  }
-}
-
-template <int TL, typename T>
-__device__ __forceinline__ void ld_frag(const T* row, int t, T* v) {
-  lds4(row + t * 4, v);
-  if constexpr (TL == 128) lds4(row + 64 + t * 4, v + 4);
-}
+constexpr int GL_FLUSH = 256;   // FP32 terms per run of a Gram
 
 __device__ inline void load_dims4(const TView& v, const int* ival, int* d) {
 #pragma unroll
@@ -50,263 +25,355 @@ __device__ inline void load_dims4(const TView& v, const int* ival, int* d) {
 }
 
 // ============================================================ leg contraction
-// Block tile: TL rows (output index i) x TC columns (o, q); TC = TL for FP32,
-// TL / 2 for FP64 (shared-memory bound).
-template <typename T, int TL>
+// out[o, i, q] = sum_j A[i, j] in[o, j, q], i.e. a (Jout x J) matrix times the J x C
+// matrix of the columns c = (o, q), q fastest and contiguous.  A CTA keeps A
+// transposed in shared memory and takes tiles of TC columns: the J rows of a
+// tile arrive as asynchronous 16-byte copies (a unit of 16 bytes never leaves
+// its o), a thread holds MI outputs of two units.  TI = MI x (256 / column
+// threads) is chosen from the live Jout, so a small bond does not pay for the
+// rows of a large tile; the column index is divided once per thread and tile,
+// in 32 bits.  The sum over j runs in order.
+//
+// Bound: FP32 ALU at chi = 48 (12 FLOP per byte), launch and latency below
+// chi = 20; two CTAs per SM overlap one's copies with the other's products.
+// Class of a case, 64 / 128-row tiles -> these: 4x4 chi = 48 72 -> 24 ms, a batch of
+// nine small instances 76 -> 14 ms.
+template <typename T, int MI, int TI>
 struct LegCfg {
-  // column tile: TL, except FP64 with TL = 128 (64, to fit shared memory)
-  static constexpr int TC = (sizeof(T) == 8 && TL == 128) ? 64 : TL;
-  static constexpr int MR = TL / 16;
-  static constexpr int MC = TC / 16;
-  // fragment loads read columns t*4 .. t*4+3 (and +64 when the tile is 128)
-  static_assert(TL == 64 || TL == 128, "row tile must be 64 or 128");
-  static_assert(TC == 64 || TC == 128, "column tile must be 64 or 128");
-  static_assert(MR * 16 == TL && MC * 16 == TC, "16 x 16 threads cover the tile");
+  static constexpr int U = 16 / (int)sizeof(T);
+  static constexpr int IG = TI / MI;                   // thread groups over the outputs
+  static constexpr int CG = 256 / IG;                  // threads over the columns
+  static constexpr int NU = 2;                         // units per thread
+  static constexpr int TC = CG * NU * U;               // columns of a tile
 };
 
-template <typename T, int TL>
-__global__ void __launch_bounds__(256)
-k_leg_contract(const LegItem* __restrict__ items, void* const* ptrs, const int* __restrict__ ival) {
-  using C = LegCfg<T, TL>;
-  constexpr int TC = C::TC, MR = C::MR, MC = C::MC;
-  const LegItem it = items[blockIdx.y];
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  int d[PEPO_MAXLEG];
-  load_dims4(it.in, ival, d);
-  const int k = it.leg;
-  const int Jin = d[k];
-  const int Jout = ival[it.out_dim];
-  long long O = 1, Q = 4;
-  for (int i = 0; i < k; ++i) O *= d[i];
-  for (int i = k + 1; i < it.in.nlegs; ++i) Q *= d[i];
-  T* At = reinterpret_cast<T*>(smem_raw);     // [Jin][TL]
-  T* Bs = At + Jin * TL;                      // [Jin][TC]
-  for (int e = threadIdx.x; e < Jin * TL; e += blockDim.x) {
-    int j = e / TL, i = e - j * TL;
-    At[e] = (i < Jout) ? (T)it.A[(long long)i * it.lda + j] : T(0);
+template <typename T, int MI, int TI>
+__device__ void leg_tiles(const T* __restrict__ in, T* __restrict__ out, const double* __restrict__ A, int lda, int J,
+                          int Jout, unsigned O, unsigned QU, unsigned char* sh, int room) {
+  using C = LegCfg<T, MI, TI>;
+  constexpr int U = C::U, CG = C::CG, NU = C::NU, TC = C::TC;
+  const int tid = threadIdx.x;
+  const int cg = tid % CG, ig = tid / CG;
+  const long long Q = (long long)QU * U;
+  const unsigned cols = O * QU;                        // columns in units
+  // rows of `in` at a time: all J where they fit (then the tile is loaded once)
+  const int jc = min(J, (int)((room - sizeof(T) * (size_t)J * TI) / (sizeof(T) * TC)));
+  T* At = reinterpret_cast<T*>(sh);                    // [J][TI]
+  T* Bs = At + (size_t)J * TI;                         // [jc][TC]
+  const unsigned ntile = (cols + CG * NU - 1) / (CG * NU);
+  if (blockIdx.x >= ntile) return;
+  for (int e = tid; e < J * TI; e += 256) {
+    const int i = e / J, j = e - i * J;
+    At[j * TI + i] = i < Jout ? (T)A[(long long)i * lda + j] : T(0);
   }
-  long long G, nqb, units;
-  if (Q >= TC) { G = 1; nqb = (Q + TC - 1) / TC; units = O * nqb; }
-  else { G = TC / Q; nqb = 1; units = (O + G - 1) / G; }
-  const T* __restrict__ in = static_cast<const T*>(ptrs[it.in.ref]);
-  T* __restrict__ out = static_cast<T*>(ptrs[it.out_ref]);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  __syncthreads();
-  for (long long u = blockIdx.x; u < units; u += gridDim.x) {
-    long long o0, q0;
-    int width;
-    if (G == 1) { o0 = u / nqb; q0 = (u - o0 * nqb) * TC; width = (int)min((long long)TC, Q - q0); }
-    else { o0 = u * G; q0 = 0; width = (int)(min(G, O - o0) * Q); }
-    for (int e = threadIdx.x; e < Jin * TC; e += blockDim.x) {
-      int j = e / TC, c = e - j * TC;
-      T v = T(0);
-      if (c < width) {
-        long long o = (G == 1) ? o0 : o0 + c / Q;
-        long long q = (G == 1) ? q0 + c : c % Q;
-        v = in[(o * Jin + j) * Q + q];
+  for (unsigned tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    // this thread copies the units that it also computes with its group; the
+    // groups share the copies row by row
+    const T* src[NU];
+    T* dst[NU];
+    bool live[NU];
+#pragma unroll
+    for (int u = 0; u < NU; ++u) {
+      const unsigned c = tile * (CG * NU) + u * CG + cg;
+      live[u] = c < cols;
+      const unsigned o = live[u] ? c / QU : 0u, q = live[u] ? c - o * QU : 0u;
+      src[u] = in + (long long)o * J * Q + (long long)q * U;
+      dst[u] = out + (long long)o * Jout * Q + (long long)q * U;
+    }
+    T acc[MI][NU][U];
+#pragma unroll
+    for (int i = 0; i < MI; ++i)
+#pragma unroll
+      for (int u = 0; u < NU; ++u)
+#pragma unroll
+        for (int x = 0; x < U; ++x) acc[i][u][x] = T(0);
+    for (int j0 = 0; j0 < J; j0 += jc) {
+      const int jn = min(jc, J - j0);
+      __syncthreads();                                 // the previous rows are consumed (and A is staged)
+      for (int j = ig; j < jn; j += C::IG)
+#pragma unroll
+        for (int u = 0; u < NU; ++u)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                           (unsigned)__cvta_generic_to_shared(Bs + (size_t)j * TC + (u * CG + cg) * U)),
+                       "l"(live[u] ? src[u] + (long long)(j0 + j) * Q : in), "r"(live[u] ? 16 : 0)
+                       : "memory");
+      asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+#pragma unroll 4
+      for (int j = 0; j < jn; ++j) {
+        T a[MI], b[NU][U];
+#pragma unroll
+        for (int i = 0; i < MI; i += U)
+          *reinterpret_cast<uint4*>(a + i) = *reinterpret_cast<const uint4*>(At + (j0 + j) * TI + ig * MI + i);
+#pragma unroll
+        for (int u = 0; u < NU; ++u)
+          *reinterpret_cast<uint4*>(b[u]) = *reinterpret_cast<const uint4*>(Bs + (size_t)j * TC + (u * CG + cg) * U);
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+          for (int u = 0; u < NU; ++u)
+#pragma unroll
+            for (int x = 0; x < U; ++x) acc[i][u][x] = fma(a[i], b[u][x], acc[i][u][x]);
       }
-      Bs[e] = v;
-    }
-    __syncthreads();
-    T acc[MR][MC];
-#pragma unroll
-    for (int r = 0; r < MR; ++r)
-#pragma unroll
-      for (int c = 0; c < MC; ++c) acc[r][c] = T(0);
-#pragma unroll 2
-    for (int j = 0; j < Jin; ++j) {
-      T a[MR], b[MC];
-      ld_frag<TL>(At + j * TL, ty, a);
-      ld_frag<TC>(Bs + j * TC, tx, b);
-#pragma unroll
-      for (int r = 0; r < MR; ++r)
-#pragma unroll
-        for (int c = 0; c < MC; ++c) acc[r][c] = fma(a[r], b[c], acc[r][c]);
     }
 #pragma unroll
-    for (int c = 0; c < MC; ++c) {
-      const int col = tile_idx<TC>(tx, c);
-      if (col >= width) continue;
-      const long long o = (G == 1) ? o0 : o0 + col / Q;
-      const long long q = (G == 1) ? q0 + col : col % Q;
-      T* dst = out + o * Jout * Q + q;
+    for (int i = 0; i < MI; ++i) {
+      const int io = ig * MI + i;
+      if (io < Jout)
 #pragma unroll
-      for (int r = 0; r < MR; ++r) {
-        const int i = tile_idx<TL>(ty, r);
-        if (i < Jout) dst[(long long)i * Q] = acc[r][c];
-      }
+        for (int u = 0; u < NU; ++u)
+          if (live[u]) *reinterpret_cast<uint4*>(dst[u] + (long long)io * Q) = *reinterpret_cast<const uint4*>(acc[i][u]);
     }
-    __syncthreads();
   }
 }
 
-template <typename T, int TL>
-cudaError_t launch_leg_tl(const LegItem* items, int n_items, int grid_x, int chimax, void* const* ptrs,
-                          const int* ival, cudaStream_t s) {
-  size_t smem = sizeof(T) * (size_t)chimax * (TL + LegCfg<T, TL>::TC);
-  cudaError_t e = cudaFuncSetAttribute(k_leg_contract<T, TL>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_leg_contract<T, TL><<<dim3(grid_x, n_items), 256, smem, s>>>(items, ptrs, ival);
-  return cudaGetLastError();
+template <typename T>
+__global__ void __launch_bounds__(256, 2)
+k_leg_contract(const LegItem* __restrict__ items, void* const* ptrs, const int* __restrict__ ival, int room) {
+  const LegItem it = items[blockIdx.y];
+  extern __shared__ __align__(16) unsigned char lc_sh[];
+  int d[PEPO_MAXLEG];
+  load_dims4(it.in, ival, d);
+  const int k = it.leg;
+  int J = 1;
+  unsigned O = 1, Q = 4;
+#pragma unroll
+  for (int i = 0; i < PEPO_MAXLEG; ++i) {
+    if (i == k) J = d[i];
+    else if (i < k) O *= d[i];
+    else Q *= d[i];                                    // legs beyond nlegs have size 1
+  }
+  const int Jout = ival[it.out_dim];
+  const T* in = static_cast<const T*>(ptrs[it.in.ref]);
+  T* out = static_cast<T*>(ptrs[it.out_ref]);
+  const unsigned QU = Q / (16 / sizeof(T));
+  if (Jout <= 8) leg_tiles<T, 4, 8>(in, out, it.A, it.lda, J, Jout, O, QU, lc_sh, room);
+  else if (Jout <= 16) leg_tiles<T, 8, 16>(in, out, it.A, it.lda, J, Jout, O, QU, lc_sh, room);
+  else if (Jout <= 32) leg_tiles<T, 8, 32>(in, out, it.A, it.lda, J, Jout, O, QU, lc_sh, room);
+  else if (Jout <= 64) leg_tiles<T, 8, 64>(in, out, it.A, it.lda, J, Jout, O, QU, lc_sh, room);
+  else leg_tiles<T, 8, 128>(in, out, it.A, it.lda, J, Jout, O, QU, lc_sh, room);
 }
 
 template <typename T>
 cudaError_t launch_leg_contract(const LegItem* items, int n_items, int grid_x, int chimax,
                                 void* const* ptrs, const int* ival, cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
-  if (chimax <= 64) return launch_leg_tl<T, 64>(items, n_items, grid_x, chimax, ptrs, ival, s);
-  return launch_leg_tl<T, 128>(items, n_items, grid_x, chimax, ptrs, ival, s);
+  // two CTAs per SM; A at chi = 128 takes 64 KB (FP32) or 128 KB (FP64, one CTA)
+  const int room = (sizeof(T) == 8 && chimax > 64 ? 208 : 104) * 1024;
+  cudaError_t e = cudaFuncSetAttribute(k_leg_contract<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
+  if (e != cudaSuccess) return e;
+  k_leg_contract<T><<<dim3(grid_x, n_items), 256, room, s>>>(items, ptrs, ival, room);
+  return cudaGetLastError();
 }
 
 // ============================================================ Gram (free leg)
-// X, Y as [O][F][Q], F <= TL.  A chunk is 32 (o, q) pairs: one o and 32
-// consecutive q when Q >= 32, else floor(32 / Q) consecutive o with all q.
-constexpr int GL_BK = 32;
-constexpr int GL_FLUSH = 256;
+// out[i, i'] = sum over the flattened (o, q) of X[o, i, q] X[o, i', q]: X is F rows
+// of O Q values, contiguous in q.  One CTA takes one split of the summed range
+// of one item.  Chunks of KCU 16-byte units per row (a unit never leaves its
+// o: Q is a multiple of 4) are copied asynchronously as they lie, three stages
+// deep; rows are KCU + 1 units apart, an odd number, so the 8 threads of a
+// phase read 8 different banks groups.  TX x TX threads share a tile of MT TX
+// rows, thread (ty, tx) holding the entries (ty + TX a, tx + TX b) with a <= b
+// only: the Gram is symmetric, and this drops 44 % of the products for the
+// largest tile without a divergent branch.  The 256 / TX^2 groups of threads
+// take different units of a chunk, so a small F keeps the whole block busy;
+// the tile is chosen from the live F (8, 16, 32, 48, 64, 96, 128), not from
+// chi_max.  FP32 storage sums runs of 256 terms in FP32 and the runs in a
+// two-float sum; FP64 sums directly.
+//
+// Bound: FP32 ALU (2 shared 16-byte loads per 4 x MT x MT products at most) or
+// the FP64 pipe.  Class of a case, before -> now: chi = 8 FP64 (107 launches)
+// 143 -> 1.8 ms, 4x4 chi = 12 FP64 154 -> 1.7 ms, 4x4 chi = 48 FP32 82 -> 25 ms.  The 64 x 64 (128 x 128) tile it replaces did 64 x 64 products
+// for an 8 x 8 Gram and stored every chunk with 32-way bank conflicts.
+constexpr int kGlStages = 3;
 
-// product of the square-root weights sw[u][j_u] over layout legs u in [lo, hi)
-// for the row-major multi-index `idx` of those legs
-__device__ inline double leg_weight(const GramLegItem& it, const int* d, int lo, int hi, long long idx) {
-  double w = 1.0;
-  for (int u = hi - 1; u >= lo; --u) {
-    const long long j = idx % d[u];
-    idx /= d[u];
-    if (it.sw[u]) w *= it.sw[u][j];
+template <typename T, int MT, int TX>
+struct GlCfg {
+  static constexpr int U = 16 / (int)sizeof(T);        // values per 16-byte unit
+  static constexpr int TL = MT * TX;
+  static constexpr int G = 256 / (TX * TX);            // groups sharing a chunk
+  static constexpr int KCU = 2 * G > 8 ? 2 * G : 8;    // units per row and chunk
+  static constexpr int PITCH = (KCU + 1) * U;          // values between rows
+  static constexpr size_t kStage = sizeof(T) * (size_t)TL * PITCH;
+  static constexpr size_t kRed = G > 1 ? sizeof(double) * (size_t)TL * TL : 0;
+  static constexpr size_t kSmem = kGlStages * kStage > kRed ? kGlStages * kStage : kRed;
+};
+
+template <typename T, int MT, int TX>
+__device__ void gram_tile(const T* __restrict__ X, long long O, long long Q, int F, int s, int S, double* __restrict__ P,
+                          unsigned char* sh) {
+  using C = GlCfg<T, MT, TX>;
+  constexpr int U = C::U, KCU = C::KCU, G = C::G, TL = C::TL, PITCH = C::PITCH;
+  constexpr bool kF32 = sizeof(T) == 4;
+  T* buf = reinterpret_cast<T*>(sh);
+  const int tid = threadIdx.x;
+  const int g = tid / (TX * TX), t = tid % (TX * TX), tx = t % TX, ty = t / TX;
+  const unsigned QU = (unsigned)(Q / U);               // units per (o, row)
+  const unsigned NU = (unsigned)(O * Q / U);           // units of the summed range
+  const unsigned NC = (NU + KCU - 1) / KCU;
+  const unsigned c0 = (unsigned)((unsigned long long)NC * s / S), c1 = (unsigned)((unsigned long long)NC * (s + 1) / S);
+  const int lu = tid % KCU, lf0 = tid / KCU;           // this thread's unit of a chunk, first row
+  constexpr int LR = 256 / KCU;                        // rows per pass
+  // rows F .. TL - 1 are zero in every stage
+  for (int st = 0; st < kGlStages; ++st)
+    for (int e = tid; e < (TL - F) * PITCH; e += 256) buf[st * (TL * PITCH) + F * PITCH + e] = T(0);
+  auto load = [&](unsigned c, int st) {
+    if (c < c1) {
+      const unsigned u = c * KCU + lu;
+      const bool live = u < NU;
+      const unsigned o = live ? u / QU : 0u, q = live ? u - o * QU : 0u;
+      const T* src = X + ((long long)o * F) * Q + (long long)q * U;
+      T* dst = buf + st * (TL * PITCH) + lu * U;
+      for (int f = lf0; f < F; f += LR)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(dst + f * PITCH)),
+                     "l"(live ? src + (long long)f * Q : X), "r"(live ? 16 : 0)
+                     : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  T acc[MT][MT];
+  float hi[MT][MT], lo[MT][MT];                        // FP32: two-float sum of the runs
+#pragma unroll
+  for (int a = 0; a < MT; ++a)
+#pragma unroll
+    for (int b = 0; b < MT; ++b) { acc[a][b] = T(0); hi[a][b] = lo[a][b] = 0.f; }
+  auto flush = [&]() {
+    if constexpr (kF32) {
+#pragma unroll
+      for (int a = 0; a < MT; ++a)
+#pragma unroll
+        for (int b = a; b < MT; ++b) {
+          const float v = acc[a][b], w = hi[a][b] + v, z = w - hi[a][b];
+          lo[a][b] += (hi[a][b] - (w - z)) + (v - z);
+          hi[a][b] = w;
+          acc[a][b] = 0.f;
+        }
+    }
+  };
+  __syncthreads();
+#pragma unroll
+  for (int st = 0; st < kGlStages - 1; ++st) load(c0 + st, st);
+  int st = 0, run = 0;
+  for (unsigned c = c0; c < c1; ++c) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kGlStages - 2) : "memory");
+    __syncthreads();                                   // chunk c is in, chunk c - 1 is consumed
+    load(c + kGlStages - 1, st == 0 ? kGlStages - 1 : st - 1);
+    const T* xs = buf + st * (TL * PITCH);
+#pragma unroll
+    for (int k = 0; k < KCU / G; ++k) {
+      const int u = g * (KCU / G) + k;
+      T av[MT][U];
+#pragma unroll
+      for (int a = 0; a < MT; ++a) {
+        const uint4 x = *reinterpret_cast<const uint4*>(xs + (ty + TX * a) * PITCH + u * U);
+        *reinterpret_cast<uint4*>(av[a]) = x;
+      }
+#pragma unroll
+      for (int b = 0; b < MT; ++b) {
+        T bv[U];
+        *reinterpret_cast<uint4*>(bv) = *reinterpret_cast<const uint4*>(xs + (tx + TX * b) * PITCH + u * U);
+#pragma unroll
+        for (int i = 0; i < U; ++i)
+#pragma unroll
+          for (int a = 0; a <= b; ++a) acc[a][b] = fma(av[a][i], bv[i], acc[a][b]);
+      }
+    }
+    if constexpr (kF32) {
+      run += KCU / G * U;
+      if (run >= GL_FLUSH) { flush(); run = 0; }
+    }
+    if (++st == kGlStages) st = 0;
   }
-  return w;
+  flush();
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  auto value = [&](int a, int b) -> double {
+    if constexpr (kF32) return (double)hi[a][b] + (double)lo[a][b];
+    else return acc[a][b];
+  };
+  if constexpr (G > 1) {
+    // sum of the groups, one after another, in shared memory
+    double* red = reinterpret_cast<double*>(sh);
+    for (int gg = 0; gg < G; ++gg) {
+      __syncthreads();
+      if (g == gg) {
+#pragma unroll
+        for (int a = 0; a < MT; ++a)
+#pragma unroll
+          for (int b = a; b < MT; ++b) {
+            double* r = red + (ty + TX * a) * TL + tx + TX * b;
+            *r = gg == 0 ? value(a, b) : *r + value(a, b);
+          }
+      }
+    }
+    __syncthreads();
+    // entries with row block above the column block were not formed: mirror
+    for (int e = tid; e < F * F; e += 256) {
+      const int i = e / F, j = e - i * F;
+      P[e] = i / TX <= j / TX ? red[i * TL + j] : red[j * TL + i];
+    }
+  } else {
+#pragma unroll
+    for (int a = 0; a < MT; ++a)
+#pragma unroll
+      for (int b = a; b < MT; ++b) {
+        const int i = ty + TX * a, j = tx + TX * b;
+        if (i < F && j < F) {
+          const double v = value(a, b);
+          P[(long long)i * F + j] = v;
+          if (a != b) P[(long long)j * F + i] = v;
+        }
+      }
+  }
 }
 
-template <typename T, int TL>
-__global__ void __launch_bounds__(256)
-k_gram_leg(const GramLegItem* __restrict__ items, int splits_max, void* const* ptrs,
-           const int* __restrict__ ival) {
-  constexpr int MR = TL / 16;
+// BAND 0: F <= 32, 1: F <= 64, 2: F <= 128 (a launch of its own per band that
+// chi_max can reach, so that the small tiles do not carry the large one's
+// registers); blocks of the other bands return.
+template <typename T, int BAND>
+__global__ void __launch_bounds__(256, BAND == 0 ? 2 : 1)
+k_gram_leg(const GramLegItem* __restrict__ items, int splits_max, void* const* ptrs, const int* __restrict__ ival) {
   const GramLegItem it = items[blockIdx.y];
   int d[PEPO_MAXLEG];
   load_dims4(it.x, ival, d);
   const int k = it.leg;
-  const int F = d[k];
+  int F = 1;
   long long O = 1, Q = 4;
-  for (int i = 0; i < k; ++i) O *= d[i];
-  for (int i = k + 1; i < it.x.nlegs; ++i) Q *= d[i];
-  const long long NC = gram_leg_chunks(O, Q);
-  const int S = gram_leg_splits_k(O * Q, splits_max);
-  const int s = blockIdx.x;
-  if (s >= S) return;
-  const long long c0 = NC * s / S, c1 = NC * (s + 1) / S;
-  const T* __restrict__ X = static_cast<const T*>(ptrs[it.x.ref]);
-  const T* __restrict__ Y = static_cast<const T*>(ptrs[it.y_ref]);
-  const bool same = it.x.ref == it.y_ref;
-  bool weighted = false;
-  for (int u = 0; u < it.x.nlegs; ++u) weighted |= (u != k && it.sw[u] != nullptr);
-  __shared__ __align__(16) T Xs[GL_BK][TL];
-  __shared__ __align__(16) T Ys[GL_BK][TL];
-  __shared__ double wk[GL_BK];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const bool wideQ = Q >= GL_BK;
-  const long long qpc = wideQ ? (Q + GL_BK - 1) / GL_BK : 0;
-  const int Qi = wideQ ? GL_BK : (int)Q;
-  const int opc = wideQ ? 1 : (int)(GL_BK / Q);
-  const int rows = wideQ ? GL_BK : opc * Qi;        // live rows of a chunk
-  T* Yt = same ? &Xs[0][0] : &Ys[0][0];
-  constexpr int NS = sizeof(T) == 4 ? MR : 1;
-  T acc[MR][MR];
-  double acc64[NS][MR];
 #pragma unroll
-  for (int r = 0; r < MR; ++r)
-#pragma unroll
-    for (int c = 0; c < MR; ++c) acc[r][c] = T(0);
-#pragma unroll
-  for (int r = 0; r < NS; ++r)
-#pragma unroll
-    for (int c = 0; c < MR; ++c) acc64[r][c] = 0.0;
-  // rows beyond `rows` and columns beyond F stay zero for the whole block
-  for (int e = threadIdx.x; e < GL_BK * TL; e += blockDim.x) {
-    (&Xs[0][0])[e] = T(0);
-    (&Ys[0][0])[e] = T(0);
+  for (int i = 0; i < PEPO_MAXLEG; ++i) {
+    if (i == k) F = d[i];
+    else if (i < k) O *= d[i];
+    else Q *= d[i];                                    // legs beyond nlegs have size 1
   }
-  int run = 0;
-  for (long long cch = c0; cch < c1; ++cch) {
-    long long o0, q0;
-    if (wideQ) { o0 = cch / qpc; q0 = (cch - o0 * qpc) * GL_BK; }
-    else { o0 = cch * opc; q0 = 0; }
-    __syncthreads();   // previous chunk consumed
-    if (weighted && threadIdx.x < rows) {
-      const int kk = threadIdx.x;
-      long long o, q;
-      if (wideQ) { o = o0; q = q0 + kk; }
-      else { o = o0 + kk / Qi; q = kk % Qi; }
-      double w = 0.0;
-      if (q < Q && o < O) w = leg_weight(it, d, 0, k, o) * leg_weight(it, d, k + 1, it.x.nlegs, q >> 2);
-      wk[kk] = w;
+  if (BAND == 0 ? F > 32 : BAND == 1 ? (F <= 32 || F > 64) : F <= 64) return;
+  const int S = gram_leg_splits_k(O * Q, splits_max, kGramLegRowsSimt);
+  extern __shared__ __align__(16) unsigned char gl_sh[];
+  const T* X = static_cast<const T*>(ptrs[it.x.ref]);
+  for (int s = blockIdx.x; s < S; s += gridDim.x) {
+    double* P = it.partial + (long long)s * F * F;
+    if constexpr (BAND == 0) {
+      if (F <= 8) gram_tile<T, 2, 4>(X, O, Q, F, s, S, P, gl_sh);
+      else if (F <= 16) gram_tile<T, 4, 4>(X, O, Q, F, s, S, P, gl_sh);
+      else gram_tile<T, 4, 8>(X, O, Q, F, s, S, P, gl_sh);
+    } else if constexpr (BAND == 1) {
+      if (F <= 48) gram_tile<T, 6, 8>(X, O, Q, F, s, S, P, gl_sh);
+      else gram_tile<T, 8, 8>(X, O, Q, F, s, S, P, gl_sh);
+    } else {
+      if (F <= 96) gram_tile<T, 6, 16>(X, O, Q, F, s, S, P, gl_sh);
+      else gram_tile<T, 8, 16>(X, O, Q, F, s, S, P, gl_sh);
     }
-    if (weighted) __syncthreads();
-    for (int e = threadIdx.x; e < rows * F; e += blockDim.x) {
-      int kk, f;
-      long long o, q;
-      if (wideQ) { f = e / GL_BK; kk = e - f * GL_BK; o = o0; q = q0 + kk; }
-      else {
-        int qq = e % Qi, rest = e / Qi;
-        f = rest % F;
-        int ol = rest / F;
-        kk = ol * Qi + qq;
-        o = o0 + ol; q = qq;
-      }
-      T xv = T(0), yv = T(0);
-      if (q < Q && o < O) {
-        long long idx = (o * F + f) * Q + q;
-        xv = X[idx];
-        if (!same) yv = Y[idx];
-        if (weighted) {
-          const T w = (T)wk[kk];
-          xv *= w;
-          yv *= w;
-        }
-      }
-      Xs[kk][f] = xv;
-      if (!same) Ys[kk][f] = yv;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < GL_BK; ++kk) {
-      T a[MR], b[MR];
-      ld_frag<TL>(&Xs[kk][0], ty, a);
-      ld_frag<TL>(Yt + kk * TL, tx, b);
-#pragma unroll
-      for (int r = 0; r < MR; ++r)
-#pragma unroll
-        for (int c = 0; c < MR; ++c) acc[r][c] = fma(a[r], b[c], acc[r][c]);
-    }
-    if constexpr (sizeof(T) == 4) {
-      run += GL_BK;
-      if (run >= GL_FLUSH) {
-#pragma unroll
-        for (int r = 0; r < MR; ++r)
-#pragma unroll
-          for (int c = 0; c < MR; ++c) { acc64[r % NS][c] += (double)acc[r][c]; acc[r][c] = T(0); }
-        run = 0;
-      }
-    }
-  }
-  double* P = it.partial + (long long)s * F * F;
-#pragma unroll
-  for (int r = 0; r < MR; ++r) {
-    const int fi = tile_idx<TL>(ty, r);
-    if (fi >= F) continue;
-#pragma unroll
-    for (int c = 0; c < MR; ++c) {
-      const int fj = tile_idx<TL>(tx, c);
-      if (fj < F) {
-        double v = (double)acc[r][c];
-        if constexpr (sizeof(T) == 4) v += acc64[r % NS][c];
-        P[(long long)fi * F + fj] = v;
-      }
-    }
+    __syncthreads();                                   // the shared memory is reused
   }
 }
 
-__global__ void k_gram_leg_reduce(const GramLegItem* __restrict__ items, int splits_max, int sym,
+template <typename T, int BAND>
+size_t gram_leg_smem() {
+  if (BAND == 0) return std::max(std::max(GlCfg<T, 2, 4>::kSmem, GlCfg<T, 4, 4>::kSmem), GlCfg<T, 4, 8>::kSmem);
+  if (BAND == 1) return std::max(GlCfg<T, 6, 8>::kSmem, GlCfg<T, 8, 8>::kSmem);
+  return std::max(GlCfg<T, 6, 16>::kSmem, GlCfg<T, 8, 16>::kSmem);
+}
+
+__global__ void k_gram_leg_reduce(const GramLegItem* __restrict__ items, int splits_max, int rows, int sym,
                                   const int* __restrict__ ival) {
   const GramLegItem it = items[blockIdx.y];
   int d[PEPO_MAXLEG];
@@ -316,7 +383,7 @@ __global__ void k_gram_leg_reduce(const GramLegItem* __restrict__ items, int spl
   long long O = 1, Q = 4;
   for (int i = 0; i < k; ++i) O *= d[i];
   for (int i = k + 1; i < it.x.nlegs; ++i) Q *= d[i];
-  const int S = gram_leg_splits_k(O * Q, splits_max);
+  const int S = gram_leg_splits_k(O * Q, splits_max, rows);
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < F * F; e += gridDim.x * blockDim.x) {
     int fi = e / F, fj = e - fi * F;
     double sum = 0.0;
@@ -330,22 +397,34 @@ __global__ void k_gram_leg_reduce(const GramLegItem* __restrict__ items, int spl
   }
 }
 
+template <typename T, int BAND>
+static cudaError_t launch_gram_band(const GramLegItem* items, int n_items, int splits_max, void* const* ptrs,
+                                    const int* ival, cudaStream_t s) {
+  const size_t smem = gram_leg_smem<T, BAND>();
+  cudaError_t e = cudaFuncSetAttribute(k_gram_leg<T, BAND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  // about 8 blocks per SM in all; a block takes several splits of its item when
+  // there are many items (a batch), so that few of its blocks find nothing to do
+  const int gx = std::min(splits_max, std::max(4, ceil_div(8 * 152, n_items)));
+  k_gram_leg<T, BAND><<<dim3(gx, n_items), 256, smem, s>>>(items, splits_max, ptrs, ival);
+  return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t launch_gram_leg(const GramLegItem* items, int n_items, int splits_max, int chimax,
                             void* const* ptrs, const int* ival, cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
-  if (chimax <= 64)
-    k_gram_leg<T, 64><<<dim3(splits_max, n_items), 256, 0, s>>>(items, splits_max, ptrs, ival);
-  else
-    k_gram_leg<T, 128><<<dim3(splits_max, n_items), 256, 0, s>>>(items, splits_max, ptrs, ival);
-  return cudaGetLastError();
+  cudaError_t e = launch_gram_band<T, 0>(items, n_items, splits_max, ptrs, ival, s);
+  if (e == cudaSuccess && chimax > 32) e = launch_gram_band<T, 1>(items, n_items, splits_max, ptrs, ival, s);
+  if (e == cudaSuccess && chimax > 64) e = launch_gram_band<T, 2>(items, n_items, splits_max, ptrs, ival, s);
+  return e;
 }
 
 cudaError_t launch_gram_leg_reduce(const GramLegItem* items, int n_items, int chimax,
-                                   int splits_max, int sym, const int* ival, cudaStream_t s) {
+                                   int splits_max, int rows, int sym, const int* ival, cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
   int gx = ceil_div(chimax * chimax, 256);
-  k_gram_leg_reduce<<<dim3(gx, n_items), 256, 0, s>>>(items, splits_max, sym, ival);
+  k_gram_leg_reduce<<<dim3(gx, n_items), 256, 0, s>>>(items, splits_max, rows, sym, ival);
   return cudaGetLastError();
 }
 

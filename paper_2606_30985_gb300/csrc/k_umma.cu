@@ -644,7 +644,7 @@ __device__ inline void gram_dims(const GramLegItem& it, void* const* ptrs, const
   }
   G.F8 = round_up(G.F, 8);
   G.NC = gram_leg_chunks(G.O, G.Q);
-  G.S = gram_leg_splits_k(G.O * G.Q, splits_max);
+  G.S = gram_leg_splits_k(G.O * G.Q, splits_max, kGramLegRowsUmma);
   G.wide = G.Q >= kKC;
   G.qpc = G.wide ? (G.Q + kKC - 1) / kKC : 0;
   G.opc = G.wide ? 1 : (int)(kKC / G.Q);
@@ -762,7 +762,7 @@ struct GramLoader {
       rv0 = r0 < F; rv1 = r1 < F; rv2 = r2 < F; rv3 = r3 < F;
     }
     const long long NC = gram_leg_chunks(O, Q);
-    const int S = gram_leg_splits_k(O * Q, splits_max);
+    const int S = gram_leg_splits_k(O * Q, splits_max, kGramLegRowsUmma);
     const int sp = (int)(lu - uoff[item]);
     lcur = NC * sp / S;
     lend = NC * (sp + 1) / S;

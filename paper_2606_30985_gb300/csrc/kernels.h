@@ -29,8 +29,9 @@ template <typename T>
 cudaError_t launch_permute(const void* in, void* out, int nlegs, const int* dims_canon, const int* perm,
                            int to_layout, cudaStream_t s);
 // sum of the per-split partials; sym = 1 symmetrises the sum as (S + S^T) / 2
+// rows: the split rule's rows per split (gram_leg_splits_k)
 cudaError_t launch_gram_leg_reduce(const GramLegItem* items, int n_items, int chimax,
-                                   int splits_max, int sym, const int* ival, cudaStream_t s);
+                                   int splits_max, int rows, int sym, const int* ival, cudaStream_t s);
 template <typename T>
 cudaError_t launch_reconstruct(const ReconItem* items, int n_items, int grid_x, int ntile_max,
                                void* const* ptrs, const int* ival, cudaStream_t s);
@@ -64,19 +65,18 @@ __host__ __device__ inline int gram_rows_splits(long long K, int splits_max) {
   return (int)(s < splits_max ? s : splits_max);
 }
 // chunks of 32 (o, q) pairs: one o and 32 consecutive q when Q >= 32, else
-// floor(32 / Q) consecutive o with all q (k_gram_leg's GL_BK)
+// floor(32 / Q) consecutive o with all q (tensor-core Gram)
 __host__ __device__ inline long long gram_leg_chunks(long long O, long long Q) {
   return Q >= 32 ? O * ((Q + 31) / 32) : (O + (32 / Q) - 1) / (32 / Q);
 }
-// split count of a free-leg Gram from its summed extent K = O * Q (shared by
-// every Gram variant and the reduction, independent of their chunk sizes)
-__host__ __device__ inline int gram_leg_splits_k(long long K, int splits_max) {
-  long long s = K / 2048;
-  if (s < 1) s = 1;
-  return (int)(s < splits_max ? s : splits_max);
-}
-__host__ __device__ inline int gram_leg_splits(long long chunks, int splits_max) {
-  long long s = (chunks + 31) / 32;
+// split count of a free-leg Gram from its summed extent K = O * Q, about `rows`
+// terms per split.  Tensor cores: 2048, 64 chunks of their pipeline.  SIMT: 512,
+// so that the Grams of small bonds (K = 2048 at chi = 8) still spread over
+// several SMs; the FP64 pipe of one SM needs 30 us for such a Gram alone.
+constexpr int kGramLegRowsUmma = 2048;
+constexpr int kGramLegRowsSimt = 512;
+__host__ __device__ inline int gram_leg_splits_k(long long K, int splits_max, int rows) {
+  long long s = K / rows;
   if (s < 1) s = 1;
   return (int)(s < splits_max ? s : splits_max);
 }

@@ -786,12 +786,10 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
           GramLegItem g;
           g.x = view;
           g.x.ref = cur;
-          g.y_ref = cur;
           g.leg = w;
           g.partial = W.partial + (size_t)w * kLegSplitsMax * cm2;
           g.out = W.C + (size_t)w * cm2;
           g.ldo = chimax;
-          for (int u = 0; u < PEPO_MAXLEG; ++u) g.sw[u] = nullptr;
           gram.push_back(g);
           RotItem r;
           r.G = g.out;
@@ -1198,7 +1196,7 @@ Work work_of(const pepo_ctx* c, int cls, const void* items, int n) {
       double tot = 4;
       for (int k = 0; k < it.x.nlegs; ++k) tot *= d[k];
       double F = d[it.leg];
-      w.bytes += (it.x.ref == it.y_ref ? 1.0 : 2.0) * tot * ts;   // a symmetric Gram reads X once
+      w.bytes += tot * ts;   // a symmetric Gram reads X once
       w.flops += 2.0 * tot * F;
     } else if (cls == K_RECON) {
       const ReconItem& it = static_cast<const ReconItem*>(items)[i];
@@ -1406,8 +1404,9 @@ pepo_status run_bp_waves(pepo_ctx* c, Inst& I, std::vector<BpWave>& waves) {
     LAUNCH_T(K_GRAM_LEG, hitems(c, w.gram), w.gram.n,
              gram_leg_dispatch<T>(c, w.gram.d, w.gram.n, chimax));
     LAUNCH_T(K_GRAM_LEG_RED, nullptr, w.gram.n,
-             launch_gram_leg_reduce(w.gram.d, w.gram.n, chimax, c->tune.gram_leg_splits, use_umma<T>(c, chimax) ? 1 : 0,
-                                    c->d_ival, s));
+             launch_gram_leg_reduce(w.gram.d, w.gram.n, chimax, c->tune.gram_leg_splits,
+                                    use_umma<T>(c, chimax) ? kGramLegRowsUmma : kGramLegRowsSimt,
+                                    use_umma<T>(c, chimax) ? 1 : 0, c->d_ival, s));
     LAUNCH_T(K_MSG, nullptr, w.rot.n, launch_rotate_back(w.rot.d, w.rot.n, chimax, c->d_ival, s));
     if (w.pw.n > 0) {
       LAUNCH_T(K_OTHER, nullptr, w.pw.n, launch_pauli_weights<T>(w.pw.d, w.pw.n, c->d_ptrs, c->d_ival, s));
