@@ -16,6 +16,8 @@
 //   k_core         per bond: R1 R2^T, one-sided Jacobi SVD, truncation
 //                  (Eq. 11), lambda (Eq. 12), reconstruct matrices W1, W2
 //                  (Sec. 2.5 steps 5-8 in Q-less form), messages diag(lambda).
+#include <algorithm>
+
 #include "kernels.h"
 #include "linalg.h"
 
@@ -1756,40 +1758,62 @@ cudaError_t launch_env_eig(const EnvEigItem* items, int n_items, int chimax, int
   return cudaGetLastError();
 }
 
-// out = V G V^T = Vt^T G Vt
-__global__ void k_rotate_back(const RotItem* __restrict__ items, const int* ival) {
+// out = V G' V^T = Vt^T (G' Vt), G' = G / (sd sd^T).  A block forms a strip of the
+// output's columns: its strip of G' Vt in shared memory, then Vt^T times that, so
+// the strips of a message need nothing from each other.  Bound: the FP64 pipe
+// (4 n^3 operations a message), shared by as many SMs as the strips fill; the
+// divisions by sd are n per block (they were one per product, ~16
+// multiply-adds each, on one SM per message: 2.7 ms a launch at chi = 100, now
+// 0.2).
+__global__ void __launch_bounds__(256)
+k_rotate_back(const RotItem* __restrict__ items, const int* ival) {
   const RotItem it = items[blockIdx.x];
   const int n = ival[it.chi_idx];
+  const int w = (n + gridDim.y - 1) / gridDim.y;
+  const int j0 = blockIdx.y * w, nj = min(w, n - j0);
+  if (nj <= 0) return;
   extern __shared__ __align__(16) double sm[];
-  double* T = sm;   // n x n: T = G' Vt
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    int i = e / n, j = e - i * n;
-    double s = 0.0;
-    if (it.sd) {
-      for (int k = 0; k < n; ++k) s = fma(it.G[i * it.ld + k] / it.sd[k], it.Vt[k * it.ld + j], s);
-      s /= it.sd[i];
-    } else {
-      for (int k = 0; k < n; ++k) s = fma(it.G[i * it.ld + k], it.Vt[k * it.ld + j], s);
-    }
-    T[e] = s;
+  double* T = sm;            // n x nj: T = G' Vt[:, j0 ..]
+  double* B = sm + n * w;    // n x nj: Vt[:, j0 ..] with row k divided by sd[k]
+  double* isd = B + n * w;   // 1 / sd
+  for (int i = threadIdx.x; i < n; i += blockDim.x) isd[i] = it.sd ? 1.0 / it.sd[i] : 1.0;
+  __syncthreads();
+  for (int e = threadIdx.x; e < n * nj; e += blockDim.x) {
+    const int k = e / nj, j = e - k * nj;
+    B[e] = it.Vt[k * it.ld + j0 + j] * isd[k];
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    int i = e / n, j = e - i * n;
+  for (int e = threadIdx.x; e < n * nj; e += blockDim.x) {
+    const int i = e / nj, j = e - i * nj;
+    const double* g = it.G + i * it.ld;
     double s = 0.0;
-    for (int k = 0; k < n; ++k) s = fma(it.Vt[k * it.ld + i], T[k * n + j], s);
-    it.out[i * it.ld + j] = s;
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) s = fma(g[k], B[k * nj + j], s);
+    T[e] = s * isd[i];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < n * nj; e += blockDim.x) {
+    const int i = e / nj, j = e - i * nj;
+    const double* v = it.Vt + i;
+    double s = 0.0;
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) s = fma(v[k * it.ld], T[k * nj + j], s);
+    it.out[i * it.ld + j0 + j] = s;
   }
 }
 
 cudaError_t launch_rotate_back(const RotItem* items, int n_items, int chimax, const int* ival,
                                cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
-  size_t smem = sizeof(double) * (size_t)chimax * chimax;
+  // strips: enough blocks for two per SM, columns of a strip at least four
+  int strips = ceil_div(2 * 152, n_items);
+  strips = std::max(1, std::min(strips, std::min(16, chimax / 4)));
+  if (strips < 2 && chimax > 96) strips = 2;   // two strips of chi^2 / strips doubles in shared memory
+  const size_t smem = sizeof(double) * ((size_t)2 * chimax * ceil_div(chimax, strips) + chimax);
   cudaError_t e = cudaFuncSetAttribute(k_rotate_back, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  k_rotate_back<<<n_items, 256, smem, s>>>(items, ival);
+  k_rotate_back<<<dim3(n_items, strips), 256, smem, s>>>(items, ival);
   return cudaGetLastError();
 }
 }  // namespace pepo
