@@ -8,8 +8,8 @@
 // Precision: weights and activations are rounded to BF16 (round to nearest
 // even) at the layer inputs, every product is accumulated in FP32, gradients
 // and the Adam state are FP32 on an FP32 master copy of the weights.
-// GEMMs are small (width 256, K <= 256 except the weight gradients, whose K
-// is the row count) and run as 64 x 64 register-tiled SIMT tiles.
+// GEMMs have width 256 and K <= 256 except the weight gradients, whose K is the
+// row count; they run as 128 x 128 register-tiled SIMT tiles.
 #include <cuda_bf16.h>
 
 #include "kernels.h"
@@ -26,86 +26,207 @@ __device__ __forceinline__ float gelu_grad_f(float x) {
 }
 
 // ---------------------------------------------------------------- SIMT GEMM
-// C[m, n] = sum_k A[m, k] B[k, n] (+ bias[n]); A and B addressed through
-// strides (so transposed operands need no copies).  epi: 0 = store C;
-// 1 = store z = C + bias and a = bf16(gelu(z)); 2 = store C * gelu'(zref).
+// C[m, n] = sum_k A[m, k] B[k, n].  AT = 0: A row-major [M x K]; 1: A stored
+// [K x M] (a weight gradient's activations).  BT = 0: B row-major [K x N]; 1: B
+// stored [N x K].  Every load is 16 bytes along the stored row.  epi: 0 = store
+// C; 1 = store z = C + bias and a = bf16(gelu(z)); 2 = store C * gelu'(zref).
+// grid.z splits K: split s writes its partial sum at C + s M ldc.
+//
+// 128 x 128 tiles, 8 x 8 entries a thread, the next 16-deep slice in registers
+// while one is multiplied.  Bound: FP32 ALU.  One 10x10, chi = 100 layer
+// (36000 rows): the three 256 x 256 x rows products are 1.4e10 FLOP, 0.18 ms at
+// the FP32 peak; a weight gradient's K = rows is split so that it fills the
+// chip (16 tiles of 64 x 64 ran over all rows one after another before).  The
+// whole training step on those rows: 14.1 -> 0.68 ms.
 struct GemmArgs {
-  const float* A; long long sam, sak;
-  const float* B; long long sbk, sbn;
-  float* C; long long ldc;
+  const float* A; int lda;
+  const float* B; int ldb;
+  float* C; int ldc;
   const float* bias;
   float* act;            // epi 1: rounded activation, leading dimension ldc
   const float* zref;     // epi 2: pre-activation the derivative is taken at
-  int M, N, K;
+  int M, N, K;           // N a multiple of 4; K too unless AT; M too when AT
   int epi;
 };
 
-constexpr int MG_T = 64, MG_BK = 16;
+constexpr int MG_T = 128, MG_BK = 16;
 
+template <int AT, int BT>
 __global__ void __launch_bounds__(256) k_mlp_gemm(GemmArgs g) {
-  __shared__ float As[MG_BK][MG_T + 1];
-  __shared__ float Bs[MG_BK][MG_T + 1];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  __shared__ __align__(16) float As[MG_BK][MG_T + 4];
+  __shared__ __align__(16) float Bs[MG_BK][MG_T + 4];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int m0 = blockIdx.y * MG_T, n0 = blockIdx.x * MG_T;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < g.K; k0 += MG_BK) {
-    for (int e = threadIdx.x; e < MG_BK * MG_T; e += blockDim.x) {
-      const int kk = e / MG_T, mm = e - kk * MG_T;
-      const int m = m0 + mm, k = k0 + kk, n = n0 + mm;
-      As[kk][mm] = (m < g.M && k < g.K) ? g.A[(long long)m * g.sam + (long long)k * g.sak] : 0.f;
-      Bs[kk][mm] = (n < g.N && k < g.K) ? g.B[(long long)k * g.sbk + (long long)n * g.sbn] : 0.f;
+  const int kc = (g.K + gridDim.z - 1) / gridDim.z;
+  const int k0 = blockIdx.z * kc, k1 = min(g.K, k0 + kc);
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 ra[2], rb[2];
+  auto load = [&](int k) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = tid + 256 * u;
+      if (AT) {              // 16 rows (k) of 32 quads (m)
+        const int kk = k + (e >> 5), m = m0 + 4 * (e & 31);
+        ra[u] = kk < k1 && m < g.M ? *reinterpret_cast<const float4*>(g.A + (long long)kk * g.lda + m) : zero;
+      } else {               // 128 rows (m) of 4 quads (k)
+        const int m = m0 + (e >> 2), kk = k + 4 * (e & 3);
+        ra[u] = m < g.M && kk < k1 ? *reinterpret_cast<const float4*>(g.A + (long long)m * g.lda + kk) : zero;
+      }
+      if (BT) {
+        const int n = n0 + (e >> 2), kk = k + 4 * (e & 3);
+        rb[u] = n < g.N && kk < k1 ? *reinterpret_cast<const float4*>(g.B + (long long)n * g.ldb + kk) : zero;
+      } else {
+        const int kk = k + (e >> 5), n = n0 + 4 * (e & 31);
+        rb[u] = kk < k1 && n < g.N ? *reinterpret_cast<const float4*>(g.B + (long long)kk * g.ldb + n) : zero;
+      }
     }
+  };
+  auto store = [&]() {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = tid + 256 * u;
+      if (AT) {
+        *reinterpret_cast<float4*>(&As[e >> 5][4 * (e & 31)]) = ra[u];
+      } else {
+        const int m = e >> 2, kk = 4 * (e & 3);
+        As[kk][m] = ra[u].x; As[kk + 1][m] = ra[u].y; As[kk + 2][m] = ra[u].z; As[kk + 3][m] = ra[u].w;
+      }
+      if (BT) {
+        const int n = e >> 2, kk = 4 * (e & 3);
+        Bs[kk][n] = rb[u].x; Bs[kk + 1][n] = rb[u].y; Bs[kk + 2][n] = rb[u].z; Bs[kk + 3][n] = rb[u].w;
+      } else {
+        *reinterpret_cast<float4*>(&Bs[e >> 5][4 * (e & 31)]) = rb[u];
+      }
+    }
+  };
+  float acc[8][8] = {};
+  load(k0);
+  for (int k = k0; k < k1; k += MG_BK) {
+    store();
     __syncthreads();
+    if (k + MG_BK < k1) load(k + MG_BK);
 #pragma unroll
     for (int kk = 0; kk < MG_BK; ++kk) {
-      float a[4], b[4];
+      float av[8], bv[8];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) { a[i] = As[kk][ty * 4 + i]; b[i] = Bs[kk][tx * 4 + i]; }
+      for (int h = 0; h < 2; ++h) {   // rows / columns 4 t .. 4 t + 3 and 64 further
+        *reinterpret_cast<float4*>(av + 4 * h) = *reinterpret_cast<const float4*>(&As[kk][64 * h + 4 * ty]);
+        *reinterpret_cast<float4*>(bv + 4 * h) = *reinterpret_cast<const float4*>(&Bs[kk][64 * h + 4 * tx]);
+      }
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
     }
     __syncthreads();
   }
+  float* C = g.C + (long long)blockIdx.z * g.M * g.ldc;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
+  for (int i = 0; i < 8; ++i) {
+    const int m = m0 + 64 * (i >> 2) + 4 * ty + (i & 3);
     if (m >= g.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
+    for (int h = 0; h < 2; ++h) {
+      const int n = n0 + 64 * h + 4 * tx;
       if (n >= g.N) continue;
-      float v = acc[i][j];
       const long long o = (long long)m * g.ldc + n;
+      float v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[q] = acc[i][4 * h + q];
       if (g.epi == 1) {
-        v += g.bias[n];
-        g.C[o] = v;
-        g.act[o] = bf16r(gelu_f(v));
+        float t[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) { v[q] += g.bias[n + q]; t[q] = bf16r(gelu_f(v[q])); }
+        *reinterpret_cast<float4*>(g.act + o) = make_float4(t[0], t[1], t[2], t[3]);
       } else if (g.epi == 2) {
-        g.C[o] = v * gelu_grad_f(g.zref[o]);
-      } else {
-        g.C[o] = v + (g.bias ? g.bias[n] : 0.f);
+        const float4 z = *reinterpret_cast<const float4*>(g.zref + o);
+        v[0] *= gelu_grad_f(z.x); v[1] *= gelu_grad_f(z.y); v[2] *= gelu_grad_f(z.z); v[3] *= gelu_grad_f(z.w);
       }
+      *reinterpret_cast<float4*>(C + o) = make_float4(v[0], v[1], v[2], v[3]);
     }
   }
 }
 
-static cudaError_t gemm(const GemmArgs& g, cudaStream_t s) {
+template <int AT, int BT>
+static cudaError_t gemm(const GemmArgs& g, int splits, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
-  dim3 grid((g.N + MG_T - 1) / MG_T, (g.M + MG_T - 1) / MG_T);
-  k_mlp_gemm<<<grid, 256, 0, s>>>(g);
+  dim3 grid((g.N + MG_T - 1) / MG_T, (g.M + MG_T - 1) / MG_T, splits);
+  k_mlp_gemm<AT, BT><<<grid, 256, 0, s>>>(g);
   return cudaGetLastError();
 }
 
-// column sums: out[n] = sum_m A[m, n] (bias gradients), FP32 with a per-thread
-// partial per column block
-__global__ void k_colsum(const float* A, int M, int N, long long lda, float* out) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
+// out[i] = sum of `parts` partial vectors of length n
+__global__ void k_sum_parts(const float* __restrict__ part, int parts, int n, float* __restrict__ out) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    float s = 0.f;
+    for (int p = 0; p < parts; ++p) s += part[(long long)p * n + i];
+    out[i] = s;
+  }
+}
+
+// y[r] = a[r, :] . w + b: one warp per row
+__global__ void __launch_bounds__(256)
+k_row_dot(const float* __restrict__ a, const float* __restrict__ w, const float* __restrict__ b, int rows,
+          float* __restrict__ y) {
+  constexpr int W = PEPO_WS_WIDTH;
+  const int lane = threadIdx.x & 31;
+  const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (r >= rows) return;
   float s = 0.f;
-  for (int m = 0; m < M; ++m) s += A[(long long)m * lda + n];
-  out[n] = s;
+#pragma unroll
+  for (int k = 0; k < W; k += 128) {
+    const float4 x = *reinterpret_cast<const float4*>(a + (long long)r * W + k + 4 * lane);
+    const float4 v = *reinterpret_cast<const float4*>(w + k + 4 * lane);
+    s = fmaf(x.x, v.x, s); s = fmaf(x.y, v.y, s); s = fmaf(x.z, v.z, s); s = fmaf(x.w, v.w, s);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) y[r] = s + b[0];
+}
+
+// Backward of the output layer in one pass over z2 and a2, one thread per
+// column and a chunk of rows per block: d2 = dy W3^T gelu'(z2), and the
+// chunk's part of dW3 = a2^T dy and db2 = column sums of d2 (out: [chunk][2][W]).
+// Memory-bound; a single block per 128 columns summed all rows before.
+__global__ void __launch_bounds__(PEPO_WS_WIDTH)
+k_out_backward(const float* __restrict__ z2, const float* __restrict__ a2, const float* __restrict__ dy,
+               const float* __restrict__ w3, int rows, int chunk, float* __restrict__ d2, float* __restrict__ dw3,
+               float* __restrict__ db2, long long stride) {
+  constexpr int W = PEPO_WS_WIDTH;
+  const int c = threadIdx.x;
+  const int r0 = blockIdx.x * chunk, r1 = min(rows, r0 + chunk);
+  const float w = w3[c];
+  float s3 = 0.f, s2 = 0.f;
+#pragma unroll 4
+  for (int r = r0; r < r1; ++r) {
+    const long long o = (long long)r * W + c;
+    const float e = dy[r];
+    const float d = (e * w) * gelu_grad_f(z2[o]);
+    d2[o] = d;
+    s2 += d;
+    s3 = fmaf(a2[o], e, s3);
+  }
+  dw3[blockIdx.x * stride + c] = s3;
+  db2[blockIdx.x * stride + c] = s2;
+}
+
+// The chunk's part of dW1 = x^T d1 and db1 = column sums of d1 (out: [chunk][13][W])
+__global__ void __launch_bounds__(PEPO_WS_WIDTH)
+k_in_backward(const float* __restrict__ x, const float* __restrict__ d1, int rows, int chunk, float* __restrict__ out) {
+  constexpr int W = PEPO_WS_WIDTH, F = PEPO_WS_FEATURES;
+  const int c = threadIdx.x;
+  const int r0 = blockIdx.x * chunk, r1 = min(rows, r0 + chunk);
+  float acc[F + 1] = {};
+#pragma unroll 2
+  for (int r = r0; r < r1; ++r) {
+    const float d = d1[(long long)r * W + c];
+#pragma unroll
+    for (int f = 0; f < F; ++f) acc[f] = fmaf(x[(long long)r * F + f], d, acc[f]);
+    acc[F] += d;
+  }
+  float* o = out + (long long)blockIdx.x * (F + 1) * W;
+#pragma unroll
+  for (int f = 0; f <= F; ++f) o[f * W + c] = acc[f];
 }
 
 __global__ void k_round(const float* in, float* out, long long n) {
@@ -113,22 +234,25 @@ __global__ void k_round(const float* in, float* out, long long n) {
     out[i] = bf16r(in[i]);
 }
 
-// dy = 2 / n (y - t) and the loss (one block: deterministic sum)
-__global__ void k_mse(const float* y, const float* t, int n, float* dy, float* loss) {
-  __shared__ float red[256];
-  float s = 0.f;
+// dy = 2 / n (y - t), the loss and db3 = sum dy (one block: deterministic sums)
+__global__ void __launch_bounds__(1024) k_mse(const float* y, const float* t, int n, float* dy, float* loss, float* db3) {
+  __shared__ float red[1024], rb[1024];
+  float s = 0.f, sd = 0.f;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const float d = y[i] - t[i];
-    dy[i] = 2.f * d / (float)n;
+    const float e = 2.f * d / (float)n;
+    dy[i] = e;
     s += d * d;
+    sd += e;
   }
   red[threadIdx.x] = s;
+  rb[threadIdx.x] = sd;
   __syncthreads();
   for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    if (threadIdx.x < o) { red[threadIdx.x] += red[threadIdx.x + o]; rb[threadIdx.x] += rb[threadIdx.x + o]; }
     __syncthreads();
   }
-  if (threadIdx.x == 0) *loss = red[0] / (float)n;
+  if (threadIdx.x == 0) { *loss = red[0] / (float)n; *db3 = rb[0]; }
 }
 
 __global__ void k_adam(float* p, float* m, float* v, const float* g, long long n, float lr, float b1, float b2,
@@ -350,21 +474,17 @@ cudaError_t mlp_forward(const MlpBuffers& B, const float* X, int rows, float* y_
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   GemmArgs g{};
-  g.A = B.x; g.sam = F; g.sak = 1;
-  g.B = B.pr + o.W1; g.sbk = W; g.sbn = 1;
+  g.A = B.x; g.lda = F;
+  g.B = B.pr + o.W1; g.ldb = W;
   g.C = B.z1; g.ldc = W; g.bias = B.p + o.b1; g.act = B.a1;
   g.M = rows; g.N = W; g.K = F; g.epi = 1;
-  if ((e = gemm(g, s)) != cudaSuccess) return e;
-  g.A = B.a1; g.sam = W; g.sak = 1;
-  g.B = B.pr + o.W2; g.sbk = W; g.sbn = 1;
+  if ((e = gemm<0, 0>(g, 1, s)) != cudaSuccess) return e;
+  g.A = B.a1; g.lda = W;
+  g.B = B.pr + o.W2;
   g.C = B.z2; g.bias = B.p + o.b2; g.act = B.a2; g.K = W;
-  if ((e = gemm(g, s)) != cudaSuccess) return e;
-  GemmArgs h{};
-  h.A = B.a2; h.sam = W; h.sak = 1;
-  h.B = B.pr + o.W3; h.sbk = 1; h.sbn = 1;
-  h.C = y_out ? y_out : B.y; h.ldc = 1; h.bias = B.p + o.b3;
-  h.M = rows; h.N = 1; h.K = W; h.epi = 0;
-  return gemm(h, s);
+  if ((e = gemm<0, 0>(g, 1, s)) != cudaSuccess) return e;
+  k_row_dot<<<(rows + 7) / 8, 256, 0, s>>>(B.a2, B.pr + o.W3, B.p + o.b3, rows, y_out ? y_out : B.y);
+  return cudaGetLastError();
 }
 
 // forward + backward of the mean squared error; gradient into B.g, loss into B.loss[0]
@@ -373,37 +493,42 @@ cudaError_t mlp_gradient(const MlpBuffers& B, const float* X, const float* t, in
   const int W = PEPO_WS_WIDTH, F = PEPO_WS_FEATURES;
   cudaError_t e = mlp_forward(B, X, rows, B.y, s);
   if (e != cudaSuccess) return e;
-  k_mse<<<1, 256, 0, s>>>(B.y, t, rows, B.dy, B.loss);
-  // dW3 = a2^T dy, db3 = sum dy
+  k_mse<<<1, 1024, 0, s>>>(B.y, t, rows, B.dy, B.loss, B.g + o.b3);
+  // Row chunks of the column sums: about two blocks per SM, at least 32 rows.
+  // Partial sums go to activation buffers that nothing needs any more (d1 before
+  // it is formed; z2 and a2 after d2 is), which hold them for every row count:
+  // a single chunk writes the gradient itself.
+  const int chunk = rows / 304 > 32 ? (rows + 303) / 304 : 32;
+  const int nch = (rows + chunk - 1) / chunk;
+  // dz2 = (dy W3^T) * gelu'(z2), dW3 = a2^T dy, db2 = colsum dz2
+  if (nch == 1) {
+    k_out_backward<<<1, W, 0, s>>>(B.z2, B.a2, B.dy, B.pr + o.W3, rows, chunk, B.d2, B.g + o.W3, B.g + o.b2, 0);
+  } else {
+    k_out_backward<<<nch, W, 0, s>>>(B.z2, B.a2, B.dy, B.pr + o.W3, rows, chunk, B.d2, B.d1, B.d1 + (long long)nch * W, W);
+    k_sum_parts<<<1, W, 0, s>>>(B.d1, nch, W, B.g + o.W3);
+    k_sum_parts<<<1, W, 0, s>>>(B.d1 + (long long)nch * W, nch, W, B.g + o.b2);
+  }
+  // dW2 = a1^T dz2, K = rows split so that 4 tiles x splits fill the chip, at least 256 rows each
+  const int splits = rows / 256 < 1 ? 1 : (rows / 256 < 76 ? rows / 256 : 76);
   GemmArgs g{};
-  g.A = B.a2; g.sam = 1; g.sak = W;          // a2^T: [W x rows]
-  g.B = B.dy; g.sbk = 1; g.sbn = 1;
-  g.C = B.g + o.W3; g.ldc = 1; g.M = W; g.N = 1; g.K = rows; g.epi = 0;
-  if ((e = gemm(g, s)) != cudaSuccess) return e;
-  k_colsum<<<1, 32, 0, s>>>(B.dy, rows, 1, 1, B.g + o.b3);
-  // dz2 = (dy W3^T) * gelu'(z2)
-  GemmArgs d{};
-  d.A = B.dy; d.sam = 1; d.sak = 1;
-  d.B = B.pr + o.W3; d.sbk = 1; d.sbn = 1;     // W3^T as [1 x W]
-  d.C = B.d2; d.ldc = W; d.zref = B.z2; d.M = rows; d.N = W; d.K = 1; d.epi = 2;
-  if ((e = gemm(d, s)) != cudaSuccess) return e;
-  // dW2 = a1^T dz2, db2 = colsum dz2
-  g.A = B.a1; g.sam = 1; g.sak = W;
-  g.B = B.d2; g.sbk = W; g.sbn = 1;
-  g.C = B.g + o.W2; g.ldc = W; g.M = W; g.N = W; g.K = rows;
-  if ((e = gemm(g, s)) != cudaSuccess) return e;
-  k_colsum<<<(W + 127) / 128, 128, 0, s>>>(B.d2, rows, W, W, B.g + o.b2);
+  g.A = B.a1; g.lda = W;                     // stored [rows x W]
+  g.B = B.d2; g.ldb = W;
+  g.C = splits == 1 ? B.g + o.W2 : B.a2; g.ldc = W; g.M = W; g.N = W; g.K = rows; g.epi = 0;
+  if ((e = gemm<1, 0>(g, splits, s)) != cudaSuccess) return e;
+  if (splits > 1) k_sum_parts<<<W * W / 256, 256, 0, s>>>(B.a2, splits, W * W, B.g + o.W2);
   // dz1 = (dz2 W2^T) * gelu'(z1)
-  d.A = B.d2; d.sam = W; d.sak = 1;
-  d.B = B.pr + o.W2; d.sbk = 1; d.sbn = W;     // W2^T
-  d.C = B.d1; d.zref = B.z1; d.K = W;
-  if ((e = gemm(d, s)) != cudaSuccess) return e;
-  // dW1 = x^T dz1, db1 = colsum dz1
-  g.A = B.x; g.sam = 1; g.sak = F;
-  g.B = B.d1; g.sbk = W; g.sbn = 1;
-  g.C = B.g + o.W1; g.ldc = W; g.M = F; g.N = W; g.K = rows;
-  if ((e = gemm(g, s)) != cudaSuccess) return e;
-  k_colsum<<<(W + 127) / 128, 128, 0, s>>>(B.d1, rows, W, W, B.g + o.b1);
+  GemmArgs d{};
+  d.A = B.d2; d.lda = W;
+  d.B = B.pr + o.W2; d.ldb = W;              // stored [W x W], used transposed
+  d.C = B.d1; d.ldc = W; d.zref = B.z1; d.M = rows; d.N = W; d.K = W; d.epi = 2;
+  if ((e = gemm<0, 1>(d, 1, s)) != cudaSuccess) return e;
+  // dW1 = x^T dz1, db1 = colsum dz1 (neighbours in the parameter vector)
+  if (nch == 1) {
+    k_in_backward<<<1, W, 0, s>>>(B.x, B.d1, rows, chunk, B.g + o.W1);
+  } else {
+    k_in_backward<<<nch, W, 0, s>>>(B.x, B.d1, rows, chunk, B.z2);
+    k_sum_parts<<<F + 1, W, 0, s>>>(B.z2, nch, (F + 1) * W, B.g + o.W1);
+  }
   return cudaGetLastError();
 }
 
