@@ -106,9 +106,11 @@ struct ReconItem {
   float* Wp;               // tensor-core path: W packed into swizzled B blocks (recon_packed_floats(nmax))
 };
 
-// Vector contraction of one leg of an FP64 tensor: out[o, q] = sum_j in[o, j, q] v[j].
+// Vector contraction of one leg of an FP64 tensor: out[o, q] = sum_j in[o, j, q] v[j]
+// (the later contractions of single-layer BP), or a copy of a one-leg site's
+// pinned slice.
 struct VecItem {
-  int in_ref;              // >= 0: site tensor (storage type) read at stride 4, offset pin
+  int in_ref;              // >= 0: one-leg site (storage type) read at stride 4, offset pin
   int pin;                 // Pauli index read when in_ref >= 0
   const double* in_d;      // FP64 input when in_ref < 0
   int ndims;
@@ -116,6 +118,20 @@ struct VecItem {
   int leg;
   const double* v;
   double* out;
+};
+
+// First contraction of a site's pinned slice x[o, j2, j3] (its last two legs j2,
+// j3) in single-layer BP, both ways in one read: out_prev[o, j2] = sum_j3 x v_last[j3]
+// and out_last[o, j3] = sum_j2 x v_prev[j2].
+struct VecPairItem {
+  int in_ref;              // site tensor (storage type), read at stride 4, offset pin
+  int pin;
+  int ndims;               // >= 2
+  int dim[PEPO_MAXLEG];    // ival indices (layout order)
+  const double* v_last;
+  const double* v_prev;
+  double* out_prev;
+  double* out_last;
 };
 
 // ------------------------------------------------------------ linear algebra

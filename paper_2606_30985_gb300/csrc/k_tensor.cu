@@ -3,7 +3,7 @@
 //   k_gram_rows      cv^T cv with FP64 accumulation (Eq. 10, Cholesky-QR Gram)
 //   k_reconstruct    psi_new = psi W written in the next update's layout
 //                    (Sec. 2.5 steps 6-7 in Q-less form, Alg. 1 lines 9-12)
-//   k_vec_contract   one-leg vector contraction (single-layer BP, Sec. 2.6)
+//   k_vec_pair, k_vec_contract   vector contractions of single-layer BP (Sec. 2.6)
 //
 // All sizes are read on the device (see common.cuh).  Accumulation: FP32
 // storage accumulates with FP32 FMAs over short runs that are flushed into
@@ -551,6 +551,132 @@ cudaError_t launch_reconstruct(const ReconItem* items, int n_items, int grid_x, 
 }
 
 // ========================================================= vector contraction
+// Sum of products x v, x of the storage type, v FP64.  FP32 storage: v as two FP32
+// parts and a two-float sum (12 FP32 operations a product, ~2^-45 of the sum's
+// terms; an FP64 multiply-add and the conversion take 128 issue slots here).
+template <typename T> struct VecSum;
+template <> struct VecSum<double> {
+  double s = 0.0;
+  __device__ void add(double x, double v) { s = fma(x, v, s); }
+  __device__ void merge(int o) { s += __shfl_xor_sync(0xffffffffu, s, o); }
+  __device__ double value() const { return s; }
+  static __device__ double split(double v) { return v; }
+  using V = double;
+};
+template <> struct VecSum<float> {
+  float s = 0.f, c = 0.f;
+  using V = float2;
+  static __device__ float2 split(double v) {
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
+  }
+  __device__ void take(float p) {
+    const float t = s + p, b = t - s;
+    c += (s - (t - b)) + (p - b);
+    s = t;
+  }
+  __device__ void add(float x, float2 v) {
+    const float p = x * v.x;
+    c += fmaf(x, v.x, -p);
+    take(p);
+    c = fmaf(x, v.y, c);
+  }
+  __device__ void merge(int o) {
+    const float p = __shfl_xor_sync(0xffffffffu, s, o), q = __shfl_xor_sync(0xffffffffu, c, o);
+    take(p);
+    c += q;
+  }
+  __device__ double value() const { return (double)s + (double)c; }
+};
+
+// One pass over the pinned slice feeds both first contractions: lanes hold the
+// columns j3, so a row's product with v_last is a warp sum and the products with
+// v_prev accumulate per lane.  A block shares the rows of one o when there are
+// 32 or more, else each of its warps takes an o of its own.  Bound: HBM (every
+// 32-byte sector of the site tensor holds two pinned values); separate passes
+// read the tensor twice and kept the FP64 pipe busy for 4 slots a value.
+// Class of the correlator of a 4x4, chi = 64 grid (11 passes): 7.2 -> 4.3 ms; of a
+// batch of nine small instances 53 -> 5.5 ms (blocks per item by their number).
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_vec_pair(const VecPairItem* __restrict__ items, void* const* ptrs, const int* __restrict__ ival) {
+  using A = VecSum<T>;
+  const VecPairItem it = items[blockIdx.y];
+  int d[PEPO_MAXLEG];
+#pragma unroll
+  for (int k = 0; k < PEPO_MAXLEG; ++k) d[k] = (k < it.ndims) ? ival[it.dim[k]] : 1;
+  long long O = 1;
+  int J2 = 1, J3 = 1;
+#pragma unroll
+  for (int k = 0; k < PEPO_MAXLEG; ++k) {
+    if (k == it.ndims - 1) J3 = d[k];
+    else if (k == it.ndims - 2) J2 = d[k];
+    else if (k < it.ndims) O *= d[k];
+  }
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const bool share = J2 >= 32;
+  if ((share ? (long long)blockIdx.x : (long long)blockIdx.x * 8) >= O) return;
+  __shared__ typename A::V vl[128], vp[128];
+  __shared__ double part[8][128];
+  for (int i = tid; i < J3; i += 256) vl[i] = A::split(it.v_last[i]);
+  for (int i = tid; i < J2; i += 256) vp[i] = A::split(it.v_prev[i]);
+  __syncthreads();
+  const T* site = static_cast<const T*>(ptrs[it.in_ref]) + it.pin;
+  const long long step = share ? gridDim.x : (long long)gridDim.x * 8;
+  for (long long o = share ? blockIdx.x : (long long)blockIdx.x * 8 + w; o < O; o += step) {
+    const T* base = site + o * J2 * J3 * 4;
+    A col[4];
+    for (int j2 = share ? w : 0; j2 < J2; j2 += share ? 8 : 1) {
+      T x[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int j3 = lane + 32 * c;
+        x[c] = j3 < J3 ? __ldg(base + ((long long)j2 * J3 + j3) * 4) : T(0);
+      }
+      A row;
+      const typename A::V q = vp[j2];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int j3 = lane + 32 * c;
+        if (j3 < J3) {
+          row.add(x[c], vl[j3]);
+          col[c].add(x[c], q);
+        }
+      }
+#pragma unroll
+      for (int m = 16; m > 0; m >>= 1) row.merge(m);
+      if (lane == 0) it.out_prev[o * J2 + j2] = row.value();
+    }
+    if (share) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (lane + 32 * c < J3) part[w][lane + 32 * c] = col[c].value();
+      __syncthreads();
+      for (int j = tid; j < J3; j += 256) {
+        double t = 0.0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) t += part[i][j];
+        it.out_last[o * J3 + j] = t;
+      }
+      __syncthreads();
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (lane + 32 * c < J3) it.out_last[o * J3 + lane + 32 * c] = col[c].value();
+    }
+  }
+}
+
+// blocks per item: about 16 per SM in all, few per item when a batch has many
+static int vec_blocks(int n_items) { return max(4, min(256, ceil_div(16 * 152, n_items))); }
+
+template <typename T>
+cudaError_t launch_vec_pair(const VecPairItem* items, int n_items, void* const* ptrs, const int* ival, cudaStream_t s) {
+  if (n_items == 0) return cudaSuccess;
+  k_vec_pair<T><<<dim3(vec_blocks(n_items), n_items), 256, 0, s>>>(items, ptrs, ival);
+  return cudaGetLastError();
+}
+
 template <typename T>
 __global__ void k_vec_contract(const VecItem* __restrict__ items, void* const* ptrs,
                                const int* __restrict__ ival) {
@@ -559,37 +685,34 @@ __global__ void k_vec_contract(const VecItem* __restrict__ items, void* const* p
 #pragma unroll
   for (int k = 0; k < PEPO_MAXLEG; ++k) d[k] = (k < it.ndims) ? ival[it.dim[k]] : 1;
   const int k = it.leg;
-  const int J = k >= 0 ? d[k] : 1;
-  long long O = 1, Q = 1;
-  for (int i = 0; i < k; ++i) O *= d[i];
-  for (int i = k + 1; i < it.ndims; ++i) Q *= d[i];
-  const T* site = it.in_ref >= 0 ? static_cast<const T*>(ptrs[it.in_ref]) : nullptr;
-  if (k < 0) {  // no contraction: copy (the pinned slice of a one-leg site)
-    long long n = 1;
-    for (int i = 0; i < it.ndims; ++i) n *= d[i];
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-         e += (long long)gridDim.x * blockDim.x)
-      it.out[e] = site ? (double)site[e * 4 + it.pin] : it.in_d[e];
+  if (k < 0) {  // no contraction: the pinned slice of a one-leg site
+    const T* site = static_cast<const T*>(ptrs[it.in_ref]);
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < d[0]; e += gridDim.x * blockDim.x)
+      it.out[e] = (double)site[e * 4 + it.pin];
     return;
   }
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < O * Q;
-       e += (long long)gridDim.x * blockDim.x) {
-    long long o = e / Q, q = e - o * Q;
+  unsigned O = 1, Q = 1;
+  int J = 1;
+#pragma unroll
+  for (int i = 0; i < PEPO_MAXLEG; ++i) {
+    if (i == k) J = d[i];
+    else if (i < k) O *= d[i];
+    else if (i < it.ndims) Q *= d[i];
+  }
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < O * Q; e += gridDim.x * blockDim.x) {
+    const unsigned o = e / Q, q = e - o * Q;
+    const double* x = it.in_d + (long long)o * J * Q + q;
     double sum = 0.0;
-    for (int j = 0; j < J; ++j) {
-      long long idx = (o * J + j) * Q + q;
-      double x = site ? (double)site[idx * 4 + it.pin] : it.in_d[idx];
-      sum = fma(x, it.v[j], sum);
-    }
+#pragma unroll 4
+    for (int j = 0; j < J; ++j) sum = fma(x[(long long)j * Q], it.v[j], sum);
     it.out[e] = sum;
   }
 }
 
 template <typename T>
-cudaError_t launch_vec_contract(const VecItem* items, int n_items, int grid_x, void* const* ptrs,
-                                const int* ival, cudaStream_t s) {
+cudaError_t launch_vec_contract(const VecItem* items, int n_items, void* const* ptrs, const int* ival, cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
-  k_vec_contract<T><<<dim3(grid_x, n_items), 256, 0, s>>>(items, ptrs, ival);
+  k_vec_contract<T><<<dim3(min(32, vec_blocks(n_items)), n_items), 256, 0, s>>>(items, ptrs, ival);
   return cudaGetLastError();
 }
 
@@ -601,8 +724,10 @@ cudaError_t launch_vec_contract(const VecItem* items, int n_items, int grid_x, v
                                            const int*, cudaStream_t);                             \
   template cudaError_t launch_reconstruct<T>(const ReconItem*, int, int, int, void* const*,       \
                                              const int*, cudaStream_t);                           \
-  template cudaError_t launch_vec_contract<T>(const VecItem*, int, int, void* const*, const int*, \
-                                              cudaStream_t);
+  template cudaError_t launch_vec_contract<T>(const VecItem*, int, void* const*, const int*,      \
+                                              cudaStream_t);                                      \
+  template cudaError_t launch_vec_pair<T>(const VecPairItem*, int, void* const*, const int*,      \
+                                          cudaStream_t);
 PEPO_INST(float)
 PEPO_INST(double)
 

@@ -36,8 +36,9 @@ template <typename T>
 cudaError_t launch_reconstruct(const ReconItem* items, int n_items, int grid_x, int ntile_max,
                                void* const* ptrs, const int* ival, cudaStream_t s);
 template <typename T>
-cudaError_t launch_vec_contract(const VecItem* items, int n_items, int grid_x,
-                                void* const* ptrs, const int* ival, cudaStream_t s);
+cudaError_t launch_vec_contract(const VecItem* items, int n_items, void* const* ptrs, const int* ival, cudaStream_t s);
+template <typename T>
+cudaError_t launch_vec_pair(const VecPairItem* items, int n_items, void* const* ptrs, const int* ival, cudaStream_t s);
 
 // ---- k_umma.cu (FP32 storage, TF32x3 on tcgen05 tensor cores, chi <= 128)
 bool umma_supported(int chimax);

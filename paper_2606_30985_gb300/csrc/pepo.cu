@@ -110,8 +110,11 @@ struct BpWave {
   DArr<PauliWItem> pw;     // final waves only: Pauli weights of the rotated sites
 };
 
+// single-layer BP: level 0 copies (one-leg sites), level 1 the first contractions
+// of every other site (pairs), levels 2 and 3 the later ones
 struct SlLevel {
   DArr<VecItem> items;
+  DArr<VecPairItem> pairs;   // level 1 only
 };
 
 struct Inst {
@@ -888,7 +891,26 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
         }
       }
     }
+    // every site with two or more legs put two items into level 1: its last leg
+    // contracted, then the one before it
+    std::vector<VecPairItem> pairs;
+    for (size_t i = 0; i + 1 < lv[1].size(); i += 2) {
+      const VecItem &a = lv[1][i], &b = lv[1][i + 1];
+      VecPairItem p;
+      p.in_ref = a.in_ref;
+      p.pin = a.pin;
+      p.ndims = a.ndims;
+      for (int k = 0; k < a.ndims; ++k) p.dim[k] = a.dim[k];
+      p.v_last = a.v;
+      p.out_prev = a.out;
+      p.v_prev = b.v;
+      p.out_last = b.out;
+      if (b.in_ref != a.in_ref || a.leg != a.ndims - 1 || b.leg != a.ndims - 2) return false;   // cannot happen
+      pairs.push_back(p);
+    }
+    lv[1].clear();
     for (int l = 0; l < 4; ++l) I.sl[l].items = stage(P, lv[l]);
+    I.sl[1].pairs = stage(P, pairs);
   }
 
   // ---- message / scalar / Bethe items
@@ -991,7 +1013,10 @@ void resolve_all(pepo_ctx* c) {
         resolve(w.rot, d);
         resolve(w.pw, d);
       }
-    for (int l = 0; l < 4; ++l) resolve(I.sl[l].items, d);
+    for (int l = 0; l < 4; ++l) {
+      resolve(I.sl[l].items, d);
+      resolve(I.sl[l].pairs, d);
+    }
     resolve(I.msgs, d); resolve(I.sscal, d); resolve(I.escal, d); resolve(I.bethe, d);
     resolve(I.gates, d);
   }
@@ -1087,8 +1112,10 @@ void build_group(Planner& P, pepo_ctx* c) {
   }
   for (int l = 0; l < 4; ++l) {
     std::vector<const DArr<VecItem>*> v;
-    for (auto& I : c->inst) v.push_back(&I.sl[l].items);
+    std::vector<const DArr<VecPairItem>*> q;
+    for (auto& I : c->inst) { v.push_back(&I.sl[l].items); q.push_back(&I.sl[l].pairs); }
     G.sl[l].items = cat_items(P, v);
+    G.sl[l].pairs = cat_items(P, q);
   }
   {
     std::vector<const DArr<MsgItem>*> m;
@@ -1419,8 +1446,8 @@ pepo_status run_bp_waves(pepo_ctx* c, Inst& I, std::vector<BpWave>& waves) {
 template <typename T>
 pepo_status run_sl_pass(pepo_ctx* c, Inst& I) {
   for (int l = 0; l < 4; ++l) {
-    if (I.sl[l].items.n == 0) continue;
-    LAUNCH_T(K_VEC, nullptr, I.sl[l].items.n, launch_vec_contract<T>(I.sl[l].items.d, I.sl[l].items.n, 256, c->d_ptrs, c->d_ival, c->stream));
+    LAUNCH_T(K_VEC, nullptr, I.sl[l].pairs.n, launch_vec_pair<T>(I.sl[l].pairs.d, I.sl[l].pairs.n, c->d_ptrs, c->d_ival, c->stream));
+    LAUNCH_T(K_VEC, nullptr, I.sl[l].items.n, launch_vec_contract<T>(I.sl[l].items.d, I.sl[l].items.n, c->d_ptrs, c->d_ival, c->stream));
   }
   return PEPO_OK;
 }
