@@ -906,104 +906,109 @@ cudaError_t launch_factor(const SiteFacItem* items, int n_items, int rmax, int n
 // the ranks of any input form a permutation (every order[] slot written once).
 __device__ inline double rank_key(double x) { return x == x ? x : -1.0; }
 
-// One-sided Jacobi (Hestenes) on the columns of A (m x n, column-major, m >= n),
-// accumulating V (n x n, column-major).  Returns the sweep count; sets
-// *capped when the sweep budget ran out.  abs_rel > 0 also skips a pair whose
-// coupling |a_p . a_q| is below abs_rel ||A||_F^2: such a pair moves no
-// singular value by more than that absolute amount, and without the cut the
-// columns of tiny singular values (their content mostly rounding noise from
-// rotations with the large ones) are chased for many sweeps without ever
-// reaching relative orthogonality.
-template <typename R>
-__device__ int jacobi_svd(R* A, int m, int n, R* V, int max_sweeps, int* capped, double* red,
-                          double abs_rel = 0.0) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  // V == nullptr: rotations are not accumulated (the caller recovers the other
-  // side's vectors from a copy of the input)
-  if (V)
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) V[e] = (e % (n + 1) == 0) ? R(1) : R(0);
-  __syncthreads();
+// One-sided Jacobi (Hestenes) on the columns of A (n x n, column-major),
+// accumulating V (n x n, column-major), by one block.  Returns the sweep count;
+// sets *capped when the sweep budget ran out.
+//
+// A pair of columns belongs to L lanes (32 up to n = 64, 16 above, so that the
+// n / 2 <= 64 pairs of a tournament round run at once on 1024 threads), which
+// hold both columns in registers from the dot product to the rotation; the
+// squared norms are recomputed every sweep and updated by the rotations
+// between, so a pair costs one reduction.  Bound: shared-memory bandwidth (8
+// column passes a rotation) and the latency of one round at small n.
+template <typename R, int L>
+__device__ int jacobi_block_l(R* A, int n, R* V, R* nrm, int max_sweeps, int* capped) {
+  constexpr int E = L == 32 ? 2 : 8;                        // column values per lane: n <= 64, n <= 128
+  const int l = threadIdx.x % L, grp = threadIdx.x / L, ng = blockDim.x / L;
+  const unsigned mask = L == 32 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) V[e] = (e % (n + 1) == 0) ? R(1) : R(0);
+  auto norms = [&]() {
+    for (int c = grp; c < n; c += ng) {
+      R q = 0;
+      for (int i = l; i < n; i += L) q = fma(A[c * n + i], A[c * n + i], q);
+#pragma unroll
+      for (int o = L / 2; o > 0; o >>= 1) q += __shfl_xor_sync(mask, q, o);
+      if (l == 0) nrm[c] = q;
+    }
+    __syncthreads();
+  };
+  norms();
   if (n < 2) return 0;
+  // ||A||_F^2 (the same bits whatever the block's size)
+  R fro = 0;
+  for (int c = threadIdx.x & 31; c < n; c += 32) fro += nrm[c];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) fro += __shfl_xor_sync(0xffffffffu, fro, o);
+  __syncthreads();
   const int np = (n % 2) ? n + 1 : n;   // players incl. a dummy
-  // orthogonality target: above the rounding noise of a length-m dot product
-  // in the working precision (FP32 columns: ~sqrt(m) 6e-8 relative)
-  const double tol = (sizeof(R) == 4 ? 3e-7 : 1e-15) * sqrt((double)m);
-  // columns below 1e-30 (FP64) or 1e-13 (FP32) of the total squared norm are
+  // orthogonality target: above the rounding noise of a length-n dot product
+  // in the working precision (FP32 columns: ~sqrt(n) 6e-8 relative); columns
+  // below 1e-30 (FP64) or 1e-13 (FP32) of the total squared norm are
   // numerically zero in that precision: rotating them only stirs rounding
   // noise and never converges
-  double fro = 0.0;
-  for (long long e = threadIdx.x; e < (long long)m * n; e += blockDim.x) fro = fma((double)A[e], (double)A[e], fro);
-  {
-    fro = warp_sum(fro);
-    __shared__ double fr[32];
-    if (lane == 0) fr[wid] = fro;
-    __syncthreads();
-    fro = 0.0;
-    for (int i = 0; i < nw; ++i) fro += fr[i];
-    __syncthreads();
-  }
-  const double negligible = (sizeof(R) == 4 ? 1e-13 : 1e-30) * fro;
-  const R abs_cut = (R)(abs_rel * fro);
-  __shared__ int sh_rot;
+  const R tol = (R)((sizeof(R) == 4 ? 3e-7 : 1e-15) * sqrt((double)n));
+  const R negligible = (R)(sizeof(R) == 4 ? 1e-13 : 1e-30) * fro;
   int sweep = 0;
   for (; sweep < max_sweeps; ++sweep) {
-    if (threadIdx.x == 0) sh_rot = 0;
-    __syncthreads();
+    if (sweep > 0) norms();
     int rotated = 0;
     for (int round = 0; round < np - 1; ++round) {
-      for (int pi = wid; pi < np / 2; pi += nw) {
+      for (int pi = grp; pi < np / 2; pi += ng) {
         int a, b;
         if (pi == 0) { a = np - 1; b = round; }
-        else { a = (round + pi) % (np - 1); b = (round - pi + np - 1) % (np - 1); }
+        else {
+          a = round + pi; if (a >= np - 1) a -= np - 1;
+          b = round - pi; if (b < 0) b += np - 1;
+        }
         if (a >= n || b >= n) continue;
-        int p = a < b ? a : b, q = a < b ? b : a;
-        R* Ap = A + (long long)p * m;
-        R* Aq = A + (long long)q * m;
-        R al = 0, be = 0, ga = 0;
-        for (int i = lane; i < m; i += 32) {
-          R x = Ap[i], y = Aq[i];
-          al = fma(x, x, al); be = fma(y, y, be); ga = fma(x, y, ga);
-        }
+        const int p = a < b ? a : b, q = a < b ? b : a;
+        R* Ap = A + p * n;
+        R* Aq = A + q * n;
+        R x[E], y[E], ga = 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          al += __shfl_xor_sync(0xffffffffu, al, o);
-          be += __shfl_xor_sync(0xffffffffu, be, o);
-          ga += __shfl_xor_sync(0xffffffffu, ga, o);
+        for (int u = 0; u < E; ++u) {
+          const int i = l + L * u;
+          x[u] = i < n ? Ap[i] : R(0);
+          y[u] = i < n ? Aq[i] : R(0);
+          ga = fma(x[u], y[u], ga);
         }
-        // rotation parameters in the working precision (FP64 division and
-        // square root are slow on this part; FP32 columns need no more)
-        if (ga != R(0) && al > (R)negligible && be > (R)negligible &&
-            fabs(ga) > (R)tol * sqrt(al * be) && fabs(ga) > abs_cut) {
+        const R al = nrm[p], be = nrm[q];
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) ga += __shfl_xor_sync(mask, ga, o);
+        if (ga != R(0) && al > negligible && be > negligible && fabs(ga) > tol * sqrt(al * be)) {
           rotated = 1;
           const R zeta = (be - al) / (R(2) * ga);
           const R t = (zeta >= R(0) ? R(1) : R(-1)) / (fabs(zeta) + sqrt(R(1) + zeta * zeta));
           const R c = R(1) / sqrt(R(1) + t * t), s = c * t;
-          for (int i = lane; i < m; i += 32) {
-            R x = Ap[i], y = Aq[i];
-            Ap[i] = c * x - s * y;
-            Aq[i] = s * x + c * y;
-          }
-          if (V) {
-            R* Vp = V + (long long)p * n;
-            R* Vq = V + (long long)q * n;
-            for (int i = lane; i < n; i += 32) {
-              R x = Vp[i], y = Vq[i];
-              Vp[i] = c * x - s * y;
-              Vq[i] = s * x + c * y;
+          R* Vp = V + p * n;
+          R* Vq = V + q * n;
+#pragma unroll
+          for (int u = 0; u < E; ++u) {
+            const int i = l + L * u;
+            if (i < n) {
+              Ap[i] = c * x[u] - s * y[u];
+              Aq[i] = s * x[u] + c * y[u];
+              const R vx = Vp[i], vy = Vq[i];
+              Vp[i] = c * vx - s * vy;
+              Vq[i] = s * vx + c * vy;
             }
           }
+          __syncwarp(mask);
+          if (l == 0) { nrm[p] = al - t * ga; nrm[q] = be + t * ga; }
         }
       }
       __syncthreads();
     }
-    if (rotated) atomicOr(&sh_rot, 1);
-    __syncthreads();
-    if (sh_rot == 0) break;
-    __syncthreads();
+    if (!__syncthreads_or(rotated)) break;
   }
   if (sweep >= max_sweeps && threadIdx.x == 0) *capped = 1;
-  (void)red;
+  __syncthreads();
   return sweep;
+}
+template <typename R>
+__device__ int jacobi_block(R* A, int n, R* V, R* nrm, int max_sweeps, int* capped) {
+  return n <= 64 ? jacobi_block_l<R, 32>(A, n, V, nrm, max_sweeps, capped)
+                 : jacobi_block_l<R, 16>(A, n, V, nrm, max_sweeps, capped);
 }
 
 // ---- the same on the CTAs of one cluster --------------------------------
@@ -1096,7 +1101,7 @@ __device__ bool jac_pair(R* x, R* y, int m, R* vx, R* vy, int nv, R* nx, R* ny, 
 // The order of the rotations of a column depends on n alone, so every cluster
 // size gives the same bits.
 //
-// Rotation and stopping rules as jacobi_svd, plus abs_rel > 0: a pair whose
+// Rotation and stopping rules as jacobi_block, plus abs_rel > 0: a pair whose
 // coupling |a_p . a_q| is below abs_rel ||A||_F^2 is skipped too.  Such a pair
 // moves no singular value by more than that, and without the cut the columns of
 // tiny singular values (mostly rounding noise from rotations with the large
@@ -1690,72 +1695,61 @@ __device__ void scaled_rotation(const EnvEigItem& it, int n) {
 
 // M (symmetrised, PSD) -> one-sided Jacobi on its columns: M V = U S with
 // S = |eigenvalues| and V the eigenvectors (U = V up to signs of numerically
-// zero eigenvalues).  Outputs Vt (row i = column i of V) and sqrt(S).
+// zero eigenvalues).  Outputs Vt (row i = column i of V) and sqrt(S).  FP32
+// (R = float, FP32-storage modes): the eigenbasis only rotates FP32 tensors.
+// The matrices live in shared memory; FP64 ones that do not fit (chi > 112) in
+// the item's workspace.
+constexpr size_t kEigSmem = (size_t)220 * 1024;
+template <typename R>
 __global__ void __launch_bounds__(1024)
-k_env_eig(const EnvEigItem* __restrict__ items, const int* ival, int fp32) {
+k_env_eig(const EnvEigItem* __restrict__ items, const int* ival, int chimax) {
   const EnvEigItem it = items[blockIdx.x];
   const int n = ival[it.chi_idx];
+  extern __shared__ __align__(16) unsigned char eig_sh[];
   __shared__ double red[32];
   __shared__ int capped;
   if (threadIdx.x == 0) capped = 0;
-  if (fp32) {
-    // FP32-storage modes: the eigenbasis only rotates FP32 tensors, so the
-    // Jacobi runs in FP32 entirely in shared memory
-    extern __shared__ __align__(16) float sm32[];
-    float* A = sm32;                       // n x n column-major
-    float* V = sm32 + (long long)n * n;
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-      int i = e / n, j = e - i * n;
-      A[(long long)j * n + i] = (float)(0.5 * (it.M[i * it.ld + j] + it.M[j * it.ld + i]));
-    }
-    __syncthreads();
-    jacobi_svd<float>(A, n, n, V, 60, &capped, red);
-    __syncthreads();
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-      double s = 0.0;
-      for (int i = 0; i < n; ++i) s = fma((double)A[(long long)j * n + i], (double)A[(long long)j * n + i], s);
-      it.sqrtD[j] = sqrt(sqrt(s));
-    }
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-      int i = e / n, j = e - i * n;
-      it.Vt[i * it.ld + j] = (double)V[(long long)i * n + j];
-    }
-    floor_sqrt_eigs(it.sqrtD, n, red);
-    scaled_rotation(it, n);
-    return;
-  }
-  double* A = it.work;                      // n x n column-major
-  double* V = it.work + (long long)n * n;   // n x n column-major
+  R* nrm = reinterpret_cast<R*>(eig_sh);                   // 128 values
+  const bool in = sizeof(R) * (2 * (size_t)chimax * chimax + 128) <= kEigSmem;
+  R* A = in ? nrm + 128 : reinterpret_cast<R*>(it.work);   // n x n column-major
+  R* V = A + n * n;
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    int i = e / n, j = e - i * n;   // A column j, row i
-    A[(long long)j * n + i] = 0.5 * (it.M[i * it.ld + j] + it.M[j * it.ld + i]);
+    const int i = e / n, j = e - i * n;
+    A[j * n + i] = (R)(0.5 * (it.M[i * it.ld + j] + it.M[j * it.ld + i]));
   }
   __syncthreads();
-  jacobi_svd<double>(A, n, n, V, 60, &capped, red);
-  __syncthreads();
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+  jacobi_block<R>(A, n, V, nrm, 60, &capped);
+  for (int j = threadIdx.x >> 5; j < n; j += (int)(blockDim.x >> 5)) {
     double s = 0.0;
-    for (int i = 0; i < n; ++i) s = fma(A[(long long)j * n + i], A[(long long)j * n + i], s);
-    it.sqrtD[j] = sqrt(sqrt(s));   // sqrt of the eigenvalue |lambda_j| = ||A v_j||
+    for (int i = threadIdx.x & 31; i < n; i += 32) s = fma((double)A[j * n + i], (double)A[j * n + i], s);
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) it.sqrtD[j] = sqrt(sqrt(s));   // sqrt of the eigenvalue |lambda_j| = ||A v_j||
   }
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    int i = e / n, j = e - i * n;
-    it.Vt[i * it.ld + j] = V[(long long)i * n + j];   // row i of Vt = column i of V
+    const int i = e / n, j = e - i * n;
+    it.Vt[i * it.ld + j] = (double)V[i * n + j];           // row i of Vt = column i of V
   }
   floor_sqrt_eigs(it.sqrtD, n, red);
   scaled_rotation(it, n);
 }
 
+template <typename R>
+static cudaError_t launch_eig(const EnvEigItem* items, int n_items, int chimax, const int* ival, cudaStream_t s) {
+  const size_t want = sizeof(R) * (2 * (size_t)chimax * chimax + 128);
+  const size_t smem = want <= kEigSmem ? want : sizeof(R) * 128;
+  cudaError_t e = cudaFuncSetAttribute(k_env_eig<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  // a warp per pair of columns up to chi = 64, half a warp above
+  const int pairs = (chimax + 1) / 2;
+  const int threads = chimax <= 64 ? std::max(64, 32 * pairs) : 16 * ((pairs + 1) & ~1);
+  k_env_eig<R><<<n_items, threads, smem, s>>>(items, ival, chimax);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_env_eig(const EnvEigItem* items, int n_items, int chimax, int fp32, const int* ival,
                            cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
-  size_t smem = fp32 ? 2 * sizeof(float) * (size_t)chimax * chimax : 0;
-  if (smem > 0) {
-    cudaError_t e = cudaFuncSetAttribute(k_env_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  k_env_eig<<<n_items, 1024, smem, s>>>(items, ival, fp32);
-  return cudaGetLastError();
+  return fp32 ? launch_eig<float>(items, n_items, chimax, ival, s) : launch_eig<double>(items, n_items, chimax, ival, s);
 }
 
 // out = V G' V^T = Vt^T (G' Vt), G' = G / (sd sd^T).  A block forms a strip of the
