@@ -30,6 +30,24 @@ struct TView {
   int dim[PEPO_MAXLEG];
 };
 
+// Sum of FP32 values in two floats (Knuth's two-sum; s + c holds ~46 bits of the
+// largest partial sum): where a long sum of FP32 data needs more than FP32, for
+// 8 to 10 FP32 operations instead of an FP64 addition, which takes 64 slots here.
+struct TwoFloat {
+  float s = 0.f, c = 0.f;
+  __device__ void take(float p) {
+    const float t = s + p, b = t - s;
+    c += (s - (t - b)) + (p - b);
+    s = t;
+  }
+  __device__ void take_product(float x, float y) {
+    const float p = x * y;
+    c += fmaf(x, y, -p);
+    take(p);
+  }
+  __device__ double value() const { return (double)s + (double)c; }
+};
+
 __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 __host__ __device__ inline long long ceil_divl(long long a, long long b) { return (a + b - 1) / b; }
 

@@ -14,14 +14,6 @@
 
 namespace pepo {
 
-template <typename T> struct Flush;
-template <> struct Flush<float> {
-  static constexpr bool kFlush = true;
-};
-template <> struct Flush<double> {
-  static constexpr bool kFlush = false;
-};
-
 __device__ inline void load_dims(const TView& v, const int* ival, int* d) {
 #pragma unroll
   for (int k = 0; k < PEPO_MAXLEG; ++k) d[k] = (k < v.nlegs) ? ival[v.dim[k]] : 1;
@@ -52,8 +44,7 @@ cudaError_t launch_copy(const TView* items, const int* out_refs, int n_items, in
 }
 
 // ================================================================ Gram (rows)
-// 64 x 64 output tile per block, 16 x 16 threads with 4 x 4 micro-tiles,
-// K streamed 16 rows at a time.
+// Tiles of 64 x 64, the rows K split over blocks (gram_rows_splits).
 constexpr int GR_T = 64;
 constexpr int GR_BK = 16;
 constexpr int GR_FLUSH = 256;   // FP32 run length before the FP64 flush
@@ -66,10 +57,10 @@ __device__ inline void tile_of(int t, int nt, int sym, int& ti, int& tj) {
   ti = r; tj = r + (t - base);
 }
 
-template <typename T>
+// FP64 storage: bound by the FP64 pipe whatever the tile.
 __global__ void __launch_bounds__(256)
-k_gram_rows(const GramRowsItem* __restrict__ items, int splits_max, int sym, void* const* ptrs,
-            const int* __restrict__ ival) {
+k_gram_rows64(const GramRowsItem* __restrict__ items, int splits_max, int sym, void* const* ptrs,
+              const int* __restrict__ ival) {
   const GramRowsItem it = items[blockIdx.z];
   if (it.active >= 0 && ival[it.active] == 0) return;
   int d[PEPO_MAXLEG];
@@ -87,31 +78,28 @@ k_gram_rows(const GramRowsItem* __restrict__ items, int splits_max, int sym, voi
   int ti, tj;
   tile_of(t, nt, sym, ti, tj);
   const long long k0 = K * s / S, k1 = K * (s + 1) / S;
-  const T* __restrict__ X = static_cast<const T*>(ptrs[it.x.ref]);
-  const T* __restrict__ Y = static_cast<const T*>(ptrs[it.y_ref]);
-  __shared__ __align__(16) T Xs[GR_BK][GR_T];
-  __shared__ __align__(16) T Ys[GR_BK][GR_T];
+  const double* __restrict__ X = static_cast<const double*>(ptrs[it.x.ref]);
+  __shared__ __align__(16) double Xs[GR_BK][GR_T];
+  __shared__ __align__(16) double Ys[GR_BK][GR_T];
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  T acc[4][4];
-  double acc64[4][4];
+  double acc[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) { acc[a][b] = T(0); acc64[a][b] = 0.0; }
-  int run = 0;
+    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
   for (long long kb = k0; kb < k1; kb += GR_BK) {
     for (int e = threadIdx.x; e < GR_BK * GR_T; e += blockDim.x) {
       int kk = e / GR_T, c = e - kk * GR_T;
       long long k = kb + kk;
       int fi = ti * GR_T + c, fj = tj * GR_T + c;
       bool okk = k < k1;
-      Xs[kk][c] = (okk && fi < F) ? X[k * F + fi] : T(0);
-      Ys[kk][c] = (okk && fj < F) ? Y[k * F + fj] : T(0);
+      Xs[kk][c] = (okk && fi < F) ? X[k * F + fi] : 0.0;
+      Ys[kk][c] = (okk && fj < F) ? X[k * F + fj] : 0.0;
     }
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < GR_BK; ++kk) {
-      T xa[4], yb[4];
+      double xa[4], yb[4];
 #pragma unroll
       for (int a = 0; a < 4; ++a) xa[a] = Xs[kk][ty * 4 + a];
 #pragma unroll
@@ -122,16 +110,6 @@ k_gram_rows(const GramRowsItem* __restrict__ items, int splits_max, int sym, voi
         for (int b = 0; b < 4; ++b) acc[a][b] = fma(xa[a], yb[b], acc[a][b]);
     }
     __syncthreads();
-    if (Flush<T>::kFlush) {
-      run += GR_BK;
-      if (run >= GR_FLUSH) {
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) { acc64[a][b] += (double)acc[a][b]; acc[a][b] = T(0); }
-        run = 0;
-      }
-    }
   }
   double* P = it.partial + (long long)s * F * F;
 #pragma unroll
@@ -141,7 +119,126 @@ k_gram_rows(const GramRowsItem* __restrict__ items, int splits_max, int sym, voi
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       int fj = tj * GR_T + tx * 4 + b;
-      if (fj < F) P[(long long)fi * F + fj] = acc64[a][b] + (double)acc[a][b];
+      if (fj < F) P[(long long)fi * F + fj] = acc[a][b];
+    }
+  }
+}
+
+// 16-byte asynchronous copy of a quad, zeros where it lies outside
+__device__ inline void copy_quad(void* dst, const void* src, bool live) {
+  const int n = live ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(n)
+               : "memory");
+}
+
+// FP32 storage.  64 x 64 tiles of the upper triangle; a chunk of 64 rows is
+// copied asynchronously, three stages deep.  Two groups of 128 threads take 32
+// rows of a chunk each, a thread 8 x 4 entries (32 multiply-adds per three
+// 16-byte shared loads, two of them broadcasts), so the FP32 pipe bounds it;
+// 4 x 4 entries and scalar, unpipelined loads ran at 18 TFLOP/s (class of a 4x4
+// chi = 64 layer 17 -> 8.3 ms, 3x3 chi = 100 55 -> 25 ms).  Runs of 256
+// terms in FP32 go into a two-float sum, the groups and splits into FP64.
+constexpr int GF_K = 64;
+constexpr int GF_STAGES = 3;
+
+__global__ void __launch_bounds__(256, 2)
+k_gram_rows32(const GramRowsItem* __restrict__ items, int splits_max, int sym, void* const* ptrs,
+              const int* __restrict__ ival) {
+  const GramRowsItem it = items[blockIdx.z];
+  if (it.active >= 0 && ival[it.active] == 0) return;
+  int d[PEPO_MAXLEG];
+  load_dims(it.x, ival, d);
+  const int nl = it.x.nlegs;
+  const int F = 4 * (nl > 0 ? d[nl - 1] : 1);
+  long long K = 1;
+  for (int i = 0; i + 1 < nl; ++i) K *= d[i];
+  const int S = gram_rows_splits(K, splits_max);
+  const int sp = blockIdx.x % splits_max;
+  const int nt = ceil_div(F, GR_T);
+  if (sp >= S || (int)(blockIdx.x / splits_max) >= (sym ? nt * (nt + 1) / 2 : nt * nt)) return;
+  int ti, tj;
+  tile_of(blockIdx.x / splits_max, nt, sym, ti, tj);
+  const bool diag = ti == tj;
+  const long long k0 = K * sp / S, k1 = K * (sp + 1) / S;
+  const float* __restrict__ X = static_cast<const float*>(ptrs[it.x.ref]);
+  extern __shared__ __align__(16) float gf_sh[];       // stages of [X | Y], 64 rows x 64 columns each
+  const int tid = threadIdx.x, g = tid >> 7, tx = tid & 15, ty = (tid >> 4) & 7;
+  auto load = [&](int st, long long kb) {
+    if (kb < k1) {
+      float* xs = gf_sh + st * (2 * GF_K * GR_T);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = tid + 256 * u;                   // 64 rows x 16 quads
+        const int row = e >> 4, q = 4 * (e & 15);
+        const long long k = kb + row;
+        const int ci = ti * GR_T + q, cj = tj * GR_T + q;
+        const bool in = k < k1;
+        copy_quad(xs + row * GR_T + q, in && ci < F ? X + k * F + ci : X, in && ci < F);
+        if (!diag) copy_quad(xs + (GF_K + row) * GR_T + q, in && cj < F ? X + k * F + cj : X, in && cj < F);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float acc[8][4];
+  TwoFloat sum[8][4];
+#pragma unroll
+  for (int a = 0; a < 8; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+  auto flush = [&]() {
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) { sum[a][b].take(acc[a][b]); acc[a][b] = 0.f; }
+  };
+#pragma unroll
+  for (int st = 0; st < GF_STAGES - 1; ++st) load(st, k0 + st * GF_K);
+  int st = 0, run = 0;
+  for (long long kb = k0; kb < k1; kb += GF_K) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(GF_STAGES - 2) : "memory");
+    __syncthreads();                                   // this chunk is in, the one before is consumed
+    load(st == 0 ? GF_STAGES - 1 : st - 1, kb + (GF_STAGES - 1) * GF_K);
+    const float* xs = gf_sh + st * (2 * GF_K * GR_T) + g * (GF_K / 2) * GR_T;
+    const float* ys = diag ? xs : xs + GF_K * GR_T;
+#pragma unroll 8
+    for (int kk = 0; kk < GF_K / 2; ++kk) {
+      float a8[8], b4[4];
+      *reinterpret_cast<float4*>(a8) = *reinterpret_cast<const float4*>(xs + kk * GR_T + 4 * ty);
+      *reinterpret_cast<float4*>(a8 + 4) = *reinterpret_cast<const float4*>(xs + kk * GR_T + 32 + 4 * ty);
+      *reinterpret_cast<float4*>(b4) = *reinterpret_cast<const float4*>(ys + kk * GR_T + 4 * tx);
+#pragma unroll
+      for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(a8[a], b4[b], acc[a][b]);
+    }
+    run += GF_K / 2;
+    if (run >= GR_FLUSH) { flush(); run = 0; }
+    if (++st == GF_STAGES) st = 0;
+  }
+  flush();
+  // the two groups' sums, then the split's tile
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  double* red = reinterpret_cast<double*>(gf_sh);
+  if (g == 1)
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        red[(4 * ty + (a & 3) + 32 * (a >> 2)) * GR_T + 4 * tx + b] = sum[a][b].value();
+  __syncthreads();
+  if (g == 0) {
+    double* P = it.partial + (long long)sp * F * F;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const int r = 4 * ty + (a & 3) + 32 * (a >> 2), fi = ti * GR_T + r;
+      if (fi >= F) continue;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int fj = tj * GR_T + 4 * tx + b;
+        if (fj < F) P[(long long)fi * F + fj] = red[r * GR_T + 4 * tx + b] + sum[a][b].value();
+      }
     }
   }
 }
@@ -172,7 +269,14 @@ cudaError_t launch_gram_rows(const GramRowsItem* items, int n_items, int tiles_m
                              int sym, void* const* ptrs, const int* ival, cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
   dim3 grid(tiles_max * splits_max, 1, n_items);
-  k_gram_rows<T><<<grid, 256, 0, s>>>(items, splits_max, sym, ptrs, ival);
+  if constexpr (sizeof(T) == 8) {
+    k_gram_rows64<<<grid, 256, 0, s>>>(items, splits_max, sym, ptrs, ival);
+  } else {
+    const size_t smem = sizeof(float) * GF_STAGES * 2 * GF_K * GR_T;
+    cudaError_t e = cudaFuncSetAttribute(k_gram_rows32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_gram_rows32<<<grid, 256, smem, s>>>(items, splits_max, sym, ptrs, ival);
+  }
   return cudaGetLastError();
 }
 
@@ -256,13 +360,6 @@ k_col_scale(const GramRowsItem* __restrict__ items, int pass, int step, void* co
 // exponent e with the column's largest magnitude in [2^(e-1), 2^e)
 __device__ inline int col_exp(unsigned bits) { return (int)(bits >> 23) - 126; }
 
-__device__ inline void gx_copy16(void* dst, const void* src, bool live) {
-  const int n = live ? 16 : 0;
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
-               "r"(n)
-               : "memory");
-}
-
 __global__ void __launch_bounds__(256, 2)
 k_gram_exact(const GramRowsItem* __restrict__ items, int pass, void* const* ptrs, const int* __restrict__ ival) {
   const GramRowsItem it = items[blockIdx.z];
@@ -300,8 +397,8 @@ k_gram_exact(const GramRowsItem* __restrict__ items, int pass, void* const* ptrs
       const long long k = kb + row;
       const int ci = ti * GX_T + 4 * qd, cj = tj * GX_T + 4 * qd;
       const bool okk = k < k1;
-      gx_copy16(xs + row * GX_T + 4 * qd, okk && ci < F ? X + k * F + ci : X, okk && ci < F);
-      if (!diag) gx_copy16(xs + (GX_RUN + row) * GX_T + 4 * qd, okk && cj < F ? X + k * F + cj : X, okk && cj < F);
+      copy_quad(xs + row * GX_T + 4 * qd, okk && ci < F ? X + k * F + ci : X, okk && ci < F);
+      if (!diag) copy_quad(xs + (GX_RUN + row) * GX_T + 4 * qd, okk && cj < F ? X + k * F + cj : X, okk && cj < F);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
