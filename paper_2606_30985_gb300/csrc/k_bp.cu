@@ -184,31 +184,45 @@ __global__ void k_edge_scalars(const EdgeItem* __restrict__ items, const int* iv
 // ======================================================= Pauli weights
 // Zero the outputs, then each block of grid.x sums its slice of one item's
 // squares per Pauli index (the index is the innermost one) and adds them in.
+// Bound: HBM; FP32 storage sums in two floats (an FP64 multiply-add and the
+// conversion per value kept the FP64 pipe busy four times as long: 1.28 -> 0.29 ms
+// for a 4x4, chi = 64 grid).
 __global__ void k_pauli_zero(const PauliWItem* __restrict__ items) {
   if (threadIdx.x < 4) items[blockIdx.x].out[threadIdx.x] = 0.0;
 }
 
+struct PlainSum {
+  double s = 0.0;
+  __device__ void take_product(double x, double y) { s = fma(x, y, s); }
+  __device__ double value() const { return s; }
+};
+template <typename T> struct PauliAcc;
+template <> struct PauliAcc<float> { using Sum = TwoFloat; using Quad = float4; };
+template <> struct PauliAcc<double> { using Sum = PlainSum; using Quad = double4; };
+
 template <typename T>
-__global__ void k_pauli_weights(const PauliWItem* __restrict__ items, void* const* ptrs, const int* ival) {
+__global__ void __launch_bounds__(256)
+k_pauli_weights(const PauliWItem* __restrict__ items, void* const* ptrs, const int* ival) {
   const PauliWItem it = items[blockIdx.y];
-  long long n = 4;
-  for (int k = 0; k < it.x.nlegs; ++k) n *= ival[it.x.dim[k]];
-  const T* x = static_cast<const T*>(ptrs[it.x.ref]);
-  // each thread visits whole groups of 4 (one J), so its p-th partial is Pauli p
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  const long long groups = n / 4;
+  long long groups = 1;
+  for (int k = 0; k < it.x.nlegs; ++k) groups *= ival[it.x.dim[k]];
+  using Quad = typename PauliAcc<T>::Quad;
+  const Quad* x = static_cast<const Quad*>(ptrs[it.x.ref]);
+  // a quad holds the four Paulis of one J, so the p-th partial is Pauli p
+  typename PauliAcc<T>::Sum acc[4];
+#pragma unroll 4
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < groups;
        g += (long long)gridDim.x * blockDim.x) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const double v = (double)x[g * 4 + q];
-      acc[q] = fma(v, v, acc[q]);
-    }
+    const Quad v = x[g];
+    acc[0].take_product(v.x, v.x);
+    acc[1].take_product(v.y, v.y);
+    acc[2].take_product(v.z, v.z);
+    acc[3].take_product(v.w, v.w);
   }
   __shared__ double red[8];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const double t = bsum(acc[q], red);
+    const double t = bsum(acc[q].value(), red);
     if (threadIdx.x == 0) atomicAdd(&it.out[q], t);
   }
 }
@@ -218,7 +232,8 @@ cudaError_t launch_pauli_weights(const PauliWItem* items, int n, void* const* pt
                                  cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   k_pauli_zero<<<n, 32, 0, s>>>(items);
-  k_pauli_weights<T><<<dim3(64, n), 256, 0, s>>>(items, ptrs, ival);
+  // about 16 blocks per SM in all
+  k_pauli_weights<T><<<dim3(max(8, min(256, ceil_div(16 * 152, n))), n), 256, 0, s>>>(items, ptrs, ival);
   return cudaGetLastError();
 }
 template cudaError_t launch_pauli_weights<float>(const PauliWItem*, int, void* const*, const int*, cudaStream_t);

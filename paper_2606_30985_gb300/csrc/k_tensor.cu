@@ -660,22 +660,14 @@ template <> struct VecSum<double> {
   static __device__ double split(double v) { return v; }
   using V = double;
 };
-template <> struct VecSum<float> {
-  float s = 0.f, c = 0.f;
+template <> struct VecSum<float> : TwoFloat {
   using V = float2;
   static __device__ float2 split(double v) {
     const float h = (float)v;
     return make_float2(h, (float)(v - (double)h));
   }
-  __device__ void take(float p) {
-    const float t = s + p, b = t - s;
-    c += (s - (t - b)) + (p - b);
-    s = t;
-  }
   __device__ void add(float x, float2 v) {
-    const float p = x * v.x;
-    c += fmaf(x, v.x, -p);
-    take(p);
+    take_product(x, v.x);
     c = fmaf(x, v.y, c);
   }
   __device__ void merge(int o) {
@@ -683,7 +675,6 @@ template <> struct VecSum<float> {
     take(p);
     c += q;
   }
-  __device__ double value() const { return (double)s + (double)c; }
 };
 
 // One pass over the pinned slice feeds both first contractions: lanes hold the
