@@ -52,6 +52,7 @@ namespace um {
 
 constexpr int kThreads = 512;
 constexpr int kConv = 256;              // converter threads (warps 8..15)
+constexpr int kGroup = 128;             // converter threads of one chunk: two groups take turns
 constexpr int kM = 128;                 // accumulator rows = TMEM lanes
 constexpr int kKC = 32;                 // K values per staged chunk
 constexpr int kTmemCols = 512;          // two accumulators of 256 columns
@@ -616,54 +617,55 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
 }
 
 // ============================================================ Gram (free leg)
-struct GramDims {
-  long long O, Q, NC;
-  int F, F8, S, k, nlegs, d[PEPO_MAXLEG];
-  bool wide;
-  long long qpc;
-  int opc;
+// A free-leg Gram sums over the flattened (o, q): NQ quads of 4 values per row,
+// Q4 per (o, row).  A chunk is 8 quads of every row; unit = (item, split) = a
+// range of chunks.
+struct GramUnit {
   const float* X;
   double* partial;
+  long long FQ, Q;     // values between two o, between two rows
+  unsigned Q4, NQ;
+  int F, F8, s;
+  unsigned c0, c1;     // chunks of the unit
 };
-
-__device__ inline void gram_dims(const GramLegItem& it, void* const* ptrs, const int* ival, int splits_max,
-                                 GramDims& G) {
-  G.nlegs = it.x.nlegs;
-  G.k = it.leg;
-  G.F = 1;
-  G.O = 1;
-  G.Q = 4;
-  // constant indices only (unrolled selects), so the dims stay in registers
+__device__ inline void gram_extent(const GramLegItem& it, const int* ival, int& F, unsigned& O, unsigned& Q4) {
+  F = 1;
+  O = 1;
+  Q4 = 1;
 #pragma unroll
   for (int k = 0; k < PEPO_MAXLEG; ++k) {
     const int dk = (k < it.x.nlegs) ? ival[it.x.dim[k]] : 1;
-    G.d[k] = dk;
-    if (k == G.k) G.F = dk;
-    else if (k < G.k) G.O *= dk;
-    else if (k < G.nlegs) G.Q *= dk;
+    if (k == it.leg) F = dk;
+    else if (k < it.leg) O *= dk;
+    else Q4 *= dk;
   }
-  G.F8 = round_up(G.F, 8);
-  G.NC = gram_leg_chunks(G.O, G.Q);
-  G.S = gram_leg_splits_k(G.O * G.Q, splits_max, kGramLegRowsUmma);
-  G.wide = G.Q >= kKC;
-  G.qpc = G.wide ? (G.Q + kKC - 1) / kKC : 0;
-  G.opc = G.wide ? 1 : (int)(kKC / G.Q);
-  G.X = static_cast<const float*>(ptrs[it.x.ref]);
-  G.partial = it.partial;
+}
+__device__ inline int gram_splits(unsigned O, unsigned Q4, int splits_max) {
+  return gram_leg_splits_k((long long)O * Q4 * 4, splits_max, kGramLegRowsUmma);
+}
+// unit u through the prefix table of split counts
+__device__ __noinline__ void gram_unit(GramUnit& g, long long u, const long long* uoff, int n, const GramLegItem* items,
+                                       void* const* ptrs, const int* ival, int splits_max) {
+  int i = 0;
+  while (i + 1 < n && uoff[i + 1] <= u) ++i;
+  const GramLegItem& it = items[i];
+  unsigned O;
+  gram_extent(it, ival, g.F, O, g.Q4);
+  g.F8 = round_up(g.F, 8);
+  g.Q = 4ll * g.Q4;
+  g.FQ = g.Q * g.F;
+  g.NQ = O * g.Q4;
+  const unsigned long long NC = (g.NQ + 7) / 8, S = (unsigned long long)gram_splits(O, g.Q4, splits_max);
+  g.s = (int)(u - uoff[i]);
+  g.c0 = (unsigned)(NC * g.s / S);
+  g.c1 = (unsigned)(NC * (g.s + 1) / S);
+  g.X = static_cast<const float*>(ptrs[it.x.ref]);
+  g.partial = it.partial;
 }
 
-// Converter raw staging: each converter thread copies its four 16-byte
-// pieces of a chunk with cp.async into its own slots of a raw stage (piece u
-// of thread t at (u kConv + t) 16 bytes, then the item's padded row count per
-// thread), kRawMax chunks ahead of the chunk it converts, so the loads of
-// several chunks are in flight without holding registers.
-constexpr int kRawMax = 6;
-constexpr size_t kRawF8Off = (size_t)kConv * 4 * 16;                      // after the pieces
-constexpr size_t kRawBytes = kRawF8Off + (size_t)kConv * 4;                 // pieces, F8
-
 struct GramSmem {
-  int f8max, stages, ld, raw;
-  size_t stage_bytes, raw_off, acc_off, bar_off, total;
+  int f8max, stages, ld;
+  size_t stage_bytes, acc_off, bar_off, total;
 };
 __host__ __device__ inline GramSmem gram_smem(int chimax) {
   GramSmem p;
@@ -673,145 +675,18 @@ __host__ __device__ inline GramSmem gram_smem(int chimax) {
   p.ld = p.f8max + 1;                                               // odd row stride (words)
   const size_t acc_bytes = 2 * (size_t)p.f8max * p.ld * 4;          // sum + compensation
   const size_t budget = 227 * 1024 - 1024 - 8 * (kMaxItems + 1) - 512 - 1024;
-  p.stages = 2;
-  const size_t fixed = acc_bytes + 2 * p.stage_bytes;
-  p.raw = fixed < budget ? (int)((budget - fixed) / kRawBytes) : 0;
-  if (p.raw > kRawMax) p.raw = kRawMax;
-  p.raw_off = p.stages * p.stage_bytes;
-  p.acc_off = p.raw_off + (size_t)p.raw * kRawBytes;
+  p.stages = acc_bytes < budget ? (int)((budget - acc_bytes) / p.stage_bytes) : 0;
+  if (p.stages > 4) p.stages = 4;
+  p.acc_off = p.stages * p.stage_bytes;
   p.bar_off = p.acc_off + acc_bytes;
   p.total = p.bar_off + 512 + 8 * (size_t)(kMaxItems + 1) + 1024 + 1024;
   return p;
-}
-
-struct GramCursor {
-  int item, s;
-  long long c, c1;    // current chunk, end of the unit's range
-  GramDims G;
-};
-
-// unit u -> (item, split) through the prefix table of split counts
-__device__ inline void gram_unit(GramCursor& g, long long u, const long long* uoff, int n,
-                                 const GramLegItem* items, void* const* ptrs, const int* ival, int splits_max) {
-  int i = 0;
-  while (i + 1 < n && uoff[i + 1] <= u) ++i;
-  if (i != g.item) {
-    g.item = i;
-    gram_dims(items[i], ptrs, ival, splits_max, g.G);
-  }
-  g.s = (int)(u - uoff[i]);
-  g.c = g.G.NC * g.s / g.G.S;
-  g.c1 = g.G.NC * (g.s + 1) / g.G.S;
 }
 
 struct GramBars {
   uint64_t full[4], empty[4], accfull[2], accempty[2], drain;
   uint32_t tmem;
   int abort_flag;
-};
-
-
-// Load side of the Gram converters: the cursor of one converter thread over
-// the chunks of its CTA's units (items x splits), kept in registers.  Per
-// chunk, issue() copies the thread's column group (4 K values) of its four
-// rows with cp.async into its slots of a raw stage, with the item's padded row
-// count F8 (0 once the CTA's work is done); the source pointer advances
-// incrementally.  The Gram is unweighted: the BP message weights are carried
-// by the rotated tensor itself (its legs are scaled by the square roots of the
-// message eigenvalues).
-struct GramLoader {
-  int kq, row0;
-  long long lu, lcur, lend, stride_u;
-  bool live;
-  int item, F, F8, Q4, qpc, opc;
-  bool wide;
-  long long Q, O, FQ;
-  const float* X;
-  long long roff0, roff1, roff2, roff3;
-  bool rv0, rv1, rv2, rv3;
-  int lqb;
-  long long lo;
-  const float* lp;
-
-  __device__ __forceinline__ void init(int kq_, int row0_, long long first_unit) {
-    kq = kq_;
-    row0 = row0_;
-    lu = first_unit;
-    stride_u = gridDim.x;
-    item = -1;
-    live = false;
-  }
-  // position the cursor at the first chunk of unit lu (item constants are
-  // reloaded when the item changes)
-  __device__ __forceinline__ void enter_unit(const GramLegItem* items, int n_items, const long long* uoff, long long U,
-                                             void* const* ptrs, const int* ival, int splits_max) {
-    live = lu < U;
-    if (!live) return;
-    int i = 0;
-    while (i + 1 < n_items && uoff[i + 1] <= lu) ++i;
-    if (i != item) {
-      item = i;
-      GramDims G;
-      gram_dims(items[i], ptrs, ival, splits_max, G);
-      F = G.F; F8 = G.F8; Q = G.Q; O = G.O; X = G.X; wide = G.wide;
-      Q4 = (int)(G.Q / 4);
-      qpc = (int)G.qpc; opc = G.opc;
-      FQ = (long long)G.F * G.Q;
-      const int r0 = row0, r1 = row0 + 32, r2 = row0 + 64, r3 = row0 + 96;
-      roff0 = (long long)r0 * Q; roff1 = (long long)r1 * Q; roff2 = (long long)r2 * Q; roff3 = (long long)r3 * Q;
-      rv0 = r0 < F; rv1 = r1 < F; rv2 = r2 < F; rv3 = r3 < F;
-    }
-    const long long NC = gram_leg_chunks(O, Q);
-    const int S = gram_leg_splits_k(O * Q, splits_max, kGramLegRowsUmma);
-    const int sp = (int)(lu - uoff[item]);
-    lcur = NC * sp / S;
-    lend = NC * (sp + 1) / S;
-    if (wide) {
-      lo = lcur / qpc;
-      lqb = (int)(lcur - lo * qpc);
-      lp = X + lo * FQ + (long long)lqb * kKC + 4 * kq;
-    } else {
-      lo = lcur * opc;
-      const int ooff = kq / Q4, q4 = kq - ooff * Q4;
-      lp = X + (lo + ooff) * FQ + 4 * q4;
-    }
-  }
-  // copy the chunk at the cursor into raw stage rb (one copy group) and
-  // advance; returns true when the unit is finished (the caller then enters
-  // the next one).  Columns outside the item are zero-filled (no read).
-  __device__ __forceinline__ bool issue(unsigned char* rb, int ct) {
-    int* f8slot = reinterpret_cast<int*>(rb + kRawF8Off + (size_t)ct * 4);
-    if (!live) {
-      *f8slot = 0;
-      cp_async_commit();   // empty group: keeps one group per chunk slot
-      return false;
-    }
-    const bool kvalid = wide ? (lqb * 8 + kq < Q4) : (kq / Q4 < opc && lo + kq / Q4 < O);
-    const void* z = (const void*)X;
-    cp_async16(rb + ((size_t)0 * kConv + ct) * 16, (kvalid && rv0) ? (const void*)(lp + roff0) : z, (kvalid && rv0) ? 16 : 0);
-    cp_async16(rb + ((size_t)1 * kConv + ct) * 16, (kvalid && rv1) ? (const void*)(lp + roff1) : z, (kvalid && rv1) ? 16 : 0);
-    cp_async16(rb + ((size_t)2 * kConv + ct) * 16, (kvalid && rv2) ? (const void*)(lp + roff2) : z, (kvalid && rv2) ? 16 : 0);
-    cp_async16(rb + ((size_t)3 * kConv + ct) * 16, (kvalid && rv3) ? (const void*)(lp + roff3) : z, (kvalid && rv3) ? 16 : 0);
-    *f8slot = F8;
-    cp_async_commit();
-    if (++lcur < lend) {
-      if (wide) {
-        if (++lqb == qpc) {
-          lqb = 0;
-          ++lo;
-          lp += FQ - (long long)(qpc - 1) * kKC;
-        } else {
-          lp += kKC;
-        }
-      } else {
-        lo += opc;
-        lp += (long long)opc * FQ;
-      }
-      return false;
-    }
-    lu += stride_u;
-    return true;
-  }
 };
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -829,16 +704,14 @@ k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NS = P.stages;
 
+  for (int i = tid; i < n_items; i += kThreads) {
+    int F;
+    unsigned O, Q4;
+    gram_extent(items[i], ival, F, O, Q4);
+    uoff[i + 1] = gram_splits(O, Q4, splits_max);
+  }
   if (tid == 0) {
-    long long a = 0;
-    for (int i = 0; i < n_items; ++i) {
-      uoff[i] = a;
-      GramDims G;
-      gram_dims(items[i], ptrs, ival, splits_max, G);
-      a += G.S;
-    }
-    uoff[n_items] = a;
-    for (int s = 0; s < NS; ++s) { mbar_init(&bars->full[s], kConv / 32); mbar_init(&bars->empty[s], 1); }
+    for (int s = 0; s < NS; ++s) { mbar_init(&bars->full[s], kGroup / 32); mbar_init(&bars->empty[s], 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(&bars->accfull[b], 1); mbar_init(&bars->accempty[b], 4); }
     mbar_init(&bars->drain, 1);
     bars->abort_flag = 0;
@@ -851,6 +724,11 @@ k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, 
   if (warp == 0) tmem_alloc(&bars->tmem);
   tc_before();
   __syncthreads();
+  if (tid == 0) {
+    uoff[0] = 0;
+    for (int i = 0; i < n_items; ++i) uoff[i + 1] += uoff[i];
+  }
+  __syncthreads();
   tc_after();
   const uint32_t tmem = bars->tmem;
   const long long U = uoff[n_items];
@@ -858,23 +736,21 @@ k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, 
   if (warp == 0) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
-      GramCursor g;
-      g.item = -1;
+      GramUnit g;
       long long rc = 0;
       int st_i = 0;            // operand stage and its phase parity (advanced per chunk)
       uint32_t st_ph = 0;
       bool ok = true;
       for (long long u = blockIdx.x; u < U && ok; u += gridDim.x) {
         gram_unit(g, u, uoff, n_items, items, ptrs, ival, splits_max);
-        const int F8 = g.G.F8;
-        const uint32_t id = idesc_tf32(kM, 2 * F8);
-        for (long long c = g.c; c < g.c1 && ok;) {
+        const uint32_t id = idesc_tf32(kM, 2 * g.F8);
+        for (unsigned c = g.c0; c < g.c1 && ok;) {
           const int b = (int)(rc & 1);
           if (!mbar_wait(&bars->accempty[b], (uint32_t)(((rc >> 1) & 1) ^ 1), abort_flag, err, lim)) { ok = false; break; }
           tc_after();
           const uint32_t d_tmem = tmem + (uint32_t)(b * 256);
-          const long long cend = min(g.c1, c + kRun);
-          for (long long cr = c; cr < cend; ++cr) {
+          const unsigned cend = min(g.c1, c + kRun);
+          for (unsigned cr = c; cr < cend; ++cr) {
             const int s = st_i;
             if (!mbar_wait(&bars->full[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
             if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
@@ -901,17 +777,16 @@ k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, 
     // -------------------------------------------------------------- epilogue
     const int row = 32 * (warp & 3) + lane;
     const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
-    GramCursor g;
-    g.item = -1;
+    GramUnit g;
     long long rc = 0;
     bool ok = true;
     for (long long u = blockIdx.x; u < U && ok; u += gridDim.x) {
       gram_unit(g, u, uoff, n_items, items, ptrs, ival, splits_max);
-      const int F = g.G.F, F8 = g.G.F8;
+      const int F = g.F, F8 = g.F8;
       const bool live_row = row < F;
       if (live_row)
         for (int c0 = 0; c0 < F8; ++c0) { acc[(size_t)row * P.ld + c0] = 0.f; cmp[(size_t)row * P.ld + c0] = 0.f; }
-      for (long long c = g.c; c < g.c1; c += kRun) {
+      for (unsigned c = g.c0; c < g.c1; c += kRun) {
         const int b = (int)(rc & 1);
         if (!warp_wait(&bars->accfull[b], (uint32_t)((rc >> 1) & 1), abort_flag, err, lim)) { ok = false; break; }
         tc_after();
@@ -943,66 +818,81 @@ k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, 
       }
       if (!ok) break;
       if (live_row) {
-        double* P0 = g.G.partial + (size_t)g.s * F * F + (size_t)row * F;
+        double* P0 = g.partial + (size_t)g.s * F * F + (size_t)row * F;
         for (int col = 0; col < F; ++col)
           P0[col] = (double)acc[(size_t)row * P.ld + col] - (double)cmp[(size_t)row * P.ld + col];
       }
     }
   } else if (warp >= 8) {
     // ------------------------------------------------------------ converters
-    // Load side: this thread's column group of each chunk (4 K values) for
-    // its four rows is copied with cp.async into its own slots of a raw stage,
-    // P.raw chunks ahead of the conversion, together with the item's padded
-    // row count F8 (0 marks the end of the CTA's work).  The cursor lives in
-    // registers and the source pointer advances incrementally.
-    const int ct = tid - 256, cw = ct >> 5;
-    const int kq = 4 * (cw & 1) + (lane >> 3);     // this thread's 4-wide K group of a chunk
-    const int i8_0 = cw >> 1;                      // row groups i8_0 + 4 u, u = 0..3
-    const int il = lane & 7;
-    unsigned char* raw = smem + P.raw_off;
-    const int DR = P.raw;
-    GramLoader ld;
-    ld.init(kq, 8 * i8_0 + il, blockIdx.x);
-    ld.enter_unit(items, n_items, uoff, U, ptrs, ival, splits_max);
-    auto issue_next = [&](int rs) {
-      if (ld.issue(raw + (size_t)rs * kRawBytes, ct))
-        ld.enter_unit(items, n_items, uoff, U, ptrs, ival, splits_max);
-    };
-    for (int d = 0; d < DR; ++d) issue_next(d);
-    // conversion side: wait for this thread's copies of chunk cc, split and
-    // store into the operand stage, then refill the raw stage
-    int rs = 0;                // raw stage of the chunk being converted
-    int st_i = 0;              // operand stage and its phase parity
-    uint32_t st_ph = 0;
-    while (true) {
-      cp_async_wait(DR - 1);
-      const unsigned char* rb = raw + (size_t)rs * kRawBytes;
-      const int F8 = *reinterpret_cast<const int*>(rb + kRawF8Off + (size_t)ct * 4);
-      if (F8 == 0) break;
-      float4 vs[4];
+    // This thread copies quad kq of the rows r0 + 16 u of every other chunk of
+    // the unit: the eight lanes of a row read 128 consecutive bytes (or eight
+    // consecutive o), store one swizzled 128-byte row without bank conflicts.
+    const int ct = tid - 256, grp = ct / kGroup, t = ct % kGroup;
+    const int kq = t & 7, r0 = t >> 3;
+    constexpr int MU = kM / (kGroup / 8);             // row steps of 16
+    unsigned n = 0;                                   // chunks of the CTA before this unit
+    GramUnit g;
+    bool ok = true;
+    for (long long u = blockIdx.x; u < U && ok; u += gridDim.x) {
+      gram_unit(g, u, uoff, n_items, items, ptrs, ival, splits_max);
+      unsigned c = g.c0 + ((n ^ (unsigned)grp) & 1u);  // this group's first chunk
+      unsigned nn = n + (c - g.c0);                    // its number in the CTA
+      n += g.c1 - g.c0;
+      unsigned qi = 8 * c + kq;
+      const unsigned o = qi / g.Q4;
+      unsigned q4 = qi - o * g.Q4;
+      const float* src = g.X + (long long)o * g.FQ + 4ll * q4 + (long long)r0 * g.Q;
+      // the quad 16 further on: dO o's and dq quads
+      const unsigned dO = 16 / g.Q4, dq = 16 - dO * g.Q4;
+      const long long step = (long long)dO * g.FQ + 4ll * dq, wrap = g.FQ - g.Q, rows16 = 16 * g.Q;
+      const unsigned Q4 = g.Q4, NQ = g.NQ, c1 = g.c1;
+      const int F = g.F, F8 = g.F8;
+      auto load = [&](float4 (&v)[MU]) {
+        const bool live = qi < NQ;
+        const float* p = src;
 #pragma unroll
-      for (int u4 = 0; u4 < 4; ++u4) vs[u4] = *reinterpret_cast<const float4*>(rb + ((size_t)u4 * kConv + ct) * 16);
-      const int s = st_i;
-      if (!warp_wait(&bars->empty[s], st_ph ^ 1u, abort_flag, err, lim)) break;
-      if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
-      unsigned char* st = Xs + (size_t)s * P.stage_bytes;
-#pragma unroll
-      for (int u4 = 0; u4 < 4; ++u4) {
-        const int i = 8 * (i8_0 + 4 * u4) + il;
-        if (i < F8) {
-          const float4 x = vs[u4];
-          const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
-          const float4 l = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
-          *reinterpret_cast<float4*>(st + swz(i, kq)) = h;
-          *reinterpret_cast<float4*>(st + swz(i + F8, kq)) = l;
+        for (int i = 0; i < MU; ++i) {
+          v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (live && r0 + 16 * i < F) v[i] = __ldg(reinterpret_cast<const float4*>(p));
+          p += rows16;
         }
+        qi += 16;
+        q4 += dq;
+        src += step;
+        if (q4 >= Q4) { q4 -= Q4; src += wrap; }
+      };
+      auto convert = [&](const float4 (&v)[MU]) -> bool {
+        const unsigned s = nn % (unsigned)NS;
+        if (!warp_wait(&bars->empty[s], ((nn / (unsigned)NS) & 1u) ^ 1u, abort_flag, err, lim)) return false;
+        unsigned char* st = Xs + (size_t)s * P.stage_bytes;
+#pragma unroll
+        for (int i = 0; i < MU; ++i) {
+          const int r = r0 + 16 * i;
+          if (r < F8) {
+            const float4 x = v[i];
+            const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
+            *reinterpret_cast<float4*>(st + swz(r, kq)) = h;
+            *reinterpret_cast<float4*>(st + swz(r + F8, kq)) = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
+          }
+        }
+        fence_async_smem();
+        warp_arrive(&bars->full[s]);
+        nn += 2;
+        return true;
+      };
+      float4 v0[MU], v1[MU];
+      if (c < c1) load(v0);
+      while (c < c1) {
+        if (c + 2 < c1) load(v1);
+        if (!convert(v0)) { ok = false; break; }
+        c += 2;
+        if (c >= c1) break;
+        if (c + 2 < c1) load(v0);
+        if (!convert(v1)) { ok = false; break; }
+        c += 2;
       }
-      fence_async_smem();
-      warp_arrive(&bars->full[s]);
-      issue_next(rs);
-      if (++rs == DR) rs = 0;
     }
-    cp_async_wait(0);   // no copy may land after the kernel's shared memory is gone
   }
   tc_before();
   __syncthreads();
@@ -1523,7 +1413,7 @@ cudaError_t launch_gram_umma(const GramLegItem* items, int n_items, int splits_m
   if (n_items == 0) return cudaSuccess;
   if (!umma_supported(chimax)) return cudaErrorInvalidValue;
   const um::GramSmem P = um::gram_smem(chimax);
-  if (P.raw < 1) return cudaErrorInvalidValue;
+  if (P.stages < 2) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(um::k_gram_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.total);
   if (e != cudaSuccess) return e;
   for (int i0 = 0; i0 < n_items; i0 += um::kMaxItems) {
