@@ -254,34 +254,53 @@ __device__ __forceinline__ float tf32_hi(float x) {
 __host__ __device__ inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
 // ============================================================ leg contraction
-struct LegDims {
-  long long O, Q, R, tiles;
-  int J, Jout, K8, N16;
+struct LegPlan {
   const float* in;
   float* out;
   const double* A;
-  int lda;
+  unsigned R, Q;       // rows (o, q) of the item, values between two j
+  int J, Jout, K8, N16, nkc, lda;
 };
 
-__device__ inline void leg_dims(const LegItem& it, void* const* ptrs, const int* ival, LegDims& L) {
-  int d[PEPO_MAXLEG];
-  for (int k = 0; k < PEPO_MAXLEG; ++k) d[k] = (k < it.in.nlegs) ? ival[it.in.dim[k]] : 1;
-  const int k = it.leg;
-  L.J = d[k];
+__device__ inline unsigned leg_rows(const LegItem& it, const int* ival, unsigned& Q, int& J) {
+  unsigned O = 1;
+  Q = 4;
+  J = 1;
+#pragma unroll
+  for (int k = 0; k < PEPO_MAXLEG; ++k) {
+    const int dk = (k < it.in.nlegs) ? ival[it.in.dim[k]] : 1;
+    if (k == it.leg) J = dk;
+    else if (k < it.leg) O *= dk;
+    else Q *= dk;
+  }
+  return O * Q;
+}
+__device__ __noinline__ void leg_plan(const LegItem* items, int i, void* const* ptrs, const int* ival, LegPlan& L) {
+  const LegItem& it = items[i];
+  L.R = leg_rows(it, ival, L.Q, L.J);
   L.Jout = ival[it.out_dim];
-  L.O = 1;
-  L.Q = 4;
-  for (int i = 0; i < k; ++i) L.O *= d[i];
-  for (int i = k + 1; i < it.in.nlegs; ++i) L.Q *= d[i];
-  L.R = L.O * L.Q;
-  L.tiles = (L.R + kM - 1) / kM;
   L.K8 = round_up(L.J, 8);
   // N >= 16: a factor of rank 0 (a message that is not finite) still issues MMAs
   L.N16 = round_up(L.Jout > 0 ? L.Jout : 1, 16);
+  L.nkc = (L.K8 + kKC - 1) / kKC;
   L.in = static_cast<const float*>(ptrs[it.in.ref]);
   L.out = static_cast<float*>(ptrs[it.out_ref]);
   L.A = it.A;
   L.lda = it.lda;
+}
+
+// The CTA's tiles t0 .. t1 of the launch, item by item: tiles lo .. hi of `item`.
+struct ItemRange {
+  int item;
+  unsigned lo, hi, t, t1;
+};
+__device__ inline bool range_next(ItemRange& r, const unsigned* toff, int n) {   // false when the CTA is done
+  if (r.t >= r.t1) return false;
+  while (r.item + 1 < n && toff[r.item + 1] <= r.t) ++r.item;
+  r.lo = r.t - toff[r.item];
+  r.hi = min(r.t1, toff[r.item + 1]) - toff[r.item];
+  r.t += r.hi - r.lo;
+  return true;
 }
 
 // Shared-memory plan of k_leg_umma for a given chi bound.
@@ -304,39 +323,6 @@ __host__ __device__ inline LegSmem leg_smem(int chimax) {
   return p;
 }
 
-struct LegCursor {   // position in the CTA's tile range
-  int item;
-  long long tile;    // tile within the item
-  long long left;    // tiles left for this CTA
-  LegDims L;
-};
-
-__device__ inline bool cursor_start(LegCursor& c, const long long* toff, int n, long long t0, long long t1,
-                                    const LegItem* items, void* const* ptrs, const int* ival) {
-  c.left = t1 - t0;
-  if (c.left <= 0) return false;
-  int i = 0;
-  while (i + 1 < n && toff[i + 1] <= t0) ++i;
-  c.item = i;
-  c.tile = t0 - toff[i];
-  leg_dims(items[i], ptrs, ival, c.L);
-  return true;
-}
-// advance to the next tile; returns true when the item changed
-__device__ inline bool cursor_next(LegCursor& c, const long long* toff, int n, const LegItem* items,
-                                   void* const* ptrs, const int* ival) {
-  --c.left;
-  ++c.tile;
-  bool changed = false;
-  while (c.left > 0 && c.tile >= c.L.tiles && c.item + 1 < n) {
-    ++c.item;
-    c.tile = 0;
-    leg_dims(items[c.item], ptrs, ival, c.L);
-    changed = true;
-  }
-  return changed;
-}
-
 struct LegBars {
   uint64_t full[4], empty[4], accfull[2], accempty[2], bfull, bfree, drain;
   uint32_t tmem;
@@ -352,21 +338,18 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
   unsigned char* Bs = smem;                          // [Ah; Al] small matrix
   unsigned char* As = smem + P.b_bytes;              // stages: hi tile, lo tile
   LegBars* bars = reinterpret_cast<LegBars*>(smem + P.bar_off);
-  long long* toff = reinterpret_cast<long long*>(smem + P.bar_off + 512);
+  unsigned* toff = reinterpret_cast<unsigned*>(smem + P.bar_off + 512);
   volatile int* abort_flag = &bars->abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NS = P.stages;
 
+  for (int i = tid; i < n_items; i += kThreads) {
+    unsigned Q;
+    int J;
+    toff[i + 1] = (leg_rows(items[i], ival, Q, J) + kM - 1) / kM;
+  }
   if (tid == 0) {
-    long long acc = 0;
-    for (int i = 0; i < n_items; ++i) {
-      toff[i] = acc;
-      LegDims L;
-      leg_dims(items[i], ptrs, ival, L);
-      acc += L.tiles;
-    }
-    toff[n_items] = acc;
-    for (int s = 0; s < NS; ++s) { mbar_init(&bars->full[s], kConv / 32); mbar_init(&bars->empty[s], 1); }
+    for (int s = 0; s < NS; ++s) { mbar_init(&bars->full[s], kGroup / 32); mbar_init(&bars->empty[s], 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(&bars->accfull[b], 1); mbar_init(&bars->accempty[b], 4); }
     mbar_init(&bars->bfull, kConv / 32);
     mbar_init(&bars->bfree, 1);
@@ -377,61 +360,60 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
   if (warp == 0) tmem_alloc(&bars->tmem);
   tc_before();
   __syncthreads();
+  if (tid == 0) {
+    toff[0] = 0;
+    for (int i = 0; i < n_items; ++i) toff[i + 1] += toff[i];
+  }
+  __syncthreads();
   tc_after();
   const uint32_t tmem = bars->tmem;
-  const long long T = toff[n_items];
-  const long long t0 = T * blockIdx.x / gridDim.x, t1 = T * (blockIdx.x + 1) / gridDim.x;
+  const unsigned long long T = toff[n_items];
+  ItemRange rg;
+  rg.item = 0;
+  rg.t = (unsigned)(T * blockIdx.x / gridDim.x);
+  rg.t1 = (unsigned)(T * (blockIdx.x + 1) / gridDim.x);
+  LegPlan L;
 
   if (warp == 0) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
-      LegCursor c;
-      bool live = cursor_start(c, toff, n_items, t0, t1, items, ptrs, ival);
-      long long tc = 0;
+      unsigned tc = 0;
       int st_i = 0;            // operand stage and its phase parity (advanced per chunk)
       uint32_t st_ph = 0;
-      int item_n = 0;
       bool ok = true;
-      if (live) ok = mbar_wait(&bars->bfull, 0, abort_flag, err, lim);
-      while (live && ok) {
-        const int b = (int)(tc & 1);
-        if (!mbar_wait(&bars->accempty[b], (uint32_t)(((tc >> 1) & 1) ^ 1), abort_flag, err, lim)) break;
-        tc_after();
-        const uint32_t d_tmem = tmem + (uint32_t)(b * 256);
-        const int N16 = c.L.N16, K8 = c.L.K8;
+      for (unsigned item_n = 0; ok && range_next(rg, toff, n_items); ++item_n) {
+        leg_plan(items, rg.item, ptrs, ival, L);
+        const int N16 = L.N16, K8 = L.K8, nkc = L.nkc;
         const uint32_t bblk = (uint32_t)(2 * N16) * 128;   // B block per K chunk
         const uint32_t id_wide = idesc_tf32(kM, 2 * N16), id_half = idesc_tf32(kM, N16);
-        const int nkc = (K8 + kKC - 1) / kKC;
-        for (int kc = 0; kc < nkc && ok; ++kc) {
-          const int s = st_i;
-          if (!mbar_wait(&bars->full[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
-          if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
+        if (!mbar_wait(&bars->bfull, item_n & 1u, abort_flag, err, lim)) break;
+        tc_after();
+        for (unsigned tile = rg.lo; tile < rg.hi && ok; ++tile, ++tc) {
+          const int b = (int)(tc & 1);
+          if (!mbar_wait(&bars->accempty[b], ((tc >> 1) & 1u) ^ 1u, abort_flag, err, lim)) { ok = false; break; }
           tc_after();
-          const uint32_t a_hi = su32(As + (size_t)s * P.stage_bytes);
-          const uint32_t a_lo = a_hi + (uint32_t)(P.stage_bytes / 2);
-          const uint32_t b0 = su32(Bs);
-          const int ksteps = min(kKC, K8 - kc * kKC) / 8;
-          for (int st = 0; st < ksteps; ++st) {
-            const uint64_t dah = sdesc(a_hi + (uint32_t)st * 32u);
-            const uint64_t dal = sdesc(a_lo + (uint32_t)st * 32u);
-            const uint64_t db = sdesc(b0 + (uint32_t)kc * bblk + (uint32_t)st * 32u);
-            mma_tf32(d_tmem, dah, db, id_wide, (kc > 0 || st > 0) ? 1u : 0u);
-            mma_tf32(d_tmem, dal, db, id_half, 1u);
+          const uint32_t d_tmem = tmem + (uint32_t)(b * 256);
+          for (int kc = 0; kc < nkc; ++kc) {
+            const int s = st_i;
+            if (!mbar_wait(&bars->full[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
+            if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
+            tc_after();
+            const uint32_t a_hi = su32(As + (size_t)s * P.stage_bytes);
+            const uint32_t a_lo = a_hi + (uint32_t)(P.stage_bytes / 2);
+            const uint32_t b0 = su32(Bs) + (uint32_t)kc * bblk;
+            const int ksteps = min(kKC, K8 - kc * kKC) / 8;
+            for (int st = 0; st < ksteps; ++st) {
+              const uint64_t dah = sdesc(a_hi + (uint32_t)st * 32u);
+              const uint64_t dal = sdesc(a_lo + (uint32_t)st * 32u);
+              const uint64_t db = sdesc(b0 + (uint32_t)st * 32u);
+              mma_tf32(d_tmem, dah, db, id_wide, (kc > 0 || st > 0) ? 1u : 0u);
+              mma_tf32(d_tmem, dal, db, id_half, 1u);
+            }
+            mma_commit(&bars->empty[s]);
           }
-          mma_commit(&bars->empty[s]);
+          if (ok) mma_commit(&bars->accfull[b]);
         }
-        if (!ok) break;
-        mma_commit(&bars->accfull[b]);
-        ++tc;
-        const bool last = (c.left == 1);
-        const bool changed = cursor_next(c, toff, n_items, items, ptrs, ival);
-        if (changed || last) mma_commit(&bars->bfree);
-        if (last) break;
-        if (changed) {
-          ++item_n;
-          if (!mbar_wait(&bars->bfull, (uint32_t)(item_n & 1), abort_flag, err, lim)) break;
-          tc_after();
-        }
+        if (ok) mma_commit(&bars->bfree);
       }
       // every issued MMA completes before tensor memory is released
       mma_commit(&bars->drain);
@@ -440,172 +422,162 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
     __syncwarp();
   } else if (warp >= 4 && warp < 8) {
     // -------------------------------------------------------------- epilogue
-    LegCursor c;
-    bool live = cursor_start(c, toff, n_items, t0, t1, items, ptrs, ival);
     const int row = 32 * (warp & 3) + lane;
     const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
-    long long tc = 0;
-    while (live) {
-      const int b = (int)(tc & 1);
-      if (!warp_wait(&bars->accfull[b], (uint32_t)((tc >> 1) & 1), abort_flag, err, lim)) break;
-      tc_after();
-      const LegDims& L = c.L;
-      const long long rg = c.tile * kM + row;
-      const bool valid = rg < L.R;
-      long long o = 0, q = 0;
-      if (valid) { o = rg / L.Q; q = rg - o * L.Q; }
-      float* dst = L.out + (o * L.Jout) * L.Q + q;
-      const uint32_t tbase = tmem + lane_base + (uint32_t)(b * 256);
-      // 16-column blocks; the TMEM loads of block i+1 are in flight while
-      // block i is stored (two register sets, unrolled so none is copied)
-      uint32_t a1[16], a2[16], b1[16], b2[16];
-      auto store_blk = [&](const uint32_t* p1, const uint32_t* p2, int c0) {
-        if (!valid) return;
+    unsigned tc = 0;
+    bool ok = true;
+    while (ok && range_next(rg, toff, n_items)) {
+      leg_plan(items, rg.item, ptrs, ival, L);
+      const int N16 = L.N16, Jout = L.Jout;
+      const unsigned Q = L.Q;
+      for (unsigned tile = rg.lo; tile < rg.hi; ++tile, ++tc) {
+        const int b = (int)(tc & 1);
+        if (!warp_wait(&bars->accfull[b], (tc >> 1) & 1u, abort_flag, err, lim)) { ok = false; break; }
+        tc_after();
+        const unsigned r = tile * kM + row;
+        const bool valid = r < L.R;
+        const unsigned o = valid ? r / Q : 0u, q = valid ? r - o * Q : 0u;
+        float* dst = L.out + (long long)o * Jout * Q + q;
+        const uint32_t tbase = tmem + lane_base + (uint32_t)(b * 256);
+        // 16-column blocks; the TMEM loads of block i+1 are in flight while
+        // block i is stored (two register sets, unrolled so none is copied)
+        uint32_t a1[16], a2[16], b1[16], b2[16];
+        auto store_blk = [&](const uint32_t* p1, const uint32_t* p2, int c0) {
+          if (!valid) return;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int col = c0 + i;
-          if (col < L.Jout) dst[(long long)col * L.Q] = __uint_as_float(p1[i]) + __uint_as_float(p2[i]);
-        }
-      };
-      tmem_ld16(tbase, a1);
-      tmem_ld16(tbase + (uint32_t)L.N16, a2);
-      tmem_wait32(a1, a2);
-      for (int c0 = 0; c0 < L.N16; c0 += 32) {
-        const bool m1 = c0 + 16 < L.N16;
-        if (m1) {
-          tmem_ld16(tbase + (uint32_t)(c0 + 16), b1);
-          tmem_ld16(tbase + (uint32_t)(L.N16 + c0 + 16), b2);
-        }
-        store_blk(a1, a2, c0);
-        if (!m1) break;
-        tmem_wait32(b1, b2);
-        const bool m2 = c0 + 32 < L.N16;
-        if (m2) {
-          tmem_ld16(tbase + (uint32_t)(c0 + 32), a1);
-          tmem_ld16(tbase + (uint32_t)(L.N16 + c0 + 32), a2);
-        }
-        store_blk(b1, b2, c0 + 16);
-        if (!m2) break;
+          for (int i = 0; i < 16; ++i) {
+            if (c0 + i < Jout) *dst = __uint_as_float(p1[i]) + __uint_as_float(p2[i]);
+            dst += Q;
+          }
+        };
+        tmem_ld16(tbase, a1);
+        tmem_ld16(tbase + (uint32_t)N16, a2);
         tmem_wait32(a1, a2);
+        for (int c0 = 0; c0 < N16; c0 += 32) {
+          const bool m1 = c0 + 16 < N16;
+          if (m1) {
+            tmem_ld16(tbase + (uint32_t)(c0 + 16), b1);
+            tmem_ld16(tbase + (uint32_t)(N16 + c0 + 16), b2);
+          }
+          store_blk(a1, a2, c0);
+          if (!m1) break;
+          tmem_wait32(b1, b2);
+          const bool m2 = c0 + 32 < N16;
+          if (m2) {
+            tmem_ld16(tbase + (uint32_t)(c0 + 32), a1);
+            tmem_ld16(tbase + (uint32_t)(N16 + c0 + 32), a2);
+          }
+          store_blk(b1, b2, c0 + 16);
+          if (!m2) break;
+          tmem_wait32(a1, a2);
+        }
+        tc_before();
+        warp_arrive(&bars->accempty[b]);
       }
-      tc_before();
-      warp_arrive(&bars->accempty[b]);
-      ++tc;
-      if (c.left == 1) break;
-      cursor_next(c, toff, n_items, items, ptrs, ival);
     }
   } else if (warp >= 8) {
     // ------------------------------------------------------------ converters
-    // Each thread owns one row r of the tile and, per chunk, four 4-wide K
-    // groups (jq = jq0 + 2 u): four coalesced 4-byte loads per group (the
-    // lanes of a warp read 32 consecutive rows), then one 16-byte store per
-    // group into the K-major layout (8 consecutive rows per quarter warp: no
-    // bank conflicts).  Loads run two chunks ahead of the stores (register
-    // ring v0, v1, v2).
-    const int ct = tid - 256, cw = ct >> 5;
-    const int r = 32 * (cw & 3) + lane;             // this thread's row
-    const int jq0 = cw >> 2;                        // K groups jq0, jq0 + 2, +4, +6
-    // load cursor
-    LegCursor lc;
-    bool lc_live = cursor_start(lc, toff, n_items, t0, t1, items, ptrs, ival);
-    int lkc = 0;
-    bool lvalid = false;
-    const float* lsrc = nullptr;
-    auto enter_tile = [&]() {
-      const long long rg = lc.tile * kM + r;
-      lvalid = rg < lc.L.R;
-      lsrc = lc.L.in;
-      if (lvalid) {
-        const long long o = rg / lc.L.Q, q = rg - o * lc.L.Q;
-        lsrc = lc.L.in + o * lc.L.J * lc.L.Q + q;
-      }
-      lkc = 0;
-    };
-    if (lc_live) enter_tile();
-    auto load_next = [&](float4* v) {
+    // This thread owns row r of every other chunk: 32 coalesced 4-byte loads
+    // (the lanes of a warp read 32 consecutive rows), then 16-byte stores into
+    // the K-major layout (8 consecutive rows per quarter warp: no bank conflicts).
+    // The loads of the group's next chunk are in flight while one is converted.
+    const int ct = tid - 256, grp = ct / kGroup, r = ct % kGroup;
+    unsigned n = 0;                                   // chunks of the CTA before this item
+    bool ok = true;
+    for (unsigned item_n = 0; ok && range_next(rg, toff, n_items); ++item_n) {
+      leg_plan(items, rg.item, ptrs, ival, L);
+      const int nkc = L.nkc, J = L.J, K8 = L.K8;
+      const unsigned Q = L.Q;
+      const unsigned total = (rg.hi - rg.lo) * (unsigned)nkc;
+      unsigned j = (n ^ (unsigned)grp) & 1u;           // this group's first chunk of the item
+      unsigned nn = n + j;                             // its number in the CTA
+      n += total;
+      // load cursor: chunk (tile, kc) and this thread's source row
+      unsigned tile = rg.lo, lj = j;
+      int kc = (int)j;
+      const float* src = L.in;
+      bool valid = false;
+      auto enter = [&]() {
+        while (kc >= nkc) { kc -= nkc; ++tile; }
+        const unsigned rr = tile * kM + r;
+        valid = rr < L.R;
+        const unsigned o = valid ? rr / Q : 0u;
+        src = L.in + (long long)o * J * Q + (valid ? rr - o * Q : 0u);
+      };
+      auto load = [&](float4 (&v)[8]) {
+        const int m = valid ? J - kc * kKC : 0;        // values of this row in the chunk
+        const float* p = src + (long long)(kc * kKC) * Q;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (!lc_live) return;
-      if (lvalid) {
-        const int J = lc.L.J;
-        const long long Q = lc.L.Q;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int j = lkc * kKC + 4 * (jq0 + 2 * u);
-          const float* p0 = lsrc + (long long)j * Q;
-          if (j < J) v[u].x = __ldg(p0);
-          if (j + 1 < J) v[u].y = __ldg(p0 + Q);
-          if (j + 2 < J) v[u].z = __ldg(p0 + 2 * Q);
-          if (j + 3 < J) v[u].w = __ldg(p0 + 3 * Q);
+        for (int u = 0; u < 8; ++u) {
+          v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (4 * u < m) v[u].x = __ldg(p);
+          p += Q;
+          if (4 * u + 1 < m) v[u].y = __ldg(p);
+          p += Q;
+          if (4 * u + 2 < m) v[u].z = __ldg(p);
+          p += Q;
+          if (4 * u + 3 < m) v[u].w = __ldg(p);
+          p += Q;
         }
+        lj += 2;
+        kc += 2;
+        if (lj < total) enter();
+      };
+      int ckc = (int)(j % (unsigned)nkc);              // K chunk of the chunk being converted
+      auto convert = [&](const float4 (&v)[8]) -> bool {
+        const unsigned s = nn % (unsigned)NS;
+        if (!warp_wait(&bars->empty[s], ((nn / (unsigned)NS) & 1u) ^ 1u, abort_flag, err, lim)) return false;
+        unsigned char* hi = As + (size_t)s * P.stage_bytes;
+        unsigned char* lo = hi + P.stage_bytes / 2;
+        const int kw = K8 - ckc * kKC;                 // columns the MMAs of this chunk read
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          if (4 * u < kw) {
+            const uint32_t off = swz(r, u);
+            const float4 x = v[u];
+            const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
+            *reinterpret_cast<float4*>(hi + off) = h;
+            *reinterpret_cast<float4*>(lo + off) = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
+          }
+        }
+        fence_async_smem();
+        warp_arrive(&bars->full[s]);
+        nn += 2;
+        ckc += 2;
+        while (ckc >= nkc) ckc -= nkc;
+        return true;
+      };
+      float4 v0[8], v1[8];
+      if (j < total) {
+        enter();
+        load(v0);
       }
-      if (++lkc < (lc.L.K8 + kKC - 1) / kKC) return;
-      if (lc.left == 1) { lc_live = false; return; }
-      cursor_next(lc, toff, n_items, items, ptrs, ival);
-      enter_tile();
-    };
-    float4 v0[4], v1[4], v2[4];
-    load_next(v0);
-    load_next(v1);
-    // store cursor
-    LegCursor c;
-    bool live = cursor_start(c, toff, n_items, t0, t1, items, ptrs, ival);
-    int st_i = 0;              // operand stage and its phase parity
-    uint32_t st_ph = 0;
-    int item_n = 0, kc = 0;
-    bool need_b = true;
-    // one chunk: issue the loads two chunks ahead into vl, convert and store
-    // vs (the ring is rotated by unrolling, never by copying registers, so
-    // no load is waited on before its turn); returns false at the end
-    auto step = [&](float4 (&vl)[4], float4 (&vs)[4]) -> bool {
-      const LegDims& L = c.L;
-      load_next(vl);
-      if (need_b) {
-        if (item_n > 0 && !warp_wait(&bars->bfree, (uint32_t)((item_n - 1) & 1), abort_flag, err, lim)) return false;
-        // [Ah; Al]: rows n < N16 hold hi(A[n, :]), rows N16 + n hold lo(A[n, :]);
-        // one block of 2 N16 rows per 32-wide K chunk
+      // the item's small matrix [Ah; Al]: rows q < N16 hold hi(A[q, :]), rows N16 + q
+      // hold lo(A[q, :]); one block of 2 N16 rows per 32-wide K chunk
+      if (item_n > 0 && !warp_wait(&bars->bfree, (item_n - 1) & 1u, abort_flag, err, lim)) break;
+      {
         const size_t bblk = (size_t)(2 * L.N16) * 128;
-        const int K32 = (L.K8 + kKC - 1) / kKC * kKC;
+        const int K32 = nkc * kKC;
         for (int e = ct; e < L.N16 * K32; e += kConv) {
-          const int n = e / K32, j = e - n * K32;
+          const int q = e / K32, k = e - q * K32;
           float x = 0.f;
-          if (n < L.Jout && j < L.J) x = (float)L.A[(long long)n * L.lda + j];
+          if (q < L.Jout && k < J) x = (float)L.A[(long long)q * L.lda + k];
           const float h = tf32_hi(x);
-          const float l = x - h;
-          unsigned char* blk = Bs + (size_t)(j / kKC) * bblk + (size_t)(j & 3) * 4;
-          const int piece = (j % kKC) >> 2;
-          *reinterpret_cast<float*>(blk + swz(n, piece)) = h;
-          *reinterpret_cast<float*>(blk + swz(n + L.N16, piece)) = l;
+          unsigned char* blk = Bs + (size_t)(k / kKC) * bblk + (size_t)(k & 3) * 4;
+          const int piece = (k % kKC) >> 2;
+          *reinterpret_cast<float*>(blk + swz(q, piece)) = h;
+          *reinterpret_cast<float*>(blk + swz(q + L.N16, piece)) = x - h;
         }
         fence_async_smem();
         warp_arrive(&bars->bfull);
-        need_b = false;
       }
-      const int s = st_i;
-      if (!warp_wait(&bars->empty[s], st_ph ^ 1u, abort_flag, err, lim)) return false;
-      if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
-      unsigned char* hi = As + (size_t)s * P.stage_bytes;
-      unsigned char* lo = hi + P.stage_bytes / 2;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const size_t off = swz(r, jq0 + 2 * u);
-        const float4 x = vs[u];
-        const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
-        *reinterpret_cast<float4*>(hi + off) = h;
-        *reinterpret_cast<float4*>(lo + off) = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
+      for (; j < total; j += 4) {
+        if (j + 2 < total) load(v1);
+        if (!convert(v0)) { ok = false; break; }
+        if (j + 2 >= total) break;
+        if (j + 4 < total) load(v0);
+        if (!convert(v1)) { ok = false; break; }
       }
-      fence_async_smem();
-      warp_arrive(&bars->full[s]);
-      if (++kc < (L.K8 + kKC - 1) / kKC) return true;
-      kc = 0;
-      if (c.left == 1) return false;
-      if (cursor_next(c, toff, n_items, items, ptrs, ival)) { ++item_n; need_b = true; }
-      return true;
-    };
-    while (live) {
-      if (!step(v2, v0)) break;
-      if (!step(v0, v1)) break;
-      if (!step(v1, v2)) break;
     }
   }
   tc_before();
