@@ -882,83 +882,63 @@ k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, 
 // converters (row-contiguous, 16-byte loads), B = [hi(W^T); lo(W^T)] of the
 // tile's N block as one bulk copy of a block pre-packed by k_pack_w (the
 // swizzled shared-memory image, so the copy is linear).
-struct RecDims {
-  long long R, tiles, nrb;
-  int n, np, K8, nnb, NB, cut, nl;
-  int d[PEPO_MAXLEG];
-  long long rstride[PEPO_MAXLEG], ostride[PEPO_MAXLEG];
+struct RecPlan {
   const float* in;
   float* out;
   const double* W;
-  int ldw;
   const float* Wp;
-  int nkc;
+  unsigned R, nrb;         // rows, row blocks of 128
+  int n, np, K8, nkc, nnb, NB, ldw;
+  unsigned d1, d2;         // extents of the last two of the (up to three) row legs
+  long long os0, os1, os2, ocut;   // output strides of the row legs and of the new cut leg
 };
 
-__device__ __forceinline__ void rec_dims(const ReconItem& it, void* const* ptrs, const int* ival, RecDims& D) {
-  // every array below is indexed with constants only (unrolled loops and
-  // selects), so a cursor holding RecDims stays in registers
-  D.nl = it.in.nlegs;
-  D.cut = D.nl - 1;
+__device__ inline unsigned rec_rows(const ReconItem& it, const int* ival) {
+  unsigned R = 1;
+#pragma unroll
+  for (int i = 0; i < PEPO_MAXLEG; ++i)
+    if (i + 1 < it.in.nlegs) R *= (unsigned)ival[it.in.dim[i]];
+  return R;
+}
+__device__ inline void rec_blocks(int np, int& nnb, int& NB) {
+  nnb = (np + 127) / 128;
+  NB = round_up((np + nnb - 1) / nnb, 8);
+}
+__device__ __noinline__ void rec_plan(const ReconItem* items, int i, void* const* ptrs, const int* ival, RecPlan& D) {
+  const ReconItem& it = items[i];
+  const int nl = it.in.nlegs, cut = nl - 1;
   const int chin = ival[it.new_dim];
-  int od[PEPO_MAXLEG];
-#pragma unroll
-  for (int k = 0; k < PEPO_MAXLEG; ++k) {
-    D.d[k] = (k < D.nl) ? ival[it.in.dim[k]] : 1;
-    od[k] = (k == D.cut) ? chin : D.d[k];
-  }
-  int dcut = 1;
-#pragma unroll
-  for (int k = 0; k < PEPO_MAXLEG; ++k) if (k == D.cut) dcut = D.d[k];
-  D.n = 4 * dcut;
+  D.n = 4 * ival[it.in.dim[cut]];
   D.np = 4 * chin;
-  D.R = 1;
-#pragma unroll
-  for (int i = 0; i < PEPO_MAXLEG; ++i) if (i < D.cut) D.R *= D.d[i];
-  // output stride of layout leg l: 4 x the product of the output extents of
-  // the legs that follow l in the output order out_perm
-  int pos[PEPO_MAXLEG], pdim[PEPO_MAXLEG];
-#pragma unroll
-  for (int kk = 0; kk < PEPO_MAXLEG; ++kk) {
-    pos[kk] = PEPO_MAXLEG;
-    pdim[kk] = 1;
-  }
-#pragma unroll
-  for (int kk = 0; kk < PEPO_MAXLEG; ++kk) {
-    if (kk >= D.nl) continue;
-    const int li = it.out_perm[kk];
-#pragma unroll
-    for (int l = 0; l < PEPO_MAXLEG; ++l)
-      if (l == li) { pos[l] = kk; pdim[kk] = od[l]; }
-  }
-#pragma unroll
-  for (int l = 0; l < PEPO_MAXLEG; ++l) {
-    long long st = 4;
-#pragma unroll
-    for (int kk = 0; kk < PEPO_MAXLEG; ++kk)
-      if (kk > pos[l] && kk < D.nl) st *= pdim[kk];
-    D.ostride[l] = st;
-  }
-  // row stride of layout leg i < cut in the input (cut leg last, row-major)
-#pragma unroll
-  for (int i = 0; i < PEPO_MAXLEG; ++i) {
-    long long st = 1;
-#pragma unroll
-    for (int j = 0; j < PEPO_MAXLEG; ++j)
-      if (j > i && j < D.cut) st *= D.d[j];
-    D.rstride[i] = st;
-  }
-  D.K8 = round_up(D.n, 8);
-  D.nnb = (D.np + 127) / 128;
-  D.NB = round_up((D.np + D.nnb - 1) / D.nnb, 8);
+  D.R = rec_rows(it, ival);
   D.nrb = (D.R + kM - 1) / kM;
-  D.tiles = D.nrb * D.nnb;
+  D.K8 = round_up(D.n, 8);
+  D.nkc = (D.K8 + kKC - 1) / kKC;
+  rec_blocks(D.np, D.nnb, D.NB);
+  // output stride of input leg l: 4 x the product of the output extents of the
+  // legs that follow it in the output order out_perm
+  long long os[PEPO_MAXLEG] = {0, 0, 0, 0};
+  int dd[PEPO_MAXLEG] = {1, 1, 1, 1};
+  long long st = 4;
+  for (int kk = nl - 1; kk >= 0; --kk) {
+    const int l = it.out_perm[kk];
+    const int e = l == cut ? chin : ival[it.in.dim[l]];
+    os[l] = st;
+    dd[l] = e;
+    st *= e;
+  }
+  D.ocut = os[cut];
+  // the row legs 0 .. cut - 1, right-aligned in three places (missing ones: extent 1)
+  D.os2 = cut >= 1 ? os[cut - 1] : 0;
+  D.d2 = cut >= 1 ? dd[cut - 1] : 1;
+  D.os1 = cut >= 2 ? os[cut - 2] : 0;
+  D.d1 = cut >= 2 ? dd[cut - 2] : 1;
+  D.os0 = cut >= 3 ? os[cut - 3] : 0;
   D.in = static_cast<const float*>(ptrs[it.in.ref]);
   D.out = static_cast<float*>(ptrs[it.out_ref]);
   D.W = it.W;
   D.ldw = it.ldw;
   D.Wp = it.Wp;
-  D.nkc = (D.K8 + kKC - 1) / kKC;
 }
 
 struct RecSmem {
@@ -973,33 +953,6 @@ __host__ __device__ inline RecSmem rec_smem() {
   p.bar_off = p.stages * p.stage_bytes;
   p.total = p.bar_off + 512 + 8 * (size_t)(kMaxItems + 1) + 1024;
   return p;
-}
-
-struct RecCursor {
-  int item;
-  long long tile, left;
-  RecDims D;
-};
-__device__ __forceinline__ bool rec_start(RecCursor& c, const long long* toff, int n, long long t0, long long t1,
-                                 const ReconItem* items, void* const* ptrs, const int* ival) {
-  c.left = t1 - t0;
-  if (c.left <= 0) return false;
-  int i = 0;
-  while (i + 1 < n && toff[i + 1] <= t0) ++i;
-  c.item = i;
-  c.tile = t0 - toff[i];
-  rec_dims(items[i], ptrs, ival, c.D);
-  return true;
-}
-__device__ __forceinline__ void rec_next(RecCursor& c, const long long* toff, int n, const ReconItem* items,
-                                void* const* ptrs, const int* ival) {
-  --c.left;
-  ++c.tile;
-  while (c.left > 0 && c.tile >= c.D.tiles && c.item + 1 < n) {
-    ++c.item;
-    c.tile = 0;
-    rec_dims(items[c.item], ptrs, ival, c.D);
-  }
 }
 
 struct RecBars {
@@ -1018,21 +971,18 @@ k_recon_umma(const ReconItem* __restrict__ items, int n_items, void* const* ptrs
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const RecSmem P = rec_smem();
   RecBars* bars = reinterpret_cast<RecBars*>(smem + P.bar_off);
-  long long* toff = reinterpret_cast<long long*>(smem + P.bar_off + 512);
+  unsigned* toff = reinterpret_cast<unsigned*>(smem + P.bar_off + 512);
   volatile int* abort_flag = &bars->abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NS = P.stages;
+  for (int i = tid; i < n_items; i += kThreads) {
+    int nnb, NB;
+    rec_blocks(4 * ival[items[i].new_dim], nnb, NB);
+    toff[i + 1] = (rec_rows(items[i], ival) + kM - 1) / kM * nnb;
+  }
   if (tid == 0) {
-    long long acc = 0;
-    for (int i = 0; i < n_items; ++i) {
-      toff[i] = acc;
-      RecDims D;
-      rec_dims(items[i], ptrs, ival, D);
-      acc += D.tiles;
-    }
-    toff[n_items] = acc;
     for (int s = 0; s < NS; ++s) {
-      mbar_init(&bars->full[s], kConv / 32);
+      mbar_init(&bars->full[s], kGroup / 32);
       mbar_init(&bars->wfull[s], 1);
       mbar_init(&bars->empty[s], 1);
     }
@@ -1044,243 +994,227 @@ k_recon_umma(const ReconItem* __restrict__ items, int n_items, void* const* ptrs
   if (warp == 0) tmem_alloc(&bars->tmem);
   tc_before();
   __syncthreads();
+  if (tid == 0) {
+    toff[0] = 0;
+    for (int i = 0; i < n_items; ++i) toff[i + 1] += toff[i];
+  }
+  __syncthreads();
   tc_after();
   const uint32_t tmem = bars->tmem;
-  const long long T = toff[n_items];
-  const long long t0 = T * blockIdx.x / gridDim.x, t1 = T * (blockIdx.x + 1) / gridDim.x;
+  const unsigned long long T = toff[n_items];
+  ItemRange rg;
+  rg.item = 0;
+  rg.t = (unsigned)(T * blockIdx.x / gridDim.x);
+  rg.t1 = (unsigned)(T * (blockIdx.x + 1) / gridDim.x);
+  RecPlan D;
 
   if (warp == 0) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
-      RecCursor c;
-      bool live = rec_start(c, toff, n_items, t0, t1, items, ptrs, ival);
-      long long tc = 0;
+      unsigned tc = 0;
       int st_i = 0;            // operand stage and its phase parity (advanced per chunk)
       uint32_t st_ph = 0;
       bool ok = true;
-      while (live && ok) {
-        const int b = (int)(tc & 1);
-        if (!mbar_wait(&bars->accempty[b], (uint32_t)(((tc >> 1) & 1) ^ 1), abort_flag, err, lim)) break;
-        tc_after();
-        const uint32_t d_tmem = tmem + (uint32_t)(b * 256);
-        const int NB = c.D.NB, K8 = c.D.K8;
+      while (ok && range_next(rg, toff, n_items)) {
+        rec_plan(items, rg.item, ptrs, ival, D);
+        const int NB = D.NB, K8 = D.K8, nkc = D.nkc;
         const uint32_t id_wide = idesc_tf32(kM, 2 * NB), id_half = idesc_tf32(kM, NB);
-        const int nkc = (K8 + kKC - 1) / kKC;
-        for (int kc = 0; kc < nkc; ++kc) {
-          const int s = st_i;
-          if (!mbar_wait(&bars->full[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
-          if (!mbar_wait(&bars->wfull[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
-          if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
+        for (unsigned tile = rg.lo; tile < rg.hi && ok; ++tile, ++tc) {
+          const int b = (int)(tc & 1);
+          if (!mbar_wait(&bars->accempty[b], ((tc >> 1) & 1u) ^ 1u, abort_flag, err, lim)) { ok = false; break; }
           tc_after();
-          const uint32_t a_hi = su32(smem + (size_t)s * P.stage_bytes);
-          const uint32_t a_lo = a_hi + (uint32_t)P.a_bytes;
-          const uint32_t bb = a_hi + (uint32_t)(2 * P.a_bytes);
-          const int ksteps = min(kKC, K8 - kc * kKC) / 8;
-          for (int st = 0; st < ksteps; ++st) {
-            const uint64_t dah = sdesc(a_hi + (uint32_t)st * 32u);
-            const uint64_t dal = sdesc(a_lo + (uint32_t)st * 32u);
-            const uint64_t db = sdesc(bb + (uint32_t)st * 32u);
-            mma_tf32(d_tmem, dah, db, id_wide, (kc > 0 || st > 0) ? 1u : 0u);
-            mma_tf32(d_tmem, dal, db, id_half, 1u);
+          const uint32_t d_tmem = tmem + (uint32_t)(b * 256);
+          for (int kc = 0; kc < nkc; ++kc) {
+            const int s = st_i;
+            if (!mbar_wait(&bars->full[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
+            if (!mbar_wait(&bars->wfull[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
+            if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
+            tc_after();
+            const uint32_t a_hi = su32(smem + (size_t)s * P.stage_bytes);
+            const uint32_t a_lo = a_hi + (uint32_t)P.a_bytes;
+            const uint32_t bb = a_hi + (uint32_t)(2 * P.a_bytes);
+            const int ksteps = min(kKC, K8 - kc * kKC) / 8;
+            for (int st = 0; st < ksteps; ++st) {
+              const uint64_t dah = sdesc(a_hi + (uint32_t)st * 32u);
+              const uint64_t dal = sdesc(a_lo + (uint32_t)st * 32u);
+              const uint64_t db = sdesc(bb + (uint32_t)st * 32u);
+              mma_tf32(d_tmem, dah, db, id_wide, (kc > 0 || st > 0) ? 1u : 0u);
+              mma_tf32(d_tmem, dal, db, id_half, 1u);
+            }
+            mma_commit(&bars->empty[s]);
           }
-          mma_commit(&bars->empty[s]);
+          if (ok) mma_commit(&bars->accfull[b]);
         }
-        if (!ok) break;
-        mma_commit(&bars->accfull[b]);
-        ++tc;
-        if (c.left == 1) break;
-        rec_next(c, toff, n_items, items, ptrs, ival);
       }
       mma_commit(&bars->drain);
       mbar_drain(&bars->drain, 0, err);
     }
     __syncwarp();
-  } else if (warp >= 4 && warp < 8) {
-    // -------------------------------------------------------------- epilogue
-    RecCursor c;
-    bool live = rec_start(c, toff, n_items, t0, t1, items, ptrs, ival);
-    const int row = 32 * (warp & 3) + lane;
-    const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
-    long long tc = 0;
-    while (live) {
-      const int b = (int)(tc & 1);
-      if (!warp_wait(&bars->accfull[b], (uint32_t)((tc >> 1) & 1), abort_flag, err, lim)) break;
-      tc_after();
-      const RecDims& D = c.D;
-      const long long rb = c.tile / D.nnb;
-      const int nb = (int)(c.tile - rb * D.nnb);
-      const long long rg = rb * kM + row;
-      const bool valid = rg < D.R;
-      long long base = 0;
-      long long ocut = 0;
-#pragma unroll
-      for (int i = 0; i < PEPO_MAXLEG; ++i) if (i == D.cut) ocut = D.ostride[i];
-      if (valid) {
-        long long rem = rg;
-#pragma unroll
-        for (int i = 0; i < PEPO_MAXLEG; ++i) {
-          if (i < D.cut) {
-            const long long idx = rem / D.rstride[i];
-            rem -= idx * D.rstride[i];
-            base += idx * D.ostride[i];
+  } else if (warp == 1) {
+    // ------------------------------------------------- W blocks, bulk copies
+    if (lane == 0) {
+      unsigned n = 0;          // copies issued
+      bool ok = true;
+      while (ok && range_next(rg, toff, n_items)) {
+        rec_plan(items, rg.item, ptrs, ival, D);
+        const uint32_t bytes = (uint32_t)(2 * D.NB) * 128u;
+        for (unsigned tile = rg.lo; tile < rg.hi && ok; ++tile) {
+          const float* blk = D.Wp + (size_t)(tile % (unsigned)D.nnb) * D.nkc * (size_t)(2 * D.NB) * 32;
+          for (int kc = 0; kc < D.nkc; ++kc) {
+            const unsigned s = n % (unsigned)NS;
+            if (!mbar_wait(&bars->empty[s], ((n / (unsigned)NS) & 1u) ^ 1u, abort_flag, err, lim)) { ok = false; break; }
+            if (D.Wp) {
+              mbar_arrive_tx(&bars->wfull[s], bytes);
+              bulk_g2s(smem + (size_t)s * P.stage_bytes + 2 * P.a_bytes, blk + (size_t)kc * (2 * D.NB) * 32, bytes,
+                       &bars->wfull[s]);
+            } else {   // no packed W workspace: flag it and keep the pipeline moving
+              atomicOr(err, 2);
+              mbar_arrive(&bars->wfull[s]);
+            }
+            ++n;
           }
         }
       }
-      const uint32_t tbase = tmem + lane_base + (uint32_t)(b * 256);
-      // 16-column blocks, loads of block i+1 in flight while block i is stored
-      uint32_t a1[16], a2[16], b1[16], b2[16];
-      auto store_blk = [&](const uint32_t* p1, const uint32_t* p2, int c0) {
-        if (!valid) return;
+      // no bulk copy may land after the kernel's shared memory is gone: the last
+      // copy of every stage (a stage is armed again only after the MMAs that
+      // consumed its previous copy)
+      for (unsigned k = n > (unsigned)NS ? n - NS : 0; k < n; ++k)
+        mbar_drain(&bars->wfull[k % (unsigned)NS], (k / (unsigned)NS) & 1u, err);
+    }
+    __syncwarp();
+  } else if (warp >= 4 && warp < 8) {
+    // -------------------------------------------------------------- epilogue
+    const int row = 32 * (warp & 3) + lane;
+    const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
+    unsigned tc = 0;
+    bool ok = true;
+    while (ok && range_next(rg, toff, n_items)) {
+      rec_plan(items, rg.item, ptrs, ival, D);
+      const int NB = D.NB;
+      const long long ocut = D.ocut;
+      for (unsigned tile = rg.lo; tile < rg.hi; ++tile, ++tc) {
+        const int b = (int)(tc & 1);
+        if (!warp_wait(&bars->accfull[b], (tc >> 1) & 1u, abort_flag, err, lim)) { ok = false; break; }
+        tc_after();
+        const unsigned rb = tile / (unsigned)D.nnb;
+        const int nb = (int)(tile - rb * D.nnb);
+        const unsigned r = rb * kM + row;
+        const bool valid = r < D.R;
+        const unsigned r1 = r / D.d2, i2 = r - r1 * D.d2, i0 = r1 / D.d1, i1 = r1 - i0 * D.d1;
+        // first column of the tile (a multiple of 8): its cut index and Paulis
+        float* dst = D.out + (i0 * D.os0 + i1 * D.os1 + i2 * D.os2) + (long long)(nb * NB / 4) * ocut;
+        const int cols = valid ? min(NB, D.np - nb * NB) : 0;
+        const uint32_t tbase = tmem + lane_base + (uint32_t)(b * 256);
+        // 16-column blocks, loads of block i+1 in flight while block i is stored;
+        // the four Paulis of a cut index are one 16-byte store
+        uint32_t a1[16], a2[16], b1[16], b2[16];
+        auto store_blk = [&](const uint32_t* p1, const uint32_t* p2, int c0) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int cg = nb * D.NB + c0 + i;
-          if (c0 + i < D.NB && cg < D.np)
-            D.out[base + (long long)(cg >> 2) * ocut + (cg & 3)] = __uint_as_float(p1[i]) + __uint_as_float(p2[i]);
-        }
-      };
-      tmem_ld16(tbase, a1);
-      tmem_ld16(tbase + (uint32_t)D.NB, a2);
-      tmem_wait32(a1, a2);
-      for (int c0 = 0; c0 < D.NB; c0 += 32) {
-        const bool m1 = c0 + 16 < D.NB;
-        if (m1) {
-          tmem_ld16(tbase + (uint32_t)(c0 + 16), b1);
-          tmem_ld16(tbase + (uint32_t)(D.NB + c0 + 16), b2);
-        }
-        store_blk(a1, a2, c0);
-        if (!m1) break;
-        tmem_wait32(b1, b2);
-        const bool m2 = c0 + 32 < D.NB;
-        if (m2) {
-          tmem_ld16(tbase + (uint32_t)(c0 + 32), a1);
-          tmem_ld16(tbase + (uint32_t)(D.NB + c0 + 32), a2);
-        }
-        store_blk(b1, b2, c0 + 16);
-        if (!m2) break;
+          for (int i = 0; i < 16; i += 4) {
+            if (c0 + i < cols)
+              *reinterpret_cast<float4*>(dst) = make_float4(__uint_as_float(p1[i]) + __uint_as_float(p2[i]),
+                                                            __uint_as_float(p1[i + 1]) + __uint_as_float(p2[i + 1]),
+                                                            __uint_as_float(p1[i + 2]) + __uint_as_float(p2[i + 2]),
+                                                            __uint_as_float(p1[i + 3]) + __uint_as_float(p2[i + 3]));
+            dst += ocut;
+          }
+        };
+        tmem_ld16(tbase, a1);
+        tmem_ld16(tbase + (uint32_t)NB, a2);
         tmem_wait32(a1, a2);
+        for (int c0 = 0; c0 < NB; c0 += 32) {
+          const bool m1 = c0 + 16 < NB;
+          if (m1) {
+            tmem_ld16(tbase + (uint32_t)(c0 + 16), b1);
+            tmem_ld16(tbase + (uint32_t)(NB + c0 + 16), b2);
+          }
+          store_blk(a1, a2, c0);
+          if (!m1) break;
+          tmem_wait32(b1, b2);
+          const bool m2 = c0 + 32 < NB;
+          if (m2) {
+            tmem_ld16(tbase + (uint32_t)(c0 + 32), a1);
+            tmem_ld16(tbase + (uint32_t)(NB + c0 + 32), a2);
+          }
+          store_blk(b1, b2, c0 + 16);
+          if (!m2) break;
+          tmem_wait32(a1, a2);
+        }
+        tc_before();
+        warp_arrive(&bars->accempty[b]);
       }
-      tc_before();
-      warp_arrive(&bars->accempty[b]);
-      ++tc;
-      if (c.left == 1) break;
-      rec_next(c, toff, n_items, items, ptrs, ival);
     }
   } else if (warp >= 8) {
     // ------------------------------------------------------------ converters
-    const int cw = (tid - 256) >> 5;
-    const int kq = 4 * (cw & 1) + (lane >> 3);     // 4-wide K group of A handled by this thread
-    const int i8_0 = cw >> 1;                      // A row groups i8_0 + 4 u
-    const int il = lane & 7;
-    const bool issuer = (tid == 256);               // issues the bulk copy of the B block
-    // stages whose wfull barrier the issuer has armed, and per stage the
-    // parity of its last arming (flipped at every arming): at most one copy
-    // per stage is in flight (a stage is re-armed only after the MMA that
-    // consumed its previous copy), so the last phase of each armed stage
-    // covers every copy this CTA issued
-    uint32_t warmed = 0, wpar = 0;
-    RecCursor c;
-    bool live = rec_start(c, toff, n_items, t0, t1, items, ptrs, ival);
-    int st_i = 0;              // operand stage and its phase parity
-    uint32_t st_ph = 0;
-    int kc = 0;
-    // row block rb and N block nb of the store cursor's tile, advanced per
-    // tile (tiles run nb fastest; an item change restarts at tile 0)
-    long long s_rb = 0;
-    int s_nb = 0;
-    if (live) { s_rb = c.tile / c.D.nnb; s_nb = (int)(c.tile - s_rb * c.D.nnb); }
-    auto advance = [&](RecCursor& cur, long long& rb, int& nb) {
-      const int it0 = cur.item;
-      rec_next(cur, toff, n_items, items, ptrs, ival);
-      if (cur.item != it0) { rb = 0; nb = 0; }
-      else if (++nb == cur.D.nnb) { nb = 0; ++rb; }
-    };
-    // loads of the next chunk run one chunk ahead (ring rotated by unrolling);
-    // the four source rows of this thread are set up once per tile
-    RecCursor lcur = c;
-    int lkc = 0;
-    bool l_live = live;
-    long long l_rb = s_rb;
-    int l_nb = s_nb;
-    const float* lrow[4];
-    bool lrv[4];
-    auto l_rows = [&]() {
-      const RecDims& D = lcur.D;
+    // This thread copies quad kq of the rows r0 + 16 u of every other chunk: the
+    // eight lanes of a row read its 128 bytes and store one swizzled row.
+    const int ct = tid - 256, grp = ct / kGroup, t = ct % kGroup;
+    const int kq = t & 7, r0 = t >> 3;
+    constexpr int MU = kM / (kGroup / 8);
+    unsigned n = 0;                                   // chunks of the CTA before this item
+    bool ok = true;
+    while (ok && range_next(rg, toff, n_items)) {
+      rec_plan(items, rg.item, ptrs, ival, D);
+      const int nkc = D.nkc, K = D.n;
+      const unsigned R = D.R;
+      const unsigned total = (rg.hi - rg.lo) * (unsigned)nkc;
+      unsigned j = (n ^ (unsigned)grp) & 1u;
+      unsigned nn = n + j;
+      n += total;
+      unsigned tile = rg.lo, lj = j;
+      int kc = (int)j;
+      unsigned row = 0;                                // first row of this thread in the load cursor's tile
+      const float* src = D.in;
+      auto enter = [&]() {
+        while (kc >= nkc) { kc -= nkc; ++tile; }
+        row = tile / (unsigned)D.nnb * kM + r0;
+        src = D.in + (long long)row * K + 4 * kq;
+      };
+      auto load = [&](float4 (&v)[MU]) {
+        const int k = kc * kKC;
+        const bool live = k + 4 * kq < K;
+        const float* p = src + k;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const long long r = l_rb * kM + 8 * (i8_0 + 4 * u) + il;
-        lrv[u] = r < D.R;
-        lrow[u] = D.in + (lrv[u] ? r * D.n : 0);
-      }
-    };
-    if (l_live) l_rows();
-    auto load_next = [&](float4 (&v)[4]) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (!l_live) return;
-      const RecDims& D = lcur.D;
-      const int k = lkc * kKC + 4 * kq;
-      if (k < D.n) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (lrv[u]) v[u] = __ldg(reinterpret_cast<const float4*>(lrow[u] + k));
-      }
-      if (++lkc < D.nkc) return;
-      lkc = 0;
-      if (lcur.left == 1) { l_live = false; return; }
-      const long long rb0 = l_rb;
-      const int item0 = lcur.item;
-      advance(lcur, l_rb, l_nb);
-      if (l_rb != rb0 || lcur.item != item0) l_rows();
-    };
-    auto step = [&](float4 (&vl)[4], float4 (&vs)[4]) -> bool {
-      load_next(vl);
-      const RecDims& D = c.D;
-      const int nb = s_nb;
-      const int s = st_i;
-      if (!warp_wait(&bars->empty[s], st_ph ^ 1u, abort_flag, err, lim)) return false;
-      if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
-      unsigned char* hi = smem + (size_t)s * P.stage_bytes;
-      unsigned char* lo = hi + P.a_bytes;
-      unsigned char* bs = hi + 2 * P.a_bytes;
-      if (issuer) {
-        if (D.Wp) {
-          const uint32_t bytes = (uint32_t)(2 * D.NB) * 128u;
-          mbar_arrive_tx(&bars->wfull[s], bytes);
-          bulk_g2s(bs, D.Wp + ((size_t)nb * D.nkc + kc) * (size_t)(2 * D.NB) * 32, bytes, &bars->wfull[s]);
-        } else {   // no packed W workspace: flag it and keep the pipeline moving
-          atomicOr(err, 2);
-          mbar_arrive(&bars->wfull[s]);
+        for (int i = 0; i < MU; ++i) {
+          v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (live && row + 16 * i < R) v[i] = __ldg(reinterpret_cast<const float4*>(p));
+          p += 16 * K;
         }
-        warmed |= 1u << s;
-        wpar ^= 1u << s;
-      }
+        lj += 2;
+        kc += 2;
+        if (lj < total) enter();
+      };
+      auto convert = [&](const float4 (&v)[MU]) -> bool {
+        const unsigned s = nn % (unsigned)NS;
+        if (!warp_wait(&bars->empty[s], ((nn / (unsigned)NS) & 1u) ^ 1u, abort_flag, err, lim)) return false;
+        unsigned char* hi = smem + (size_t)s * P.stage_bytes;
+        unsigned char* lo = hi + P.a_bytes;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int i = 8 * (i8_0 + 4 * u) + il;
-        const float4 x = vs[u];
-        const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
-        const float4 l = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
-        *reinterpret_cast<float4*>(hi + swz(i, kq)) = h;
-        *reinterpret_cast<float4*>(lo + swz(i, kq)) = l;
+        for (int i = 0; i < MU; ++i) {
+          const uint32_t off = swz(r0 + 16 * i, kq);
+          const float4 x = v[i];
+          const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
+          *reinterpret_cast<float4*>(hi + off) = h;
+          *reinterpret_cast<float4*>(lo + off) = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
+        }
+        fence_async_smem();
+        warp_arrive(&bars->full[s]);
+        nn += 2;
+        return true;
+      };
+      float4 v0[MU], v1[MU];
+      if (j < total) {
+        enter();
+        load(v0);
       }
-      fence_async_smem();
-      warp_arrive(&bars->full[s]);
-      if (++kc < D.nkc) return true;
-      kc = 0;
-      if (c.left == 1) return false;
-      advance(c, s_rb, s_nb);
-      return true;
-    };
-    float4 v0[4], v1[4];
-    load_next(v0);
-    while (live) {
-      if (!step(v1, v0)) break;
-      if (!step(v0, v1)) break;
+      for (; j < total; j += 4) {
+        if (j + 2 < total) load(v1);
+        if (!convert(v0)) { ok = false; break; }
+        if (j + 2 >= total) break;
+        if (j + 4 < total) load(v0);
+        if (!convert(v1)) { ok = false; break; }
+      }
     }
-    // no bulk copy may land after the kernel's shared memory is gone
-    if (issuer)
-      for (int q = 0; q < NS; ++q)
-        if (warmed & (1u << q)) mbar_drain(&bars->wfull[q], ((wpar >> q) & 1u) ^ 1u, err);
   }
   tc_before();
   __syncthreads();
@@ -1304,10 +1238,9 @@ int sm_count() {
 // N block nb and K chunk kc a (2 NB rows x 128 B) image with rows c < NB
 // = hi(W[k, nb NB + c]) and rows NB + c = the lo part, k in the chunk.
 __global__ void k_pack_w(const ReconItem* __restrict__ items, void* const* ptrs, const int* __restrict__ ival) {
-  const ReconItem it = items[blockIdx.y];
-  if (it.Wp == nullptr) return;
-  RecDims D;
-  rec_dims(it, ptrs, ival, D);
+  if (items[blockIdx.y].Wp == nullptr) return;
+  RecPlan D;
+  rec_plan(items, blockIdx.y, ptrs, ival, D);
   const long long per_blk = (long long)(2 * D.NB) * 32;
   const long long total = (long long)D.nnb * D.nkc * per_blk;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
