@@ -906,6 +906,61 @@ cudaError_t launch_factor(const SiteFacItem* items, int n_items, int rmax, int n
 // the ranks of any input form a permutation (every order[] slot written once).
 __device__ inline double rank_key(double x) { return x == x ? x : -1.0; }
 
+// Rotation of a Jacobi pair from its squared norms and product: h = tan(theta / 2) and
+// s = sin theta of the smaller angle that makes the columns orthogonal, and the new
+// squared norms.  False when the pair is orthogonal to tol (tol2 = tol^2),
+// numerically zero or coupled by less than cut.
+//
+// The rotation is applied as x -= s (y + h x), y += s (x - h y) (the old x): four
+// multiply-adds like the c, s form, but what rounding does to the columns' norms
+// and angles scales with s, so the thousands of small late rotations leave V
+// more orthogonal.  h may be off by 1e-7 of itself (the next sweep sees what that
+// leaves); s has to belong to h.
+__device__ __forceinline__ bool rot_params(float al, float be, float ga, float tol2, float negligible, float cut, float& h,
+                                           float& s, float& na, float& nb) {
+  if (!(ga != 0.f && al > negligible && be > negligible && fabsf(ga) > cut &&
+        fabsf(ga) * rsqrtf(al) * rsqrtf(be) * fabsf(ga) * rsqrtf(al) * rsqrtf(be) > tol2))
+    return false;
+  const float z = __fdividef(be - al, 2.f * ga), az = fabsf(z);
+  const float t = copysignf(az > 1e8f ? 0.5f / az : __fdividef(1.f, az + sqrtf(fmaf(z, z, 1.f))), z);
+  h = __fdividef(t, 1.f + sqrtf(fmaf(t, t, 1.f)));
+  s = 2.f * h / fmaf(h, h, 1.f);
+  na = al - t * ga;
+  nb = be + t * ga;
+  return true;
+}
+// FP64: h in FP32, s from it by a reciprocal with two Newton steps.  A division or
+// a root in FP64 is ~20 operations of 16 clocks a warp here, and the textbook
+// form has five.
+__device__ __forceinline__ bool rot_params(double al, double be, double ga, double tol2, double negligible, double cut,
+                                           double& h, double& s, double& na, double& nb) {
+  if (!(ga != 0.0 && al > negligible && be > negligible && fabs(ga) > cut && ga * ga > tol2 * (al * be))) return false;
+  const double d = be - al, g = 2.0 * ga;
+  const int e = max(__double2hiint(d) & 0x7ff00000, __double2hiint(g) & 0x7ff00000);
+  const double sc = __hiloint2double(max(0x7fe00000 - e, 0x00100000), 0);      // 2^-exponent
+  const float df = (float)(d * sc), gf = (float)(g * sc);
+  if (gf == 0.f) return false;                                                 // |zeta| > 1e38
+  const float z = df / gf, az = fabsf(z);
+  const float t = copysignf(az > 1e8f ? 0.5f / az : 1.f / (az + sqrtf(fmaf(z, z, 1.f))), z);
+  h = (double)(t / (1.f + sqrtf(fmaf(t, t, 1.f))));
+  const double x = fma(h, h, 1.0);
+  double y = (double)__frcp_rn((float)x);
+  y = fma(y, fma(-x, y, 1.0), y);
+  y = fma(y, fma(-x, y, 1.0), y);
+  s = 2.0 * h * y;
+  const double c = fma(-s, h, 1.0);
+  const double cs = 2.0 * c * s * ga, cc = c * c, ss = s * s;
+  na = fma(cc, al, fma(ss, be, -cs));
+  nb = fma(ss, al, fma(cc, be, cs));
+  return true;
+}
+template <typename R>
+__device__ __forceinline__ void rot_apply(R& x, R& y, R h, R s) {
+  const R u = fma(h, x, y), v = fma(-h, y, x);
+  x = fma(-s, u, x);
+  y = fma(s, v, y);
+}
+
 // One-sided Jacobi (Hestenes) on the columns of A (n x n, column-major),
 // accumulating V (n x n, column-major), by one block.  Returns the sweep count;
 // sets *capped when the sweep budget ran out.
@@ -946,7 +1001,8 @@ __device__ int jacobi_block_l(R* A, int n, R* V, R* nrm, int max_sweeps, int* ca
   // below 1e-30 (FP64) or 1e-13 (FP32) of the total squared norm are
   // numerically zero in that precision: rotating them only stirs rounding
   // noise and never converges
-  const R tol = (R)((sizeof(R) == 4 ? 3e-7 : 1e-15) * sqrt((double)n));
+  const double tol = (sizeof(R) == 4 ? 3e-7 : 1e-15) * sqrt((double)n);
+  const R tol2 = (R)(tol * tol);
   const R negligible = (R)(sizeof(R) == 4 ? 1e-13 : 1e-30) * fro;
   int sweep = 0;
   for (; sweep < max_sweeps; ++sweep) {
@@ -975,26 +1031,26 @@ __device__ int jacobi_block_l(R* A, int n, R* V, R* nrm, int max_sweeps, int* ca
         const R al = nrm[p], be = nrm[q];
 #pragma unroll
         for (int o = L / 2; o > 0; o >>= 1) ga += __shfl_xor_sync(mask, ga, o);
-        if (ga != R(0) && al > negligible && be > negligible && fabs(ga) > tol * sqrt(al * be)) {
+        R h, s, na, nb;
+        if (rot_params(al, be, ga, tol2, negligible, R(0), h, s, na, nb)) {
           rotated = 1;
-          const R zeta = (be - al) / (R(2) * ga);
-          const R t = (zeta >= R(0) ? R(1) : R(-1)) / (fabs(zeta) + sqrt(R(1) + zeta * zeta));
-          const R c = R(1) / sqrt(R(1) + t * t), s = c * t;
           R* Vp = V + p * n;
           R* Vq = V + q * n;
 #pragma unroll
           for (int u = 0; u < E; ++u) {
             const int i = l + L * u;
             if (i < n) {
-              Ap[i] = c * x[u] - s * y[u];
-              Aq[i] = s * x[u] + c * y[u];
-              const R vx = Vp[i], vy = Vq[i];
-              Vp[i] = c * vx - s * vy;
-              Vq[i] = s * vx + c * vy;
+              rot_apply(x[u], y[u], h, s);
+              Ap[i] = x[u];
+              Aq[i] = y[u];
+              R vx = Vp[i], vy = Vq[i];
+              rot_apply(vx, vy, h, s);
+              Vp[i] = vx;
+              Vq[i] = vy;
             }
           }
           __syncwarp(mask);
-          if (l == 0) { nrm[p] = al - t * ga; nrm[q] = be + t * ga; }
+          if (l == 0) { nrm[p] = na; nrm[q] = nb; }
         }
       }
       __syncthreads();
@@ -1031,60 +1087,102 @@ constexpr int kCoreThreads = 1024;
 constexpr size_t kCoreSmem = (size_t)192 * 1024;
 constexpr int kCoreMaxDim = 512;                   // columns and rows of a core: rg * chi <= 512
 
-// One warp's rotation of the columns x and y (length m, shared memory) of A and
-// vx, vy (length nv, may be null) of V; nx, ny are their squared norms, kept
-// up to date.  Returns whether it rotated.  FP32 columns are held in registers
-// between the dot product and the rotation (shared-memory bandwidth bounds that
-// pass; the FP64 one is bound by its pipe), so each is read and written once.
-template <typename R>
-__device__ bool jac_pair(R* x, R* y, int m, R* vx, R* vy, int nv, R* nx, R* ny, R tol, R negligible, R abs_cut) {
+// One warp's FP32 rotation of the columns x and y (length m, shared memory) of A
+// and vx, vy (length nv) of V; nx, ny are their squared norms, kept up to date.
+// Returns whether it rotated.  The columns are held in registers between the dot
+// product and the rotation (shared-memory bandwidth bounds the pass), so each
+// is read and written once.
+__device__ bool jac_pair(float* x, float* y, int m, float* vx, float* vy, int nv, float* nx, float* ny, float tol2,
+                         float negligible, float cut) {
   const int lane = threadIdx.x & 31;
-  constexpr int U = sizeof(R) == 4 ? kCoreMaxDim / 32 : 1;
-  R a[U], b[U];
-  R ga = 0;
-  if constexpr (U > 1) {
+  constexpr int U = kCoreMaxDim / 32;
+  float a[U], b[U];
+  float ga = 0;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int i = lane + 32 * u;
-      a[u] = b[u] = R(0);
-      if (32 * u < m) {
-        if (i < m) { a[u] = x[i]; b[u] = y[i]; }
-        ga = fma(a[u], b[u], ga);
-      }
+  for (int u = 0; u < U; ++u) {
+    const int i = lane + 32 * u;
+    a[u] = b[u] = 0.f;
+    if (32 * u < m) {
+      if (i < m) { a[u] = x[i]; b[u] = y[i]; }
+      ga = fmaf(a[u], b[u], ga);
     }
-  } else {
-    for (int i = lane; i < m; i += 32) ga = fma(x[i], y[i], ga);
   }
-  const R al = *nx, be = *ny;
+  const float al = *nx, be = *ny;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
-  if (!(ga != R(0) && al > negligible && be > negligible && fabs(ga) > tol * sqrt(al * be) && fabs(ga) > abs_cut))
-    return false;
-  const R zeta = (be - al) / (R(2) * ga);
-  const R t = (zeta >= R(0) ? R(1) : R(-1)) / (fabs(zeta) + sqrt(R(1) + zeta * zeta));
-  const R c = R(1) / sqrt(R(1) + t * t), s = c * t;
-  if constexpr (U > 1) {
+  float h, s, na, nb;
+  if (!rot_params(al, be, ga, tol2, negligible, cut, h, s, na, nb)) return false;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int i = lane + 32 * u;
-      if (i < m) { x[i] = c * a[u] - s * b[u]; y[i] = s * a[u] + c * b[u]; }
-    }
-  } else {
-    for (int i = lane; i < m; i += 32) {
-      const R p = x[i], q = y[i];
-      x[i] = c * p - s * q;
-      y[i] = s * p + c * q;
+  for (int u = 0; u < U; ++u) {
+    const int i = lane + 32 * u;
+    if (i < m) {
+      rot_apply(a[u], b[u], h, s);
+      x[i] = a[u];
+      y[i] = b[u];
     }
   }
-  if (vx)
-    for (int i = lane; i < nv; i += 32) {
-      const R p = vx[i], q = vy[i];
-      vx[i] = c * p - s * q;
-      vy[i] = s * p + c * q;
-    }
+  for (int i = lane; i < nv; i += 32) {
+    float p = vx[i], q = vy[i];
+    rot_apply(p, q, h, s);
+    vx[i] = p;
+    vy[i] = q;
+  }
   __syncwarp();
-  if (lane == 0) { *nx = al - t * ga; *ny = be + t * ga; }
+  if (lane == 0) { *nx = na; *ny = nb; }
   return true;
+}
+
+// The pairs of one inner round in FP64 (pair k: the columns pq[k].x, pq[k].y of buf,
+// per values each, m of A then nv of V), by the whole block: half a warp per dot
+// product, one lane per pair for the rotation, half a warp per rotated pair.  The
+// FP64 pipe bounds it: an operation that all lanes repeat costs as much as 32
+// useful ones, so the scalars of all pairs share a warp.
+struct JacRound {
+  int2 pq[64];
+  double ga[64], h[64], s[64];                             // s > 1.5: no rotation
+};
+__device__ int jac_round64(JacRound& R, int pairs, double* buf, int per, int m, int nv, double* nrm, double tol2,
+                           double negligible, double cut) {
+  const int l = threadIdx.x & 15, h = threadIdx.x >> 4, nh = blockDim.x >> 4;
+  const unsigned mask = 0xffffu << (threadIdx.x & 16);
+  int rot = 0;
+  for (int k = h; k < pairs; k += nh) {
+    const double* x = buf + R.pq[k].x * per;
+    const double* y = buf + R.pq[k].y * per;
+    double ga = 0.0;
+    for (int i = l; i < m; i += 16) ga = fma(x[i], y[i], ga);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) ga += __shfl_xor_sync(mask, ga, o);
+    if (l == 0) R.ga[k] = ga;
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < pairs; k += blockDim.x) {
+    double* nx = nrm + R.pq[k].x;
+    double* ny = nrm + R.pq[k].y;
+    double h = 0.0, s = 2.0, na, nb;
+    if (rot_params(*nx, *ny, R.ga[k], tol2, negligible, cut, h, s, na, nb)) {
+      *nx = na;
+      *ny = nb;
+      rot = 1;
+    }
+    R.h[k] = h;
+    R.s[k] = s;
+  }
+  __syncthreads();
+  for (int k = h; k < pairs; k += nh) {
+    const double h = R.h[k], s = R.s[k];
+    if (s > 1.5) continue;
+    double* x = buf + R.pq[k].x * per;
+    double* y = buf + R.pq[k].y * per;
+    for (int i = l; i < m + nv; i += 16) {
+      double p = x[i], q = y[i];
+      rot_apply(p, q, h, s);
+      x[i] = p;
+      y[i] = q;
+    }
+  }
+  __syncthreads();
+  return rot;
 }
 
 // One-sided Jacobi of A (m x n, column-major, leading dimension m, global
@@ -1126,7 +1224,10 @@ __device__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* cap
   double fro = 0.0;
   for (int j = threadIdx.x; j < n; j += blockDim.x) fro += cnorm[j];
   fro = block_sum(fro, fr);
-  const R tol = (R)((sizeof(R) == 4 ? 3e-7 : 1e-15) * sqrt((double)m));
+  const double tol = (sizeof(R) == 4 ? 3e-7 : 1e-15) * sqrt((double)m);
+  const R tol2 = (R)(tol * tol);
+  __shared__ JacRound jr;
+  __shared__ int jr_count;
   // columns below 1e-30 (FP64) or 1e-13 (FP32) of the total squared norm are
   // numerically zero in that precision
   const R negligible = (R)((sizeof(R) == 4 ? 1e-13 : 1e-30) * fro);
@@ -1177,14 +1278,29 @@ __device__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* cap
   // the pairs f(0) .. f(cnt - 1) (slots of disjoint columns; x < 0: none), then a block barrier
   auto round_of = [&](int cnt, auto f) -> int {
     int rot = 0;
-    for (int k = wid; k < cnt; k += nw) {
-      const int2 v = f(k);
-      if (v.x < 0) continue;
-      R* x = buf + v.x * per;
-      R* y = buf + v.y * per;
-      rot |= jac_pair<R>(x, y, m, x + m, y + m, n, nrm + v.x, nrm + v.y, tol, negligible, abs_cut) ? 1 : 0;
+    if constexpr (sizeof(R) == 4) {
+      for (int k = wid; k < cnt; k += nw) {
+        const int2 v = f(k);
+        if (v.x < 0) continue;
+        R* x = buf + v.x * per;
+        R* y = buf + v.y * per;
+        rot |= jac_pair(x, y, m, x + m, y + m, n, nrm + v.x, nrm + v.y, tol2, negligible, abs_cut) ? 1 : 0;
+      }
+      __syncthreads();
+    } else {
+      if (wid == 0) {                                      // list the round's pairs (at most 64 = n / 2)
+        int at = 0;
+        for (int k0 = 0; k0 < cnt; k0 += 32) {
+          const int2 v = k0 + lane < cnt ? f(k0 + lane) : make_int2(-1, -1);
+          const unsigned live = __ballot_sync(0xffffffffu, v.x >= 0);
+          if (v.x >= 0) jr.pq[at + __popc(live & ((1u << lane) - 1u))] = v;
+          at += __popc(live);
+        }
+        if (lane == 0) jr_count = at;
+      }
+      __syncthreads();
+      rot = jac_round64(jr, jr_count, buf, per, m, n, nrm, tol2, negligible, abs_cut);
     }
-    __syncthreads();
     return rot;
   };
   // inner round `k` of block pair (P, Q) at slots p0, q0: pair i of it
