@@ -17,6 +17,8 @@
 //                  (Eq. 11), lambda (Eq. 12), reconstruct matrices W1, W2
 //                  (Sec. 2.5 steps 5-8 in Q-less form), messages diag(lambda).
 #include <algorithm>
+#include <cstddef>
+#include <type_traits>
 
 #include "kernels.h"
 #include "linalg.h"
@@ -574,123 +576,183 @@ cudaError_t launch_form(const SiteFacItem* items, int n_items, int grid_x, const
   return cudaGetLastError();
 }
 
-// =================================================================== factor
-constexpr int kFacThreads = 512;     // one thread per column: n, r <= 512
-
-// Shared-memory plan of k_factor: the vectors first, then whatever is left
-// for the factor itself (U of the Cholesky branch, the matrix of the
-// Householder branch) when it fits.
-struct FacSmem {
-  size_t dg, od, uc, perm, v, mat, total;
+// ------------------------------------------------------------ clusters
+// The CTAs that share a site's factor or a bond core meet at the hardware cluster barrier (its
+// arrive / wait pair orders their global-memory accesses); a cluster of one
+// meets at the block barrier.
+struct Cta {
+  int rank, size;        // this CTA in its cluster, CTAs in it
+  long long tid, nthr;   // this thread among the cluster's threads
 };
-__host__ __device__ inline FacSmem fac_smem(int rmax, int nmax, int householder) {
+__device__ __forceinline__ void cta_sync(const Cta& c) {
+  if (c.size > 1) {
+    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+  } else {
+    __syncthreads();
+  }
+}
+
+// =================================================================== factor
+constexpr int kFacThreads = 512;
+constexpr int kFacSlices = 4;
+
+// Shared memory of k_factor: the vectors of the cluster Cholesky (or of the
+// Householder QR, FP64 storage), then what is left for the factor itself (a
+// CTA's columns of U, or the Householder branch's matrix) when it fits.
+struct FacSmem {
+  size_t cand, uc, part, dq, oq, pos, perm, v, mat, total;
+};
+__host__ __device__ inline FacSmem fac_smem(int rmax, int nmax, int householder, int csize) {
   FacSmem m;
   const int w = rmax > nmax ? rmax : nmax;
   size_t o = 0;
-  m.dg = o;   o += sizeof(double) * w;
-  m.od = o;   o += sizeof(double) * w;
+  m.cand = o; o += 2 * sizeof(double) * w;
   m.uc = o;   o += sizeof(double) * w;
-  m.perm = o; o += sizeof(int) * (size_t)(w + (w & 1));
+  m.part = o; o += sizeof(double) * kFacSlices * (size_t)((w + csize - 1) / csize);
+  m.dq = o;   o += sizeof(double) * w;
+  m.oq = o;   o += sizeof(double) * w;
+  m.pos = o;  o += sizeof(int) * (size_t)w;
+  m.perm = o; o += sizeof(int) * (size_t)w;
   m.v = o;
   if (householder) o += sizeof(double) * ((size_t)4 * nmax + (size_t)(kFacThreads / 32) * rmax);
+  o = (o + 15) & ~(size_t)15;
   m.mat = o;
-  const size_t cap = (size_t)200 * 1024;
-  const size_t want = householder ? sizeof(double) * (size_t)4 * nmax * rmax : sizeof(double) * (size_t)rmax * rmax;
+  const size_t cap = (size_t)216 * 1024;
+  const size_t want = householder ? sizeof(double) * (size_t)4 * nmax * rmax
+                                  : sizeof(double) * (size_t)w * ((w + csize - 1) / csize);
   o += want < cap - o ? want : cap - o;
   m.total = o;
   return m;
 }
 
+// a CTA's candidate for the next pivot
+struct Pivot {
+  double value, own;     // remaining and original diagonal
+  int col;
+};
+
+__device__ __forceinline__ unsigned cluster_addr(const void* p, int rank) {   // p's address in CTA `rank`
+  unsigned a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+template <typename R> __device__ __forceinline__ R cluster_ld(unsigned a);
+template <> __device__ __forceinline__ double cluster_ld<double>(unsigned a) {
+  double x;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(x) : "r"(a) : "memory");
+  return x;
+}
+template <> __device__ __forceinline__ float cluster_ld<float>(unsigned a) {
+  float x;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(a) : "memory");
+  return x;
+}
+template <> __device__ __forceinline__ int cluster_ld<int>(unsigned a) {
+  int x;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(x) : "r"(a) : "memory");
+  return x;
+}
+
 // Pivoted Cholesky of a symmetric n x n matrix A (leading dimension lda, read
-// only) in precision R: U (leading dimension ldu) receives the upper factor in
-// pivoted column order, perm the original column at each position; returns the
-// rank (pivots <= rel times the first end it), or -1 when an accepted pivot
-// keeps less than `safe` of its own column's diagonal (safe < 0: not tested).
+// only) in precision R by the CTAs of a cluster; returns the rank (pivots <= rel
+// times the first end it), or -1 when an accepted pivot keeps less than `safe`
+// of its own column's diagonal (safe < 0: not tested).  CTA k owns the w columns
+// from k w on: U[j][c] (j steps, c its column, in shared memory where w n values
+// fit) is its part of the upper factor, pos[c] the step at which the column
+// became a pivot (-1: never), perm[j] the pivot column of step j.
 //
-// Left-looking: step j forms only row j, U[j, q] = (A[p_j, p_q] - sum_l<j
-// U[l, j] U[l, q]) / U[j, j], one thread per column q.  The right-looking form
-// rewrites the whole trailing square at every step (r^3 / 3 multiply-adds and
-// as many read-modify-writes through L2 with an index division each); this one
-// does r^3 / 6 multiply-adds and only reads U, which stays in shared memory up
-// to r = 150 or so.  The terms of an entry are subtracted in the same order.
-// Bound: the FP64 pipe of one SM (2 multiply-adds per clock: 2.6 ms at
-// r = 400), two barriers per step below that.
+// Left-looking: step j forms only row j, U[j, q] = (A[p_j, q] - sum_l<j U[l, p_j]
+// U[l, q]) / U[j, p_j], the sum in four interleaved parts (the same bits for every
+// cluster size), and nothing is rewritten (the right-looking form updates the trailing square through L2
+// at every step).  Columns stay where they are, so a step moves only the
+// candidates: every CTA offers its largest remaining diagonal with that column
+// of U, the cluster meets once, and all read the winner's column from its
+// shared memory (offers alternate between two buffers, so one meeting per
+// step is enough).  Bound: the FP64 pipe, r^3 / 6 multiply-adds at 2 per clock
+// and SM, plus ~2 us of meeting and latency per step.
 template <typename R>
-__device__ int chol_pivoted(const double* __restrict__ A, int lda, int n, R* U, int ldu, R* dg, R* od, R* uc, int* perm,
-                            double rel, double safe) {
-  __shared__ double rv[kFacThreads / 32];
-  __shared__ int ri[kFacThreads / 32];
-  const int q = threadIdx.x, lane = q & 31, wid = q >> 5;
-  const int nw = (n + 31) >> 5;
-  int pq = q;                                   // original column at this thread's position
-  R dq = R(0), oq = R(0);
-  if (q < n) {
-    dq = oq = (R)A[(long long)q * lda + q];
-    dg[q] = dq;
-    od[q] = oq;
-    perm[q] = q;
+__device__ int chol_cluster(const double* __restrict__ A, int lda, int n, int w, R* U, const Cta& ct, Pivot* offer,
+                            R* offer_u, int ldo, R* uc, R* part, R* dq, R* oq, int* pos, int* perm, double rel,
+                            double safe) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int c0 = ct.rank * w;
+  const int nl = min(w, n - c0) > 0 ? min(w, n - c0) : 0;
+  __shared__ int sh_best;
+  for (int i = tid; i < nl; i += kFacThreads) {
+    dq[i] = oq[i] = (R)A[(long long)(c0 + i) * lda + c0 + i];
+    pos[i] = -1;
   }
+  __syncthreads();
   double d0 = 0.0;
   for (int j = 0; j < n; ++j) {
-    // pivot: the largest remaining diagonal, smallest position among ties;
-    // position j when every candidate is NaN (the test below then stops)
-    double best = -1.0;
-    int bi = n;
-    if (q >= j && q < n && (double)dq > best) { best = (double)dq; bi = q; }
+    Pivot* of = offer + (j & 1);
+    R* ofu = offer_u + (j & 1) * ldo;
+    if (tid < 32) {
+      // this CTA's largest remaining diagonal (smallest column among ties; none
+      // when every candidate is NaN)
+      double best = -1.0;
+      int bi = n;
+      for (int i = lane; i < nl; i += 32)
+        if (pos[i] < 0 && (double)dq[i] > best) { best = (double)dq[i]; bi = i; }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-    }
-    if (lane == 0 && wid < nw) { rv[wid] = best; ri[wid] = bi; }
-    __syncthreads();
-    double b = -1.0;
-    int p = n;
-    for (int i = j >> 5; i < nw; ++i)
-      if (rv[i] > b || (rv[i] == b && ri[i] < p)) { b = rv[i]; p = ri[i]; }
-    if (p >= n) p = j;
-    const R dp = dg[p];
-    if (j == 0) d0 = (double)dp;
-    if (!((double)dp > rel * d0) || !((double)dp > 0.0)) return j;
-    if (safe >= 0.0 && !((double)dp >= safe * (double)od[p])) return -1;
-    const int pp = perm[p], pj = perm[j];
-    const R dj = dg[j], oj = od[j], op = od[p];
-    // column p of the finished rows, staged for the broadcast reads below, and
-    // the swap of the positions j and p in those rows
-    for (int l = q; l < j; l += kFacThreads) {
-      const R x = U[(long long)l * ldu + p];
-      uc[l] = x;
-      if (p != j) {
-        U[(long long)l * ldu + p] = U[(long long)l * ldu + j];
-        U[(long long)l * ldu + j] = x;
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+      }
+      if (lane == 0) {
+        of->value = best;
+        of->own = bi < n ? (double)oq[bi] : 0.0;
+        of->col = bi < n ? c0 + bi : n;
+        sh_best = bi;
       }
     }
-    if (p != j) {
-      if (q == p) { pq = pj; dq = dj; oq = oj; }
-      if (q == j) { pq = pp; dq = dp; oq = op; }
+    __syncthreads();
+    if (sh_best < n)
+      for (int l = tid; l < j; l += kFacThreads) ofu[l] = U[l * w + sh_best];
+    cta_sync(ct);
+    // the winner of the cluster
+    double dp = -1.0, op = 0.0;
+    int p = n, from = 0;
+    for (int k = 0; k < ct.size; ++k) {
+      const unsigned a = cluster_addr(of, k);
+      const double v = cluster_ld<double>(a);
+      const int q = cluster_ld<int>(a + (unsigned)offsetof(Pivot, col));
+      if (v > dp || (v == dp && q < p)) { dp = v; p = q; from = k; op = cluster_ld<double>(a + (unsigned)offsetof(Pivot, own)); }
+    }
+    if (j == 0) d0 = dp;
+    if (p >= n || !(dp > rel * d0) || !(dp > 0.0)) return j;
+    if (safe >= 0.0 && !(dp >= safe * op)) return -1;
+    R a_pc = R(0);
+    if (tid < nl) a_pc = (R)A[(long long)p * lda + c0 + tid];
+    {
+      const unsigned a = cluster_addr(ofu, from);
+      for (int l = tid; l < j; l += kFacThreads) uc[l] = cluster_ld<R>(a + (unsigned)(l * sizeof(R)));
+    }
+    if (tid == 0) perm[j] = p;
+    __syncthreads();
+    for (int e = tid; e < kFacSlices * nl; e += kFacThreads) {
+      const int sl = e / nl, c = e - sl * nl;
+      R acc = R(0);
+#pragma unroll 8
+      for (int l = sl; l < j; l += kFacSlices) acc = fma(uc[l], U[l * w + c], acc);
+      part[e] = acc;
     }
     __syncthreads();
-    const R rjj = sqrt(dp);
-    if (q == j) U[(long long)j * ldu + j] = rjj;
-    if (q > j && q < n) {
-      R acc = (R)A[(long long)pp * lda + pq];
-      const R* uq = U + q;
-      int l = 0;
-      for (; l + 16 <= j; l += 16) {            // 16 loads in flight before their uses
-        R x[16];
+    if (tid < nl) {
+      if (c0 + tid == p) {
+        U[j * w + tid] = sqrt(dq[tid]);
+        pos[tid] = j;
+      } else if (pos[tid] < 0) {
+        R acc = a_pc;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = uq[(long long)(l + i) * ldu];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) acc = fma(-uc[l + i], x[i], acc);
+        for (int k = 0; k < kFacSlices; ++k) acc -= part[k * nl + tid];
+        acc /= sqrt((R)dp);
+        U[j * w + tid] = acc;
+        dq[tid] = fma(-acc, acc, dq[tid]);
       }
-      for (; l < j; ++l) acc = fma(-uc[l], uq[(long long)l * ldu], acc);
-      acc /= rjj;
-      U[(long long)j * ldu + q] = acc;
-      dq = fma(-acc, acc, dq);
     }
-    if (p != j && (q == p || q == j)) { perm[q] = pq; od[q] = oq; }
-    if (q < n) dg[q] = dq;
+    __syncthreads();
   }
   return n;
 }
@@ -815,11 +877,16 @@ __device__ int qrcp(double* B, int ld, int M, int r, double* dg, double* w, doub
 // Householder branch).
 __global__ void __launch_bounds__(kFacThreads)
 k_factor(const SiteFacItem* __restrict__ items, int* ival, int only, unsigned long long* qcount, int rmax, int nmax,
-         int householder) {
-  const SiteFacItem it = items[blockIdx.x];
+         int householder, int csize) {
+  const SiteFacItem it = items[blockIdx.x / csize];
   const int branch = ival[it.branch_idx];
   if (only >= 0 && branch != only) return;
-  if (qcount && threadIdx.x == 0 && branch == 0) atomicAdd(&qcount[0], 1ull);
+  Cta ct;
+  ct.rank = blockIdx.x % csize;
+  ct.size = csize;
+  ct.tid = (long long)ct.rank * blockDim.x + threadIdx.x;
+  ct.nthr = (long long)csize * blockDim.x;
+  if (qcount && ct.tid == 0 && branch == 0) atomicAdd(&qcount[0], 1ull);
   long long m;
   int n;
   cv_shape(it.cv, ival, m, n);
@@ -829,64 +896,88 @@ k_factor(const SiteFacItem* __restrict__ items, int* ival, int only, unsigned lo
   double* T = it.T;
   const int ld = it.ldt;
   extern __shared__ __align__(16) unsigned char fsh[];
-  const FacSmem S = fac_smem(rmax, nmax, householder);
-  double* dg = reinterpret_cast<double*>(fsh + S.dg);
-  double* od = reinterpret_cast<double*>(fsh + S.od);
-  double* uc = reinterpret_cast<double*>(fsh + S.uc);
-  int* perm = reinterpret_cast<int*>(fsh + S.perm);
+  __shared__ Pivot offer[2];
+  const FacSmem S = fac_smem(rmax, nmax, householder, csize);
+  const int ldo = rmax > nmax ? rmax : nmax;
   double* mat = reinterpret_cast<double*>(fsh + S.mat);
+  int* pos = reinterpret_cast<int*>(fsh + S.pos);
+  int* perm = reinterpret_cast<int*>(fsh + S.perm);
   const size_t room = S.total - S.mat;
-  int rank = 0;
+  auto chol = [&](auto* zero, const double* A, int lda, int k, auto* scratch, double safe, auto*& U) -> int {
+    using R = std::remove_reference_t<decltype(*zero)>;
+    const int w = (k + csize - 1) / csize;
+    U = sizeof(R) * (size_t)k * w <= room ? reinterpret_cast<R*>(mat) : scratch + (long long)ct.rank * w * k;
+    return chol_cluster<R>(A, lda, k, w, U, ct, offer, reinterpret_cast<R*>(fsh + S.cand), ldo,
+                           reinterpret_cast<R*>(fsh + S.uc), reinterpret_cast<R*>(fsh + S.part),
+                           reinterpret_cast<R*>(fsh + S.dq), reinterpret_cast<R*>(fsh + S.oq), pos, perm, it.rel, safe);
+  };
+  double* scratch = T + (long long)2 * ld * ld;      // behind T and G: 2 ld^2 doubles
   if (branch == 1) {
-    double* scratch = T + (long long)2 * ld * ld;    // behind T and G: 2 ld^2 doubles
     int ok;
     if (it.rel_safe >= 1e-6) {
-      const bool in = sizeof(float) * (size_t)n * n <= room;
-      ok = chol_pivoted<float>(it.C, it.ldc, n, in ? reinterpret_cast<float*>(mat) : reinterpret_cast<float*>(scratch), n,
-                               reinterpret_cast<float*>(dg), reinterpret_cast<float*>(od), reinterpret_cast<float*>(uc),
-                               perm, it.rel, it.rel_safe);
+      float* U;
+      ok = chol((float*)nullptr, it.C, it.ldc, n, reinterpret_cast<float*>(scratch), it.rel_safe, U);
     } else {
-      const bool in = sizeof(double) * (size_t)n * n <= room;
-      ok = chol_pivoted<double>(it.C, it.ldc, n, in ? mat : scratch, n, dg, od, uc, perm, it.rel, it.rel_safe);
+      double* U;
+      ok = chol((double*)nullptr, it.C, it.ldc, n, scratch, it.rel_safe, U);
     }
-    if (threadIdx.x == 0 && qcount) atomicAdd(&qcount[ok >= 0 ? 1 : 2], 1ull);
+    if (ct.tid == 0 && qcount) atomicAdd(&qcount[ok >= 0 ? 1 : 2], 1ull);
+    cta_sync(ct);                                    // the last offers are read, every CTA has its branch
     if (ok < 0) {
-      if (threadIdx.x == 0) ival[it.branch_idx] = 2;
+      if (ct.tid == 0) ival[it.branch_idx] = 2;
       return;
     }
-    __syncthreads();
   }
   if (branch == 1 || !householder) {
-    const bool in = sizeof(double) * (size_t)r * r <= room;
-    double* U = in ? mat : T;
-    const int ldu = in ? r : ld;
-    rank = chol_pivoted<double>(T + (long long)ld * ld, ld, r, U, ldu, dg, od, uc, perm, it.rel, -1.0);
+    double* U;
+    const int rank = chol((double*)nullptr, T + (long long)ld * ld, ld, r, scratch, -1.0, U);
+    // columns that never became a pivot follow in their own order
+    const int w = (r + csize - 1) / csize, c0 = ct.rank * w;
+    const int nl = min(w, r - c0);
+    int* taken = reinterpret_cast<int*>(fsh + S.uc);
     __syncthreads();
-    if (in)
-      for (long long e = threadIdx.x; e < (long long)rank * r; e += blockDim.x) {
-        const int a = (int)(e / r), q = (int)(e - (long long)a * r);
-        if (q >= a) T[(long long)a * ld + q] = mat[e];
+    for (int i = threadIdx.x; i < r; i += blockDim.x) taken[i] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < rank; i += blockDim.x) taken[perm[i]] = 1;
+    __syncthreads();
+    for (int c = threadIdx.x; c < nl; c += blockDim.x) {
+      int q = pos[c];
+      if (q < 0) {
+        q = rank;
+        for (int i = 0; i < c0 + c; ++i) q += 1 - taken[i];
+        pos[c] = q;
       }
-  } else {
-    const int M = 4 * ival[it.kfac_idx];
-    double* v = reinterpret_cast<double*>(fsh + S.v);
-    double* part = v + (size_t)4 * nmax;
-    const bool in = sizeof(double) * (size_t)M * r <= room;
-    if (in) {
-      for (long long e = threadIdx.x; e < (long long)M * r; e += blockDim.x) {
-        const int a = (int)(e / r), q = (int)(e - (long long)a * r);
-        mat[e] = T[(long long)a * ld + q];
-      }
-      __syncthreads();
+      it.perm[q] = c0 + c;
     }
-    rank = qrcp(in ? mat : T, in ? r : ld, M, r, dg, od, v, part, perm, it.rel);
     __syncthreads();
-    if (in)
-      for (long long e = threadIdx.x; e < (long long)rank * r; e += blockDim.x) {
-        const int a = (int)(e / r), q = (int)(e - (long long)a * r);
-        T[(long long)a * ld + q] = mat[e];
-      }
+    for (int e = threadIdx.x; e < rank * nl; e += blockDim.x) {
+      const int a = e / nl, c = e - a * nl, q = pos[c];
+      if (a <= q) T[(long long)a * ld + q] = U[a * w + c];
+    }
+    if (ct.tid == 0) ival[it.rank_idx] = rank;
+    cta_sync(ct);                                    // no CTA leaves while its offers may be read
+    return;
   }
+  const int M = 4 * ival[it.kfac_idx];
+  double* v = reinterpret_cast<double*>(fsh + S.v);
+  double* part = v + (size_t)4 * nmax;
+  double* dg = reinterpret_cast<double*>(fsh + S.dq);
+  double* od = reinterpret_cast<double*>(fsh + S.oq);
+  const bool in = sizeof(double) * (size_t)M * r <= room;
+  if (in) {
+    for (long long e = threadIdx.x; e < (long long)M * r; e += blockDim.x) {
+      const int a = (int)(e / r), q = (int)(e - (long long)a * r);
+      mat[e] = T[(long long)a * ld + q];
+    }
+    __syncthreads();
+  }
+  const int rank = qrcp(in ? mat : T, in ? r : ld, M, r, dg, od, v, part, perm, it.rel);
+  __syncthreads();
+  if (in)
+    for (long long e = threadIdx.x; e < (long long)rank * r; e += blockDim.x) {
+      const int a = (int)(e / r), q = (int)(e - (long long)a * r);
+      T[(long long)a * ld + q] = mat[e];
+    }
   for (int i = threadIdx.x; i < r; i += blockDim.x) it.perm[i] = perm[i];
   if (threadIdx.x == 0) ival[it.rank_idx] = rank;
 }
@@ -894,11 +985,29 @@ k_factor(const SiteFacItem* __restrict__ items, int* ival, int only, unsigned lo
 cudaError_t launch_factor(const SiteFacItem* items, int n_items, int rmax, int nmax, int* ival,
                           cudaStream_t s, int only, int householder, unsigned long long* qcount) {
   if (n_items == 0) return cudaSuccess;
-  const FacSmem S = fac_smem(rmax, nmax, householder);
+  // FP32 storage: up to eight CTAs a site while they all find an SM (a factor of
+  // r = 4 chi columns below 128 is latency-bound on one); the Householder QR of
+  // FP64 storage is one block's
+  int csize = 1;
+  if (!householder && rmax > 128)
+    for (csize = 8; csize > 1 && n_items * csize > 2 * 152; csize /= 2) {}
+  const FacSmem S = fac_smem(rmax, nmax, householder, csize);
   cudaError_t e = cudaFuncSetAttribute(k_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.total);
   if (e != cudaSuccess) return e;
-  k_factor<<<n_items, kFacThreads, S.total, s>>>(items, ival, only, qcount, rmax, nmax, householder);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_items * csize);
+  cfg.blockDim = dim3(kFacThreads);
+  cfg.dynamicSmemBytes = S.total;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = csize;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, k_factor, items, ival, only, qcount, rmax, nmax, householder, csize);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // ===================================================================== core
@@ -1065,22 +1174,6 @@ template <typename R>
 __device__ int jacobi_block(R* A, int n, R* V, R* nrm, int max_sweeps, int* capped) {
   return n <= 64 ? jacobi_block_l<R, 32>(A, n, V, nrm, max_sweeps, capped)
                  : jacobi_block_l<R, 16>(A, n, V, nrm, max_sweeps, capped);
-}
-
-// ---- the same on the CTAs of one cluster --------------------------------
-// The CTAs that share a bond core meet at the hardware cluster barrier (its
-// arrive / wait pair orders their global-memory accesses); a cluster of one
-// meets at the block barrier.
-struct Cta {
-  int rank, size;        // this CTA in its cluster, CTAs in it
-  long long tid, nthr;   // this thread among the cluster's threads
-};
-__device__ __forceinline__ void cta_sync(const Cta& c) {
-  if (c.size > 1) {
-    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
-  } else {
-    __syncthreads();
-  }
 }
 
 constexpr int kCoreThreads = 1024;
