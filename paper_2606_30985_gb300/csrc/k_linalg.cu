@@ -32,44 +32,66 @@ __device__ inline double warp_sum(double v) {
   return v;
 }
 
-// Block-wide sum; `red` must hold blockDim.x / 32 doubles.  All threads return it.
+// FP64 here issues one warp instruction per 16 clocks and SM, whatever the number
+// of useful lanes: scalars that the whole block needs (a root, a quotient, the sum
+// of the warps' partials) are formed by one warp and read from shared memory, and
+// magnitudes are compared as integers.
+
+// Block-wide sum; `red` must hold 32 doubles.  All threads return it.
 __device__ inline double block_sum(double v, double* red) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   v = warp_sum(v);
   __syncthreads();
   if (lane == 0) red[w] = v;
   __syncthreads();
-  double t = 0.0;
-  for (int i = 0; i < nw; ++i) t += red[i];
+  if (w == 0) {
+    double t = lane < nw ? red[lane] : 0.0;
+    t = warp_sum(t);
+    __syncwarp();
+    if (lane == 0) red[0] = t;
+  }
   __syncthreads();
-  return t;
+  return red[0];
+}
+
+// Order of a magnitude (>= 0) as an integer; NaN and negative values below every number.
+__device__ __forceinline__ long long mag_key(double x) {
+  const long long b = __double_as_longlong(x);
+  return b >= 0 && b <= 0x7ff0000000000000ll ? b : (b == (long long)0x8000000000000000ull ? 0ll : -1ll);
 }
 
 // Block-wide argmax over values[i] for i in [lo, hi) (hi > lo); returns the
 // index (smallest index among ties), always inside [lo, hi): lo when no value
-// exceeds -1 (every value NaN), where the callers' pivot test then stops.
-// `ri` needs blockDim.x / 32 ints, `rv` doubles.
-__device__ inline int block_argmax(const double* values, int lo, int hi, double* rv, int* ri) {
+// is a number >= 0, where the callers' pivot test then stops.  `rk` needs 32
+// long longs, `ri` 32 ints.
+__device__ inline int block_argmax(const double* values, int lo, int hi, long long* rk, int* ri) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  double best = -1.0;
+  long long best = -1;
   int bi = hi;
   for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-    double x = values[i];
-    if (x > best || (x == best && i < bi)) { best = x; bi = i; }
+    const long long x = mag_key(values[i]);
+    if (x > best) { best = x; bi = i; }
   }
+  auto fold = [&]() {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    double ob = __shfl_xor_sync(0xffffffffu, best, o);
-    int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+    }
+  };
+  fold();
+  if (lane == 0) { rk[w] = best; ri[w] = bi; }
+  __syncthreads();
+  if (w == 0) {
+    best = lane < nw ? rk[lane] : -1;
+    bi = lane < nw ? ri[lane] : hi;
+    fold();
+    __syncwarp();
+    if (lane == 0) ri[0] = bi;
   }
   __syncthreads();
-  if (lane == 0) { rv[w] = best; ri[w] = bi; }
-  __syncthreads();
-  double b = -1.0;
-  int idx = hi;
-  for (int i = 0; i < nw; ++i)
-    if (rv[i] > b || (rv[i] == b && ri[i] < idx)) { b = rv[i]; idx = ri[i]; }
+  const int idx = ri[0];
   __syncthreads();
   return idx < hi ? idx : lo;
 }
@@ -85,8 +107,9 @@ k_env_factor(const EnvFactorItem* __restrict__ items, int* ival) {
   double* A = sm;                 // n x n
   double* dg = A + n * n;         // n
   int* perm = reinterpret_cast<int*>(dg + n);
-  __shared__ double rv[8];
-  __shared__ int ri[8];
+  __shared__ long long rv[32];
+  __shared__ int ri[32];
+  __shared__ double sh_r[2];
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
     int i = e / n, j = e - i * n;
     A[e] = 0.5 * (it.M[i * it.ld + j] + it.M[j * it.ld + i]);
@@ -113,15 +136,18 @@ k_env_factor(const EnvFactorItem* __restrict__ items, int* ival) {
       if (threadIdx.x == 0) { int t = perm[j]; perm[j] = perm[p]; perm[p] = t; }
       __syncthreads();
     }
-    const double rjj = sqrt(A[j * n + j]);
+    if (threadIdx.x == 0) {
+      sh_r[0] = sqrt(A[j * n + j]);
+      sh_r[1] = 1.0 / sh_r[0];
+    }
     __syncthreads();
-    for (int k = j + 1 + threadIdx.x; k < n; k += blockDim.x) A[j * n + k] /= rjj;
-    if (threadIdx.x == 0) A[j * n + j] = rjj;
+    const double inv = sh_r[1];
+    for (int k = j + 1 + threadIdx.x; k < n; k += blockDim.x) A[j * n + k] *= inv;
+    if (threadIdx.x == 0) A[j * n + j] = sh_r[0];
     __syncthreads();
-    const int m = n - j - 1;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-      int a = j + 1 + e / m, b = j + 1 + e % m;
-      A[a * n + b] -= A[j * n + a] * A[j * n + b];
+    for (int a = j + 1 + (int)(threadIdx.x >> 5); a < n; a += (int)(blockDim.x >> 5)) {
+      const double x = A[j * n + a];
+      for (int b = j + 1 + (int)(threadIdx.x & 31); b < n; b += 32) A[a * n + b] -= x * A[j * n + b];
     }
     __syncthreads();
   }
@@ -203,7 +229,7 @@ __host__ __device__ inline HhSmem hh_smem(long long L) {
   m.vtv = o;  o += sizeof(double) * (size_t)NB * NB;
   m.tm = o;   o += sizeof(double) * (size_t)NB * NB;
   m.tau = o;  o += sizeof(double) * (size_t)NB;
-  m.bred = o; o += sizeof(double) * (size_t)(kHhThreads / 32);
+  m.bred = o; o += sizeof(double) * 32;
   m.total = o;
   return m;
 }
@@ -257,20 +283,23 @@ __device__ void hh_block_qr(T* A, long long rows, int n, unsigned char* smem, co
         s = fma(x, x, s);
       }
       s = block_sum(s, bred);
-      const double alpha = (double)col[jj];
-      const double normx = sqrt(s);
-      double beta = alpha, tj = 0.0, v0 = 1.0;
-      if (normx > 0.0) {
-        beta = alpha >= 0.0 ? -normx : normx;
-        v0 = alpha - beta;
-        tj = (beta - alpha) / beta;
-      }
-      __syncthreads();
-      if (normx > 0.0)
-        for (int i = jj + 1 + tid; i < pr; i += blockDim.x) col[i] = (T)((double)col[i] / v0);
       if (tid == 0) {
+        const double alpha = (double)col[jj], normx = sqrt(s);
+        double beta = alpha, tj = 0.0, inv = 1.0;
+        if (normx > 0.0) {
+          beta = alpha >= 0.0 ? -normx : normx;
+          inv = 1.0 / (alpha - beta);
+          tj = (beta - alpha) / beta;
+        }
         col[jj] = (T)beta;
         tau[jj] = tj;
+        bred[1] = inv;
+      }
+      __syncthreads();
+      const double tj = tau[jj];
+      if (tj != 0.0) {
+        const double inv = bred[1];
+        for (int i = jj + 1 + tid; i < pr; i += blockDim.x) col[i] = (T)((double)col[i] * inv);
       }
       __syncthreads();
       // the reflection on the panel's later columns, one warp per column
@@ -678,6 +707,9 @@ __device__ int chol_cluster(const double* __restrict__ A, int lda, int n, int w,
   const int c0 = ct.rank * w;
   const int nl = min(w, n - c0) > 0 ? min(w, n - c0) : 0;
   __shared__ int sh_best;
+  __shared__ Pivot sh_win;
+  __shared__ int sh_from;
+  __shared__ R sh_rs;
   for (int i = tid; i < nl; i += kFacThreads) {
     dq[i] = oq[i] = (R)A[(long long)(c0 + i) * lda + c0 + i];
     pos[i] = -1;
@@ -690,18 +722,21 @@ __device__ int chol_cluster(const double* __restrict__ A, int lda, int n, int w,
     if (tid < 32) {
       // this CTA's largest remaining diagonal (smallest column among ties; none
       // when every candidate is NaN)
-      double best = -1.0;
+      long long best = -1;
       int bi = n;
       for (int i = lane; i < nl; i += 32)
-        if (pos[i] < 0 && (double)dq[i] > best) { best = (double)dq[i]; bi = i; }
+        if (pos[i] < 0) {
+          const long long x = mag_key((double)dq[i]);
+          if (x > best) { best = x; bi = i; }
+        }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
       }
       if (lane == 0) {
-        of->value = best;
+        of->value = bi < n ? (double)dq[bi] : -1.0;
         of->own = bi < n ? (double)oq[bi] : 0.0;
         of->col = bi < n ? c0 + bi : n;
         sh_best = bi;
@@ -712,17 +747,35 @@ __device__ int chol_cluster(const double* __restrict__ A, int lda, int n, int w,
       for (int l = tid; l < j; l += kFacThreads) ofu[l] = U[l * w + sh_best];
     cta_sync(ct);
     // the winner of the cluster
-    double dp = -1.0, op = 0.0;
-    int p = n, from = 0;
-    for (int k = 0; k < ct.size; ++k) {
-      const unsigned a = cluster_addr(of, k);
-      const double v = cluster_ld<double>(a);
-      const int q = cluster_ld<int>(a + (unsigned)offsetof(Pivot, col));
-      if (v > dp || (v == dp && q < p)) { dp = v; p = q; from = k; op = cluster_ld<double>(a + (unsigned)offsetof(Pivot, own)); }
+    if (tid < 32) {
+      const unsigned a = cluster_addr(of, lane < ct.size ? lane : ct.rank);
+      const double v = lane < ct.size ? cluster_ld<double>(a) : -1.0;
+      const double own = cluster_ld<double>(a + (unsigned)offsetof(Pivot, own));
+      const int col = lane < ct.size ? cluster_ld<int>(a + (unsigned)offsetof(Pivot, col)) : n;
+      long long best = mag_key(v);
+      int bi = col, bl = lane;
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o), ol = __shfl_xor_sync(0xffffffffu, bl, o);
+        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; bl = ol; }
+      }
+      bl = __shfl_sync(0xffffffffu, bl, 0);
+      if (lane == bl) {
+        sh_win.value = v;
+        sh_win.own = own;
+        sh_win.col = col;
+        sh_from = lane;
+        sh_rs = R(1) / sqrt((R)v);
+      }
     }
+    __syncthreads();
+    const double dp = sh_win.value, op = sh_win.own;
+    const int p = sh_win.col, from = sh_from;
     if (j == 0) d0 = dp;
     if (p >= n || !(dp > rel * d0) || !(dp > 0.0)) return j;
     if (safe >= 0.0 && !(dp >= safe * op)) return -1;
+    const R rs = sh_rs;
     R a_pc = R(0);
     if (tid < nl) a_pc = (R)A[(long long)p * lda + c0 + tid];
     {
@@ -741,13 +794,13 @@ __device__ int chol_cluster(const double* __restrict__ A, int lda, int n, int w,
     __syncthreads();
     if (tid < nl) {
       if (c0 + tid == p) {
-        U[j * w + tid] = sqrt(dq[tid]);
+        U[j * w + tid] = dq[tid] * rs;
         pos[tid] = j;
       } else if (pos[tid] < 0) {
         R acc = a_pc;
 #pragma unroll
         for (int k = 0; k < kFacSlices; ++k) acc -= part[k * nl + tid];
-        acc /= sqrt((R)dp);
+        acc *= rs;
         U[j * w + tid] = acc;
         dq[tid] = fma(-acc, acc, dq[tid]);
       }
@@ -764,9 +817,10 @@ __device__ int chol_cluster(const double* __restrict__ A, int lda, int n, int w,
 // per column left all but r threads idle on two serial passes of M rows).
 __device__ int qrcp(double* B, int ld, int M, int r, double* dg, double* w, double* v, double* part, int* perm,
                     double rel) {
-  __shared__ double rv[kFacThreads / 32];
-  __shared__ int ri[kFacThreads / 32];
-  __shared__ double red[kFacThreads / 32];
+  __shared__ long long rv[32];
+  __shared__ int ri[32];
+  __shared__ double red[32];
+  __shared__ double sh_h[3];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   constexpr int NW = kFacThreads / 32;
   for (int i = threadIdx.x; i < r; i += blockDim.x) perm[i] = i;
@@ -811,12 +865,16 @@ __device__ int qrcp(double* B, int ld, int M, int r, double* dg, double* w, doub
       s = fma(x, x, s);
     }
     s = block_sum(s, red);
-    const double alpha = B[(long long)j * ld + j];
-    const double normx = sqrt(s);
-    const double beta = alpha >= 0.0 ? -normx : normx;
-    const double v0 = alpha - beta;
-    const double tau = (beta - alpha) / beta;
-    for (int i = j + threadIdx.x; i < M; i += blockDim.x) v[i] = (i == j) ? 1.0 : B[(long long)i * ld + j] / v0;
+    if (threadIdx.x == 0) {
+      const double alpha = B[(long long)j * ld + j], normx = sqrt(s);
+      const double b = alpha >= 0.0 ? -normx : normx;
+      sh_h[0] = b;
+      sh_h[1] = 1.0 / (alpha - b);
+      sh_h[2] = (b - alpha) / b;
+    }
+    __syncthreads();
+    const double beta = sh_h[0], inv = sh_h[1], tau = sh_h[2];
+    for (int i = j + threadIdx.x; i < M; i += blockDim.x) v[i] = (i == j) ? 1.0 : B[(long long)i * ld + j] * inv;
     __syncthreads();
     for (int i = j + threadIdx.x; i < M; i += blockDim.x) B[(long long)i * ld + j] = (i == j) ? beta : 0.0;
     for (int k0 = j + 1; k0 < r; k0 += 32) {
@@ -1011,10 +1069,6 @@ cudaError_t launch_factor(const SiteFacItem* items, int n_items, int rmax, int n
 }
 
 // ===================================================================== core
-// Sort key of a singular-value estimate (a norm, >= 0): NaN ranks last, so
-// the ranks of any input form a permutation (every order[] slot written once).
-__device__ inline double rank_key(double x) { return x == x ? x : -1.0; }
-
 // Rotation of a Jacobi pair from its squared norms and product: h = tan(theta / 2) and
 // s = sin theta of the smaller angle that makes the columns orthogonal, and the new
 // squared norms.  False when the pair is orthogonal to tol (tol2 = tol^2),
@@ -1533,13 +1587,14 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize
     }
     cta_sync(ct);
   };
-  // descending order of sv[0 .. cols)
+  // descending order of sv[0 .. cols), NaN last, so that any input gives a
+  // permutation (every order[] slot written once)
   auto rank_order = [&](int cols) {
     for (int j = threadIdx.x; j < cols; j += blockDim.x) {
       int rk = 0;
-      const double kj = rank_key(sv[j]);
+      const long long kj = mag_key(sv[j]);
       for (int i = 0; i < cols; ++i) {
-        const double ki = rank_key(sv[i]);
+        const long long ki = mag_key(sv[i]);
         if (ki > kj || (ki == kj && i < j)) ++rk;
       }
       order[rk] = j;
@@ -1618,12 +1673,16 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize
       if (l <= i) L[i * (i + 1) / 2 + l] = G[e];
     }
     __syncthreads();
+    double* Li = reinterpret_cast<double*>(core_sh) + 160 * 161 / 2;   // reciprocal diagonals
     for (int j = 0; j < NK; ++j) {
       const int jj = j * (j + 1) / 2;
-      const double djj = sqrt(L[jj + j]);
+      if (threadIdx.x == 0) {
+        L[jj + j] = sqrt(L[jj + j]);
+        Li[j] = 1.0 / L[jj + j];
+      }
       __syncthreads();
-      if (threadIdx.x == 0) L[jj + j] = djj;
-      for (int i = j + 1 + threadIdx.x; i < NK; i += blockDim.x) L[i * (i + 1) / 2 + j] /= djj;
+      const double dinv = Li[j];
+      for (int i = j + 1 + threadIdx.x; i < NK; i += blockDim.x) L[i * (i + 1) / 2 + j] *= dinv;
       __syncthreads();
       for (int i = j + 1 + (int)(threadIdx.x >> 5); i < NK; i += (int)(blockDim.x >> 5)) {
         const double lij = L[i * (i + 1) / 2 + j];
@@ -1637,7 +1696,7 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize
         const double* lc = L + c * (c + 1) / 2;
 #pragma unroll 8
         for (int l = 0; l < c; ++l) x -= Qk[(long long)l * N + i] * lc[l];
-        Qk[(long long)c * N + i] = x / lc[c];
+        Qk[(long long)c * N + i] = x * Li[c];
       }
     }
     cta_sync(ct);
@@ -1705,13 +1764,22 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize
   }
   __syncthreads();
   const int chi = sh_chi;
-  const double inv = 1.0 / sqrt(sh_sum);
-  for (long long i = ct.tid; i < it.chimax; i += ct.nthr) it.lam[i] = (i < chi) ? sv[order[i]] / sh_nrm : 0.0;
+  // per kept value c: lambda_c, and the factor of its vector in W, sqrt(s_c) / sqrt(sum s),
+  // divided by s_c for the side whose vectors are the unscaled columns
+  __shared__ double lam[128], fac[2][128];
+  for (int c = threadIdx.x; c < chi; c += blockDim.x) {
+    const double sc = sv[order[c]];
+    lam[c] = sc / sh_nrm;
+    fac[0][c] = sqrt(sc / sh_sum);
+    fac[1][c] = sc > 0.0 ? fac[0][c] / sc : 0.0;
+  }
+  __syncthreads();
+  for (long long i = ct.tid; i < it.chimax; i += ct.nthr) it.lam[i] = (i < chi) ? lam[i] : 0.0;
   for (long long i = ct.tid; i < N; i += ct.nthr) it.svals[i] = i < NK ? sv[order[i]] : sv[512 + i];
   // messages diag(lambda)
   for (long long e = ct.tid; e < (long long)it.chimax * it.chimax; e += ct.nthr) {
     const int i = (int)(e / it.chimax), j = (int)(e % it.chimax);
-    const double x = (i == j && i < chi) ? sv[order[i]] / sh_nrm : 0.0;
+    const double x = (i == j && i < chi) ? lam[i] : 0.0;
     it.msg12[e] = x;
     it.msg21[e] = x;
   }
@@ -1742,8 +1810,12 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize
   double* Zs[2] = {Z, Z + (long long)rmax * it.chimax};
   {
     constexpr int kZld = kCoreMaxDim + 1;                  // odd: lanes on one row of several columns
+    // reciprocal diagonals of both triangles
+    double* di = reinterpret_cast<double*>(core_sh + kCoreSmem) - 2 * kCoreMaxDim;
+    for (int a = threadIdx.x; a < k1; a += blockDim.x) di[a] = 1.0 / it.T1[(long long)a * it.ldt1 + a];
+    for (int a = threadIdx.x; a < k2; a += blockDim.x) di[kCoreMaxDim + a] = 1.0 / it.T2[(long long)a * it.ldt2 + a];
     double* zc = reinterpret_cast<double*>(core_sh);       // this CTA's columns, ks each
-    const int fit = (int)(kCoreSmem / sizeof(double)) / kZld;   // 47 columns at a time
+    const int fit = ((int)(kCoreSmem / sizeof(double)) - 2 * kCoreMaxDim) / kZld;   // 45 columns at a time
     const int total = 2 * chi;
     const int per = min(fit, (total + ct.size - 1) / ct.size);
     for (int g0 = ct.rank * per; g0 < total; g0 += ct.size * per) {
@@ -1761,12 +1833,11 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize
         for (int e = threadIdx.x; e < ks * nc; e += blockDim.x) {
           const int c = e / ks, a = e - c * ks;
           const int j = order[c0 + c];
-          const double s = sv[j];
           double x;
-          if (from_cols) x = s > 0.0 ? Tc[(long long)j * M + a] / s : 0.0;
+          if (from_cols) x = Tc[(long long)j * M + a];
           else if (it.mixed_svd) x = Vr[(long long)(c0 + c) * N + a];   // Ritz right vector (above)
           else x = V[(long long)j * N + a];                             // accumulated right vector j
-          zc[c * kZld + a] = x * sqrt(s) * inv;
+          zc[c * kZld + a] = x * fac[from_cols ? 1 : 0][c0 + c];
         }
         __syncthreads();
         for (int b1 = ks; b1 > 0; b1 -= 32) {
@@ -1776,8 +1847,7 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize
             double* z = zc + c * kZld;
             double x = b0 + lane < b1 ? z[b0 + lane] : 0.0;
             for (int a = b1 - 1; a >= b0; --a) {
-              const double* trow = Ts + (long long)a * ldts;
-              double y = __shfl_sync(0xffffffffu, x, a - b0) / trow[a];
+              const double y = __shfl_sync(0xffffffffu, x, a - b0) * di[side * kCoreMaxDim + a];
               if (b0 + lane == a) x = y;
               else if (b0 + lane < a) x -= Ts[(long long)(b0 + lane) * ldts + a] * y;
             }
