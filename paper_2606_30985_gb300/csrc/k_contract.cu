@@ -38,12 +38,18 @@ __device__ inline void load_dims4(const TView& v, const int* ival, int* d) {
 // chi = 20; two CTAs per SM overlap one's copies with the other's products.
 // Class of a case, 64 / 128-row tiles -> these: 4x4 chi = 48 72 -> 24 ms, a batch of
 // nine small instances 76 -> 14 ms.
+// FP64 is bound by its pipe, two multiply-adds per clock and SM, so its tiles
+// are small (64 threads, one unit each) and a small site still spreads over
+// many SMs: at chi = 8 a tile of 512 columns took one SM 8 us (class 6.0 -> 3.5 ms).
+template <typename T> struct LegBlock;
+template <> struct LegBlock<float> { static constexpr int NT = 256, NU = 2; };
+template <> struct LegBlock<double> { static constexpr int NT = 64, NU = 1; };
 template <typename T, int MI, int TI>
 struct LegCfg {
   static constexpr int U = 16 / (int)sizeof(T);
   static constexpr int IG = TI / MI;                   // thread groups over the outputs
-  static constexpr int CG = 256 / IG;                  // threads over the columns
-  static constexpr int NU = 2;                         // units per thread
+  static constexpr int CG = LegBlock<T>::NT / IG;      // threads over the columns
+  static constexpr int NU = LegBlock<T>::NU;           // units per thread
   static constexpr int TC = CG * NU * U;               // columns of a tile
 };
 
@@ -51,7 +57,7 @@ template <typename T, int MI, int TI>
 __device__ void leg_tiles(const T* __restrict__ in, T* __restrict__ out, const double* __restrict__ A, int lda, int J,
                           int Jout, unsigned O, unsigned QU, unsigned char* sh, int room) {
   using C = LegCfg<T, MI, TI>;
-  constexpr int U = C::U, CG = C::CG, NU = C::NU, TC = C::TC;
+  constexpr int U = C::U, CG = C::CG, NU = C::NU, TC = C::TC, NT = LegBlock<T>::NT;
   const int tid = threadIdx.x;
   const int cg = tid % CG, ig = tid / CG;
   const long long Q = (long long)QU * U;
@@ -62,7 +68,7 @@ __device__ void leg_tiles(const T* __restrict__ in, T* __restrict__ out, const d
   T* Bs = At + (size_t)J * TI;                         // [jc][TC]
   const unsigned ntile = (cols + CG * NU - 1) / (CG * NU);
   if (blockIdx.x >= ntile) return;
-  for (int e = tid; e < J * TI; e += 256) {
+  for (int e = tid; e < J * TI; e += NT) {
     const int i = e / J, j = e - i * J;
     At[j * TI + i] = i < Jout ? (T)A[(long long)i * lda + j] : T(0);
   }
@@ -128,7 +134,7 @@ __device__ void leg_tiles(const T* __restrict__ in, T* __restrict__ out, const d
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(LegBlock<T>::NT, sizeof(T) == 4 ? 2 : 8)
 k_leg_contract(const LegItem* __restrict__ items, void* const* ptrs, const int* __restrict__ ival, int room) {
   const LegItem it = items[blockIdx.y];
   extern __shared__ __align__(16) unsigned char lc_sh[];
@@ -158,11 +164,18 @@ template <typename T>
 cudaError_t launch_leg_contract(const LegItem* items, int n_items, int grid_x, int chimax,
                                 void* const* ptrs, const int* ival, cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
-  // two CTAs per SM; A at chi = 128 takes 64 KB (FP32) or 128 KB (FP64, one CTA)
-  const int room = (sizeof(T) == 8 && chimax > 64 ? 208 : 104) * 1024;
-  cudaError_t e = cudaFuncSetAttribute(k_leg_contract<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
+  // A and the J rows of a tile, at most half an SM's shared memory (the rows then
+  // come in parts); A at chi = 128 takes 64 KB (FP32) or 128 KB (FP64)
+  const int ti = chimax <= 8 ? 8 : chimax <= 16 ? 16 : chimax <= 32 ? 32 : chimax <= 64 ? 64 : 128;
+  const int tc = LegBlock<T>::NT * (ti == 8 ? 4 : 8) / ti * LegBlock<T>::NU * (16 / (int)sizeof(T));
+  const size_t a_bytes = sizeof(T) * (size_t)chimax * ti;
+  size_t room = a_bytes + sizeof(T) * (size_t)chimax * tc;
+  // a smaller live bond takes a wider tile with fewer rows
+  room = std::max(room, (size_t)(sizeof(T) == 4 ? 72 : 20) * 1024);
+  room = std::min(room, std::max((size_t)104 * 1024, a_bytes + 16 * 1024));
+  cudaError_t e = cudaFuncSetAttribute(k_leg_contract<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
   if (e != cudaSuccess) return e;
-  k_leg_contract<T><<<dim3(grid_x, n_items), 256, room, s>>>(items, ptrs, ival, room);
+  k_leg_contract<T><<<dim3(grid_x, n_items), LegBlock<T>::NT, room, s>>>(items, ptrs, ival, (int)room);
   return cudaGetLastError();
 }
 
