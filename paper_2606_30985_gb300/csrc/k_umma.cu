@@ -289,19 +289,39 @@ __device__ __noinline__ void leg_plan(const LegItem* items, int i, void* const* 
   L.lda = it.lda;
 }
 
-// The CTA's tiles t0 .. t1 of the launch, item by item: tiles lo .. hi of `item`.
+// The CTA's tiles of the launch, item by item: lo, lo + step, .. (cnt of them) of
+// `item`.  Tile g of the launch goes to CTA g mod grid where the items are large
+// (at least 8 tiles per CTA on average): the CTAs then work on neighbouring
+// tiles, whose 512-byte pieces of a row share DRAM pages, instead of streaming
+// through 152 places of the tensor at once.  Small items are cut into
+// contiguous ranges, so that a CTA sees few of them (each brings its own small
+// matrix).
 struct ItemRange {
   int item;
-  unsigned lo, hi, t, t1;
+  unsigned lo, cnt, step, t, t1;
+  __device__ void start(const unsigned* toff, int n) {
+    const unsigned long long T = toff[n];
+    item = -1;
+    if (T >= 8ull * n * gridDim.x) {
+      step = gridDim.x;
+      t = blockIdx.x;
+      t1 = (unsigned)T;
+    } else {
+      step = 1;
+      t = (unsigned)(T * blockIdx.x / gridDim.x);
+      t1 = (unsigned)(T * (blockIdx.x + 1) / gridDim.x);
+    }
+  }
+  __device__ bool next(const unsigned* toff, int n) {      // false when the CTA is done
+    if (t >= t1) return false;
+    if (item < 0) item = 0;
+    while (item + 1 < n && toff[item + 1] <= t) ++item;
+    lo = t - toff[item];
+    cnt = (min(t1, toff[item + 1]) - t + step - 1) / step;
+    t += cnt * step;
+    return true;
+  }
 };
-__device__ inline bool range_next(ItemRange& r, const unsigned* toff, int n) {   // false when the CTA is done
-  if (r.t >= r.t1) return false;
-  while (r.item + 1 < n && toff[r.item + 1] <= r.t) ++r.item;
-  r.lo = r.t - toff[r.item];
-  r.hi = min(r.t1, toff[r.item + 1]) - toff[r.item];
-  r.t += r.hi - r.lo;
-  return true;
-}
 
 // Shared-memory plan of k_leg_umma for a given chi bound.
 struct LegSmem {
@@ -367,11 +387,8 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
   __syncthreads();
   tc_after();
   const uint32_t tmem = bars->tmem;
-  const unsigned long long T = toff[n_items];
   ItemRange rg;
-  rg.item = 0;
-  rg.t = (unsigned)(T * blockIdx.x / gridDim.x);
-  rg.t1 = (unsigned)(T * (blockIdx.x + 1) / gridDim.x);
+  rg.start(toff, n_items);
   LegPlan L;
 
   if (warp == 0) {
@@ -381,14 +398,14 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
       int st_i = 0;            // operand stage and its phase parity (advanced per chunk)
       uint32_t st_ph = 0;
       bool ok = true;
-      for (unsigned item_n = 0; ok && range_next(rg, toff, n_items); ++item_n) {
+      for (unsigned item_n = 0; ok && rg.next(toff, n_items); ++item_n) {
         leg_plan(items, rg.item, ptrs, ival, L);
         const int N16 = L.N16, K8 = L.K8, nkc = L.nkc;
         const uint32_t bblk = (uint32_t)(2 * N16) * 128;   // B block per K chunk
         const uint32_t id_wide = idesc_tf32(kM, 2 * N16), id_half = idesc_tf32(kM, N16);
         if (!mbar_wait(&bars->bfull, item_n & 1u, abort_flag, err, lim)) break;
         tc_after();
-        for (unsigned tile = rg.lo; tile < rg.hi && ok; ++tile, ++tc) {
+        for (unsigned i = 0; i < rg.cnt && ok; ++i, ++tc) {
           const int b = (int)(tc & 1);
           if (!mbar_wait(&bars->accempty[b], ((tc >> 1) & 1u) ^ 1u, abort_flag, err, lim)) { ok = false; break; }
           tc_after();
@@ -426,11 +443,11 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
     const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
     unsigned tc = 0;
     bool ok = true;
-    while (ok && range_next(rg, toff, n_items)) {
+    while (ok && rg.next(toff, n_items)) {
       leg_plan(items, rg.item, ptrs, ival, L);
       const int N16 = L.N16, Jout = L.Jout;
       const unsigned Q = L.Q;
-      for (unsigned tile = rg.lo; tile < rg.hi; ++tile, ++tc) {
+      for (unsigned i = 0, tile = rg.lo; i < rg.cnt; ++i, tile += rg.step, ++tc) {
         const int b = (int)(tc & 1);
         if (!warp_wait(&bars->accfull[b], (tc >> 1) & 1u, abort_flag, err, lim)) { ok = false; break; }
         tc_after();
@@ -484,11 +501,11 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
     const int ct = tid - 256, grp = ct / kGroup, r = ct % kGroup;
     unsigned n = 0;                                   // chunks of the CTA before this item
     bool ok = true;
-    for (unsigned item_n = 0; ok && range_next(rg, toff, n_items); ++item_n) {
+    for (unsigned item_n = 0; ok && rg.next(toff, n_items); ++item_n) {
       leg_plan(items, rg.item, ptrs, ival, L);
       const int nkc = L.nkc, J = L.J, K8 = L.K8;
       const unsigned Q = L.Q;
-      const unsigned total = (rg.hi - rg.lo) * (unsigned)nkc;
+      const unsigned total = rg.cnt * (unsigned)nkc;
       unsigned j = (n ^ (unsigned)grp) & 1u;           // this group's first chunk of the item
       unsigned nn = n + j;                             // its number in the CTA
       n += total;
@@ -498,7 +515,7 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
       const float* src = L.in;
       bool valid = false;
       auto enter = [&]() {
-        while (kc >= nkc) { kc -= nkc; ++tile; }
+        while (kc >= nkc) { kc -= nkc; tile += rg.step; }
         const unsigned rr = tile * kM + r;
         valid = rr < L.R;
         const unsigned o = valid ? rr / Q : 0u;
@@ -889,8 +906,12 @@ struct RecPlan {
   const float* Wp;
   unsigned R, nrb;         // rows, row blocks of 128
   int n, np, K8, nkc, nnb, NB, ldw;
-  unsigned d1, d2;         // extents of the last two of the (up to three) row legs
-  long long os0, os1, os2, ocut;   // output strides of the row legs and of the new cut leg
+  // Row r of the launch is (a0, a1, a2), a2 fastest, over the (up to three) row legs
+  // ordered so that the one that is innermost in the output is a2: the lanes of
+  // a warp then write 16-byte neighbours.
+  unsigned d1, d2;                 // extents of a1, a2
+  unsigned rs0, rs1, rs2;          // their strides among the input's rows
+  long long os0, os1, os2, ocut;   // and in the output; the new cut leg's
 };
 
 __device__ inline unsigned rec_rows(const ReconItem& it, const int* ival) {
@@ -928,12 +949,25 @@ __device__ __noinline__ void rec_plan(const ReconItem* items, int i, void* const
     st *= e;
   }
   D.ocut = os[cut];
-  // the row legs 0 .. cut - 1, right-aligned in three places (missing ones: extent 1)
-  D.os2 = cut >= 1 ? os[cut - 1] : 0;
-  D.d2 = cut >= 1 ? dd[cut - 1] : 1;
-  D.os1 = cut >= 2 ? os[cut - 2] : 0;
-  D.d1 = cut >= 2 ? dd[cut - 2] : 1;
-  D.os0 = cut >= 3 ? os[cut - 3] : 0;
+  // the row legs, right-aligned in three places (missing ones: extent 1), the
+  // output's innermost one moved to the end
+  unsigned rs[PEPO_MAXLEG] = {0, 0, 0, 0};
+  unsigned q = 1;
+  for (int l = cut - 1; l >= 0; --l) { rs[l] = q; q *= (unsigned)dd[l]; }
+  int leg[3] = {-1, -1, -1};
+  const int inner = it.out_perm[nl - 1];
+  int at = 2;
+  if (inner != cut && cut > 0) leg[at--] = inner;
+  for (int l = cut - 1; l >= 0 && at >= 0; --l)
+    if (l != inner) leg[at--] = l;
+  D.rs0 = leg[0] >= 0 ? rs[leg[0]] : 0;
+  D.os0 = leg[0] >= 0 ? os[leg[0]] : 0;
+  D.rs1 = leg[1] >= 0 ? rs[leg[1]] : 0;
+  D.os1 = leg[1] >= 0 ? os[leg[1]] : 0;
+  D.d1 = leg[1] >= 0 ? dd[leg[1]] : 1;
+  D.rs2 = leg[2] >= 0 ? rs[leg[2]] : 0;
+  D.os2 = leg[2] >= 0 ? os[leg[2]] : 0;
+  D.d2 = leg[2] >= 0 ? dd[leg[2]] : 1;
   D.in = static_cast<const float*>(ptrs[it.in.ref]);
   D.out = static_cast<float*>(ptrs[it.out_ref]);
   D.W = it.W;
@@ -1001,11 +1035,8 @@ k_recon_umma(const ReconItem* __restrict__ items, int n_items, void* const* ptrs
   __syncthreads();
   tc_after();
   const uint32_t tmem = bars->tmem;
-  const unsigned long long T = toff[n_items];
   ItemRange rg;
-  rg.item = 0;
-  rg.t = (unsigned)(T * blockIdx.x / gridDim.x);
-  rg.t1 = (unsigned)(T * (blockIdx.x + 1) / gridDim.x);
+  rg.start(toff, n_items);
   RecPlan D;
 
   if (warp == 0) {
@@ -1015,11 +1046,11 @@ k_recon_umma(const ReconItem* __restrict__ items, int n_items, void* const* ptrs
       int st_i = 0;            // operand stage and its phase parity (advanced per chunk)
       uint32_t st_ph = 0;
       bool ok = true;
-      while (ok && range_next(rg, toff, n_items)) {
+      while (ok && rg.next(toff, n_items)) {
         rec_plan(items, rg.item, ptrs, ival, D);
         const int NB = D.NB, K8 = D.K8, nkc = D.nkc;
         const uint32_t id_wide = idesc_tf32(kM, 2 * NB), id_half = idesc_tf32(kM, NB);
-        for (unsigned tile = rg.lo; tile < rg.hi && ok; ++tile, ++tc) {
+        for (unsigned i = 0; i < rg.cnt && ok; ++i, ++tc) {
           const int b = (int)(tc & 1);
           if (!mbar_wait(&bars->accempty[b], ((tc >> 1) & 1u) ^ 1u, abort_flag, err, lim)) { ok = false; break; }
           tc_after();
@@ -1055,10 +1086,10 @@ k_recon_umma(const ReconItem* __restrict__ items, int n_items, void* const* ptrs
     if (lane == 0) {
       unsigned n = 0;          // copies issued
       bool ok = true;
-      while (ok && range_next(rg, toff, n_items)) {
+      while (ok && rg.next(toff, n_items)) {
         rec_plan(items, rg.item, ptrs, ival, D);
         const uint32_t bytes = (uint32_t)(2 * D.NB) * 128u;
-        for (unsigned tile = rg.lo; tile < rg.hi && ok; ++tile) {
+        for (unsigned i = 0, tile = rg.lo; i < rg.cnt && ok; ++i, tile += rg.step) {
           const float* blk = D.Wp + (size_t)(tile % (unsigned)D.nnb) * D.nkc * (size_t)(2 * D.NB) * 32;
           for (int kc = 0; kc < D.nkc; ++kc) {
             const unsigned s = n % (unsigned)NS;
@@ -1088,11 +1119,11 @@ k_recon_umma(const ReconItem* __restrict__ items, int n_items, void* const* ptrs
     const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
     unsigned tc = 0;
     bool ok = true;
-    while (ok && range_next(rg, toff, n_items)) {
+    while (ok && rg.next(toff, n_items)) {
       rec_plan(items, rg.item, ptrs, ival, D);
       const int NB = D.NB;
       const long long ocut = D.ocut;
-      for (unsigned tile = rg.lo; tile < rg.hi; ++tile, ++tc) {
+      for (unsigned i = 0, tile = rg.lo; i < rg.cnt; ++i, tile += rg.step, ++tc) {
         const int b = (int)(tc & 1);
         if (!warp_wait(&bars->accfull[b], (tc >> 1) & 1u, abort_flag, err, lim)) { ok = false; break; }
         tc_after();
@@ -1153,32 +1184,37 @@ k_recon_umma(const ReconItem* __restrict__ items, int n_items, void* const* ptrs
     constexpr int MU = kM / (kGroup / 8);
     unsigned n = 0;                                   // chunks of the CTA before this item
     bool ok = true;
-    while (ok && range_next(rg, toff, n_items)) {
+    while (ok && rg.next(toff, n_items)) {
       rec_plan(items, rg.item, ptrs, ival, D);
       const int nkc = D.nkc, K = D.n;
       const unsigned R = D.R;
-      const unsigned total = (rg.hi - rg.lo) * (unsigned)nkc;
+      const unsigned total = rg.cnt * (unsigned)nkc;
       unsigned j = (n ^ (unsigned)grp) & 1u;
       unsigned nn = n + j;
       n += total;
       unsigned tile = rg.lo, lj = j;
       int kc = (int)j;
-      unsigned row = 0;                                // first row of this thread in the load cursor's tile
-      const float* src = D.in;
+      const float* src[MU];                            // this thread's rows in the load cursor's tile (null: none)
+      unsigned blk = ~0u;                              // row block they belong to
       auto enter = [&]() {
-        while (kc >= nkc) { kc -= nkc; ++tile; }
-        row = tile / (unsigned)D.nnb * kM + r0;
-        src = D.in + (long long)row * K + 4 * kq;
+        while (kc >= nkc) { kc -= nkc; tile += rg.step; }
+        const unsigned rb = tile / (unsigned)D.nnb;
+        if (rb == blk) return;
+        blk = rb;
+#pragma unroll
+        for (int i = 0; i < MU; ++i) {
+          const unsigned r = rb * kM + r0 + 16 * i;
+          const unsigned q = r / D.d2, a2 = r - q * D.d2, a0 = q / D.d1, a1 = q - a0 * D.d1;
+          src[i] = r < R ? D.in + (long long)(a0 * D.rs0 + a1 * D.rs1 + a2 * D.rs2) * K + 4 * kq : nullptr;
+        }
       };
       auto load = [&](float4 (&v)[MU]) {
         const int k = kc * kKC;
         const bool live = k + 4 * kq < K;
-        const float* p = src + k;
 #pragma unroll
         for (int i = 0; i < MU; ++i) {
           v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (live && row + 16 * i < R) v[i] = __ldg(reinterpret_cast<const float4*>(p));
-          p += 16 * K;
+          if (live && src[i]) v[i] = __ldg(reinterpret_cast<const float4*>(src[i] + k));
         }
         lj += 2;
         kc += 2;
