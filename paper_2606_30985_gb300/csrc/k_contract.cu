@@ -205,7 +205,8 @@ struct GlCfg {
   static constexpr int U = 16 / (int)sizeof(T);        // values per 16-byte unit
   static constexpr int TL = MT * TX;
   static constexpr int G = 256 / (TX * TX);            // groups sharing a chunk
-  static constexpr int KCU = 2 * G > 8 ? 2 * G : 8;    // units per row and chunk
+  static constexpr int U0 = sizeof(T) == 4 ? 16 : 8;
+  static constexpr int KCU = (U0 / 4) * G > U0 ? (U0 / 4) * G : U0;   // units per row and chunk
   static constexpr int PITCH = (KCU + 1) * U;          // values between rows
   static constexpr size_t kStage = sizeof(T) * (size_t)TL * PITCH;
   static constexpr size_t kRed = G > 1 ? sizeof(double) * (size_t)TL * TL : 0;
@@ -340,11 +341,12 @@ __device__ void gram_tile(const T* __restrict__ X, long long O, long long Q, int
   }
 }
 
-// BAND 0: F <= 32, 1: F <= 64, 2: F <= 128 (a launch of its own per band that
-// chi_max can reach, so that the small tiles do not carry the large one's
-// registers); blocks of the other bands return.
+// Bands of F, a launch of its own for each that chi_max can reach, so that the
+// small tiles do not carry the large ones' registers (two blocks per SM up to
+// F = 48): blocks of the other bands return.
+constexpr int kGramBands[] = {32, 48, 64, 128};
 template <typename T, int BAND>
-__global__ void __launch_bounds__(256, BAND == 0 ? 2 : 1)
+__global__ void __launch_bounds__(256, BAND < 2 ? 2 : 1)
 k_gram_leg(const GramLegItem* __restrict__ items, int splits_max, void* const* ptrs, const int* __restrict__ ival) {
   const GramLegItem it = items[blockIdx.y];
   int d[PEPO_MAXLEG];
@@ -358,7 +360,8 @@ k_gram_leg(const GramLegItem* __restrict__ items, int splits_max, void* const* p
     else if (i < k) O *= d[i];
     else Q *= d[i];                                    // legs beyond nlegs have size 1
   }
-  if (BAND == 0 ? F > 32 : BAND == 1 ? (F <= 32 || F > 64) : F <= 64) return;
+  if (F > (BAND == 0 ? 32 : BAND == 1 ? 48 : BAND == 2 ? 64 : 128)) return;
+  if (F <= (BAND == 0 ? 0 : BAND == 1 ? 32 : BAND == 2 ? 48 : 64)) return;
   const int S = gram_leg_splits_k(O * Q, splits_max, kGramLegRowsSimt);
   extern __shared__ __align__(16) unsigned char gl_sh[];
   const T* X = static_cast<const T*>(ptrs[it.x.ref]);
@@ -369,8 +372,9 @@ k_gram_leg(const GramLegItem* __restrict__ items, int splits_max, void* const* p
       else if (F <= 16) gram_tile<T, 4, 4>(X, O, Q, F, s, S, P, gl_sh);
       else gram_tile<T, 4, 8>(X, O, Q, F, s, S, P, gl_sh);
     } else if constexpr (BAND == 1) {
-      if (F <= 48) gram_tile<T, 6, 8>(X, O, Q, F, s, S, P, gl_sh);
-      else gram_tile<T, 8, 8>(X, O, Q, F, s, S, P, gl_sh);
+      gram_tile<T, 6, 8>(X, O, Q, F, s, S, P, gl_sh);
+    } else if constexpr (BAND == 2) {
+      gram_tile<T, 8, 8>(X, O, Q, F, s, S, P, gl_sh);
     } else {
       if (F <= 96) gram_tile<T, 6, 16>(X, O, Q, F, s, S, P, gl_sh);
       else gram_tile<T, 8, 16>(X, O, Q, F, s, S, P, gl_sh);
@@ -382,7 +386,8 @@ k_gram_leg(const GramLegItem* __restrict__ items, int splits_max, void* const* p
 template <typename T, int BAND>
 size_t gram_leg_smem() {
   if (BAND == 0) return std::max(std::max(GlCfg<T, 2, 4>::kSmem, GlCfg<T, 4, 4>::kSmem), GlCfg<T, 4, 8>::kSmem);
-  if (BAND == 1) return std::max(GlCfg<T, 6, 8>::kSmem, GlCfg<T, 8, 8>::kSmem);
+  if (BAND == 1) return GlCfg<T, 6, 8>::kSmem;
+  if (BAND == 2) return GlCfg<T, 8, 8>::kSmem;
   return std::max(GlCfg<T, 6, 16>::kSmem, GlCfg<T, 8, 16>::kSmem);
 }
 
@@ -416,9 +421,9 @@ static cudaError_t launch_gram_band(const GramLegItem* items, int n_items, int s
   const size_t smem = gram_leg_smem<T, BAND>();
   cudaError_t e = cudaFuncSetAttribute(k_gram_leg<T, BAND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  // about 8 blocks per SM in all; a block takes several splits of its item when
+  // about 16 blocks per SM in all; a block takes several splits of its item when
   // there are many items (a batch), so that few of its blocks find nothing to do
-  const int gx = std::min(splits_max, std::max(4, ceil_div(8 * 152, n_items)));
+  const int gx = std::min(splits_max, std::max(8, ceil_div(16 * 152, n_items)));
   k_gram_leg<T, BAND><<<dim3(gx, n_items), 256, smem, s>>>(items, splits_max, ptrs, ival);
   return cudaGetLastError();
 }
@@ -428,8 +433,9 @@ cudaError_t launch_gram_leg(const GramLegItem* items, int n_items, int splits_ma
                             void* const* ptrs, const int* ival, cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
   cudaError_t e = launch_gram_band<T, 0>(items, n_items, splits_max, ptrs, ival, s);
-  if (e == cudaSuccess && chimax > 32) e = launch_gram_band<T, 1>(items, n_items, splits_max, ptrs, ival, s);
-  if (e == cudaSuccess && chimax > 64) e = launch_gram_band<T, 2>(items, n_items, splits_max, ptrs, ival, s);
+  if (e == cudaSuccess && chimax > kGramBands[0]) e = launch_gram_band<T, 1>(items, n_items, splits_max, ptrs, ival, s);
+  if (e == cudaSuccess && chimax > kGramBands[1]) e = launch_gram_band<T, 2>(items, n_items, splits_max, ptrs, ival, s);
+  if (e == cudaSuccess && chimax > kGramBands[2]) e = launch_gram_band<T, 3>(items, n_items, splits_max, ptrs, ival, s);
   return e;
 }
 
