@@ -183,15 +183,13 @@ __device__ __forceinline__ void tmem_free(uint32_t taddr) {
 
 // shared-memory matrix descriptor: K-major, 128-byte swizzle, atoms 1024
 // bytes apart (the leading offset is unused for this layout: one atom spans
-// the MMA's K)
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-  uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1 << 16;                   // leading byte offset (unused), 16 bytes
-  d |= (uint64_t)(1024u >> 4) << 32;        // stride byte offset: 8-row atoms
-  d |= (uint64_t)1 << 46;                   // descriptor version of the sm_100 family
-  d |= (uint64_t)2 << 61;                   // layout: 128-byte swizzle
-  return d;
-}
+// the MMA's K).  The high word is the same for every operand; the low word is
+// the address in 16-byte units and the leading offset (16 bytes, unused), so
+// a K step of 32 bytes adds 2 to it.
+constexpr uint32_t kDescHi = (1024u >> 4)          // stride byte offset: 8-row atoms
+                             | (1u << 14)          // descriptor version of the sm_100 family
+                             | (2u << 29);         // layout: 128-byte swizzle
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | (1u << 16); }
 // byte offset of the 16-byte piece `piece` (K / 4) of row `row` in a tile
 __host__ __device__ __forceinline__ uint32_t swz(int row, int piece) {
   return (uint32_t)((row >> 3) * 1024 + (row & 7) * 128 + ((piece ^ (row & 7)) << 4));
@@ -200,17 +198,54 @@ __host__ __device__ __forceinline__ uint32_t swz(int row, int piece) {
 __device__ __forceinline__ uint32_t idesc_tf32(int m, int n) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+// D (+)= A B over one K step; a and b are descriptor low words
+__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      "mov.b64 da, {%1, %5};\n\t"
+      "mov.b64 db, {%2, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %3, p;\n\t}\n" ::"r"(d_tmem),
+      "r"(a), "r"(b), "r"(idesc), "r"(acc), "r"(kDescHi)
       : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint64_t* b) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(b))
                : "memory");
+}
+// One lane of the converged warp, always the same one.  The MMA warp runs its
+// loops and waits as a whole and elects the issuing lane around each chunk's
+// MMAs, so that descriptors and loop state stay warp-uniform: a branch on the
+// lane around the whole role kept them per thread, and the issue of a chunk
+// then took longer (1180 cycles for 8 MMAs) than the tensor core needs (510).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(ok));
+  return ok != 0;
+}
+// the three TF32 products of one K chunk of a split operand pair (KS K steps):
+// [Dhh | Dhl] (+)= Ahi [Bhi; Blo]^T, Dhh += Alo Bhi^T
+template <int KS>
+__device__ __forceinline__ void mma_split(uint32_t d_tmem, uint32_t ah, uint32_t al, uint32_t b, uint32_t id_wide,
+                                          uint32_t id_half, uint32_t acc0) {
+#pragma unroll
+  for (int st = 0; st < KS; ++st) {
+    mma_tf32(d_tmem, ah + 2u * st, b + 2u * st, id_wide, st > 0 ? 1u : acc0);
+    mma_tf32(d_tmem, al + 2u * st, b + 2u * st, id_half, 1u);
+  }
+}
+__device__ __forceinline__ void mma_split_chunk(int ksteps, uint32_t d_tmem, uint32_t ah, uint32_t al, uint32_t b,
+                                                uint32_t id_wide, uint32_t id_half, uint32_t acc0) {
+  switch (ksteps) {
+    case 4: mma_split<4>(d_tmem, ah, al, b, id_wide, id_half, acc0); break;
+    case 3: mma_split<3>(d_tmem, ah, al, b, id_wide, id_half, acc0); break;
+    case 2: mma_split<2>(d_tmem, ah, al, b, id_wide, id_half, acc0); break;
+    default: mma_split<1>(d_tmem, ah, al, b, id_wide, id_half, acc0); break;
+  }
 }
 // 32 TMEM lanes x 16 consecutive 32-bit columns; thread t receives lane
 // (lane base + t).  The registers are valid after tmem_wait16.
@@ -393,46 +428,44 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
 
   if (warp == 0) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      unsigned tc = 0;
-      int st_i = 0;            // operand stage and its phase parity (advanced per chunk)
-      uint32_t st_ph = 0;
-      bool ok = true;
-      for (unsigned item_n = 0; ok && rg.next(toff, n_items); ++item_n) {
-        leg_plan(items, rg.item, ptrs, ival, L);
-        const int N16 = L.N16, K8 = L.K8, nkc = L.nkc;
-        const uint32_t bblk = (uint32_t)(2 * N16) * 128;   // B block per K chunk
-        const uint32_t id_wide = idesc_tf32(kM, 2 * N16), id_half = idesc_tf32(kM, N16);
-        if (!mbar_wait(&bars->bfull, item_n & 1u, abort_flag, err, lim)) break;
+    unsigned tc = 0;
+    int st_i = 0;            // operand stage and its phase parity (advanced per chunk)
+    uint32_t st_ph = 0;
+    bool ok = true;
+    for (unsigned item_n = 0; ok && rg.next(toff, n_items); ++item_n) {
+      leg_plan(items, rg.item, ptrs, ival, L);
+      const int N16 = L.N16, K8 = L.K8, nkc = L.nkc;
+      const uint32_t bstep = (uint32_t)(2 * N16) * 8;    // B block per K chunk (16-byte units)
+      const uint32_t id_wide = idesc_tf32(kM, 2 * N16), id_half = idesc_tf32(kM, N16);
+      if (!warp_wait(&bars->bfull, item_n & 1u, abort_flag, err, lim)) break;
+      tc_after();
+      for (unsigned i = 0; i < rg.cnt && ok; ++i, ++tc) {
+        const int b = (int)(tc & 1);
+        if (!warp_wait(&bars->accempty[b], ((tc >> 1) & 1u) ^ 1u, abort_flag, err, lim)) { ok = false; break; }
         tc_after();
-        for (unsigned i = 0; i < rg.cnt && ok; ++i, ++tc) {
-          const int b = (int)(tc & 1);
-          if (!mbar_wait(&bars->accempty[b], ((tc >> 1) & 1u) ^ 1u, abort_flag, err, lim)) { ok = false; break; }
+        const uint32_t d_tmem = tmem + (uint32_t)(b * 256);
+        uint32_t db = desc_lo(su32(Bs));
+        for (int kc = 0; kc < nkc; ++kc, db += bstep) {
+          const int s = st_i;
+          if (!warp_wait(&bars->full[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
+          if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
           tc_after();
-          const uint32_t d_tmem = tmem + (uint32_t)(b * 256);
-          for (int kc = 0; kc < nkc; ++kc) {
-            const int s = st_i;
-            if (!mbar_wait(&bars->full[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
-            if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
-            tc_after();
-            const uint32_t a_hi = su32(As + (size_t)s * P.stage_bytes);
-            const uint32_t a_lo = a_hi + (uint32_t)(P.stage_bytes / 2);
-            const uint32_t b0 = su32(Bs) + (uint32_t)kc * bblk;
-            const int ksteps = min(kKC, K8 - kc * kKC) / 8;
-            for (int st = 0; st < ksteps; ++st) {
-              const uint64_t dah = sdesc(a_hi + (uint32_t)st * 32u);
-              const uint64_t dal = sdesc(a_lo + (uint32_t)st * 32u);
-              const uint64_t db = sdesc(b0 + (uint32_t)st * 32u);
-              mma_tf32(d_tmem, dah, db, id_wide, (kc > 0 || st > 0) ? 1u : 0u);
-              mma_tf32(d_tmem, dal, db, id_half, 1u);
-            }
+          const uint32_t da = desc_lo(su32(As) + (uint32_t)s * (uint32_t)P.stage_bytes);
+          if (elect_one()) {
+            mma_split_chunk(min(kKC, K8 - kc * kKC) / 8, d_tmem, da, da + (uint32_t)(P.stage_bytes / 32), db, id_wide,
+                            id_half, kc > 0 ? 1u : 0u);
             mma_commit(&bars->empty[s]);
           }
-          if (ok) mma_commit(&bars->accfull[b]);
+          __syncwarp();
         }
-        if (ok) mma_commit(&bars->bfree);
+        if (ok && elect_one()) mma_commit(&bars->accfull[b]);
+        __syncwarp();
       }
-      // every issued MMA completes before tensor memory is released
+      if (ok && elect_one()) mma_commit(&bars->bfree);
+      __syncwarp();
+    }
+    // every issued MMA completes before tensor memory is released
+    if (elect_one()) {
       mma_commit(&bars->drain);
       mbar_drain(&bars->drain, 0, err);
     }
@@ -724,40 +757,41 @@ k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, 
 
   if (warp == 0) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      GramUnit g;
-      long long rc = 0;
-      int st_i = 0;            // operand stage and its phase parity (advanced per chunk)
-      uint32_t st_ph = 0;
-      bool ok = true;
-      for (long long u = blockIdx.x; u < U && ok; u += gridDim.x) {
-        gram_unit(g, u, uoff, n_items, items, ptrs, ival, splits_max);
-        const uint32_t id = idesc_tf32(kM, 2 * g.F8);
-        for (unsigned c = g.c0; c < g.c1 && ok;) {
-          const int b = (int)(rc & 1);
-          if (!mbar_wait(&bars->accempty[b], (uint32_t)(((rc >> 1) & 1) ^ 1), abort_flag, err, lim)) { ok = false; break; }
+    GramUnit g;
+    long long rc = 0;
+    int st_i = 0;            // operand stage and its phase parity (advanced per chunk)
+    uint32_t st_ph = 0;
+    bool ok = true;
+    for (long long u = blockIdx.x; u < U && ok; u += gridDim.x) {
+      gram_unit(g, u, uoff, n_items, items, ptrs, ival, splits_max);
+      const uint32_t id = idesc_tf32(kM, 2 * g.F8);
+      for (unsigned c = g.c0; c < g.c1 && ok;) {
+        const int b = (int)(rc & 1);
+        if (!warp_wait(&bars->accempty[b], (uint32_t)(((rc >> 1) & 1) ^ 1), abort_flag, err, lim)) { ok = false; break; }
+        tc_after();
+        const uint32_t d_tmem = tmem + (uint32_t)(b * 256);
+        const unsigned cend = min(g.c1, c + kRun);
+        for (unsigned cr = c; cr < cend; ++cr) {
+          const int s = st_i;
+          if (!warp_wait(&bars->full[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
+          if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
           tc_after();
-          const uint32_t d_tmem = tmem + (uint32_t)(b * 256);
-          const unsigned cend = min(g.c1, c + kRun);
-          for (unsigned cr = c; cr < cend; ++cr) {
-            const int s = st_i;
-            if (!mbar_wait(&bars->full[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
-            if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
-            tc_after();
-            const uint32_t x0 = su32(Xs + (size_t)s * P.stage_bytes);
+          const uint32_t dx = desc_lo(su32(Xs) + (uint32_t)s * (uint32_t)P.stage_bytes);
+          if (elect_one()) {
+            const uint32_t acc0 = cr > c ? 1u : 0u;
 #pragma unroll
-            for (int st = 0; st < kKC / 8; ++st) {
-              const uint64_t d = sdesc(x0 + (uint32_t)st * 32u);
-              mma_tf32(d_tmem, d, d, id, (cr > c || st > 0) ? 1u : 0u);
-            }
+            for (uint32_t st = 0; st < kKC / 8; ++st)
+              mma_tf32(d_tmem, dx + 2u * st, dx + 2u * st, id, st > 0 ? 1u : acc0);
             mma_commit(&bars->empty[s]);
+            if (cr + 1 == cend) mma_commit(&bars->accfull[b]);
           }
-          if (!ok) break;
-          mma_commit(&bars->accfull[b]);
-          ++rc;
-          c = cend;
+          __syncwarp();
         }
+        ++rc;
+        c = cend;
       }
+    }
+    if (elect_one()) {
       mma_commit(&bars->drain);
       mbar_drain(&bars->drain, 0, err);
     }
@@ -1041,42 +1075,39 @@ k_recon_umma(const ReconItem* __restrict__ items, int n_items, void* const* ptrs
 
   if (warp == 0) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      unsigned tc = 0;
-      int st_i = 0;            // operand stage and its phase parity (advanced per chunk)
-      uint32_t st_ph = 0;
-      bool ok = true;
-      while (ok && rg.next(toff, n_items)) {
-        rec_plan(items, rg.item, ptrs, ival, D);
-        const int NB = D.NB, K8 = D.K8, nkc = D.nkc;
-        const uint32_t id_wide = idesc_tf32(kM, 2 * NB), id_half = idesc_tf32(kM, NB);
-        for (unsigned i = 0; i < rg.cnt && ok; ++i, ++tc) {
-          const int b = (int)(tc & 1);
-          if (!mbar_wait(&bars->accempty[b], ((tc >> 1) & 1u) ^ 1u, abort_flag, err, lim)) { ok = false; break; }
+    unsigned tc = 0;
+    int st_i = 0;            // operand stage and its phase parity (advanced per chunk)
+    uint32_t st_ph = 0;
+    bool ok = true;
+    while (ok && rg.next(toff, n_items)) {
+      rec_plan(items, rg.item, ptrs, ival, D);
+      const int NB = D.NB, K8 = D.K8, nkc = D.nkc;
+      const uint32_t id_wide = idesc_tf32(kM, 2 * NB), id_half = idesc_tf32(kM, NB);
+      for (unsigned i = 0; i < rg.cnt && ok; ++i, ++tc) {
+        const int b = (int)(tc & 1);
+        if (!warp_wait(&bars->accempty[b], ((tc >> 1) & 1u) ^ 1u, abort_flag, err, lim)) { ok = false; break; }
+        tc_after();
+        const uint32_t d_tmem = tmem + (uint32_t)(b * 256);
+        for (int kc = 0; kc < nkc; ++kc) {
+          const int s = st_i;
+          if (!warp_wait(&bars->full[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
+          if (!warp_wait(&bars->wfull[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
+          if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
           tc_after();
-          const uint32_t d_tmem = tmem + (uint32_t)(b * 256);
-          for (int kc = 0; kc < nkc; ++kc) {
-            const int s = st_i;
-            if (!mbar_wait(&bars->full[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
-            if (!mbar_wait(&bars->wfull[s], st_ph, abort_flag, err, lim)) { ok = false; break; }
-            if (++st_i == NS) { st_i = 0; st_ph ^= 1u; }
-            tc_after();
-            const uint32_t a_hi = su32(smem + (size_t)s * P.stage_bytes);
-            const uint32_t a_lo = a_hi + (uint32_t)P.a_bytes;
-            const uint32_t bb = a_hi + (uint32_t)(2 * P.a_bytes);
-            const int ksteps = min(kKC, K8 - kc * kKC) / 8;
-            for (int st = 0; st < ksteps; ++st) {
-              const uint64_t dah = sdesc(a_hi + (uint32_t)st * 32u);
-              const uint64_t dal = sdesc(a_lo + (uint32_t)st * 32u);
-              const uint64_t db = sdesc(bb + (uint32_t)st * 32u);
-              mma_tf32(d_tmem, dah, db, id_wide, (kc > 0 || st > 0) ? 1u : 0u);
-              mma_tf32(d_tmem, dal, db, id_half, 1u);
-            }
+          const uint32_t da = desc_lo(su32(smem) + (uint32_t)s * (uint32_t)P.stage_bytes);
+          const uint32_t ab = (uint32_t)(P.a_bytes / 16);
+          if (elect_one()) {
+            mma_split_chunk(min(kKC, K8 - kc * kKC) / 8, d_tmem, da, da + ab, da + 2u * ab, id_wide, id_half,
+                            kc > 0 ? 1u : 0u);
             mma_commit(&bars->empty[s]);
           }
-          if (ok) mma_commit(&bars->accfull[b]);
+          __syncwarp();
         }
+        if (ok && elect_one()) mma_commit(&bars->accfull[b]);
+        __syncwarp();
       }
+    }
+    if (elect_one()) {
       mma_commit(&bars->drain);
       mbar_drain(&bars->drain, 0, err);
     }
