@@ -53,6 +53,11 @@ namespace um {
 constexpr int kThreads = 512;
 constexpr int kConv = 256;              // converter threads (warps 8..15)
 constexpr int kGroup = 128;             // converter threads of one chunk: two groups take turns
+// The Gram's groups of converters: four, one chunk in registers each, or as many as
+// there are stages (a group may wait for a stage's next release only, so two
+// groups never wait for the same stage).
+constexpr int kGramGroups = 4;
+constexpr int kGramThreads = 256 + kGramGroups * kGroup;
 constexpr int kM = 128;                 // accumulator rows = TMEM lanes
 constexpr int kKC = 32;                 // K values per staged chunk
 constexpr int kTmemCols = 512;          // two accumulators of 256 columns
@@ -711,7 +716,7 @@ struct GramBars {
   int abort_flag;
 };
 
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kGramThreads, 1)
 k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, int chimax, void* const* ptrs,
             const int* __restrict__ ival, int* err, unsigned long long lim) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -726,7 +731,7 @@ k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NS = P.stages;
 
-  for (int i = tid; i < n_items; i += kThreads) {
+  for (int i = tid; i < n_items; i += kGramThreads) {
     int F;
     unsigned O, Q4;
     gram_extent(items[i], ival, F, O, Q4);
@@ -741,7 +746,7 @@ k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, 
   }
   // zero the operand stages once: rows [F, F8) stay zero-filled by the
   // converters, everything else is rewritten before use
-  for (size_t e = tid; e < (size_t)NS * P.stage_bytes / 16; e += kThreads)
+  for (size_t e = tid; e < (size_t)NS * P.stage_bytes / 16; e += kGramThreads)
     reinterpret_cast<float4*>(Xs)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
   if (warp == 0) tmem_alloc(&bars->tmem);
   tc_before();
@@ -848,26 +853,29 @@ k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, 
     }
   } else if (warp >= 8) {
     // ------------------------------------------------------------ converters
-    // This thread copies quad kq of the rows r0 + 16 u of every other chunk of
+    // This thread copies quad kq of the rows r0 + 16 u of every fourth chunk of
     // the unit: the eight lanes of a row read 128 consecutive bytes (or eight
     // consecutive o), store one swizzled 128-byte row without bank conflicts.
+    // Bound: the latency of these loads.  A group requests its next chunk as soon
+    // as the one before is stored, so three or four chunks are on their way.
     const int ct = tid - 256, grp = ct / kGroup, t = ct % kGroup;
     const int kq = t & 7, r0 = t >> 3;
     constexpr int MU = kM / (kGroup / 8);             // row steps of 16
+    const unsigned G = (unsigned)min(kGramGroups, NS);
     unsigned n = 0;                                   // chunks of the CTA before this unit
     GramUnit g;
-    bool ok = true;
+    bool ok = (unsigned)grp < G;
     for (long long u = blockIdx.x; u < U && ok; u += gridDim.x) {
       gram_unit(g, u, uoff, n_items, items, ptrs, ival, splits_max);
-      unsigned c = g.c0 + ((n ^ (unsigned)grp) & 1u);  // this group's first chunk
+      unsigned c = g.c0 + ((unsigned)grp + G - n % G) % G;   // this group's first chunk
       unsigned nn = n + (c - g.c0);                    // its number in the CTA
       n += g.c1 - g.c0;
       unsigned qi = 8 * c + kq;
       const unsigned o = qi / g.Q4;
       unsigned q4 = qi - o * g.Q4;
       const float* src = g.X + (long long)o * g.FQ + 4ll * q4 + (long long)r0 * g.Q;
-      // the quad 16 further on: dO o's and dq quads
-      const unsigned dO = 16 / g.Q4, dq = 16 - dO * g.Q4;
+      // the same quad of the group's next chunk: dO o's and dq quads further on
+      const unsigned dO = 8 * G / g.Q4, dq = 8 * G - dO * g.Q4;
       const long long step = (long long)dO * g.FQ + 4ll * dq, wrap = g.FQ - g.Q, rows16 = 16 * g.Q;
       const unsigned Q4 = g.Q4, NQ = g.NQ, c1 = g.c1;
       const int F = g.F, F8 = g.F8;
@@ -880,7 +888,7 @@ k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, 
           if (live && r0 + 16 * i < F) v[i] = __ldg(reinterpret_cast<const float4*>(p));
           p += rows16;
         }
-        qi += 16;
+        qi += 8 * G;
         q4 += dq;
         src += step;
         if (q4 >= Q4) { q4 -= Q4; src += wrap; }
@@ -901,19 +909,14 @@ k_gram_umma(const GramLegItem* __restrict__ items, int n_items, int splits_max, 
         }
         fence_async_smem();
         warp_arrive(&bars->full[s]);
-        nn += 2;
+        nn += G;
         return true;
       };
-      float4 v0[MU], v1[MU];
-      if (c < c1) load(v0);
-      while (c < c1) {
-        if (c + 2 < c1) load(v1);
-        if (!convert(v0)) { ok = false; break; }
-        c += 2;
-        if (c >= c1) break;
-        if (c + 2 < c1) load(v0);
-        if (!convert(v1)) { ok = false; break; }
-        c += 2;
+      float4 v[MU];
+      if (c < c1) load(v);
+      for (; c < c1; c += G) {
+        if (!convert(v)) { ok = false; break; }
+        if (c + G < c1) load(v);
       }
     }
   }
@@ -1390,7 +1393,7 @@ cudaError_t launch_gram_umma(const GramLegItem* items, int n_items, int splits_m
   if (e != cudaSuccess) return e;
   for (int i0 = 0; i0 < n_items; i0 += um::kMaxItems) {
     const int n = std::min(um::kMaxItems, n_items - i0);
-    um::k_gram_umma<<<um::sm_count(), um::kThreads, P.total, s>>>(items + i0, n, splits_max, chimax, ptrs, ival,
+    um::k_gram_umma<<<um::sm_count(), um::kGramThreads, P.total, s>>>(items + i0, n, splits_max, chimax, ptrs, ival,
                                                                    err, wait_ns);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
