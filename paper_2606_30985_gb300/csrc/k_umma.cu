@@ -300,6 +300,12 @@ struct LegPlan {
   const double* A;
   unsigned R, Q;       // rows (o, q) of the item, values between two j
   int J, Jout, K8, N16, nkc, lda;
+  int kb, kr;          // K steps of 8 a chunk: kb, one more in the first kr chunks
+  // first K value of chunk kc.  The chunks are as even as their steps allow (J = 100: 32,
+  // 24, 24, 24 and not 32, 32, 32, 8): the loads of a group's next chunk hide
+  // behind the conversion of this one, and a chunk of 8 hides nothing.
+  __device__ __forceinline__ int k0(int kc) const { return 8 * (kb * kc + min(kc, kr)); }
+  __device__ __forceinline__ int steps(int kc) const { return kb + (kc < kr ? 1 : 0); }
 };
 
 __device__ inline unsigned leg_rows(const LegItem& it, const int* ival, unsigned& Q, int& J) {
@@ -323,6 +329,8 @@ __device__ __noinline__ void leg_plan(const LegItem* items, int i, void* const* 
   // N >= 16: a factor of rank 0 (a message that is not finite) still issues MMAs
   L.N16 = round_up(L.Jout > 0 ? L.Jout : 1, 16);
   L.nkc = (L.K8 + kKC - 1) / kKC;
+  L.kb = L.nkc > 0 ? L.K8 / 8 / L.nkc : 0;
+  L.kr = L.K8 / 8 - L.kb * L.nkc;
   L.in = static_cast<const float*>(ptrs[it.in.ref]);
   L.out = static_cast<float*>(ptrs[it.out_ref]);
   L.A = it.A;
@@ -439,7 +447,7 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
     bool ok = true;
     for (unsigned item_n = 0; ok && rg.next(toff, n_items); ++item_n) {
       leg_plan(items, rg.item, ptrs, ival, L);
-      const int N16 = L.N16, K8 = L.K8, nkc = L.nkc;
+      const int N16 = L.N16, nkc = L.nkc;
       const uint32_t bstep = (uint32_t)(2 * N16) * 8;    // B block per K chunk (16-byte units)
       const uint32_t id_wide = idesc_tf32(kM, 2 * N16), id_half = idesc_tf32(kM, N16);
       if (!warp_wait(&bars->bfull, item_n & 1u, abort_flag, err, lim)) break;
@@ -457,7 +465,7 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
           tc_after();
           const uint32_t da = desc_lo(su32(As) + (uint32_t)s * (uint32_t)P.stage_bytes);
           if (elect_one()) {
-            mma_split_chunk(min(kKC, K8 - kc * kKC) / 8, d_tmem, da, da + (uint32_t)(P.stage_bytes / 32), db, id_wide,
+            mma_split_chunk(L.steps(kc), d_tmem, da, da + (uint32_t)(P.stage_bytes / 32), db, id_wide,
                             id_half, kc > 0 ? 1u : 0u);
             mma_commit(&bars->empty[s]);
           }
@@ -541,7 +549,7 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
     bool ok = true;
     for (unsigned item_n = 0; ok && rg.next(toff, n_items); ++item_n) {
       leg_plan(items, rg.item, ptrs, ival, L);
-      const int nkc = L.nkc, J = L.J, K8 = L.K8;
+      const int nkc = L.nkc, J = L.J;
       const unsigned Q = L.Q;
       const unsigned total = rg.cnt * (unsigned)nkc;
       unsigned j = (n ^ (unsigned)grp) & 1u;           // this group's first chunk of the item
@@ -560,8 +568,9 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
         src = L.in + (long long)o * J * Q + (valid ? rr - o * Q : 0u);
       };
       auto load = [&](float4 (&v)[8]) {
-        const int m = valid ? J - kc * kKC : 0;        // values of this row in the chunk
-        const float* p = src + (long long)(kc * kKC) * Q;
+        const int k0 = L.k0(kc);
+        const int m = valid ? min(J - k0, 8 * L.steps(kc)) : 0;   // values of this row in the chunk
+        const float* p = src + (long long)k0 * Q;
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -584,7 +593,7 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
         if (!warp_wait(&bars->empty[s], ((nn / (unsigned)NS) & 1u) ^ 1u, abort_flag, err, lim)) return false;
         unsigned char* hi = As + (size_t)s * P.stage_bytes;
         unsigned char* lo = hi + P.stage_bytes / 2;
-        const int kw = K8 - ckc * kKC;                 // columns the MMAs of this chunk read
+        const int kw = 8 * L.steps(ckc);               // columns the MMAs of this chunk read
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           if (4 * u < kw) {
@@ -614,12 +623,13 @@ k_leg_umma(const LegItem* __restrict__ items, int n_items, int chimax, void* con
         const size_t bblk = (size_t)(2 * L.N16) * 128;
         const int K32 = nkc * kKC;
         for (int e = ct; e < L.N16 * K32; e += kConv) {
-          const int q = e / K32, k = e - q * K32;
+          const int q = e / K32, kk = e - q * K32;
+          const int kc = kk / kKC, k = L.k0(kc) + kk % kKC;
           float x = 0.f;
-          if (q < L.Jout && k < J) x = (float)L.A[(long long)q * L.lda + k];
+          if (q < L.Jout && k < J && kk % kKC < 8 * L.steps(kc)) x = (float)L.A[(long long)q * L.lda + k];
           const float h = tf32_hi(x);
-          unsigned char* blk = Bs + (size_t)(k / kKC) * bblk + (size_t)(k & 3) * 4;
-          const int piece = (k % kKC) >> 2;
+          unsigned char* blk = Bs + (size_t)kc * bblk + (size_t)(kk & 3) * 4;
+          const int piece = (kk % kKC) >> 2;
           *reinterpret_cast<float*>(blk + swz(q, piece)) = h;
           *reinterpret_cast<float*>(blk + swz(q + L.N16, piece)) = x - h;
         }
