@@ -1092,36 +1092,58 @@ __device__ __forceinline__ bool rot_params(float al, float be, float ga, float t
   nb = be + t * ga;
   return true;
 }
-// FP64: h in FP32, s from it by a reciprocal with two Newton steps.  A division or
-// a root in FP64 is ~20 operations of 16 clocks a warp here, and the textbook
-// form has five.
+// FP64: an operation of a warp holds its quarter of the FP64 unit for 64 clocks
+// (measured; independent ones are no faster), so what need not be FP64 is not.
+// The test and h come from the operands' leading 24 bits, scaled to the largest
+// (integer work); s = 2 h / (1 + h^2) follows from an FP32 reciprocal by one
+// cubic step, 2 h times it being exact; the norms' updates take tan theta in FP32
+// (they steer the next rotations and are recomputed every round).
+__device__ __forceinline__ float top_float(double x, int e) {   // x 2^(1023 - e), e >= its biased exponent
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int ex = (hi >> 20) & 0x7ff, f = ex - e + 127;
+  const int bits = (hi & 0x80000000) | (f << 23) | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29);
+  return ex == 0 || f <= 0 ? 0.f : __int_as_float(bits);
+}
+__device__ __forceinline__ double wide(float x) {               // (double)x of a normal number or zero
+  const int b = __float_as_int(x);
+  return (b & 0x7fffffff) == 0 ? 0.0
+                               : __hiloint2double((b & 0x80000000) | (((b & 0x7fffffff) >> 3) + (896 << 20)), b << 29);
+}
 __device__ __forceinline__ bool rot_params(double al, double be, double ga, double tol2, double negligible, double cut,
                                            double& h, double& s, double& na, double& nb) {
-  if (!(ga != 0.0 && al > negligible && be > negligible && fabs(ga) > cut && ga * ga > tol2 * (al * be))) return false;
-  const double d = be - al, g = 2.0 * ga;
-  const int e = max(__double2hiint(d) & 0x7ff00000, __double2hiint(g) & 0x7ff00000);
-  const double sc = __hiloint2double(max(0x7fe00000 - e, 0x00100000), 0);      // 2^-exponent
-  const float df = (float)(d * sc), gf = (float)(g * sc);
-  if (gf == 0.f) return false;                                                 // |zeta| > 1e38
-  const float z = df / gf, az = fabsf(z);
+  // al, be, |ga| and the bounds are not negative: their bits order like their values
+  const long long ia = __double_as_longlong(al), ib = __double_as_longlong(be);
+  const long long ig = __double_as_longlong(ga) & 0x7fffffffffffffffll;
+  const int e = (int)(max(max(ia, ib), ig) >> 52);
+  if (e >= 0x7ff || ig == 0 || min(ia, ib) <= __double_as_longlong(negligible) || ig <= __double_as_longlong(cut)) return false;
+  const float fa = top_float(al, e), fb = top_float(be, e), fg = top_float(ga, e);
+  const float rel = fabsf(fg) * rsqrtf(fa) * rsqrtf(fb);
+  if (!(rel * rel > (float)tol2)) return false;
+  const double d = be - al;
+  const float df = top_float(d, e), z = __fdividef(df, 2.f * fg), az = fabsf(z);
   const float t = copysignf(az > 1e8f ? 0.5f / az : 1.f / (az + sqrtf(fmaf(z, z, 1.f))), z);
-  h = (double)(t / (1.f + sqrtf(fmaf(t, t, 1.f))));
-  const double x = fma(h, h, 1.0);
-  double y = (double)__frcp_rn((float)x);
-  y = fma(y, fma(-x, y, 1.0), y);
-  y = fma(y, fma(-x, y, 1.0), y);
-  s = 2.0 * h * y;
-  const double c = fma(-s, h, 1.0);
-  const double cs = 2.0 * c * s * ga, cc = c * c, ss = s * s;
-  na = fma(cc, al, fma(ss, be, -cs));
-  nb = fma(ss, al, fma(cc, be, cs));
+  const float hf = t / (1.f + sqrtf(fmaf(t, t, 1.f)));
+  if (!(fabsf(hf) > 1e-30f)) return false;                      // beyond FP32's range: no rotation either
+  h = wide(hf);
+  const double y = wide(__frcp_rn(fmaf(hf, hf, 1.f)));
+  const double r = fma(-fma(h, h, 1.0), y, 1.0);
+  const double w = wide(2.f * hf) * y;
+  s = fma(w, fma(r, r, r), w);
+  const double tg = wide(t) * ga;
+  na = al - tg;
+  nb = be + tg;
   return true;
 }
-template <typename R>
-__device__ __forceinline__ void rot_apply(R& x, R& y, R h, R s) {
-  const R u = fma(h, x, y), v = fma(-h, y, x);
-  x = fma(-s, u, x);
-  y = fma(s, v, y);
+__device__ __forceinline__ void rot_apply(float& x, float& y, float h, float s) {
+  const float u = fmaf(h, x, y), v = fmaf(-h, y, x);
+  x = fmaf(-s, u, x);
+  y = fmaf(s, v, y);
+}
+// the same rotation as three shears: three FP64 operations a pair instead of four
+__device__ __forceinline__ void rot_apply(double& x, double& y, double h, double s) {
+  x = fma(-h, y, x);
+  y = fma(s, x, y);
+  x = fma(-h, y, x);
 }
 
 // One-sided Jacobi (Hestenes) on the columns of A (n x n, column-major),
@@ -1230,102 +1252,259 @@ __device__ int jacobi_block(R* A, int n, R* V, R* nrm, int max_sweeps, int* capp
                  : jacobi_block_l<R, 16>(A, n, V, nrm, max_sweeps, capped);
 }
 
-constexpr int kCoreThreads = 1024;
+constexpr int kCoreThreads = 512;                  // 128 registers: columns stay in them
 constexpr size_t kCoreSmem = (size_t)192 * 1024;
 constexpr int kCoreMaxDim = 512;                   // columns and rows of a core: rg * chi <= 512
 
-// One warp's FP32 rotation of the columns x and y (length m, shared memory) of A
-// and vx, vy (length nv) of V; nx, ny are their squared norms, kept up to date.
-// Returns whether it rotated.  The columns are held in registers between the dot
-// product and the rotation (shared-memory bandwidth bounds the pass), so each
-// is read and written once.
-__device__ bool jac_pair(float* x, float* y, int m, float* vx, float* vy, int nv, float* nx, float* ny, float tol2,
-                         float negligible, float cut) {
-  const int lane = threadIdx.x & 31;
-  constexpr int U = kCoreMaxDim / 32;
-  float a[U], b[U];
+// Column of up to 32 U values, 32 apart per lane (zeros past len).
+template <int U>
+__device__ __forceinline__ void col_load(float (&a)[U], const float* x, int len) {
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int i = (threadIdx.x & 31) + 32 * u;
+    a[u] = i < len ? x[i] : 0.f;
+  }
+}
+template <int U>
+__device__ __forceinline__ void col_store(const float (&a)[U], float* x, int len) {
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int i = (threadIdx.x & 31) + 32 * u;
+    if (i < len) x[i] = a[u];
+  }
+}
+template <int U>
+__device__ __forceinline__ float col_dot(const float (&a)[U], const float (&b)[U]) {
   float ga = 0;
 #pragma unroll
-  for (int u = 0; u < U; ++u) {
-    const int i = lane + 32 * u;
-    a[u] = b[u] = 0.f;
-    if (32 * u < m) {
-      if (i < m) { a[u] = x[i]; b[u] = y[i]; }
-      ga = fmaf(a[u], b[u], ga);
-    }
-  }
-  const float al = *nx, be = *ny;
+  for (int u = 0; u < U; ++u) ga = fmaf(a[u], b[u], ga);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
-  float h, s, na, nb;
-  if (!rot_params(al, be, ga, tol2, negligible, cut, h, s, na, nb)) return false;
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    const int i = lane + 32 * u;
-    if (i < m) {
-      rot_apply(a[u], b[u], h, s);
-      x[i] = a[u];
-      y[i] = b[u];
-    }
-  }
-  for (int i = lane; i < nv; i += 32) {
-    float p = vx[i], q = vy[i];
-    rot_apply(p, q, h, s);
-    vx[i] = p;
-    vy[i] = q;
-  }
-  __syncwarp();
-  if (lane == 0) { *nx = na; *ny = nb; }
-  return true;
+  return ga;
 }
 
-// The pairs of one inner round in FP64 (pair k: the columns pq[k].x, pq[k].y of buf,
-// per values each, m of A then nv of V), by the whole block: half a warp per dot
-// product, one lane per pair for the rotation, half a warp per rotated pair.  The
-// FP64 pipe bounds it: an operation that all lanes repeat costs as much as 32
-// useful ones, so the scalars of all pairs share a warp.
-struct JacRound {
-  int2 pq[64];
-  double ga[64], h[64], s[64];                             // s > 1.5: no rotation
-};
-__device__ int jac_round64(JacRound& R, int pairs, double* buf, int per, int m, int nv, double* nrm, double tol2,
-                           double negligible, double cut) {
-  const int l = threadIdx.x & 15, h = threadIdx.x >> 4, nh = blockDim.x >> 4;
-  const unsigned mask = 0xffffu << (threadIdx.x & 16);
-  int rot = 0;
-  for (int k = h; k < pairs; k += nh) {
-    const double* x = buf + R.pq[k].x * per;
-    const double* y = buf + R.pq[k].y * per;
-    double ga = 0.0;
-    for (int i = l; i < m; i += 16) ga = fma(x[i], y[i], ga);
+// One warp's FP32 rotation of the columns x and y (length m, shared memory) of A
+// and vx, vy (length nv) of V; nx, ny are their squared norms, kept up to date.
+// Returns whether it rotated.  m and nv are at most 32 U.
+template <int U>
+__device__ __noinline__ int jac_pair(float* x, float* y, int m, float* vx, float* vy, int nv, float* nx, float* ny,
+                                     float tol2, float negligible, float cut) {
+  float a[U], b[U];
+  col_load(a, x, m);
+  col_load(b, y, m);
+  float h, s, na, nb;
+  if (!rot_params(*nx, *ny, col_dot(a, b), tol2, negligible, cut, h, s, na, nb)) return 0;
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) ga += __shfl_xor_sync(mask, ga, o);
-    if (l == 0) R.ga[k] = ga;
+  for (int u = 0; u < U; ++u) rot_apply(a[u], b[u], h, s);
+  col_store(a, x, m);
+  col_store(b, y, m);
+  col_load(a, vx, nv);
+  col_load(b, vy, nv);
+#pragma unroll
+  for (int u = 0; u < U; ++u) rot_apply(a[u], b[u], h, s);
+  col_store(a, vx, nv);
+  col_store(b, vy, nv);
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) { *nx = na; *ny = nb; }
+  return 1;
+}
+
+// The cross pairs of two blocks of columns in shared memory (cp columns at slot
+// 0, then cq; per values each: m of A, nv of V): step k pairs column i of the first
+// with column (i + k) mod bs of the second.  Bound: the latency of a step (load,
+// product, rotation, store, barrier), then shared-memory bandwidth.  So a warp
+// keeps its column of the first block in registers over all steps and moves only
+// the other one.  Up to 256 rows it holds A's and V's; above that (up to 32
+// columns a block: two per warp) the rotations are kept and V follows in a
+// pass of its own.  hs: (h, s) of step k and column i at 32 k + i, s = 2: none.
+template <int U>
+__device__ __noinline__ int jac_cross(float* buf, int per, int m, int nv, int cp, int cq, int bs, float* nrm,
+                                      float tol2, float negligible, float cut, float2* hs) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  constexpr int NW = kCoreThreads / 32;
+  int rot = 0;
+  if constexpr (U <= 8) {                                   // 32 U >= n: bs <= 16 = NW
+    const int i = wid;
+    const bool on = i < cp;
+    float* xc = buf + i * per;
+    float x[U], vx[U], nx = 0.f;
+    if (on) {
+      col_load(x, xc, m);
+      col_load(vx, xc + m, nv);
+      nx = nrm[i];
+    }
+    int q = i;                                              // (i + k) mod bs
+    for (int k = 0; k < bs; ++k) {
+      if (on && q < cq) {
+        float* yc = buf + (cp + q) * per;
+        float* ny = nrm + cp + q;
+        float y[U], vy[U], h, s, na, nb;
+        col_load(y, yc, m);
+        col_load(vy, yc + m, nv);
+        if (rot_params(nx, *ny, col_dot(x, y), tol2, negligible, cut, h, s, na, nb)) {
+          rot = 1;
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            rot_apply(x[u], y[u], h, s);
+            rot_apply(vx[u], vy[u], h, s);
+          }
+          col_store(y, yc, m);
+          col_store(vy, yc + m, nv);
+          nx = na;
+          __syncwarp();
+          if (lane == 0) *ny = nb;
+        }
+      }
+      if (++q >= bs) q = 0;
+      __syncthreads();
+    }
+    if (on) {
+      col_store(x, xc, m);
+      col_store(vx, xc + m, nv);
+    }
+  } else {
+    float x[2][U], nx[2];
+    int q[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int i = wid + NW * c;
+      q[c] = i;
+      col_load(x[c], buf + i * per, i < cp ? m : 0);
+      nx[c] = i < cp ? nrm[i] : 0.f;
+    }
+    for (int k = 0; k < bs; ++k) {
+      float y[2][U], ga[2];
+#pragma unroll
+      for (int c = 0; c < 2; ++c) col_load(y[c], buf + (cp + q[c]) * per, wid + NW * c < cp && q[c] < cq ? m : 0);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) ga[c] = col_dot(x[c], y[c]);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int i = wid + NW * c;
+        if (i < cp && q[c] < cq) {
+          float* ny = nrm + cp + q[c];
+          float2 r;
+          float na, nb;
+          if (rot_params(nx[c], *ny, ga[c], tol2, negligible, cut, r.x, r.y, na, nb)) {
+            rot = 1;
+#pragma unroll
+            for (int u = 0; u < U; ++u) rot_apply(x[c][u], y[c][u], r.x, r.y);
+            col_store(y[c], buf + (cp + q[c]) * per, m);
+            nx[c] = na;
+            __syncwarp();
+            if (lane == 0) *ny = nb;
+          } else {
+            r.y = 2.f;
+          }
+          if (lane == 0) hs[32 * k + i] = r;
+        }
+        if (++q[c] >= bs) q[c] -= bs;
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int i = wid + NW * c;
+      if (i < cp) col_store(x[c], buf + i * per, m);
+      q[c] = i;
+      col_load(x[c], buf + i * per + m, i < cp ? nv : 0);
+    }
+    for (int k = 0; k < bs; ++k) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int i = wid + NW * c;
+        if (i < cp && q[c] < cq) {
+          const float2 r = hs[32 * k + i];
+          if (r.y < 1.5f) {
+            float y[U];
+            float* yc = buf + (cp + q[c]) * per + m;
+            col_load(y, yc, nv);
+#pragma unroll
+            for (int u = 0; u < U; ++u) rot_apply(x[c][u], y[u], r.x, r.y);
+            col_store(y, yc, nv);
+          }
+        }
+        if (++q[c] >= bs) q[c] -= bs;
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int i = wid + NW * c;
+      if (i < cp) col_store(x[c], buf + i * per + m, nv);
+    }
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < pairs; k += blockDim.x) {
-    double* nx = nrm + R.pq[k].x;
-    double* ny = nrm + R.pq[k].y;
+  return rot;
+}
+
+// The pairs f(0) .. f(cnt - 1) of one inner round in FP64 (the columns .x and .y of
+// buf, x < 0: none; per values each, m of A then nv of V), by the whole block: half
+// a warp per dot product (a warp above 64 rows), one lane per pair for the
+// rotation, a warp per 32 rows of a pair to rotate.  Bound: the FP64 units, one
+// warp operation per 64 clocks and quarter of the SM: an operation that all lanes
+// repeat costs as much as 32 useful ones, and the quarters share the work by
+// warps.
+struct JacRound {
+  double ga[64], h[64], s[64];                             // s > 1.5: no rotation
+};
+template <class F>
+__device__ __forceinline__ int jac_round64(JacRound& R, int cnt, F f, double* buf, int per, int m, int nv, double* nrm,
+                                           double tol2, double negligible, double cut) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int rot = 0;
+  if (m > 64) {
+    for (int k = wid; k < cnt; k += nw) {
+      const int2 v = f(k);
+      if (v.x < 0) continue;
+      const double* x = buf + v.x * per;
+      const double* y = buf + v.y * per;
+      double ga = 0.0;
+      for (int i = lane; i < m; i += 32) ga = fma(x[i], y[i], ga);
+      ga = warp_sum(ga);
+      if (lane == 0) R.ga[k] = ga;
+    }
+  } else {
+    const int l = threadIdx.x & 15;
+    const unsigned mask = 0xffffu << (threadIdx.x & 16);
+    for (int k = threadIdx.x >> 4; k < cnt; k += 2 * nw) {
+      const int2 v = f(k);
+      if (v.x < 0) continue;
+      const double* x = buf + v.x * per;
+      const double* y = buf + v.y * per;
+      double ga = 0.0;
+      for (int i = l; i < m; i += 16) ga = fma(x[i], y[i], ga);
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) ga += __shfl_xor_sync(mask, ga, o);
+      if (l == 0) R.ga[k] = ga;
+    }
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
+    const int2 v = f(k);
     double h = 0.0, s = 2.0, na, nb;
-    if (rot_params(*nx, *ny, R.ga[k], tol2, negligible, cut, h, s, na, nb)) {
-      *nx = na;
-      *ny = nb;
+    if (v.x >= 0 && rot_params(nrm[v.x], nrm[v.y], R.ga[k], tol2, negligible, cut, h, s, na, nb)) {
+      nrm[v.x] = na;
+      nrm[v.y] = nb;
       rot = 1;
     }
     R.h[k] = h;
     R.s[k] = s;
   }
   __syncthreads();
-  for (int k = h; k < pairs; k += nh) {
-    const double h = R.h[k], s = R.s[k];
+  const int segs = (m + nv + 31) >> 5;
+  for (int e = wid; e < cnt * segs; e += nw) {
+    const int k = e / segs, i = 32 * (e - k * segs) + lane;
+    const double s = R.s[k];
     if (s > 1.5) continue;
-    double* x = buf + R.pq[k].x * per;
-    double* y = buf + R.pq[k].y * per;
-    for (int i = l; i < m + nv; i += 16) {
-      double p = x[i], q = y[i];
-      rot_apply(p, q, h, s);
-      x[i] = p;
-      y[i] = q;
+    const int2 v = f(k);
+    if (i < m + nv) {
+      double* x = buf + v.x * per + i;
+      double* y = buf + v.y * per + i;
+      double p = *x, q = *y;
+      rot_apply(p, q, R.h[k], s);
+      *x = p;
+      *y = q;
     }
   }
   __syncthreads();
@@ -1354,7 +1533,7 @@ __device__ int jac_round64(JacRound& R, int pairs, double* buf, int per, int m, 
 // orthogonality.  Squared norms are recomputed every round and updated by the
 // rotations between.  flags: 3 ints, zeroed by the caller; cnorm: n doubles.
 template <typename R>
-__device__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* capped, double abs_rel, const Cta& ct,
+__device__ __noinline__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* capped, double abs_rel, const Cta& ct,
                               int* flags, double* cnorm, unsigned char* sh) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   __shared__ double fr[32];
@@ -1373,12 +1552,15 @@ __device__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* cap
   fro = block_sum(fro, fr);
   const double tol = (sizeof(R) == 4 ? 3e-7 : 1e-15) * sqrt((double)m);
   const R tol2 = (R)(tol * tol);
-  __shared__ JacRound jr;
-  __shared__ int jr_count;
+  __shared__ union {
+    JacRound jr;                                            // FP64
+    float2 hs[32 * 32];                                     // FP32
+  } rs;
   // columns below 1e-30 (FP64) or 1e-13 (FP32) of the total squared norm are
   // numerically zero in that precision
   const R negligible = (R)((sizeof(R) == 4 ? 1e-13 : 1e-30) * fro);
   const R abs_cut = (R)(abs_rel * fro);
+  const int longest = max(m, n);                            // of a column: registers per lane
   const int room = (int)((kCoreSmem - 4096) / sizeof(R));
   R* nrm = reinterpret_cast<R*>(sh);                        // squared norms of the columns at hand
   R* buf = reinterpret_cast<R*>(sh + 4096);
@@ -1394,30 +1576,51 @@ __device__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* cap
   // blocks P < Q of pair pi in a round
   auto blocks = [&](int round, int pi, int& P, int& Q) {
     if (pi == 0) { P = nblk - 1; Q = round; }
-    else { P = (round + pi) % (nblk - 1); Q = (round - pi + nblk - 1) % (nblk - 1); }
+    else {
+      P = round + pi; if (P >= nblk - 1) P -= nblk - 1;
+      Q = round - pi; if (Q < 0) Q += nblk - 1;
+    }
     if (P > Q) { const int t = P; P = Q; Q = t; }
   };
-  auto bring = [&](int c0, int cnt, int at) {               // columns c0.. to slots at..
-    for (int e = threadIdx.x; e < cnt * per; e += blockDim.x) {
-      const int c = e / per, i = e - c * per;
-      buf[(at + c) * per + i] = i < m ? A[(long long)(c0 + c) * m + i] : V[(long long)(c0 + c) * n + i - m];
-    }
+  auto col_sq = [&](const R* x) -> R {                      // squared norm of a column of A, by a warp
+    R q = 0;
+    for (int i = lane; i < m; i += 32) q = fma(x[i], x[i], q);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    return q;
   };
-  auto back = [&](int c0, int cnt, int at) {
-    for (int e = threadIdx.x; e < cnt * per; e += blockDim.x) {
-      const int c = e / per, i = e - c * per;
-      const R x = buf[(at + c) * per + i];
-      if (i < m) A[(long long)(c0 + c) * m + i] = x;
-      else V[(long long)(c0 + c) * n + i - m] = x;
+  // columns c0 .. of the first cnt0 slots and d0 .. of the next cnt1 between global and
+  // shared memory: a warp per column of A or V, eight values of a lane in flight; on the
+  // way in, also the squared norms
+  auto move = [&](bool in, int c0, int cnt0, int d0, int cnt1) {
+    for (int t = wid; t < 2 * (cnt0 + cnt1); t += nw) {
+      const int c = t >> 1;
+      const long long col = c < cnt0 ? c0 + c : d0 + c - cnt0;
+      R* g = (t & 1) ? V + col * n : A + col * m;
+      R* l = buf + c * per + ((t & 1) ? m : 0);
+      const int len = (t & 1) ? n : m;
+      const R* src = in ? g : l;
+      R* dst = in ? l : g;
+      for (int i0 = lane; i0 < len; i0 += 256) {
+        R v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (i0 + 32 * u < len) v[u] = src[i0 + 32 * u];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (i0 + 32 * u < len) dst[i0 + 32 * u] = v[u];
+      }
+      if (in && !(t & 1)) {
+        __syncwarp();
+        const R q = col_sq(l);
+        if (lane == 0) nrm[c] = q;
+      }
     }
+    __syncthreads();
   };
   auto norms = [&](int cnt) {
     for (int c = wid; c < cnt; c += nw) {
-      const R* x = buf + c * per;
-      R q = 0;
-      for (int i = lane; i < m; i += 32) q = fma(x[i], x[i], q);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+      const R q = col_sq(buf + c * per);
       if (lane == 0) nrm[c] = q;
     }
     __syncthreads();
@@ -1431,22 +1634,15 @@ __device__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* cap
         if (v.x < 0) continue;
         R* x = buf + v.x * per;
         R* y = buf + v.y * per;
-        rot |= jac_pair(x, y, m, x + m, y + m, n, nrm + v.x, nrm + v.y, tol2, negligible, abs_cut) ? 1 : 0;
+        R* nx = nrm + v.x;
+        R* ny = nrm + v.y;
+        if (longest <= 128) rot |= jac_pair<4>(x, y, m, x + m, y + m, n, nx, ny, tol2, negligible, abs_cut);
+        else if (longest <= 256) rot |= jac_pair<8>(x, y, m, x + m, y + m, n, nx, ny, tol2, negligible, abs_cut);
+        else rot |= jac_pair<16>(x, y, m, x + m, y + m, n, nx, ny, tol2, negligible, abs_cut);
       }
       __syncthreads();
     } else {
-      if (wid == 0) {                                      // list the round's pairs (at most 64 = n / 2)
-        int at = 0;
-        for (int k0 = 0; k0 < cnt; k0 += 32) {
-          const int2 v = k0 + lane < cnt ? f(k0 + lane) : make_int2(-1, -1);
-          const unsigned live = __ballot_sync(0xffffffffu, v.x >= 0);
-          if (v.x >= 0) jr.pq[at + __popc(live & ((1u << lane) - 1u))] = v;
-          at += __popc(live);
-        }
-        if (lane == 0) jr_count = at;
-      }
-      __syncthreads();
-      rot = jac_round64(jr, jr_count, buf, per, m, n, nrm, tol2, negligible, abs_cut);
+      rot = jac_round64(rs.jr, cnt, f, buf, per, m, n, nrm, tol2, negligible, abs_cut);
     }
     return rot;
   };
@@ -1454,24 +1650,24 @@ __device__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* cap
   auto inner = [&](bool all, int k, int i, int P, int Q, int p0, int q0) -> int2 {
     const int cp = count(P), cq = count(Q);
     if (!all) {                                             // column i of P with column (i + k) mod bs of Q
-      const int q = (i + k) % bs;
+      const int q = i + k < bs ? i + k : i + k - bs;
       return i < cp && q < cq ? make_int2(p0 + i, q0 + q) : make_int2(-1, -1);
     }
     const int cnt = cp + cq, np = cnt + (cnt & 1);          // tournament (a dummy if odd)
     if (k >= np - 1 || i >= np / 2) return make_int2(-1, -1);
     int x, y;
     if (i == 0) { x = np - 1; y = k; }
-    else { x = (k + i) % (np - 1); y = (k - i + np - 1) % (np - 1); }
+    else {
+      x = k + i; if (x >= np - 1) x -= np - 1;
+      y = k - i; if (y < 0) y += np - 1;
+    }
     if (x >= cnt || y >= cnt) return make_int2(-1, -1);
     if (x > y) { const int t = x; x = y; y = t; }
     return make_int2(x < cp ? p0 + x : q0 + x - cp, y < cp ? p0 + y : q0 + y - cp);
   };
   const int steps0 = 2 * bs - 1;                            // inner rounds of round 0; later: bs
   int sweep = 0;
-  if (resident && ct.rank == 0) {
-    bring(0, n, 0);
-    __syncthreads();
-  }
+  if (resident && ct.rank == 0) move(true, 0, n, 0, 0);
   for (; sweep < max_sweeps; ++sweep) {
     int* flag = flags + sweep % 3;
     if (ct.rank == 0 && threadIdx.x == 0) flags[(sweep + 1) % 3] = 0;
@@ -1496,15 +1692,19 @@ __device__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* cap
           blocks(round, pi, P, Q);
           const int cp = count(P), cq = count(Q);
           if (cp == 0 || (cq == 0 && !all)) continue;
-          bring(first(P), cp, 0);
-          bring(first(Q), cq, cp);
-          __syncthreads();
-          norms(cp + cq);
-          for (int k = 0; k < steps; ++k)
+          move(true, first(P), cp, first(Q), cq);
+          bool cross = false;
+          if constexpr (sizeof(R) == 4) {
+            cross = !all;
+            if (cross) {
+              if (longest <= 128) rot |= jac_cross<4>(buf, per, m, n, cp, cq, bs, nrm, tol2, negligible, abs_cut, rs.hs);
+              else if (longest <= 256) rot |= jac_cross<8>(buf, per, m, n, cp, cq, bs, nrm, tol2, negligible, abs_cut, rs.hs);
+              else rot |= jac_cross<16>(buf, per, m, n, cp, cq, bs, nrm, tol2, negligible, abs_cut, rs.hs);
+            }
+          }
+          for (int k = 0; !cross && k < steps; ++k)
             rot |= round_of(bs, [&](int i) { return inner(all, k, i, P, Q, 0, cp); });
-          back(first(P), cp, 0);
-          back(first(Q), cq, cp);
-          __syncthreads();
+          move(false, first(P), cp, first(Q), cq);
         }
         cta_sync(ct);
       }
@@ -1513,7 +1713,7 @@ __device__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* cap
     cta_sync(ct);
     if (*reinterpret_cast<volatile int*>(flag) == 0) break;
   }
-  if (resident && ct.rank == 0) back(0, n, 0);
+  if (resident && ct.rank == 0) move(false, 0, n, 0, 0);
   if (sweep >= max_sweeps && threadIdx.x == 0) *capped = 1;
   cta_sync(ct);
   return sweep;
@@ -1523,8 +1723,9 @@ __device__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* cap
 // and the FP64 Jacobi: 2 multiply-adds per clock and SM) and the shared-memory
 // bandwidth of the FP32 Jacobi, both spread over the cluster's SMs; one CTA
 // per bond left 150 of 152 SMs idle on a small grid and kept the Jacobi's
-// columns in L2.  Core class of a saturated layer, one CTA -> cluster: 3x3 chi = 100
-// 652 -> 101 ms, 4x4 chi = 64 197 -> 40 ms, 3x5 chi = 27 29.5 -> 13 ms.
+// columns in L2.  Core class of a saturated layer, one CTA -> cluster -> columns in
+// registers (512 threads): 3x3 chi = 100 652 -> 93 -> 80 ms, 4x4 chi = 64 197 -> 39 ->
+// 23 ms, 3x5 chi = 27 29.5 -> 13 -> 7.8 ms, 4x4 chi = 12 in FP64 30 -> 7.3 -> 3.9 ms.
 __global__ void __launch_bounds__(kCoreThreads, 1)
 k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize) {
   const CoreItem it = items[blockIdx.x / csize];
