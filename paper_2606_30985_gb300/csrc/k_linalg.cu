@@ -1146,26 +1146,50 @@ __device__ __forceinline__ void rot_apply(double& x, double& y, double h, double
   x = fma(-h, y, x);
 }
 
-// One-sided Jacobi (Hestenes) on the columns of A (n x n, column-major),
-// accumulating V (n x n, column-major), by one block.  Returns the sweep count;
-// sets *capped when the sweep budget ran out.
+// Pair pi of a round of the tournament of n columns (np = n rounded up to even);
+// x < 0: the one with the dummy.
+__device__ __forceinline__ int2 tournament(int round, int pi, int n, int np) {
+  int a, b;
+  if (pi == 0) { a = np - 1; b = round; }
+  else {
+    a = round + pi; if (a >= np - 1) a -= np - 1;
+    b = round - pi; if (b < 0) b += np - 1;
+  }
+  if (a >= n || b >= n) return make_int2(-1, -1);
+  return a < b ? make_int2(a, b) : make_int2(b, a);
+}
+
+// One-sided Jacobi (Hestenes) on the columns of A (n x n, column-major, leading
+// dimension ld), accumulating V (the same), by one block.  Returns the
+// sweep count; sets *capped when the sweep budget ran out.
 //
-// A pair of columns belongs to L lanes (32 up to n = 64, 16 above, so that the
-// n / 2 <= 64 pairs of a tournament round run at once on 1024 threads), which
-// hold both columns in registers from the dot product to the rotation; the
-// squared norms are recomputed every sweep and updated by the rotations
-// between, so a pair costs one reduction.  Bound: shared-memory bandwidth (8
-// column passes a rotation) and the latency of one round at small n.
-template <typename R, int L>
-__device__ int jacobi_block_l(R* A, int n, R* V, R* nrm, int max_sweeps, int* capped) {
-  constexpr int E = L == 32 ? 2 : 8;                        // column values per lane: n <= 64, n <= 128
+// A pair of columns belongs to L lanes that hold E values of both in registers
+// from the dot product to the rotation (V's too, requested before the product is
+// summed, where the registers hold them: up to four values a lane); the squared norms are recomputed every sweep and updated by the
+// rotations between, so a pair costs one reduction.  Bound: the instructions of
+// a round (the scalars of a rotation are ~80 and repeat per warp, so a warp takes
+// 32 / L pairs) and its latency, then shared-memory bandwidth.  ld is L more
+// than a multiple of 32, so that the L-lane groups of a warp, whose columns are
+// neighbours, read different banks.  FP64 goes this way up to n = 16 (the pairs'
+// warps then have a quarter of the FP64 unit each; one barrier a round).
+__host__ __device__ inline int jac_lanes(int n) { return n <= 32 ? 8 : 16; }
+__host__ __device__ inline int jac_ld(int n) {
+  const int L = jac_lanes(n);
+  return n <= L ? L : (n - L + 31) / 32 * 32 + L;
+}
+template <typename R, int L, int E>
+__device__ int jacobi_block_l(R* A, int n, int ld, R* V, R* nrm, int max_sweeps, int* capped) {
   const int l = threadIdx.x % L, grp = threadIdx.x / L, ng = blockDim.x / L;
-  const unsigned mask = L == 32 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) V[e] = (e % (n + 1) == 0) ? R(1) : R(0);
+  const unsigned mask = (L == 16 ? 0xffffu : 0xffu) << (threadIdx.x & 31 & ~(L - 1));
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) V[e / n * ld + e % n] = e % (n + 1) == 0 ? R(1) : R(0);
   auto norms = [&]() {
     for (int c = grp; c < n; c += ng) {
       R q = 0;
-      for (int i = l; i < n; i += L) q = fma(A[c * n + i], A[c * n + i], q);
+#pragma unroll
+      for (int u = 0; u < E; ++u) {
+        const int i = l + L * u;
+        if (i < n) q = fma(A[c * ld + i], A[c * ld + i], q);
+      }
 #pragma unroll
       for (int o = L / 2; o > 0; o >>= 1) q += __shfl_xor_sync(mask, q, o);
       if (l == 0) nrm[c] = q;
@@ -1181,11 +1205,10 @@ __device__ int jacobi_block_l(R* A, int n, R* V, R* nrm, int max_sweeps, int* ca
   for (int o = 16; o > 0; o >>= 1) fro += __shfl_xor_sync(0xffffffffu, fro, o);
   __syncthreads();
   const int np = (n % 2) ? n + 1 : n;   // players incl. a dummy
-  // orthogonality target: above the rounding noise of a length-n dot product
-  // in the working precision (FP32 columns: ~sqrt(n) 6e-8 relative); columns
-  // below 1e-30 (FP64) or 1e-13 (FP32) of the total squared norm are
-  // numerically zero in that precision: rotating them only stirs rounding
-  // noise and never converges
+  // orthogonality target: above the rounding noise of a length-n dot product in
+  // the working precision (FP32 columns: ~sqrt(n) 6e-8 relative); columns below
+  // 1e-30 (FP64) or 1e-13 (FP32) of the total squared norm are numerically zero:
+  // rotating them only stirs rounding noise and never converges
   const double tol = (sizeof(R) == 4 ? 3e-7 : 1e-15) * sqrt((double)n);
   const R tol2 = (R)(tol * tol);
   const R negligible = (R)(sizeof(R) == 4 ? 1e-13 : 1e-30) * fro;
@@ -1195,47 +1218,47 @@ __device__ int jacobi_block_l(R* A, int n, R* V, R* nrm, int max_sweeps, int* ca
     int rotated = 0;
     for (int round = 0; round < np - 1; ++round) {
       for (int pi = grp; pi < np / 2; pi += ng) {
-        int a, b;
-        if (pi == 0) { a = np - 1; b = round; }
-        else {
-          a = round + pi; if (a >= np - 1) a -= np - 1;
-          b = round - pi; if (b < 0) b += np - 1;
-        }
-        if (a >= n || b >= n) continue;
-        const int p = a < b ? a : b, q = a < b ? b : a;
-        R* Ap = A + p * n;
-        R* Aq = A + q * n;
-        R x[E], y[E], ga = 0;
+        const int2 pq = tournament(round, pi, n, np);
+        if (pq.x < 0) continue;
+        R* Ap = A + pq.x * ld + l;
+        R* Aq = A + pq.y * ld + l;
+        R* Vp = V + pq.x * ld + l;
+        R* Vq = V + pq.y * ld + l;
+        R x[E], y[E], vx[E], vy[E], ga = 0;
 #pragma unroll
         for (int u = 0; u < E; ++u) {
-          const int i = l + L * u;
-          x[u] = i < n ? Ap[i] : R(0);
-          y[u] = i < n ? Aq[i] : R(0);
-          ga = fma(x[u], y[u], ga);
+          const bool in = l + L * u < n;
+          x[u] = in ? Ap[L * u] : R(0);
+          y[u] = in ? Aq[L * u] : R(0);
+          if (E <= 4) {
+            vx[u] = in ? Vp[L * u] : R(0);
+            vy[u] = in ? Vq[L * u] : R(0);
+          }
         }
-        const R al = nrm[p], be = nrm[q];
+        const R al = nrm[pq.x], be = nrm[pq.y];
+#pragma unroll
+        for (int u = 0; u < E; ++u) ga = fma(x[u], y[u], ga);
 #pragma unroll
         for (int o = L / 2; o > 0; o >>= 1) ga += __shfl_xor_sync(mask, ga, o);
         R h, s, na, nb;
         if (rot_params(al, be, ga, tol2, negligible, R(0), h, s, na, nb)) {
           rotated = 1;
-          R* Vp = V + p * n;
-          R* Vq = V + q * n;
 #pragma unroll
           for (int u = 0; u < E; ++u) {
-            const int i = l + L * u;
-            if (i < n) {
+            if (l + L * u < n) {
+              if (E > 4) {
+                vx[u] = Vp[L * u];
+                vy[u] = Vq[L * u];
+              }
               rot_apply(x[u], y[u], h, s);
-              Ap[i] = x[u];
-              Aq[i] = y[u];
-              R vx = Vp[i], vy = Vq[i];
-              rot_apply(vx, vy, h, s);
-              Vp[i] = vx;
-              Vq[i] = vy;
+              rot_apply(vx[u], vy[u], h, s);
+              Ap[L * u] = x[u];
+              Aq[L * u] = y[u];
+              Vp[L * u] = vx[u];
+              Vq[L * u] = vy[u];
             }
           }
-          __syncwarp(mask);
-          if (l == 0) { nrm[p] = na; nrm[q] = nb; }
+          if (l == 0) { nrm[pq.x] = na; nrm[pq.y] = nb; }
         }
       }
       __syncthreads();
@@ -1245,11 +1268,6 @@ __device__ int jacobi_block_l(R* A, int n, R* V, R* nrm, int max_sweeps, int* ca
   if (sweep >= max_sweeps && threadIdx.x == 0) *capped = 1;
   __syncthreads();
   return sweep;
-}
-template <typename R>
-__device__ int jacobi_block(R* A, int n, R* V, R* nrm, int max_sweeps, int* capped) {
-  return n <= 64 ? jacobi_block_l<R, 32>(A, n, V, nrm, max_sweeps, capped)
-                 : jacobi_block_l<R, 16>(A, n, V, nrm, max_sweeps, capped);
 }
 
 constexpr int kCoreThreads = 512;                  // 128 registers: columns stay in them
@@ -1511,6 +1529,42 @@ __device__ __forceinline__ int jac_round64(JacRound& R, int cnt, F f, double* bu
   return rot;
 }
 
+// The same in FP64, in rounds of jac_round64.  buf: columns of 2 n values, A's then V's
+// (A filled in by the caller).
+__device__ int jacobi_block64(double* buf, int n, double* nrm, int max_sweeps, int* capped, JacRound& R) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int per = 2 * n, np = n + (n & 1);
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) buf[e / n * per + n + e % n] = e % (n + 1) == 0 ? 1.0 : 0.0;
+  auto norms = [&]() {
+    for (int c = wid; c < n; c += nw) {
+      double q = 0.0;
+      for (int i = lane; i < n; i += 32) q = fma(buf[c * per + i], buf[c * per + i], q);
+      q = warp_sum(q);
+      if (lane == 0) nrm[c] = q;
+    }
+    __syncthreads();
+  };
+  norms();
+  if (n < 2) return 0;
+  double fro = 0.0;
+  for (int c = lane; c < n; c += 32) fro += nrm[c];
+  fro = warp_sum(fro);
+  __syncthreads();
+  const double tol = 1e-15 * sqrt((double)n), negligible = 1e-30 * fro;
+  int sweep = 0;
+  for (; sweep < max_sweeps; ++sweep) {
+    if (sweep > 0) norms();
+    int rotated = 0;
+    for (int round = 0; round < np - 1; ++round)
+      rotated |= jac_round64(R, np / 2, [&](int pi) { return tournament(round, pi, n, np); }, buf, per, n, n, nrm,
+                             tol * tol, negligible, 0.0);
+    if (!__syncthreads_or(rotated)) break;
+  }
+  if (sweep >= max_sweeps && threadIdx.x == 0) *capped = 1;
+  __syncthreads();
+  return sweep;
+}
+
 // One-sided Jacobi of A (m x n, column-major, leading dimension m, global
 // memory) with the rotations accumulated in V (n x n), on all CTAs of the
 // cluster.  The columns are cut into (at most) 16 blocks; a round of the block
@@ -1525,7 +1579,7 @@ __device__ __forceinline__ int jac_round64(JacRound& R, int cnt, F f, double* bu
 // The order of the rotations of a column depends on n alone, so every cluster
 // size gives the same bits.
 //
-// Rotation and stopping rules as jacobi_block, plus abs_rel > 0: a pair whose
+// Rotation and stopping rules as jacobi_block_l, plus abs_rel > 0: a pair whose
 // coupling |a_p . a_q| is below abs_rel ||A||_F^2 is skipped too.  Such a pair
 // moves no singular value by more than that, and without the cut the columns of
 // tiny singular values (mostly rounding noise from rotations with the large
@@ -2181,33 +2235,51 @@ __device__ void scaled_rotation(const EnvEigItem& it, int n) {
 // the item's workspace.
 constexpr size_t kEigSmem = (size_t)220 * 1024;
 template <typename R>
-__global__ void __launch_bounds__(1024)
+__host__ __device__ inline size_t eig_smem(int chimax) {   // norms, A and V
+  return sizeof(R) == 4 ? sizeof(float) * (128 + 2 * (size_t)chimax * jac_ld(chimax))
+                        : sizeof(double) * (128 + 2 * (size_t)chimax * chimax);
+}
+template <typename R>
+__global__ void __launch_bounds__(sizeof(R) == 4 ? 1024 : 512)
 k_env_eig(const EnvEigItem* __restrict__ items, const int* ival, int chimax) {
   const EnvEigItem it = items[blockIdx.x];
   const int n = ival[it.chi_idx];
   extern __shared__ __align__(16) unsigned char eig_sh[];
-  __shared__ double red[32];
+  __shared__ double red[32], sq[128];
   __shared__ int capped;
   if (threadIdx.x == 0) capped = 0;
   R* nrm = reinterpret_cast<R*>(eig_sh);                   // 128 values
-  const bool in = sizeof(R) * (2 * (size_t)chimax * chimax + 128) <= kEigSmem;
-  R* A = in ? nrm + 128 : reinterpret_cast<R*>(it.work);   // n x n column-major
-  R* V = A + n * n;
+  R* A = eig_smem<R>(chimax) <= kEigSmem ? nrm + 128 : reinterpret_cast<R*>(it.work);
+  int ld;
+  R* V;
+  if constexpr (sizeof(R) == 4) { ld = jac_ld(n); V = A + n * ld; }
+  else { ld = 2 * n; V = A + n; }
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
     const int i = e / n, j = e - i * n;
-    A[j * n + i] = (R)(0.5 * (it.M[i * it.ld + j] + it.M[j * it.ld + i]));
+    A[j * ld + i] = (R)(0.5 * (it.M[i * it.ld + j] + it.M[j * it.ld + i]));
   }
   __syncthreads();
-  jacobi_block<R>(A, n, V, nrm, 60, &capped);
+  if constexpr (sizeof(R) == 4) {
+    if (n <= 32) jacobi_block_l<float, 8, 4>(A, n, ld, V, nrm, 60, &capped);
+    else if (n <= 64) jacobi_block_l<float, 16, 4>(A, n, ld, V, nrm, 60, &capped);
+    else jacobi_block_l<float, 16, 8>(A, n, ld, V, nrm, 60, &capped);
+  } else {
+    __shared__ JacRound jr;
+    if (n <= 8) jacobi_block_l<double, 8, 1>(A, n, ld, V, nrm, 60, &capped);
+    else if (n <= 16) jacobi_block_l<double, 16, 1>(A, n, ld, V, nrm, 60, &capped);
+    else jacobi_block64(A, n, nrm, 60, &capped, jr);
+  }
   for (int j = threadIdx.x >> 5; j < n; j += (int)(blockDim.x >> 5)) {
     double s = 0.0;
-    for (int i = threadIdx.x & 31; i < n; i += 32) s = fma((double)A[j * n + i], (double)A[j * n + i], s);
+    for (int i = threadIdx.x & 31; i < n; i += 32) s = fma((double)A[j * ld + i], (double)A[j * ld + i], s);
     s = warp_sum(s);
-    if ((threadIdx.x & 31) == 0) it.sqrtD[j] = sqrt(sqrt(s));   // sqrt of the eigenvalue |lambda_j| = ||A v_j||
+    if ((threadIdx.x & 31) == 0) sq[j] = s;
   }
+  __syncthreads();
+  for (int j = threadIdx.x; j < n; j += blockDim.x) it.sqrtD[j] = sqrt(sqrt(sq[j]));   // of |lambda_j| = ||A v_j||
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
     const int i = e / n, j = e - i * n;
-    it.Vt[i * it.ld + j] = (double)V[i * n + j];           // row i of Vt = column i of V
+    it.Vt[i * it.ld + j] = (double)V[i * ld + j];          // row i of Vt = column i of V
   }
   floor_sqrt_eigs(it.sqrtD, n, red);
   scaled_rotation(it, n);
@@ -2215,13 +2287,14 @@ k_env_eig(const EnvEigItem* __restrict__ items, const int* ival, int chimax) {
 
 template <typename R>
 static cudaError_t launch_eig(const EnvEigItem* items, int n_items, int chimax, const int* ival, cudaStream_t s) {
-  const size_t want = sizeof(R) * (2 * (size_t)chimax * chimax + 128);
+  const size_t want = eig_smem<R>(chimax);
   const size_t smem = want <= kEigSmem ? want : sizeof(R) * 128;
   cudaError_t e = cudaFuncSetAttribute(k_env_eig<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  // a warp per pair of columns up to chi = 64, half a warp above
+  // FP32: every pair of a round its lanes; FP64: a warp per pair of columns
   const int pairs = (chimax + 1) / 2;
-  const int threads = chimax <= 64 ? std::max(64, 32 * pairs) : 16 * ((pairs + 1) & ~1);
+  const int threads = sizeof(R) == 4 ? std::max(64, (jac_lanes(chimax) * pairs + 31) / 32 * 32)
+                                     : std::min(512, std::max(128, 32 * pairs));
   k_env_eig<R><<<n_items, threads, smem, s>>>(items, ival, chimax);
   return cudaGetLastError();
 }
