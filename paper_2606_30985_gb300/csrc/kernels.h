@@ -33,8 +33,8 @@ cudaError_t launch_permute(const void* in, void* out, int nlegs, const int* dims
 cudaError_t launch_gram_leg_reduce(const GramLegItem* items, int n_items, int chimax,
                                    int splits_max, int rows, int sym, const int* ival, cudaStream_t s);
 template <typename T>
-cudaError_t launch_reconstruct(const ReconItem* items, int n_items, int grid_x, int ntile_max,
-                               void* const* ptrs, const int* ival, cudaStream_t s);
+cudaError_t launch_reconstruct(const ReconItem* items, int n_items, int chimax, void* const* ptrs, const int* ival,
+                               cudaStream_t s);
 template <typename T>
 cudaError_t launch_vec_contract(const VecItem* items, int n_items, void* const* ptrs, const int* ival, cudaStream_t s);
 template <typename T>

@@ -1400,18 +1400,13 @@ template <typename T>
 pepo_status run_gate_wave_tail(pepo_ctx* c, Inst& I, GateWave& w) {
   cudaStream_t s = c->stream;
   const int chimax = I.cfg.chi_max;
-  const int nmax = 4 * chimax;
   {
-    long long rows = (long long)pow_sz(chimax, 3);
-    int gx = (int)std::min<long long>(std::max<long long>(1, (rows + 63) / 64 * ceil_div(nmax, 64)),
-                                      (long long)(2 * 152 * 4 / std::max(1, w.recon.n) + 1));
-    gx = std::max(gx, 4);
     if (use_umma<T>(c, chimax))
       LAUNCH_T(K_RECON, hitems(c, w.recon), w.recon.n,
                launch_recon_umma(w.recon.d, w.recon.n, chimax, c->d_ptrs, c->d_ival, c->d_kerr, c->wait_ns, s));
     else
       LAUNCH_T(K_RECON, hitems(c, w.recon), w.recon.n,
-               launch_reconstruct<T>(w.recon.d, w.recon.n, gx, 0, c->d_ptrs, c->d_ival, s));
+               launch_reconstruct<T>(w.recon.d, w.recon.n, chimax, c->d_ptrs, c->d_ival, s));
   }
   LAUNCH_N(w.npairs, launch_commit(w.pairs.d, w.npairs, w.moves.d, w.nmoves, c->d_ptrs, c->d_ival, s));
   return PEPO_OK;
