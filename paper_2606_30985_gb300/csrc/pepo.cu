@@ -210,9 +210,13 @@ struct pepo_ctx {
   // concatenated into one launch (plan fields of grp only; grp.cfg.chi_max =
   // the context-wide chi_max)
   Inst grp;
-  int* d_active = nullptr;                 // per-instance BP activity mask
-  // CUDA graphs of one Trotter step, one BP sweep and one single-layer sweep
-  // (captured on a private stream at first use, launched on `stream`)
+  // Convergence loop (one block, uploaded and read back whole): last delta (bits) and
+  // tolerance per instance, then head (sweeps done, kernel error word), activity
+  // mask, sweeps and sweep limit per instance.
+  char* d_loop = nullptr;
+  int* d_active = nullptr;                 // the mask inside d_loop
+  // CUDA graphs of one Trotter step and of the BP and single-layer convergence
+  // loops (captured on a private stream at first use, launched on `stream`)
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t step_exec = nullptr, bp_exec = nullptr, sl_exec = nullptr;
   long long step_launches = 0, bp_launches = 0, sl_launches = 0;
@@ -225,6 +229,8 @@ struct pepo_ctx {
 };
 
 namespace {
+
+size_t loop_bytes(int n) { return 16 * (size_t)n + 4 * (2 + 3 * (size_t)n); }
 
 const char* kStaticErr = "no context";
 
@@ -1151,7 +1157,8 @@ size_t layout_arena(pepo_ctx* c, char* base, Planner* keep) {
   c->d_kerr = cv.take<int>(1);
   c->d_qr_count = cv.take<unsigned long long>(3);
   c->d_hh_acct = cv.take<double>(2);
-  c->d_active = cv.take<int>(c->n_inst);
+  c->d_loop = cv.take<char>(loop_bytes(c->n_inst));
+  c->d_active = reinterpret_cast<int*>(c->d_loop + 16 * (size_t)c->n_inst) + 2;
   c->d_items = cv.take<char>(P.st.bytes.size() + 256);
   // warm-start workspace: one network and one feature / prediction buffer
   // sized for the largest instance (instances are handled one after another)
@@ -1546,52 +1553,154 @@ pepo_status bp_sweep_launches(pepo_ctx* c) {
   return PEPO_OK;
 }
 
-template <typename T>
-pepo_status do_bp(pepo_ctx* c, int* sweeps_out, double* delta_out) {
+// The end of one sweep of a convergence loop on the device: an instance leaves the
+// mask when its delta is below its tolerance or its sweeps are used up; the loop ends
+// with the last instance or with a kernel error.
+__global__ void k_sweep_end(cudaGraphConditionalHandle handle, char* loop, int n, const unsigned long long* delta,
+                            const int* kerr) {
+  unsigned long long* last = reinterpret_cast<unsigned long long*>(loop);
+  const double* tol = reinterpret_cast<const double*>(loop + 8 * (size_t)n);
+  int* head = reinterpret_cast<int*>(loop + 16 * (size_t)n);
+  int* active = head + 2;
+  int* sweeps = active + n;
+  const int* limit = sweeps + n;
+  const int sw = head[0] + 1;
+  int any = 0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    if (!active[i]) continue;
+    sweeps[i] = sw;
+    last[i] = delta[i];
+    const bool done = __longlong_as_double((long long)delta[i]) < tol[i] || sw >= limit[i];
+    active[i] = done ? 0 : 1;
+    any |= done ? 0 : 1;
+  }
+  any = __syncthreads_or(any);
+  if (threadIdx.x == 0) {
+    head[0] = sw;
+    head[1] = *kerr;
+    cudaGraphSetConditional(handle, any && *kerr == 0 ? 1u : 0u);
+  }
+}
+
+// Capture the loop over `sweep` (launches on c->stream) into a graph whose body
+// repeats on the device while k_sweep_end says so; false when that is not possible.
+template <class F>
+bool capture_loop(pepo_ctx* c, cudaGraphExec_t* exec, long long* nlaunch, const unsigned long long* d_delta, F sweep) {
+  if (c->graphs_failed || c->cap_stream == nullptr) return false;
+  cudaGraph_t g = nullptr, captured = nullptr;
+  cudaGraphConditionalHandle h;
+  cudaGraphNodeParams p = {};
+  cudaGraphNode_t node;
+  bool ok = cudaGraphCreate(&g, 0) == cudaSuccess &&
+            cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault) == cudaSuccess;
+  if (ok) {
+    p.type = cudaGraphNodeTypeConditional;
+    p.conditional.handle = h;
+    p.conditional.type = cudaGraphCondTypeWhile;
+    p.conditional.size = 1;
+    ok = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &p) == cudaSuccess &&
+         cudaStreamBeginCaptureToGraph(c->cap_stream, p.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                       cudaStreamCaptureModeRelaxed) == cudaSuccess;
+  }
+  if (ok) {
+    cudaStream_t user = c->stream;
+    c->stream = c->cap_stream;
+    const long long l0 = c->launches;
+    ok = sweep() == PEPO_OK;
+    k_sweep_end<<<1, 256, 0, c->stream>>>(h, c->d_loop, c->n_inst, d_delta, c->d_kerr);
+    ok = cudaGetLastError() == cudaSuccess && ok;
+    c->stream = user;
+    ok = cudaStreamEndCapture(c->cap_stream, &captured) == cudaSuccess && ok;
+    *nlaunch = c->launches - l0;                           // of a sweep, as the host loop counts them
+    c->launches = l0;
+  }
+  ok = ok && cudaGraphInstantiate(exec, g, 0) == cudaSuccess;
+  if (g) cudaGraphDestroy(g);
+  if (!ok) {
+    *exec = nullptr;
+    c->graphs_failed = true;
+    cudaGetLastError();
+  }
+  return ok;
+}
+
+// Sweeps until every instance has converged or used up its sweeps.  The loop runs
+// on the device: with the host in it (mask upload, graph launch, two readbacks and
+// a synchronisation) the GPU idled ~40 us a sweep, of the ~200 us a sweep of a
+// small instance takes.  The host's loop serves timing mode and a failed capture.
+template <class F>
+pepo_status converge(pepo_ctx* c, cudaGraphExec_t* exec, long long* per_sweep, const unsigned long long* d_delta,
+                     const char* what, std::vector<int>& sweeps, std::vector<double>& delta, F sweep) {
   cudaStream_t s = c->stream;
-  std::vector<int> done(c->n_inst, 0), sweeps(c->n_inst, 0), active(c->n_inst, 1);
-  std::vector<double> delta(c->n_inst, INFINITY);
-  std::vector<unsigned long long> hd(c->n_inst);
+  const size_t n = c->n_inst;
+  std::vector<char> block(loop_bytes(c->n_inst));
+  unsigned long long* last = reinterpret_cast<unsigned long long*>(block.data());
+  double* tol = reinterpret_cast<double*>(block.data() + 8 * n);
+  int* head = reinterpret_cast<int*>(block.data() + 16 * n);
+  int *active = head + 2, *swept = active + n, *limit = swept + n;
+  head[0] = head[1] = 0;
   int maxs = 0;
-  for (auto& I : c->inst) maxs = std::max(maxs, I.cfg.bp_max_sweeps);
+  for (size_t i = 0; i < n; ++i) {
+    const auto& cfg = c->inst[i].cfg;
+    last[i] = 0x7ff0000000000000ull;                       // infinity
+    tol[i] = cfg.bp_tol;
+    limit[i] = cfg.bp_max_sweeps;
+    active[i] = limit[i] > 0 ? 1 : 0;
+    swept[i] = 0;
+    maxs = std::max(maxs, limit[i]);
+  }
+  auto result = [&] {
+    for (size_t i = 0; i < n; ++i) {
+      sweeps[i] = swept[i];
+      delta[i] = bits_to_double(last[i]);
+    }
+    return PEPO_OK;
+  };
+  if (maxs <= 0) return result();
+  if (cudaMemcpyAsync(c->d_loop, block.data(), block.size(), cudaMemcpyHostToDevice, s) != cudaSuccess)
+    return fail(c, PEPO_E_CUDA, "%s loop upload", what);
+  if (!c->timing && (*exec || capture_loop(c, exec, per_sweep, d_delta, sweep))) {
+    if (cudaGraphLaunch(*exec, s) != cudaSuccess)
+      return fail(c, PEPO_E_CUDA, "%s graph launch: %s", what, cudaGetErrorString(cudaGetLastError()));
+    if (cudaMemcpyAsync(block.data(), c->d_loop, block.size(), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+      return fail(c, PEPO_E_CUDA, "%s loop readback: %s", what, cudaGetErrorString(cudaGetLastError()));
+    c->launches += head[0] * *per_sweep;
+    if (head[1]) return kernel_error(c, head[1]);
+    return result();
+  }
+  std::vector<unsigned long long> hd(n);
   for (int sw = 1; sw <= maxs; ++sw) {
+    pepo_status st = sweep();
+    if (st != PEPO_OK) return st;
+    int kerr = 0;
+    if (cudaMemcpyAsync(hd.data(), d_delta, sizeof(unsigned long long) * n, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaMemcpyAsync(&kerr, c->d_kerr, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+      return fail(c, PEPO_E_CUDA, "%s delta readback: %s", what, cudaGetErrorString(cudaGetLastError()));
+    if (kerr) return kernel_error(c, kerr);
     bool any = false;
-    for (int i = 0; i < c->n_inst; ++i) {
-      active[i] = (!done[i] && sw <= c->inst[i].cfg.bp_max_sweeps) ? 1 : 0;
+    for (size_t i = 0; i < n; ++i) {
+      if (!active[i]) continue;
+      swept[i] = sw;
+      last[i] = hd[i];
+      if (bits_to_double(hd[i]) < tol[i] || sw == limit[i]) active[i] = 0;
       any = any || active[i];
     }
     if (!any) break;
-    if (cudaMemcpyAsync(c->d_active, active.data(), sizeof(int) * c->n_inst, cudaMemcpyHostToDevice, s) != cudaSuccess)
+    if (cudaMemcpyAsync(c->d_active, active, sizeof(int) * n, cudaMemcpyHostToDevice, s) != cudaSuccess)
       return fail(c, PEPO_E_CUDA, "active mask upload");
-    bool launched = false;
-    if (!c->timing) {
-      if (!c->bp_exec) capture_graph(c, &c->bp_exec, &c->bp_launches, [&] { return bp_sweep_launches<T>(c); });
-      if (c->bp_exec) {
-        if (cudaGraphLaunch(c->bp_exec, s) != cudaSuccess)
-          return fail(c, PEPO_E_CUDA, "BP graph launch: %s", cudaGetErrorString(cudaGetLastError()));
-        c->launches += c->bp_launches;
-        launched = true;
-      }
-    }
-    if (!launched) {
-      pepo_status st = bp_sweep_launches<T>(c);
-      if (st != PEPO_OK) return st;
-    }
-    int kerr = 0;
-    if (cudaMemcpyAsync(hd.data(), c->d_delta2, sizeof(unsigned long long) * c->n_inst,
-                        cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaMemcpyAsync(&kerr, c->d_kerr, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-      return fail(c, PEPO_E_CUDA, "BP delta readback: %s", cudaGetErrorString(cudaGetLastError()));
-    if (kerr) return kernel_error(c, kerr);
-    for (int i = 0; i < c->n_inst; ++i) {
-      if (!active[i]) continue;
-      Inst& I = c->inst[i];
-      sweeps[i] = sw;
-      delta[i] = bits_to_double(hd[i]);
-      if (delta[i] < I.cfg.bp_tol || sw == I.cfg.bp_max_sweeps) done[i] = 1;
-    }
   }
+  return result();
+}
+
+template <typename T>
+pepo_status do_bp(pepo_ctx* c, int* sweeps_out, double* delta_out) {
+  std::vector<int> sweeps(c->n_inst, 0);
+  std::vector<double> delta(c->n_inst, INFINITY);
+  pepo_status st = converge(c, &c->bp_exec, &c->bp_launches, c->d_delta2, "BP", sweeps, delta,
+                            [&] { return bp_sweep_launches<T>(c); });
+  if (st != PEPO_OK) return st;
   for (int i = 0; i < c->n_inst; ++i) {
     c->inst[i].last_sweeps = sweeps[i];
     c->inst[i].last_delta = delta[i];
@@ -1618,48 +1727,12 @@ pepo_status do_correlator(pepo_ctx* c, double* C_out, pepo_diag* diag_out) {
   cudaStream_t s = c->stream;
   Inst& G = c->grp;
   LAUNCH_N(G.msgs.n, launch_sl_init(G.msgs.d, G.msgs.n, c->d_ival, s));
-  std::vector<int> done(c->n_inst, 0), sweeps(c->n_inst, 0), active(c->n_inst, 1);
+  std::vector<int> sweeps(c->n_inst, 0);
   std::vector<double> delta(c->n_inst, INFINITY);
-  std::vector<unsigned long long> hd(c->n_inst);
-  int maxs = 0;
-  for (auto& I : c->inst) maxs = std::max(maxs, I.cfg.bp_max_sweeps);
-  for (int sw = 1; sw <= maxs; ++sw) {
-    bool any = false;
-    for (int i = 0; i < c->n_inst; ++i) {
-      active[i] = (!done[i] && sw <= c->inst[i].cfg.bp_max_sweeps) ? 1 : 0;
-      any = any || active[i];
-    }
-    if (!any) break;
-    if (cudaMemcpyAsync(c->d_active, active.data(), sizeof(int) * c->n_inst, cudaMemcpyHostToDevice, s) != cudaSuccess)
-      return fail(c, PEPO_E_CUDA, "active mask upload");
-    bool launched = false;
-    if (!c->timing) {
-      if (!c->sl_exec) capture_graph(c, &c->sl_exec, &c->sl_launches, [&] { return sl_sweep_launches<T>(c); });
-      if (c->sl_exec) {
-        if (cudaGraphLaunch(c->sl_exec, s) != cudaSuccess)
-          return fail(c, PEPO_E_CUDA, "single-layer graph launch: %s", cudaGetErrorString(cudaGetLastError()));
-        c->launches += c->sl_launches;
-        launched = true;
-      }
-    }
-    if (!launched) {
-      pepo_status st = sl_sweep_launches<T>(c);
-      if (st != PEPO_OK) return st;
-    }
-    int kerr = 0;
-    if (cudaMemcpyAsync(hd.data(), c->d_delta1, sizeof(unsigned long long) * c->n_inst,
-                        cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaMemcpyAsync(&kerr, c->d_kerr, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-      return fail(c, PEPO_E_CUDA, "single-layer delta readback");
-    if (kerr) return kernel_error(c, kerr);
-    for (int i = 0; i < c->n_inst; ++i) {
-      if (!active[i]) continue;
-      Inst& I = c->inst[i];
-      sweeps[i] = sw;
-      delta[i] = bits_to_double(hd[i]);
-      if (delta[i] < I.cfg.bp_tol || sw == I.cfg.bp_max_sweeps) done[i] = 1;
-    }
+  {
+    pepo_status st = converge(c, &c->sl_exec, &c->sl_launches, c->d_delta1, "single-layer", sweeps, delta,
+                              [&] { return sl_sweep_launches<T>(c); });
+    if (st != PEPO_OK) return st;
   }
   // final estimates from the converged messages, then the Bethe sums
   {
