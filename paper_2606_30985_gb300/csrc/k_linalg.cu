@@ -37,6 +37,20 @@ __device__ inline double warp_sum(double v) {
 // of the warps' partials) are formed by one warp and read from shared memory, and
 // magnitudes are compared as integers.
 
+// x 2^(1023 - e), e >= x's biased exponent, cut to 24 bits; (double)x of a normal
+// number or zero: by integer operations
+__device__ __forceinline__ float top_float(double x, int e) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int ex = (hi >> 20) & 0x7ff, f = ex - e + 127;
+  const int bits = (hi & 0x80000000) | (f << 23) | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29);
+  return ex == 0 || f <= 0 ? 0.f : __int_as_float(bits);
+}
+__device__ __forceinline__ double wide(float x) {
+  const int b = __float_as_int(x);
+  return (b & 0x7fffffff) == 0 ? 0.0
+                               : __hiloint2double((b & 0x80000000) | (((b & 0x7fffffff) >> 3) + (896 << 20)), b << 29);
+}
+
 // Block-wide sum; `red` must hold 32 doubles.  All threads return it.
 __device__ inline double block_sum(double v, double* red) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -195,11 +209,12 @@ cudaError_t launch_branch(const SiteFacItem* items, int n_items, int* ival, cuda
 }
 
 // ========================================================== Householder TSQR
-// Leaf rows L = max(4n, 256).  Level 0 factors each leaf in place; level l >= 1
+// FP64 storage (FP32 storage factors the exact Gram of its data, k_gram_exact).
+// Leaf rows L = max(4n, 128).  Level 0 factors each leaf in place; level l >= 1
 // gathers the R-blocks of four level-(l-1) blocks into the first one and
 // factors the stack.  R replaces the top rows of the block; entries below the
 // diagonal are zeroed (Q is never needed: the update is Q-less).
-__host__ __device__ inline long long hh_leaf_rows(int n) { return n * 4 > 256 ? (long long)n * 4 : 256; }
+__host__ __device__ inline long long hh_leaf_rows(int n) { return n * 4 > kHhLeafRows ? (long long)n * 4 : kHhLeafRows; }
 constexpr int kHhThreads = 512;   // threads of a TSQR block
 
 // Panel width of the blocked QR: the panel (L x NB) lives in shared memory.
@@ -208,28 +223,25 @@ constexpr int kHhPanel = 8;
 // Shared-memory plan of one TSQR block (leaf rows L): panel V (column-major,
 // leading dimension L + 1 so that consecutive rows of a column and the rows
 // of consecutive columns fall in different banks), per-warp partial products
-// of the trailing update, W = V^T A and W2 = T^T W, V^T V and the T factor of
-// the compact WY form, tau, a block-reduction scratch.
+// of the trailing update, W = V^T A and W2 = T^T W, V^T V, and per reflection
+// tau and the scale of its vector.
 struct HhSmem {
-  size_t p, red, wd, w2, vtv, tm, tau, bred, total;
+  size_t p, red, wd, w2, vtv, tau, inv, total;
   int lp;
 };
-template <typename T>
 __host__ __device__ inline HhSmem hh_smem(long long L) {
   constexpr int NB = kHhPanel;
   HhSmem m;
   m.lp = (int)L + 1;
   size_t o = 0;
-  m.p = o;    o += sizeof(T) * (size_t)NB * m.lp;
+  m.p = o;    o += sizeof(double) * (size_t)NB * m.lp;
   o = (o + 15) & ~(size_t)15;
-  m.red = o;  o += sizeof(T) * (size_t)(kHhThreads / 32) * NB * 32;
+  m.red = o;  o += sizeof(double) * (size_t)(kHhThreads / 32) * NB * 32;
   m.wd = o;   o += sizeof(double) * (size_t)NB * 32;
-  m.w2 = o;   o += sizeof(T) * (size_t)NB * 32;
-  o = (o + 15) & ~(size_t)15;
+  m.w2 = o;   o += sizeof(double) * (size_t)NB * 32;
   m.vtv = o;  o += sizeof(double) * (size_t)NB * NB;
-  m.tm = o;   o += sizeof(double) * (size_t)NB * NB;
   m.tau = o;  o += sizeof(double) * (size_t)NB;
-  m.bred = o; o += sizeof(double) * 32;
+  m.inv = o;  o += sizeof(double) * (size_t)NB;
   m.total = o;
   return m;
 }
@@ -243,207 +255,260 @@ __device__ inline void st4(double* p, const double (&x)[4]) {
   reinterpret_cast<double2*>(p)[1] = make_double2(x[2], x[3]);
 }
 
+// The reflection that takes a column with diagonal alpha and squared norm s (diagonal
+// included) to beta e_1: v = (1, inv x), H = 1 - tau v v^T.  1 / sqrt(s) and the
+// reciprocal come from FP32 seeds by one cubic step each (a library root and two
+// quotients take ~25 FP64 operations, this takes 11); tau = 1 - alpha / beta needs
+// no quotient.
+__device__ inline void reflector(double alpha, double s, double& beta, double& tau, double& inv) {
+  beta = alpha;
+  tau = 0.0;
+  inv = 1.0;
+  if (!(s > 0.0)) return;
+  const int es = (__double2hiint(s) >> 20) & 0x7ff;
+  if (es < 2 || es >= 0x7ff) {                              // subnormal, infinite or NaN
+    const double norm = sqrt(s);
+    beta = alpha >= 0.0 ? -norm : norm;
+    inv = 1.0 / (alpha - beta);
+    tau = (beta - alpha) / beta;
+    return;
+  }
+  const int k = (es - 1023) >> 1;                           // s = m 4^k, m in [1, 4)
+  const double m = __hiloint2double(__double2hiint(s) - k * (1 << 21), __double2loint(s));
+  const double y0 = wide(rsqrtf(top_float(m, 1024) * 2.f));
+  const double e = fma(-m * y0, y0, 1.0);
+  const double y = fma(y0 * e, fma(0.375, e, 0.5), y0);     // 1 / sqrt(m)
+  const double nm = m * y;
+  const double norm = __hiloint2double(__double2hiint(nm) + k * (1 << 20), __double2loint(nm));
+  const double a = fabs(alpha);
+  tau = fma(__hiloint2double(__double2hiint(y) - k * (1 << 20), __double2loint(y)), a, 1.0);
+  beta = alpha >= 0.0 ? -norm : norm;
+  const double d = a + norm;                                // |alpha - beta| in [norm, 2 norm]
+  const int ed = (__double2hiint(d) >> 20) & 0x7ff;
+  double z = wide(__frcp_rn(top_float(d, ed)));             // 2^(ed - 1023) / d
+  z = __hiloint2double(__double2hiint(z) - (ed - 1023) * (1 << 20), __double2loint(z));
+  const double r = fma(-d, z, 1.0);
+  z = fma(fma(r, r, r), z, z);
+  inv = alpha >= 0.0 ? z : -z;
+}
+
+// Halving exchange: sums the 2 H values of v over the lanes that differ in bit `bit`;
+// the lane with the bit clear keeps the first H sums, the other the last H (H
+// additions; summing every value on every lane takes 2 H).
+template <int H, int N>
+__device__ __forceinline__ void halve(double (&v)[N], int bit) {
+  const bool up = (threadIdx.x & bit) != 0;
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const double send = up ? v[i] : v[i + H], keep = up ? v[i + H] : v[i];
+    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+  }
+}
+
+// One pass of the trailing update over columns cb .. cb + 4 NQ - 1 (those below c0
+// stay): A <- A - V W2, W2 = T^T (V^T A).  Lanes: NQ column quads x 32 / NQ row groups.
+template <int NQ>
+__device__ __forceinline__ void hh_trailing(double* A, int n, int j0, int pr, int nb, int cb, int c0, const double* P,
+                                            int lp, double* red, double* Wd, double* W2, const double* VtV,
+                                            const double* tau) {
+  constexpr int NB = kHhPanel;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NW = kHhThreads / 32;
+  const int kq = tid % NQ, rgi = tid / NQ;
+  constexpr int nrg = kHhThreads / NQ;
+  const int cq = cb + 4 * kq;
+  const bool colok = cq < n;
+  double v[NB * 4];
+#pragma unroll
+  for (int q = 0; q < NB * 4; ++q) v[q] = 0.0;
+  if (colok) {
+    for (int i = rgi; i < pr; i += nrg) {
+      double a[4];
+      ld4(A + (long long)(j0 + i) * n + cq, a);
+#pragma unroll
+      for (int l = 0; l < NB; ++l) {
+        const double x = P[l * lp + i];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[l * 4 + q] = fma(x, a[q], v[l * 4 + q]);
+      }
+    }
+  }
+  // rows of a warp: each lane ends up with the sums of its share of the 32 values
+  halve<16>(v, 16);
+  int first = lane & 16 ? 16 : 0;
+  halve<8>(v, 8);
+  first += lane & 8 ? 8 : 0;
+  constexpr int KEEP = NQ;                                  // 32 / (32 / NQ)
+  if constexpr (NQ <= 4) { halve<4>(v, 4); first += lane & 4 ? 4 : 0; }
+  if constexpr (NQ <= 2) { halve<2>(v, 2); first += lane & 2 ? 2 : 0; }
+#pragma unroll
+  for (int i = 0; i < KEEP; ++i) {
+    const int l = (first + i) >> 2, q = (first + i) & 3;
+    red[(warp * NB + l) * 32 + 4 * kq + q] = v[i];
+  }
+  __syncthreads();
+  for (int e = tid; e < NB * 4 * NQ; e += kHhThreads) {
+    const int l = e / (4 * NQ), k = e % (4 * NQ);
+    double z = 0.0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) z += red[(w * NB + l) * 32 + k];
+    Wd[l * 32 + k] = z;
+  }
+  __syncthreads();
+  // T^T W by forward substitution: T^-T is V^T V's lower triangle with 1 / tau on the
+  // diagonal
+  if (tid < 4 * NQ) {
+    double w[NB];
+#pragma unroll
+    for (int l = 0; l < NB; ++l) {
+      double z = Wd[l * 32 + tid];
+#pragma unroll
+      for (int mm = 0; mm < l; ++mm) z = fma(-VtV[mm * NB + l], w[mm], z);
+      w[l] = l < nb ? z * tau[l] : 0.0;
+      W2[l * 32 + tid] = cb + tid < c0 ? 0.0 : w[l];
+    }
+  }
+  __syncthreads();
+  if (colok) {
+    double w2[NB][4];
+#pragma unroll
+    for (int l = 0; l < NB; ++l)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) w2[l][q] = W2[l * 32 + 4 * kq + q];
+    for (int i = rgi; i < pr; i += nrg) {
+      double* pa = A + (long long)(j0 + i) * n + cq;
+      double a[4];
+      ld4(pa, a);
+#pragma unroll
+      for (int l = 0; l < NB; ++l) {
+        const double x = P[l * lp + i];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] = fma(-x, w2[l][q], a[q]);
+      }
+      if (cq < c0) {
+        // quad straddling the panel: keep the panel's columns untouched
+        double o[4];
+        ld4(pa, o);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (cq + q < c0) a[q] = o[q];
+      }
+      st4(pa, a);
+    }
+  }
+  __syncthreads();
+}
+
 // Householder QR of one TSQR block A (rows x n, row-major, n % 4 == 0, base
 // 16-byte aligned) in place: R in the top rows, zeros below (Q is not kept).
 // Blocked by panels of NB columns in the compact WY form H_1 ... H_nb =
 // I - V T V^T: the panel is factored in shared memory, then the trailing
 // columns take all nb reflections in one pass, A <- A - V (T^T (V^T A)),
-// instead of one pass per reflection.  512 threads.  FP64 storage only: FP32
-// storage factors the exact Gram of its data instead (k_gram_exact).
-template <typename T>
-__device__ void hh_block_qr(T* A, long long rows, int n, unsigned char* smem, const HhSmem& S) {
+// instead of one pass per reflection.  512 threads.
+//
+// Bound: the FP64 units, a quarter of the SM each, one warp operation per 64
+// clocks: what counts is the operations of the busiest quarter.  So the warp of
+// a panel's next column reflects it, sums its squares and forms its reflection
+// in one go, alone on its quarter, while the other columns' warps share the rest
+// (one barrier a column); trailing sums are exchanged by halves; the last
+// columns take as many lanes as they fill.  Class: 4x4 chi = 12 layer 5.5 -> 3.4 ms, 3x3 chi = 8 evolution
+// 5.5 -> 3.4.
+__device__ void hh_block_qr(double* A, long long rows, int n, unsigned char* smem, const HhSmem& S) {
   constexpr int NB = kHhPanel;
-  T* P = reinterpret_cast<T*>(smem + S.p);
-  T* red = reinterpret_cast<T*>(smem + S.red);
+  double* P = reinterpret_cast<double*>(smem + S.p);
+  double* red = reinterpret_cast<double*>(smem + S.red);
   double* Wd = reinterpret_cast<double*>(smem + S.wd);
-  T* W2 = reinterpret_cast<T*>(smem + S.w2);
+  double* W2 = reinterpret_cast<double*>(smem + S.w2);
   double* VtV = reinterpret_cast<double*>(smem + S.vtv);
-  double* Tm = reinterpret_cast<double*>(smem + S.tm);
   double* tau = reinterpret_cast<double*>(smem + S.tau);
-  double* bred = reinterpret_cast<double*>(smem + S.bred);
+  double* inv = reinterpret_cast<double*>(smem + S.inv);
   const int lp = S.lp;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nwarp = blockDim.x >> 5;
+  constexpr int NW = kHhThreads / 32;
   const int kmax = (int)(rows < n ? rows : n);
+  // column jj of the panel: its reflection from its rows jj .. pr - 1, by a warp
+  auto reflect = [&](int jj, int pr) {
+    double* col = P + jj * lp;
+    double s = 0.0;
+    for (int i = jj + lane; i < pr; i += 32) s = fma(col[i], col[i], s);
+    s = warp_sum(s);
+    double beta, t, z;
+    reflector(col[jj], s, beta, t, z);
+    __syncwarp();
+    if (lane == 0) {
+      col[jj] = beta;
+      tau[jj] = t;
+      inv[jj] = z;
+    }
+  };
   for (int j0 = 0; j0 < kmax; j0 += NB) {
     const int nb = kmax - j0 < NB ? kmax - j0 : NB;
     const int pr = (int)(rows - j0);
     // ---- panel rows j0.., columns j0..j0+nb-1 (zero columns beyond nb)
-    for (int e = tid; e < pr * NB; e += blockDim.x) {
+    for (int e = tid; e < pr * NB; e += kHhThreads) {
       const int i = e / NB, l = e - i * NB;
-      P[l * lp + i] = (l < nb) ? A[(long long)(j0 + i) * n + j0 + l] : T(0);
+      P[l * lp + i] = (l < nb) ? A[(long long)(j0 + i) * n + j0 + l] : 0.0;
     }
     __syncthreads();
-    // ---- unblocked Householder on the panel
-    for (int jj = 0; jj < nb; ++jj) {
-      T* col = P + jj * lp;
-      double s = 0.0;
-      for (int i = jj + tid; i < pr; i += blockDim.x) {
-        const double x = (double)col[i];
-        s = fma(x, x, s);
-      }
-      s = block_sum(s, bred);
-      if (tid == 0) {
-        const double alpha = (double)col[jj], normx = sqrt(s);
-        double beta = alpha, tj = 0.0, inv = 1.0;
-        if (normx > 0.0) {
-          beta = alpha >= 0.0 ? -normx : normx;
-          inv = 1.0 / (alpha - beta);
-          tj = (beta - alpha) / beta;
-        }
-        col[jj] = (T)beta;
-        tau[jj] = tj;
-        bred[1] = inv;
-      }
-      __syncthreads();
-      const double tj = tau[jj];
-      if (tj != 0.0) {
-        const double inv = bred[1];
-        for (int i = jj + 1 + tid; i < pr; i += blockDim.x) col[i] = (T)((double)col[i] * inv);
-      }
-      __syncthreads();
-      // the reflection on the panel's later columns, one warp per column
-      if (tj != 0.0) {
-        for (int c = jj + 1 + warp; c < nb; c += nwarp) {
-          T* pc = P + c * lp;
-          T acc = T(0);
-          for (int i = jj + 1 + lane; i < pr; i += 32) acc += col[i] * pc[i];
-          const double w = tj * (warp_sum((double)acc) + (double)pc[jj]);
+    if (warp == 0) reflect(0, pr);
+    __syncthreads();
+    // ---- unblocked Householder on the panel, its vectors unscaled: x = v / inv
+    // below the diagonal.  Column jj + 1 belongs to warp 0, the others to the
+    // warps of the other quarters.
+    for (int jj = 0; jj + 1 < nb; ++jj) {
+      const int c = warp == 0 ? jj + 1 : (warp & 3) == 0 ? nb : jj + 1 + warp - (warp >> 2);
+      if (c < nb) {
+        const double* col = P + jj * lp;
+        double* pc = P + c * lp;
+        const double t = tau[jj], z = inv[jj];
+        if (t != 0.0) {
+          double acc = 0.0;
+          for (int i = jj + 1 + lane; i < pr; i += 32) acc = fma(col[i], pc[i], acc);
+          acc = warp_sum(acc);
+          const double w = t * fma(z, acc, pc[jj]), wz = w * z;
           __syncwarp();
-          if (lane == 0) pc[jj] = (T)((double)pc[jj] - w);
-          const T wt = (T)w;
-          for (int i = jj + 1 + lane; i < pr; i += 32) pc[i] -= col[i] * wt;
+          if (lane == 0) pc[jj] -= w;
+          for (int i = jj + 1 + lane; i < pr; i += 32) pc[i] = fma(-wz, col[i], pc[i]);
+          __syncwarp();
         }
+        if (c == jj + 1) reflect(c, pr);
       }
       __syncthreads();
     }
-    // ---- R of the panel and zeros below it back to A; then V explicit in P
-    // (unit diagonal, zeros above) for the WY products
-    for (int e = tid; e < pr * nb; e += blockDim.x) {
-      const int i = e / nb, l = e - i * nb;
-      A[(long long)(j0 + i) * n + j0 + l] = (i <= l) ? P[l * lp + i] : T(0);
-    }
-    __syncthreads();
-    for (int e = tid; e < NB * NB; e += blockDim.x) {
-      const int l = e / NB, i = e - l * NB;
-      if (l < nb && i <= l && i < pr) P[l * lp + i] = (i == l) ? T(1) : T(0);
+    // ---- R of the panel and zeros below it back to A; V explicit in P (scaled,
+    // unit diagonal, zeros above) for the WY products
+    for (int e = tid; e < pr * NB; e += kHhThreads) {
+      const int i = e / NB, l = e - i * NB;
+      if (l < nb) {
+        const double x = P[l * lp + i];
+        A[(long long)(j0 + i) * n + j0 + l] = (i <= l) ? x : 0.0;
+        P[l * lp + i] = i < l ? 0.0 : i == l ? 1.0 : x * inv[l];
+      }
     }
     __syncthreads();
     const int c0 = j0 + nb;
     if (c0 >= n) continue;
-    // ---- T factor: T[0:j, j] = -tau_j T[0:j, 0:j] (V[:, 0:j]^T v_j)
-    for (int q = warp; q < NB * NB; q += nwarp) {
+    // ---- V^T V above the diagonal
+    for (int q = warp; q < NB * NB; q += NW) {
       const int l = q / NB, j = q - l * NB;
       if (l >= j || j >= nb) continue;
-      const T* vl = P + l * lp;
-      const T* vj = P + j * lp;
+      const double* vl = P + l * lp;
+      const double* vj = P + j * lp;
       double acc = 0.0;
-      for (int i = j + lane; i < pr; i += 32) acc = fma((double)vl[i], (double)vj[i], acc);
+      for (int i = j + lane; i < pr; i += 32) acc = fma(vl[i], vj[i], acc);
       acc = warp_sum(acc);
       if (lane == 0) VtV[l * NB + j] = acc;
     }
+    if (tid < NB * NB && (tid % NB >= nb || tid / NB >= tid % NB)) VtV[tid] = 0.0;
     __syncthreads();
-    if (tid == 0) {
-      for (int j = 0; j < NB; ++j) {
-        for (int l = 0; l < NB; ++l) Tm[l * NB + j] = 0.0;
-        if (j >= nb) continue;
-        Tm[j * NB + j] = tau[j];
-        for (int l = 0; l < j; ++l) {
-          double z = 0.0;
-          for (int m = l; m < j; ++m) z += Tm[l * NB + m] * VtV[m * NB + j];
-          Tm[l * NB + j] = -tau[j] * z;
-        }
-      }
-    }
-    __syncthreads();
-    // ---- trailing columns in blocks of 32: 8 column quads x 64 row groups
-    const int cs = c0 & ~3;
-    const int kq = tid & 7, rgi = tid >> 3, nrg = blockDim.x >> 3;
-    for (int cb = cs; cb < n; cb += 32) {
-      const int cq = cb + 4 * kq;
-      const bool colok = cq < n;
-      T acc[NB][4];
-#pragma unroll
-      for (int l = 0; l < NB; ++l)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[l][q] = T(0);
-      if (colok) {
-        for (int i = rgi; i < pr; i += nrg) {
-          T a[4];
-          ld4(A + (long long)(j0 + i) * n + cq, a);
-#pragma unroll
-          for (int l = 0; l < NB; ++l) {
-            const T v = P[l * lp + i];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[l][q] += v * a[q];
-          }
-        }
-      }
-      // sum over the four row groups of a warp, then over the warps
-#pragma unroll
-      for (int l = 0; l < NB; ++l)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          T x = acc[l][q];
-          x += __shfl_xor_sync(0xffffffffu, x, 8);
-          x += __shfl_xor_sync(0xffffffffu, x, 16);
-          acc[l][q] = x;
-        }
-      if (lane < 8) {
-#pragma unroll
-        for (int l = 0; l < NB; ++l)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) red[(warp * NB + l) * 32 + 4 * kq + q] = acc[l][q];
-      }
-      __syncthreads();
-      for (int e = tid; e < NB * 32; e += blockDim.x) {
-        const int l = e >> 5, k = e & 31;
-        double z = 0.0;
-        for (int w = 0; w < nwarp; ++w) z += (double)red[(w * NB + l) * 32 + k];
-        Wd[e] = z;
-      }
-      __syncthreads();
-      for (int e = tid; e < NB * 32; e += blockDim.x) {
-        const int l = e >> 5, k = e & 31;
-        double z = 0.0;
-        for (int m = 0; m <= l; ++m) z += Tm[m * NB + l] * Wd[m * 32 + k];
-        // the panel's own columns (below c0, in the first block) stay as written
-        W2[e] = (cb + k < c0) ? T(0) : (T)z;
-      }
-      __syncthreads();
-      if (colok) {
-        T w2[NB][4];
-#pragma unroll
-        for (int l = 0; l < NB; ++l)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) w2[l][q] = W2[l * 32 + 4 * kq + q];
-        for (int i = rgi; i < pr; i += nrg) {
-          T* pa = A + (long long)(j0 + i) * n + cq;
-          T a[4];
-          ld4(pa, a);
-#pragma unroll
-          for (int l = 0; l < NB; ++l) {
-            const T v = P[l * lp + i];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) a[q] -= v * w2[l][q];
-          }
-          if (cq < c0) {
-            // quad straddling the panel: keep the panel's columns untouched
-            T o[4];
-            ld4(pa, o);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if (cq + q < c0) a[q] = o[q];
-          }
-          st4(pa, a);
-        }
-      }
-      __syncthreads();
+    for (int cb = c0 & ~3; cb < n; cb += 32) {
+      if (n - cb > 16) hh_trailing<8>(A, n, j0, pr, nb, cb, c0, P, lp, red, Wd, W2, VtV, tau);
+      else if (n - cb > 8) hh_trailing<4>(A, n, j0, pr, nb, cb, c0, P, lp, red, Wd, W2, VtV, tau);
+      else hh_trailing<2>(A, n, j0, pr, nb, cb, c0, P, lp, red, Wd, W2, VtV, tau);
     }
   }
 }
 
-template <typename T>
 __global__ void __launch_bounds__(kHhThreads)
 k_hh_level(const SiteFacItem* __restrict__ items, int level, void* const* ptrs, const int* ival, int pass) {
   const SiteFacItem it = items[blockIdx.y];
@@ -462,10 +527,10 @@ k_hh_level(const SiteFacItem* __restrict__ items, int level, void* const* ptrs, 
   }
   const long long g = blockIdx.x;
   if (g >= nblk) return;
-  T* A = static_cast<T*>(ptrs[it.cv.ref]);
+  double* A = static_cast<double*>(ptrs[it.cv.ref]);
   extern __shared__ __align__(16) unsigned char hh_sh[];
-  const HhSmem S = hh_smem<T>(L);            // within the launch's plan for nmax >= n
-  T* base = A + g * span * n;
+  const HhSmem S = hh_smem(L);            // within the launch's plan for nmax >= n
+  double* base = A + g * span * n;
   long long rows;
   if (level == 0) {
     long long r0 = g * span;
@@ -482,25 +547,24 @@ k_hh_level(const SiteFacItem* __restrict__ items, int level, void* const* ptrs, 
       // of a child has at most min(crows_full, ...) rows, and its R at most n
       long long rr = crows_full < n ? crows_full : n;
       if (c > 0) {
-        const T* src = A + cr0 * n;
+        const double* src = A + cr0 * n;                    // the stack (4 n rows) ends before it
         for (long long e = threadIdx.x; e < rr * n; e += blockDim.x) base[rows * n + e] = src[e];
-        __syncthreads();
       }
       rows += rr;
     }
+    __syncthreads();
   }
-  hh_block_qr<T>(base, rows, n, hh_sh, S);
+  hh_block_qr(base, rows, n, hh_sh, S);
 }
 
-template <typename T>
 cudaError_t launch_hh_level(const SiteFacItem* items, int n_items, int level, int grid_x, int nmax,
                             void* const* ptrs, const int* ival, cudaStream_t s, int pass) {
   if (n_items == 0) return cudaSuccess;
-  const size_t smem = hh_smem<T>(hh_leaf_rows(nmax)).total;
-  cudaError_t e = cudaFuncSetAttribute(k_hh_level<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const size_t smem = hh_smem(hh_leaf_rows(nmax)).total;
+  cudaError_t e = cudaFuncSetAttribute(k_hh_level, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  k_hh_level<T><<<dim3(grid_x, n_items), kHhThreads, smem, s>>>(items, level, ptrs, ival, pass);
+  k_hh_level<<<dim3(grid_x, n_items), kHhThreads, smem, s>>>(items, level, ptrs, ival, pass);
   return cudaGetLastError();
 }
 
@@ -509,7 +573,6 @@ cudaError_t launch_hh_level(const SiteFacItem* items, int n_items, int level, in
 // each factored m x n matrix (2 m n^2 - 2 n^3 / 3 for m >= n, else
 // 2 m^2 n - 2 m^3 / 3; one read of the matrix), accumulated on the device
 // because only the device knows which sites took this branch.
-template <typename T>
 __global__ void k_hh_extract(const SiteFacItem* __restrict__ items, void* const* ptrs, int* ival, int pass,
                              double* acct) {
   const SiteFacItem it = items[blockIdx.x];
@@ -523,21 +586,20 @@ __global__ void k_hh_extract(const SiteFacItem* __restrict__ items, void* const*
     const double f = m >= n ? 2.0 * dm * dn * dn - 2.0 * dn * dn * dn / 3.0
                             : 2.0 * dm * dm * dn - 2.0 * dm * dm * dm / 3.0;
     atomicAdd(&acct[0], f);
-    atomicAdd(&acct[1], dm * dn * (double)sizeof(T));
+    atomicAdd(&acct[1], dm * dn * sizeof(double));
   }
-  const T* A = static_cast<const T*>(ptrs[it.cv.ref]);
+  const double* A = static_cast<const double*>(ptrs[it.cv.ref]);
   for (int e = threadIdx.x; e < k * n; e += blockDim.x) {
     int a = e / n, q = e - a * n;
-    it.C[(long long)a * it.ldc + q] = (q >= a) ? (double)A[(long long)a * n + q] : 0.0;
+    it.C[(long long)a * it.ldc + q] = (q >= a) ? A[(long long)a * n + q] : 0.0;
   }
   if (threadIdx.x == 0) ival[it.kfac_idx] = k;
 }
 
-template <typename T>
 cudaError_t launch_hh_extract(const SiteFacItem* items, int n_items, void* const* ptrs, int* ival,
                               cudaStream_t s, int pass, double* acct) {
   if (n_items == 0) return cudaSuccess;
-  k_hh_extract<T><<<n_items, 256, 0, s>>>(items, ptrs, ival, pass, acct);
+  k_hh_extract<<<n_items, 256, 0, s>>>(items, ptrs, ival, pass, acct);
   return cudaGetLastError();
 }
 
@@ -1098,17 +1160,6 @@ __device__ __forceinline__ bool rot_params(float al, float be, float ga, float t
 // (integer work); s = 2 h / (1 + h^2) follows from an FP32 reciprocal by one
 // cubic step, 2 h times it being exact; the norms' updates take tan theta in FP32
 // (they steer the next rotations and are recomputed every round).
-__device__ __forceinline__ float top_float(double x, int e) {   // x 2^(1023 - e), e >= its biased exponent
-  const int hi = __double2hiint(x), lo = __double2loint(x);
-  const int ex = (hi >> 20) & 0x7ff, f = ex - e + 127;
-  const int bits = (hi & 0x80000000) | (f << 23) | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29);
-  return ex == 0 || f <= 0 ? 0.f : __int_as_float(bits);
-}
-__device__ __forceinline__ double wide(float x) {               // (double)x of a normal number or zero
-  const int b = __float_as_int(x);
-  return (b & 0x7fffffff) == 0 ? 0.0
-                               : __hiloint2double((b & 0x80000000) | (((b & 0x7fffffff) >> 3) + (896 << 20)), b << 29);
-}
 __device__ __forceinline__ bool rot_params(double al, double be, double ga, double tol2, double negligible, double cut,
                                            double& h, double& s, double& na, double& nb) {
   // al, be, |ga| and the bounds are not negative: their bits order like their values
@@ -2186,11 +2237,6 @@ cudaError_t launch_core(const CoreItem* items, int n_items, int chimax, int* iva
   e = cudaLaunchKernelEx(&cfg, k_core, items, ival, flags_base, csize);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
-
-template cudaError_t launch_hh_level<double>(const SiteFacItem*, int, int, int, int, void* const*,
-                                             const int*, cudaStream_t, int);
-template cudaError_t launch_hh_extract<double>(const SiteFacItem*, int, void* const*, int*,
-                                               cudaStream_t, int, double*);
 
 }  // namespace pepo
 

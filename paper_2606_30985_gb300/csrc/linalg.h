@@ -6,13 +6,12 @@ namespace pepo {
 cudaError_t launch_env_factor(const EnvFactorItem* items, int n_items, int chimax, int* ival,
                               cudaStream_t s);
 cudaError_t launch_branch(const SiteFacItem* items, int n_items, int* ival, cudaStream_t s);
-template <typename T>
+constexpr int kHhLeafRows = 128;   // least rows of a TSQR leaf
 // pass: the branch value of the sites processed (0: the Householder branch,
 // 2: the sites the Cholesky branch handed over); only < 0: every site
 cudaError_t launch_hh_level(const SiteFacItem* items, int n_items, int level, int grid_x, int nmax,
                             void* const* ptrs, const int* ival, cudaStream_t s, int pass);
 // acct (may be null): 2 doubles accumulating the QR's algorithmic FLOPs and bytes
-template <typename T>
 cudaError_t launch_hh_extract(const SiteFacItem* items, int n_items, void* const* ptrs, int* ival,
                               cudaStream_t s, int pass, double* acct);
 // householder = 1 (FP64 storage): the sites of the Householder passes hold an

@@ -1375,18 +1375,17 @@ pepo_status run_gate_wave(pepo_ctx* c, Inst& I, GateWave& w) {
       return PEPO_OK;
     }
     const long long mmax = (long long)pow_sz(chimax, 3);
-    const long long L0 = 256;
-    long long nb0 = (mmax + L0 - 1) / L0;
+    long long nb0 = (mmax + kHhLeafRows - 1) / kHhLeafRows;
     int levels = 1;
     long long nb = nb0;
     while (nb > 1) { nb = (nb + 3) / 4; ++levels; }
     long long g = nb0;
     for (int l = 0; l < levels; ++l) {
-      LAUNCH_T(K_HH, nullptr, w.fac.n, launch_hh_level<double>(w.fac.d, w.fac.n, l, (int)std::max<long long>(g, 1), nmax, c->d_ptrs,
+      LAUNCH_T(K_HH, nullptr, w.fac.n, launch_hh_level(w.fac.d, w.fac.n, l, (int)std::max<long long>(g, 1), nmax, c->d_ptrs,
                                 c->d_ival, s, pass));
       g = (g + 3) / 4;
     }
-    LAUNCH_T(K_HH, nullptr, w.fac.n, launch_hh_extract<double>(w.fac.d, w.fac.n, c->d_ptrs, c->d_ival, s, pass, c->d_hh_acct));
+    LAUNCH_T(K_HH, nullptr, w.fac.n, launch_hh_extract(w.fac.d, w.fac.n, c->d_ptrs, c->d_ival, s, pass, c->d_hh_acct));
     return PEPO_OK;
   };
   pepo_status st = factor_rows(0);
