@@ -859,7 +859,9 @@ template <> struct VecSum<float> : TwoFloat {
 // 32 or more, else each of its warps takes an o of its own.  Bound: HBM (every
 // 32-byte sector of the site tensor holds two pinned values); separate passes
 // read the tensor twice and kept the FP64 pipe busy for 4 slots a value.
-// Class of the correlator of a 4x4, chi = 64 grid (11 passes): 7.2 -> 4.3 ms; of a
+// A row's sum goes to FP64 with up to 31 others, a lane each: one at a time the three
+// FP64 operations of it cost as much as the row's load.
+// Class of the correlator of a 4x4, chi = 64 grid (11 passes): 7.2 -> 4.3 -> 3.8 ms; of a
 // batch of nine small instances 53 -> 5.5 ms (blocks per item by their number).
 template <typename T>
 __global__ void __launch_bounds__(256)
@@ -889,8 +891,10 @@ k_vec_pair(const VecPairItem* __restrict__ items, void* const* ptrs, const int* 
   const long long step = share ? gridDim.x : (long long)gridDim.x * 8;
   for (long long o = share ? blockIdx.x : (long long)blockIdx.x * 8 + w; o < O; o += step) {
     const T* base = site + o * J2 * J3 * 4;
-    A col[4];
-    for (int j2 = share ? w : 0; j2 < J2; j2 += share ? 8 : 1) {
+    A col[4], kept;                                    // lane r keeps the sum of the warp's row r mod 32
+    int r = 0;
+    const int first = share ? w : 0, by = share ? 8 : 1;
+    for (int j2 = first; j2 < J2; j2 += by) {
       T x[4];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
@@ -909,7 +913,12 @@ k_vec_pair(const VecPairItem* __restrict__ items, void* const* ptrs, const int* 
       }
 #pragma unroll
       for (int m = 16; m > 0; m >>= 1) row.merge(m);
-      if (lane == 0) it.out_prev[o * J2 + j2] = row.value();
+      if (lane == (r & 31)) kept = row;
+      ++r;
+      if ((r & 31) == 0 || j2 + by >= J2) {            // up to 32 sums go to FP64 at once
+        const int at = first + ((r - 1) / 32 * 32 + lane) * by;
+        if (lane <= ((r - 1) & 31)) it.out_prev[o * J2 + at] = kept.value();
+      }
     }
     if (share) {
 #pragma unroll
