@@ -278,4 +278,38 @@ struct GateItem {
   int* flags;
 };
 
+// One sequence of the tiles of all items, shared out evenly among resident CTAs:
+// toff[i] = tiles before item i (n + 1 entries in shared memory), from count(i).
+template <class F>
+__device__ __forceinline__ void tile_prefix(unsigned* toff, int n, F count) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) toff[i + 1] = count(i);
+  if (threadIdx.x == 0) toff[0] = 0;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    unsigned carry = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+      const int i = i0 + threadIdx.x;
+      unsigned v = i < n ? toff[i + 1] : 0u;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned w = __shfl_up_sync(0xffffffffu, v, o);
+        if ((int)threadIdx.x >= o) v += w;
+      }
+      v += carry;
+      if (i < n) toff[i + 1] = v;
+      carry = __shfl_sync(0xffffffffu, v, 31);
+    }
+  }
+  __syncthreads();
+}
+// the item of tile t: the last one that starts at or before it
+__device__ __forceinline__ int tile_item(const unsigned* toff, int n, unsigned t) {
+  int item = 0;
+  for (int lo = 0, hi = n; lo < hi;) {
+    const int mid = (lo + hi) / 2;
+    if (toff[mid] <= t) { item = mid; lo = mid + 1; } else hi = mid;
+  }
+  return item;
+}
+
 }  // namespace pepo

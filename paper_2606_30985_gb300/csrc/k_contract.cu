@@ -26,94 +26,140 @@ __device__ inline void load_dims4(const TView& v, const int* ival, int* d) {
 
 // ============================================================ leg contraction
 // out[o, i, q] = sum_j A[i, j] in[o, j, q], i.e. a (Jout x J) matrix times the J x C
-// matrix of the columns c = (o, q), q fastest and contiguous.  A CTA keeps A
-// transposed in shared memory and takes tiles of TC columns: the J rows of a
-// tile arrive as asynchronous 16-byte copies (a unit of 16 bytes never leaves
-// its o), a thread holds MI outputs of two units.  TI = MI x (256 / column
-// threads) is chosen from the live Jout, so a small bond does not pay for the
-// rows of a large tile; the column index is divided once per thread and tile,
-// in 32 bits.  The sum over j runs in order.
+// matrix of the columns c = (o, q), q fastest and contiguous.  FP32: the grid is what
+// the chip holds; the tiles of TC columns of all items, in one sequence, are
+// shared out evenly (items differ by chi^2 between a corner and the bulk).  A CTA
+// keeps its item's A transposed in shared memory; rows of `in` arrive eight at a
+// time as asynchronous 16-byte copies (a unit of 16 bytes never leaves its o),
+// three stages deep and across tiles, and a thread holds MI outputs of NU
+// units.  TI = MI x (NT / column threads) is chosen from the live Jout, so a small
+// bond does not pay for the rows of a large tile.  The sum over j runs in order.
 //
-// Bound: FP32 ALU at chi = 48 (12 FLOP per byte), launch and latency below
-// chi = 20; two CTAs per SM overlap one's copies with the other's products.
-// Class of a case, 64 / 128-row tiles -> these: 4x4 chi = 48 72 -> 24 ms, a batch of
-// nine small instances 76 -> 14 ms.
+// Bound: FP32 ALU at chi = 48 (12 FLOP per byte), HBM below, launch and latency below
+// chi = 20.  Class of a case, 64 / 128-row tiles -> whole tiles loaded, then
+// multiplied, a fixed grid per item -> these: BP legs of a 4x4 chi = 48 layer 72 -> 24 ->
+// 21 ms, of nine 4x4 instances 76 -> 14 -> 6.5 ms.
 // FP64 is bound by its pipe, two multiply-adds per clock and SM, so its tiles
 // are small (64 threads, one unit each) and a small site still spreads over
 // many SMs: at chi = 8 a tile of 512 columns took one SM 8 us (class 6.0 -> 3.5 ms).
 template <typename T> struct LegBlock;
-template <> struct LegBlock<float> { static constexpr int NT = 256, NU = 2; };
-template <> struct LegBlock<double> { static constexpr int NT = 64, NU = 1; };
+template <> struct LegBlock<float> { static constexpr int NT = 256, CTAS = 2; };
+template <> struct LegBlock<double> { static constexpr int NT = 64, CTAS = 8; };
+constexpr int kLegMaxItems = 512;                      // of a launch
+constexpr int kLegRows = 8, kLegStages = 3;
 template <typename T, int MI, int TI>
 struct LegCfg {
   static constexpr int U = 16 / (int)sizeof(T);
   static constexpr int IG = TI / MI;                   // thread groups over the outputs
   static constexpr int CG = LegBlock<T>::NT / IG;      // threads over the columns
-  static constexpr int NU = LegBlock<T>::NU;           // units per thread
-  static constexpr int TC = CG * NU * U;               // columns of a tile
+  static constexpr int NU = sizeof(T) == 4 && TI > 16 ? 2 : 1;   // units per thread
+  static constexpr int TU = CG * NU;                   // units of a tile
+  static constexpr int TC = TU * U;                    // columns
+  static constexpr int PITCH = TC + U;                 // values between staged rows (one unit off the banks)
 };
 
+// units of a tile and rows of A for a live Jout
+template <typename T>
+__host__ __device__ inline int leg_ti(int Jout) {
+  if (sizeof(T) == 4 && (Jout > 16 && Jout <= 24 || Jout > 32 && Jout <= 48 || Jout > 64 && Jout <= 96)) return Jout <= 24 ? 24 : Jout <= 48 ? 48 : 96;
+  return Jout <= 8 ? 8 : Jout <= 16 ? 16 : Jout <= 32 ? 32 : Jout <= 64 ? 64 : 128;
+}
+template <typename T>
+__host__ __device__ inline int leg_tu(int ti) {
+  return ti == 8 ? LegCfg<T, 4, 8>::TU : ti == 16 ? LegCfg<T, 8, 16>::TU : ti <= 32 ? LegCfg<T, 8, 32>::TU
+       : ti <= 64 ? LegCfg<T, 8, 64>::TU : LegCfg<T, 8, 128>::TU;   // 24, 48, 96: as many groups, six rows each
+}
+
+// tiles lo .. hi - 1 of an item
 template <typename T, int MI, int TI>
 __device__ void leg_tiles(const T* __restrict__ in, T* __restrict__ out, const double* __restrict__ A, int lda, int J,
-                          int Jout, unsigned O, unsigned QU, unsigned char* sh, int room) {
+                          int Jout, unsigned O, unsigned QU, unsigned char* sh, unsigned lo, unsigned hi) {
   using C = LegCfg<T, MI, TI>;
-  constexpr int U = C::U, CG = C::CG, NU = C::NU, TC = C::TC, NT = LegBlock<T>::NT;
+  constexpr int U = C::U, CG = C::CG, NU = C::NU, PITCH = C::PITCH, TU = C::TU, NT = LegBlock<T>::NT;
   const int tid = threadIdx.x;
   const int cg = tid % CG, ig = tid / CG;
   const long long Q = (long long)QU * U;
   const unsigned cols = O * QU;                        // columns in units
-  // rows of `in` at a time: all J where they fit (then the tile is loaded once)
-  const int jc = min(J, (int)((room - sizeof(T) * (size_t)J * TI) / (sizeof(T) * TC)));
   T* At = reinterpret_cast<T*>(sh);                    // [J][TI]
-  T* Bs = At + (size_t)J * TI;                         // [jc][TC]
-  const unsigned ntile = (cols + CG * NU - 1) / (CG * NU);
-  if (blockIdx.x >= ntile) return;
+  T* Bs = At + (size_t)J * TI;                 // [stage][row][PITCH]
+  const unsigned nch = J > kLegRows ? (J + kLegRows - 1) / kLegRows : 1;
+  const unsigned total = (hi - lo) * nch;
+  // load cursor.  Threads run along the columns, the groups share the rows; on the
+  // innermost leg (QU = 1: a column's rows are 16 bytes apart) eight threads
+  // run along the rows instead, so that they read 128 consecutive bytes.
+  unsigned ltile = lo, lch = 0, li = 0;
+  const uint4* in4 = reinterpret_cast<const uint4*>(in);
+  unsigned src[NU];                                    // first unit of the thread's column (~0: none)
+  auto load = [&]() {
+    if (li < total) {
+      const int j0 = lch * kLegRows, jn = min(kLegRows, J - j0);
+      T* dst = Bs + (size_t)(li % kLegStages) * (kLegRows * PITCH);
+      auto copy = [&](int j, int c, unsigned at, bool live) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(dst + j * PITCH + c * U)),
+                     "l"(in4 + (live ? at : 0u)), "r"(live ? 16 : 0)
+                     : "memory");
+      };
+      if (QU == 1) {
+        const int j = tid & (kLegRows - 1);
+        if (j < jn)
+#pragma unroll
+          for (int c = tid / kLegRows; c < TU; c += NT / kLegRows) {
+            const unsigned o = ltile * TU + c;
+            copy(j, c, o * (unsigned)J + j0 + j, o < cols);
+          }
+      } else {
+        if (lch == 0) {
+#pragma unroll
+          for (int u = 0; u < NU; ++u) {
+            const unsigned c = ltile * TU + u * CG + cg;
+            const unsigned o = c / QU;
+            src[u] = c < cols ? o * (J - 1) * QU + c : ~0u;   // a tensor has below 2^30 units
+          }
+        }
+        for (int j = ig; j < jn; j += C::IG)
+#pragma unroll
+          for (int u = 0; u < NU; ++u) copy(j, u * CG + cg, src[u] + (j0 + j) * QU, src[u] != ~0u);
+      }
+      if (++lch == nch) { lch = 0; ++ltile; }
+      ++li;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  __syncthreads();                                     // the item before is consumed
+#pragma unroll
+  for (int st = 0; st < kLegStages - 1; ++st) load();
   for (int e = tid; e < J * TI; e += NT) {
     const int i = e / J, j = e - i * J;
-    At[j * TI + i] = i < Jout ? (T)A[(long long)i * lda + j] : T(0);
+    const T x = i < Jout ? (T)A[(long long)i * lda + j] : T(0);
+    At[j * TI + i] = x;
   }
-  for (unsigned tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
-    // this thread copies the units that it also computes with its group; the
-    // groups share the copies row by row
-    const T* src[NU];
-    T* dst[NU];
-    bool live[NU];
+  T acc[MI][NU][U];
 #pragma unroll
-    for (int u = 0; u < NU; ++u) {
-      const unsigned c = tile * (CG * NU) + u * CG + cg;
-      live[u] = c < cols;
-      const unsigned o = live[u] ? c / QU : 0u, q = live[u] ? c - o * QU : 0u;
-      src[u] = in + (long long)o * J * Q + (long long)q * U;
-      dst[u] = out + (long long)o * Jout * Q + (long long)q * U;
-    }
-    T acc[MI][NU][U];
+  for (int i = 0; i < MI; ++i)
 #pragma unroll
-    for (int i = 0; i < MI; ++i)
+    for (int u = 0; u < NU; ++u)
+#pragma unroll
+      for (int x = 0; x < U; ++x) acc[i][u][x] = T(0);
+  unsigned tile = lo, ch = 0;
+  for (unsigned n = 0; n < total; ++n) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kLegStages - 2) : "memory");
+    __syncthreads();                                   // this chunk is in, the one before is consumed
+    load();
+    const T* b0 = Bs + (size_t)(n % kLegStages) * (kLegRows * PITCH) + cg * U;
+    const T* a0 = At + (size_t)ch * (kLegRows * TI) + ig * MI;
+    auto step = [&](int j) {
+      T b[NU][U];
 #pragma unroll
       for (int u = 0; u < NU; ++u)
+        *reinterpret_cast<uint4*>(b[u]) = *reinterpret_cast<const uint4*>(b0 + j * PITCH + u * CG * U);
+      {
+        T a[MI];
 #pragma unroll
-        for (int x = 0; x < U; ++x) acc[i][u][x] = T(0);
-    for (int j0 = 0; j0 < J; j0 += jc) {
-      const int jn = min(jc, J - j0);
-      __syncthreads();                                 // the previous rows are consumed (and A is staged)
-      for (int j = ig; j < jn; j += C::IG)
-#pragma unroll
-        for (int u = 0; u < NU; ++u)
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
-                           (unsigned)__cvta_generic_to_shared(Bs + (size_t)j * TC + (u * CG + cg) * U)),
-                       "l"(live[u] ? src[u] + (long long)(j0 + j) * Q : in), "r"(live[u] ? 16 : 0)
-                       : "memory");
-      asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-      __syncthreads();
-#pragma unroll 4
-      for (int j = 0; j < jn; ++j) {
-        T a[MI], b[NU][U];
-#pragma unroll
-        for (int i = 0; i < MI; i += U)
-          *reinterpret_cast<uint4*>(a + i) = *reinterpret_cast<const uint4*>(At + (j0 + j) * TI + ig * MI + i);
-#pragma unroll
-        for (int u = 0; u < NU; ++u)
-          *reinterpret_cast<uint4*>(b[u]) = *reinterpret_cast<const uint4*>(Bs + (size_t)j * TC + (u * CG + cg) * U);
+        for (int i = 0; i < MI; i += MI % U ? U / 2 : U) {
+          if constexpr (MI % U != 0) *reinterpret_cast<uint2*>(a + i) = *reinterpret_cast<const uint2*>(a0 + j * TI + i);
+          else *reinterpret_cast<uint4*>(a + i) = *reinterpret_cast<const uint4*>(a0 + j * TI + i);
+        }
 #pragma unroll
         for (int i = 0; i < MI; ++i)
 #pragma unroll
@@ -121,61 +167,123 @@ __device__ void leg_tiles(const T* __restrict__ in, T* __restrict__ out, const d
 #pragma unroll
             for (int x = 0; x < U; ++x) acc[i][u][x] = fma(a[i], b[u][x], acc[i][u][x]);
       }
-    }
+    };
+    const int jn = min(kLegRows, J - (int)ch * kLegRows);
+#pragma unroll 2
+    for (int j = 0; j < jn; ++j) step(j);
+    if (++ch < nch) continue;
+    ch = 0;
 #pragma unroll
-    for (int i = 0; i < MI; ++i) {
-      const int io = ig * MI + i;
-      if (io < Jout)
+    for (int u = 0; u < NU; ++u) {
+      const unsigned c = tile * TU + u * CG + cg;
+      if (c < cols) {
+        const unsigned o = c / QU, q = c - o * QU;
+        T* dst = out + (long long)o * Jout * Q + (long long)q * U;
 #pragma unroll
-        for (int u = 0; u < NU; ++u)
-          if (live[u]) *reinterpret_cast<uint4*>(dst[u] + (long long)io * Q) = *reinterpret_cast<const uint4*>(acc[i][u]);
+        for (int i = 0; i < MI; ++i) {
+          const int io = ig * MI + i;
+          if (io < Jout) *reinterpret_cast<uint4*>(dst + (long long)io * Q) = *reinterpret_cast<const uint4*>(acc[i][u]);
+        }
+      }
     }
+    ++tile;
+#pragma unroll
+    for (int i = 0; i < MI; ++i)
+#pragma unroll
+      for (int u = 0; u < NU; ++u)
+#pragma unroll
+        for (int x = 0; x < U; ++x) acc[i][u][x] = T(0);
   }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(LegBlock<T>::NT, sizeof(T) == 4 ? 2 : 8)
-k_leg_contract(const LegItem* __restrict__ items, void* const* ptrs, const int* __restrict__ ival, int room) {
-  const LegItem it = items[blockIdx.y];
+__global__ void __launch_bounds__(LegBlock<T>::NT, LegBlock<T>::CTAS)
+k_leg_contract(const LegItem* __restrict__ items, int n_items, void* const* ptrs, const int* __restrict__ ival) {
   extern __shared__ __align__(16) unsigned char lc_sh[];
-  int d[PEPO_MAXLEG];
-  load_dims4(it.in, ival, d);
-  const int k = it.leg;
-  int J = 1;
-  unsigned O = 1, Q = 4;
+  __shared__ unsigned toff[kLegMaxItems + 1];          // tiles before each item
+  auto extents = [&](const LegItem& it, int& J, unsigned& O, unsigned& QU) {
+    int d[PEPO_MAXLEG];
+    load_dims4(it.in, ival, d);
+    unsigned Q = 4;
+    J = 1;
+    O = 1;
 #pragma unroll
-  for (int i = 0; i < PEPO_MAXLEG; ++i) {
-    if (i == k) J = d[i];
-    else if (i < k) O *= d[i];
-    else Q *= d[i];                                    // legs beyond nlegs have size 1
+    for (int i = 0; i < PEPO_MAXLEG; ++i) {
+      if (i == it.leg) J = d[i];
+      else if (i < it.leg) O *= d[i];
+      else Q *= d[i];                                  // legs beyond nlegs have size 1
+    }
+    QU = Q / (16 / sizeof(T));
+  };
+  auto run = [&](const LegItem& it, int J, int Jout, unsigned O, unsigned QU, unsigned lo, unsigned hi) {
+    const int lda = it.lda;
+    const double* A = it.A;
+    const T* in = static_cast<const T*>(ptrs[it.in.ref]);
+    T* out = static_cast<T*>(ptrs[it.out_ref]);
+    switch (leg_ti<T>(Jout)) {
+      case 8: leg_tiles<T, 4, 8>(in, out, A, lda, J, Jout, O, QU, lc_sh, lo, hi); break;
+      case 16: leg_tiles<T, 8, 16>(in, out, A, lda, J, Jout, O, QU, lc_sh, lo, hi); break;
+      case 32: leg_tiles<T, 8, 32>(in, out, A, lda, J, Jout, O, QU, lc_sh, lo, hi); break;
+      case 64: leg_tiles<T, 8, 64>(in, out, A, lda, J, Jout, O, QU, lc_sh, lo, hi); break;
+      case 128: leg_tiles<T, 8, 128>(in, out, A, lda, J, Jout, O, QU, lc_sh, lo, hi); break;
+      default:
+        if constexpr (sizeof(T) == 4) {
+          if (Jout <= 24) leg_tiles<T, 6, 24>(in, out, A, lda, J, Jout, O, QU, lc_sh, lo, hi);
+          else if (Jout <= 48) leg_tiles<T, 6, 48>(in, out, A, lda, J, Jout, O, QU, lc_sh, lo, hi);
+          else leg_tiles<T, 6, 96>(in, out, A, lda, J, Jout, O, QU, lc_sh, lo, hi);
+        }
+    }
+  };
+  if constexpr (sizeof(T) == 8) {                      // a grid row per item
+    const LegItem& it = items[blockIdx.y];
+    int J;
+    unsigned O, QU;
+    extents(it, J, O, QU);
+    const int Jout = ival[it.out_dim];
+    const unsigned tu = leg_tu<T>(leg_ti<T>(Jout)), nt = (O * QU + tu - 1) / tu;
+    const unsigned per = nt / gridDim.x, more = nt - per * gridDim.x;
+    const unsigned lo = blockIdx.x * per + min(blockIdx.x, more), hi = lo + per + (blockIdx.x < more ? 1 : 0);
+    if (lo < hi) run(it, J, Jout, O, QU, lo, hi);
+  } else {
+    tile_prefix(toff, n_items, [&](int i) {
+      int J;
+      unsigned O, QU;
+      extents(items[i], J, O, QU);
+      const unsigned tu = leg_tu<T>(leg_ti<T>(ival[items[i].out_dim]));
+      return (O * QU + tu - 1) / tu;
+    });
+    const unsigned nt = toff[n_items], per = nt / gridDim.x, more = nt - per * gridDim.x;
+    unsigned t = blockIdx.x * per + min(blockIdx.x, more);
+    const unsigned t1 = t + per + (blockIdx.x < more ? 1 : 0);
+    int item = tile_item(toff, n_items, t);
+    while (t < t1) {
+      while (toff[item + 1] <= t) ++item;
+      const LegItem& it = items[item];
+      int J;
+      unsigned O, QU;
+      extents(it, J, O, QU);
+      const unsigned lo = t - toff[item], hi = min(t1, toff[item + 1]) - toff[item];
+      run(it, J, ival[it.out_dim], O, QU, lo, hi);
+      t += hi - lo;
+    }
   }
-  const int Jout = ival[it.out_dim];
-  const T* in = static_cast<const T*>(ptrs[it.in.ref]);
-  T* out = static_cast<T*>(ptrs[it.out_ref]);
-  const unsigned QU = Q / (16 / sizeof(T));
-  if (Jout <= 8) leg_tiles<T, 4, 8>(in, out, it.A, it.lda, J, Jout, O, QU, lc_sh, room);
-  else if (Jout <= 16) leg_tiles<T, 8, 16>(in, out, it.A, it.lda, J, Jout, O, QU, lc_sh, room);
-  else if (Jout <= 32) leg_tiles<T, 8, 32>(in, out, it.A, it.lda, J, Jout, O, QU, lc_sh, room);
-  else if (Jout <= 64) leg_tiles<T, 8, 64>(in, out, it.A, it.lda, J, Jout, O, QU, lc_sh, room);
-  else leg_tiles<T, 8, 128>(in, out, it.A, it.lda, J, Jout, O, QU, lc_sh, room);
 }
 
 template <typename T>
-cudaError_t launch_leg_contract(const LegItem* items, int n_items, int grid_x, int chimax,
-                                void* const* ptrs, const int* ival, cudaStream_t s) {
-  if (n_items == 0) return cudaSuccess;
-  // A and the J rows of a tile, at most half an SM's shared memory (the rows then
-  // come in parts); A at chi = 128 takes 64 KB (FP32) or 128 KB (FP64)
-  const int ti = chimax <= 8 ? 8 : chimax <= 16 ? 16 : chimax <= 32 ? 32 : chimax <= 64 ? 64 : 128;
-  const int tc = LegBlock<T>::NT * (ti == 8 ? 4 : 8) / ti * LegBlock<T>::NU * (16 / (int)sizeof(T));
-  const size_t a_bytes = sizeof(T) * (size_t)chimax * ti;
-  size_t room = a_bytes + sizeof(T) * (size_t)chimax * tc;
-  // a smaller live bond takes a wider tile with fewer rows
-  room = std::max(room, (size_t)(sizeof(T) == 4 ? 72 : 20) * 1024);
-  room = std::min(room, std::max((size_t)104 * 1024, a_bytes + 16 * 1024));
-  cudaError_t e = cudaFuncSetAttribute(k_leg_contract<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
+cudaError_t launch_leg_contract(const LegItem* items, int n_items, int chimax, void* const* ptrs, const int* ival,
+                                cudaStream_t s) {
+  size_t smem = 0;                                     // A and the stages of every tile that a live bond may take
+  for (int ti = 8; ti <= 128 && ti < 2 * chimax + 8; ti *= 2)
+    smem = std::max(smem, sizeof(T) * (size_t)chimax * ti + (size_t)kLegStages * kLegRows * (leg_tu<T>(ti) + 1) * 16);
+  cudaError_t e = cudaFuncSetAttribute(k_leg_contract<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_leg_contract<T><<<dim3(grid_x, n_items), LegBlock<T>::NT, room, s>>>(items, ptrs, ival, (int)room);
+  for (int i0 = 0; i0 < n_items; i0 += kLegMaxItems) {
+    const int n = std::min(kLegMaxItems, n_items - i0);
+    // FP64: a row of the grid per item (a small launch is all latency, and the
+    // shared sequence has more of it: 8.1 -> 11.4 us at chi = 8)
+    const dim3 grid = sizeof(T) == 8 ? dim3(std::max(8, 8 * 152 / n), n) : dim3(152 * LegBlock<T>::CTAS);
+    k_leg_contract<T><<<grid, LegBlock<T>::NT, smem, s>>>(items + i0, n, ptrs, ival);
+  }
   return cudaGetLastError();
 }
 
@@ -486,9 +594,9 @@ cudaError_t launch_permute(const void* in, void* out, int nlegs, const int* dims
   return cudaGetLastError();
 }
 
-template cudaError_t launch_leg_contract<float>(const LegItem*, int, int, int, void* const*,
+template cudaError_t launch_leg_contract<float>(const LegItem*, int, int, void* const*,
                                                 const int*, cudaStream_t);
-template cudaError_t launch_leg_contract<double>(const LegItem*, int, int, int, void* const*,
+template cudaError_t launch_leg_contract<double>(const LegItem*, int, int, void* const*,
                                                  const int*, cudaStream_t);
 template cudaError_t launch_gram_leg<float>(const GramLegItem*, int, int, int, void* const*,
                                             const int*, cudaStream_t);

@@ -6,8 +6,8 @@ namespace pepo {
 
 // ---- k_tensor.cu (storage type T = float or double) ----------------------
 template <typename T>
-cudaError_t launch_leg_contract(const LegItem* items, int n_items, int grid_x, int chimax,
-                                void* const* ptrs, const int* ival, cudaStream_t s);
+cudaError_t launch_leg_contract(const LegItem* items, int n_items, int chimax, void* const* ptrs, const int* ival,
+                                cudaStream_t s);
 template <typename T>
 cudaError_t launch_copy(const TView* items, const int* out_refs, int n_items, int grid_x,
                         void* const* ptrs, const int* ival, cudaStream_t s);

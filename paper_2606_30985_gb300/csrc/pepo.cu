@@ -1325,10 +1325,10 @@ bool use_umma(const pepo_ctx* c, int chimax) {
   return sizeof(T) == 4 && c->prec == PEPO_TF32X3 && umma_supported(chimax);
 }
 template <typename T>
-cudaError_t leg_dispatch(pepo_ctx* c, const LegItem* items, int n, int gx, int chimax) {
+cudaError_t leg_dispatch(pepo_ctx* c, const LegItem* items, int n, int chimax) {
   if (use_umma<T>(c, chimax))
     return launch_leg_umma(items, n, chimax, c->d_ptrs, c->d_ival, c->d_kerr, c->wait_ns, c->stream);
-  return launch_leg_contract<T>(items, n, gx, chimax, c->d_ptrs, c->d_ival, c->stream);
+  return launch_leg_contract<T>(items, n, chimax, c->d_ptrs, c->d_ival, c->stream);
 }
 template <typename T>
 cudaError_t gram_leg_dispatch(pepo_ctx* c, const GramLegItem* items, int n, int chimax) {
@@ -1343,14 +1343,10 @@ pepo_status run_gate_wave(pepo_ctx* c, Inst& I, GateWave& w) {
   cudaStream_t s = c->stream;
   const int chimax = I.cfg.chi_max;
   const int nmax = 4 * chimax, rmax = PEPO_RG * chimax;
-  const long long big = (long long)4 * pow_sz(chimax, 4);
-  int gx_leg = (int)std::min<long long>(std::max<long long>(1, big / (long long)(chimax * 64) + 1),
-                                        (long long)(2 * 152 * 4 / std::max(1, w.leg[0].n) + 1));
-  gx_leg = std::max(gx_leg, 8);
   LAUNCH_T(K_ENV, nullptr, w.env.n, launch_env_factor(w.env.d, w.env.n, chimax, c->d_ival, s));
   LAUNCH_N(w.copy.n, launch_copy<T>(w.copy.d, w.copy_out.d, w.copy.n, 64, c->d_ptrs, c->d_ival, s));
   for (int r = 0; r < 3; ++r)
-    LAUNCH_T(K_LEG, hitems(c, w.leg[r]), w.leg[r].n, leg_dispatch<T>(c, w.leg[r].d, w.leg[r].n, gx_leg, chimax));
+    LAUNCH_T(K_LEG, hitems(c, w.leg[r]), w.leg[r].n, leg_dispatch<T>(c, w.leg[r].d, w.leg[r].n, chimax));
   LAUNCH_N(w.fac.n, launch_branch(w.fac.d, w.fac.n, c->d_ival, s));
   {
     int nt = ceil_div(nmax, 64);
@@ -1425,9 +1421,8 @@ pepo_status run_bp_waves(pepo_ctx* c, Inst& I, std::vector<BpWave>& waves) {
   for (auto& w : waves) {
     LAUNCH_T(K_BP_EIG, nullptr, w.eig.n, launch_env_eig(w.eig.d, w.eig.n, chimax, c->tsize == 4 ? 1 : 0, c->d_ival, s));
     for (int a = 0; a < 4; ++a) {
-      int gx = std::max(8, 2 * 152 * 4 / std::max(1, w.leg[a].n));
       LAUNCH_T(K_BP_LEG, hitems(c, w.leg[a]), w.leg[a].n,
-               leg_dispatch<T>(c, w.leg[a].d, w.leg[a].n, gx, chimax));
+               leg_dispatch<T>(c, w.leg[a].d, w.leg[a].n, chimax));
     }
     LAUNCH_T(K_GRAM_LEG, hitems(c, w.gram), w.gram.n,
              gram_leg_dispatch<T>(c, w.gram.d, w.gram.n, chimax));
