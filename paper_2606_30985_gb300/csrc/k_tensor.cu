@@ -640,8 +640,10 @@ k_reconstruct(const ReconItem* __restrict__ items, void* const* ptrs, const int*
   }
 }
 
-// FP32: 256 x 64 tiles.  A CTA keeps its 64 columns of W, rounded to FP32 once, in
-// shared memory (W is FP64, and a conversion takes the FP64 unit) and goes
+// FP32: 256 x 64 tiles.  The tiles of all items, column by column, are one sequence
+// that is shared out evenly among the CTAs the chip holds (the items of a wave
+// differ by chi^2 in rows).  A CTA keeps its 64 columns of W, rounded to FP32 once,
+// in shared memory (W is FP64, and a conversion takes the FP64 unit) and goes
 // through row tiles with them; the rows arrive as they lie, 16 values of K at a
 // time, as asynchronous 16-byte copies three stages deep and across tiles.  A
 // thread holds 8 x 8 entries: per four values of K, 8 + 8 16-byte shared loads
@@ -649,7 +651,7 @@ k_reconstruct(const ReconItem* __restrict__ items, void* const* ptrs, const int*
 // multiply-adds.  The rows are numbered with the output's innermost row leg
 // fastest, so that 8 lanes store 16-byte neighbours.  The sum over K runs in order.
 // Bound: FP32 ALU.  Class of a 4x4 chi = 48 layer, 64 x 64 tiles with scalar
-// loads -> this: reconstruct 12.4 -> 5.6 ms.
+// loads -> these tiles -> one even sequence: 12.4 -> 5.6 -> 3.6 ms.
 constexpr int R3_ROWS = 256, R3_COLS = 64, R3_K = 16, R3_PITCH = R3_K + 4, R3_STAGES = 3;
 
 struct R3Plan {
@@ -658,8 +660,16 @@ struct R3Plan {
   unsigned e1, e2;                                     // row = (a0, a1, a2): extents of a1, a2
   unsigned rs[3];                                      // strides among the input's rows
   long long os[3], ocut;                               // and in the output; the new cut leg's
+  const float* in;
+  float* out;
+  const double* W;
+  int ldw;
 };
-__device__ __noinline__ void r3_plan(const ReconItem& it, const int* ival, R3Plan& p) {
+__device__ __noinline__ void r3_plan(const ReconItem& it, const int* ival, void* const* ptrs, R3Plan& p) {
+  p.in = static_cast<const float*>(ptrs[it.in.ref]);
+  p.out = static_cast<float*>(ptrs[it.out_ref]);
+  p.W = it.W;
+  p.ldw = it.ldw;
   const int nl = it.in.nlegs, cut = nl - 1;
   p.chin = ival[it.new_dim];
   p.n = 4 * ival[it.in.dim[cut]];
@@ -690,112 +700,126 @@ __device__ __noinline__ void r3_plan(const ReconItem& it, const int* ival, R3Pla
   p.ocut = os[cut];
 }
 
-__global__ void __launch_bounds__(256, 2)
-k_reconstruct32(const ReconItem* __restrict__ items, void* const* ptrs, const int* __restrict__ ival) {
-  const ReconItem& it = items[blockIdx.y];
-  __shared__ R3Plan pl;
-  if (threadIdx.x == 0) r3_plan(it, ival, pl);
-  __syncthreads();
-  const int n = pl.n, np = 4 * pl.chin;
-  const unsigned R = pl.R;
-  const int nct = ceil_div(np, R3_COLS);
-  const unsigned nrt = (R + R3_ROWS - 1) / R3_ROWS;
-  // CTAs of a column tile share its row tiles
-  const int per = max(1, (int)gridDim.x / nct);
-  const unsigned first = (int)gridDim.x >= nct ? blockIdx.x / nct : 0;
-  if (first >= (unsigned)per) return;
-  const float* __restrict__ in = static_cast<const float*>(ptrs[it.in.ref]);
-  float* __restrict__ out = static_cast<float*>(ptrs[it.out_ref]);
-  extern __shared__ __align__(16) float r3_sh[];
-  float* Ws = r3_sh;                                   // [n][64]
-  float* As = r3_sh + (size_t)n * R3_COLS;             // stages of [256][pitch]
+// Row tiles of one column tile from tile `at` of the item, at most `most`; returns how many.
+__device__ __noinline__ unsigned r3_tiles(const R3Plan& pl, float* r3_sh, unsigned at, unsigned most) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ty = 8 * (warp >> 1) + (lane & 7), tx = 4 * (warp & 1) + (lane >> 3);
+  const int n = pl.n, np = 4 * pl.chin;
+  const unsigned R = pl.R, nrt = (R + R3_ROWS - 1) / R3_ROWS;
+  const float* __restrict__ in = pl.in;
+  float* __restrict__ out = pl.out;
+  float* Ws = r3_sh;                                   // [n][64]
+  float* As = r3_sh + (size_t)n * R3_COLS;             // stages of [256][pitch]
   const unsigned nch = (unsigned)ceil_div(n, R3_K);
-  for (int ct = blockIdx.x % nct; ct < nct; ct += (int)gridDim.x >= nct ? nct : (int)gridDim.x) {
-    const unsigned tiles = nrt > first ? (nrt - first + per - 1) / per : 0u;
-    const unsigned total = tiles * nch;
-    if (total == 0) break;
-    __syncthreads();                                   // the columns before are consumed
-    for (int e = tid; e < n * R3_COLS; e += 256) {
-      const int c = ct * R3_COLS + (e & (R3_COLS - 1));
-      Ws[e] = c < np ? (float)it.W[(long long)(e / R3_COLS) * it.ldw + c] : 0.f;
-    }
-    // load cursor: this thread copies quad tid % 4 of the rows tid / 4 + 64 u
-    unsigned li = 0, lch = 0, ltile = first;
-    unsigned src[4];                                   // row of the input (~0: none)
-    auto load = [&]() {
-      if (li < total) {
-        if (lch == 0) {
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const unsigned r = ltile * R3_ROWS + (tid >> 2) + 64 * u;
-            const unsigned q = r / pl.e2, a2 = r - q * pl.e2, a0 = q / pl.e1, a1 = q - a0 * pl.e1;
-            src[u] = r < R ? a0 * pl.rs[0] + a1 * pl.rs[1] + a2 * pl.rs[2] : ~0u;
-          }
-        }
-        const int k = lch * R3_K + 4 * (tid & 3);
-        float* dst = As + (li % R3_STAGES) * (R3_ROWS * R3_PITCH) + (tid >> 2) * R3_PITCH + 4 * (tid & 3);
+  const int ct = (int)(at / nrt);
+  const unsigned first = at - ct * nrt, tiles = min(nrt - first, most), total = tiles * nch;
+  for (int e = tid; e < n * R3_COLS; e += 256) {
+    const int c = ct * R3_COLS + (e & (R3_COLS - 1));
+    Ws[e] = c < np ? (float)pl.W[(long long)(e / R3_COLS) * pl.ldw + c] : 0.f;
+  }
+  // load cursor: this thread copies quad tid % 4 of the rows tid / 4 + 64 u
+  unsigned li = 0, lch = 0, ltile = first;
+  unsigned src[4];                                   // row of the input (~0: none)
+  auto load = [&]() {
+    if (li < total) {
+      if (lch == 0) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const bool live = src[u] != ~0u && k < n;
-          copy_quad(dst + 64 * u * R3_PITCH, live ? in + (long long)src[u] * n + k : in, live);
+          const unsigned r = ltile * R3_ROWS + (tid >> 2) + 64 * u;
+          const unsigned q = r / pl.e2, a2 = r - q * pl.e2, a0 = q / pl.e1, a1 = q - a0 * pl.e1;
+          src[u] = r < R ? a0 * pl.rs[0] + a1 * pl.rs[1] + a2 * pl.rs[2] : ~0u;
         }
-        if (++lch == nch) { lch = 0; ltile += per; }
-        ++li;
       }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
+      const int k = lch * R3_K + 4 * (tid & 3);
+      float* dst = As + (li % R3_STAGES) * (R3_ROWS * R3_PITCH) + (tid >> 2) * R3_PITCH + 4 * (tid & 3);
 #pragma unroll
-    for (int st = 0; st < R3_STAGES - 1; ++st) load();
-    float acc[8][2][4];
+      for (int u = 0; u < 4; ++u) {
+        const bool live = src[u] != ~0u && k < n;
+        copy_quad(dst + 64 * u * R3_PITCH, live ? in + (long long)src[u] * n + k : in, live);
+      }
+      if (++lch == nch) { lch = 0; ++ltile; }
+      ++li;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
 #pragma unroll
-    for (int a = 0; a < 8; ++a)
+  for (int st = 0; st < R3_STAGES - 1; ++st) load();
+  float acc[8][2][4];
 #pragma unroll
-      for (int b = 0; b < 8; ++b) acc[a][b >> 2][b & 3] = 0.f;
-    unsigned tile = first, ch = 0;
-    for (unsigned m = 0; m < total; ++m) {
-      asm volatile("cp.async.wait_group %0;" ::"n"(R3_STAGES - 2) : "memory");
-      __syncthreads();                                 // this chunk is in, the one before is consumed
-      load();
-      const float* as = As + (m % R3_STAGES) * (R3_ROWS * R3_PITCH) + ty * R3_PITCH;
-      const float* ws = Ws + (size_t)ch * (R3_K * R3_COLS) + 4 * tx;
-      const int kn = min(R3_K, n - (int)ch * R3_K);    // a multiple of 4
-      for (int k = 0; k < kn; k += 4) {
-        float x[8][4];
+  for (int a = 0; a < 8; ++a)
+#pragma unroll
+    for (int b = 0; b < 8; ++b) acc[a][b >> 2][b & 3] = 0.f;
+  unsigned tile = first, ch = 0;
+  for (unsigned m = 0; m < total; ++m) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(R3_STAGES - 2) : "memory");
+    __syncthreads();                                 // this chunk is in, the one before is consumed
+    load();
+    const float* as = As + (m % R3_STAGES) * (R3_ROWS * R3_PITCH) + ty * R3_PITCH;
+    const float* ws = Ws + (size_t)ch * (R3_K * R3_COLS) + 4 * tx;
+    const int kn = min(R3_K, n - (int)ch * R3_K);    // a multiple of 4
+    for (int k = 0; k < kn; k += 4) {
+      float x[8][4];
+#pragma unroll
+      for (int a = 0; a < 8; ++a)
+        *reinterpret_cast<float4*>(x[a]) = *reinterpret_cast<const float4*>(as + 32 * a * R3_PITCH + k);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        float w[2][4];
+        *reinterpret_cast<float4*>(w[0]) = *reinterpret_cast<const float4*>(ws + (k + kk) * R3_COLS);
+        *reinterpret_cast<float4*>(w[1]) = *reinterpret_cast<const float4*>(ws + (k + kk) * R3_COLS + 32);
 #pragma unroll
         for (int a = 0; a < 8; ++a)
-          *reinterpret_cast<float4*>(x[a]) = *reinterpret_cast<const float4*>(as + 32 * a * R3_PITCH + k);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          float w[2][4];
-          *reinterpret_cast<float4*>(w[0]) = *reinterpret_cast<const float4*>(ws + (k + kk) * R3_COLS);
-          *reinterpret_cast<float4*>(w[1]) = *reinterpret_cast<const float4*>(ws + (k + kk) * R3_COLS + 32);
-#pragma unroll
-          for (int a = 0; a < 8; ++a)
-#pragma unroll
-            for (int b = 0; b < 8; ++b) acc[a][b >> 2][b & 3] = fmaf(x[a][kk], w[b >> 2][b & 3], acc[a][b >> 2][b & 3]);
-        }
+          for (int b = 0; b < 8; ++b) acc[a][b >> 2][b & 3] = fmaf(x[a][kk], w[b >> 2][b & 3], acc[a][b >> 2][b & 3]);
       }
-      if (++ch < nch) continue;
-      ch = 0;
-#pragma unroll
-      for (int a = 0; a < 8; ++a) {
-        const unsigned r = tile * R3_ROWS + ty + 32 * a;
-        if (r < R) {
-          const unsigned q = r / pl.e2, a2 = r - q * pl.e2, a0 = q / pl.e1, a1 = q - a0 * pl.e1;
-          float* dst = out + a0 * pl.os[0] + a1 * pl.os[1] + a2 * pl.os[2];
-#pragma unroll
-          for (int b = 0; b < 2; ++b) {
-            const int cn = ct * (R3_COLS / 4) + tx + 8 * b;
-            if (cn < pl.chin) *reinterpret_cast<float4*>(dst + cn * pl.ocut) = *reinterpret_cast<const float4*>(acc[a][b]);
-          }
-        }
-#pragma unroll
-        for (int b = 0; b < 8; ++b) acc[a][b >> 2][b & 3] = 0.f;
-      }
-      tile += per;
     }
+    if (++ch < nch) continue;
+    ch = 0;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const unsigned r = tile * R3_ROWS + ty + 32 * a;
+      if (r < R) {
+        const unsigned q = r / pl.e2, a2 = r - q * pl.e2, a0 = q / pl.e1, a1 = q - a0 * pl.e1;
+        float* dst = out + a0 * pl.os[0] + a1 * pl.os[1] + a2 * pl.os[2];
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          const int cn = ct * (R3_COLS / 4) + tx + 8 * b;
+          if (cn < pl.chin) *reinterpret_cast<float4*>(dst + cn * pl.ocut) = *reinterpret_cast<const float4*>(acc[a][b]);
+        }
+      }
+#pragma unroll
+      for (int b = 0; b < 8; ++b) acc[a][b >> 2][b & 3] = 0.f;
+    }
+    ++tile;
+  }
+  return tiles;
+}
+
+constexpr int kR3MaxItems = 512;                       // of a launch
+
+__global__ void __launch_bounds__(256, 2)
+k_reconstruct32(const ReconItem* __restrict__ items, int n_items, void* const* ptrs, const int* __restrict__ ival) {
+  __shared__ R3Plan pl;
+  __shared__ unsigned toff[kR3MaxItems + 1];
+  extern __shared__ __align__(16) float r3_sh[];
+  tile_prefix(toff, n_items, [&](int i) {
+    const ReconItem& it = items[i];
+    const int cut = it.in.nlegs - 1;
+    unsigned R = 1;
+    for (int l = 0; l < cut; ++l) R *= ival[it.in.dim[l]];
+    return (R + R3_ROWS - 1) / R3_ROWS * ceil_div(4 * ival[it.new_dim], R3_COLS);
+  });
+  const unsigned nt = toff[n_items], share = nt / gridDim.x, more = nt - share * gridDim.x;
+  unsigned t = blockIdx.x * share + min(blockIdx.x, more);
+  const unsigned t1 = t + share + (blockIdx.x < more ? 1 : 0);
+  if (t >= t1) return;
+  int item = tile_item(toff, n_items, t);
+  while (t < t1) {
+    while (toff[item + 1] <= t) ++item;
+    __syncthreads();                                   // the plan and the columns before are consumed
+    if (threadIdx.x == 0) r3_plan(items[item], ival, ptrs, pl);
+    __syncthreads();
+    t += r3_tiles(pl, r3_sh, t - toff[item], t1 - t);
   }
 }
 
@@ -804,18 +828,14 @@ cudaError_t launch_reconstruct(const ReconItem* items, int n_items, int chimax, 
                                cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
   const int nmax = 4 * chimax;
-  const long long rows = (long long)chimax * chimax * chimax;
   if constexpr (sizeof(T) == 4) {
     const size_t smem = sizeof(float) * ((size_t)nmax * R3_COLS + (size_t)R3_STAGES * R3_ROWS * R3_PITCH);
     cudaError_t e = cudaFuncSetAttribute(k_reconstruct32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    // twice what the chip holds (the items of a wave differ by chi^2 in rows), a
-    // multiple of the column tiles, at most a CTA per tile
-    const int nct = ceil_div(nmax, R3_COLS);
-    const long long tiles = (rows + R3_ROWS - 1) / R3_ROWS;
-    const int per = (int)std::min<long long>(tiles, std::max(1, ceil_div(4 * 152, n_items * nct)));
-    k_reconstruct32<<<dim3(per * nct, n_items), 256, smem, s>>>(items, ptrs, ival);
+    for (int i0 = 0; i0 < n_items; i0 += kR3MaxItems)
+      k_reconstruct32<<<2 * 152, 256, smem, s>>>(items + i0, std::min(kR3MaxItems, n_items - i0), ptrs, ival);
   } else {
+    const long long rows = (long long)chimax * chimax * chimax;
     const long long tiles = (rows + RC_T - 1) / RC_T * ceil_div(nmax, RC_T);
     const int gx = (int)std::max<long long>(4, std::min<long long>(tiles, 2 * 152 * 4 / n_items + 1));
     k_reconstruct<T><<<dim3(gx, n_items), 256, 0, s>>>(items, ptrs, ival);
