@@ -705,7 +705,7 @@ __host__ __device__ inline FacSmem fac_smem(int rmax, int nmax, int householder,
   m.pos = o;  o += sizeof(int) * (size_t)w;
   m.perm = o; o += sizeof(int) * (size_t)w;
   m.v = o;
-  if (householder) o += sizeof(double) * ((size_t)4 * nmax + (size_t)(kFacThreads / 32) * rmax);
+  if (householder) o += sizeof(double) * ((size_t)4 * nmax + (size_t)4 * rmax);
   o = (o + 15) & ~(size_t)15;
   m.mat = o;
   const size_t cap = (size_t)216 * 1024;
@@ -874,9 +874,12 @@ __device__ int chol_cluster(const double* __restrict__ A, int lda, int n, int w,
 
 // Column-pivoted Householder QR of the M x r matrix B (leading dimension ld)
 // in place: R in the upper trapezoid, the position order in perm; returns the
-// rank.  The 16 warps share the rows and their lanes the columns, so a
-// reflection's dot products and its update use the whole block (one thread
-// per column left all but r threads idle on two serial passes of M rows).
+// rank.  Bound: the FP64 units, a quarter of the SM each (a warp operation holds one
+// for 64 clocks).  Four warps, one per quarter, share the rows of 32 columns, so
+// that only four partial sums a column are left to add, on every lane that needs
+// them; sixteen row groups spent more on those sums than on the products.
+// Class, 16 row groups -> four: 3x3 chi = 8 evolution 4.3 -> 3.5 ms, 4x4 chi = 12
+// layer 2.4 -> 1.9.
 __device__ int qrcp(double* B, int ld, int M, int r, double* dg, double* w, double* v, double* part, int* perm,
                     double rel) {
   __shared__ long long rv[32];
@@ -884,19 +887,17 @@ __device__ int qrcp(double* B, int ld, int M, int r, double* dg, double* w, doub
   __shared__ double red[32];
   __shared__ double sh_h[3];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  constexpr int NW = kFacThreads / 32;
+  constexpr int CB = 32 * (kFacThreads / 128);              // columns of a pass
+  const int rg = wid & 3, cb = 32 * (wid >> 2) + lane;      // row group, column of a pass
   for (int i = threadIdx.x; i < r; i += blockDim.x) perm[i] = i;
-  for (int k0 = 0; k0 < r; k0 += 32) {
-    const int k = k0 + lane;
+  for (int k = cb; k < r; k += CB) {
     double s = 0.0;
-    if (k < r)
-      for (int i = wid; i < M; i += NW) { const double x = B[(long long)i * ld + k]; s = fma(x, x, s); }
-    if (k < r) part[wid * r + k] = s;
+    for (int i = rg; i < M; i += 4) { const double x = B[(long long)i * ld + k]; s = fma(x, x, s); }
+    part[rg * r + k] = s;
   }
   __syncthreads();
   for (int k = threadIdx.x; k < r; k += blockDim.x) {
-    double s = 0.0;
-    for (int g = 0; g < NW; ++g) s += part[g * r + k];
+    const double s = (part[k] + part[r + k]) + (part[2 * r + k] + part[3 * r + k]);
     dg[k] = s;
     w[k] = s;   // reference norms for the downdate safeguard
   }
@@ -921,40 +922,32 @@ __device__ int qrcp(double* B, int ld, int M, int r, double* dg, double* w, doub
       }
       __syncthreads();
     }
-    double s = 0.0;
-    for (int i = j + threadIdx.x; i < M; i += blockDim.x) {
-      const double x = B[(long long)i * ld + j];
-      s = fma(x, x, s);
+    if (wid < 4) {
+      double s = 0.0;
+      for (int i = j + threadIdx.x; i < M; i += 128) {
+        const double x = B[(long long)i * ld + j];
+        s = fma(x, x, s);
+      }
+      s = warp_sum(s);
+      if (lane == 0) red[wid] = s;
     }
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) {
-      const double alpha = B[(long long)j * ld + j], normx = sqrt(s);
-      const double b = alpha >= 0.0 ? -normx : normx;
-      sh_h[0] = b;
-      sh_h[1] = 1.0 / (alpha - b);
-      sh_h[2] = (b - alpha) / b;
-    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+      reflector(B[(long long)j * ld + j], (red[0] + red[1]) + (red[2] + red[3]), sh_h[0], sh_h[2], sh_h[1]);
     __syncthreads();
     const double beta = sh_h[0], inv = sh_h[1], tau = sh_h[2];
     for (int i = j + threadIdx.x; i < M; i += blockDim.x) v[i] = (i == j) ? 1.0 : B[(long long)i * ld + j] * inv;
     __syncthreads();
     for (int i = j + threadIdx.x; i < M; i += blockDim.x) B[(long long)i * ld + j] = (i == j) ? beta : 0.0;
-    for (int k0 = j + 1; k0 < r; k0 += 32) {
-      const int k = k0 + lane;
-      if (k >= r) continue;
+    for (int k = j + 1 + cb; k < r; k += CB) {
       double acc = 0.0;
-      for (int i = j + wid; i < M; i += NW) acc = fma(v[i], B[(long long)i * ld + k], acc);
-      part[wid * r + k] = acc;
+      for (int i = j + rg; i < M; i += 4) acc = fma(v[i], B[(long long)i * ld + k], acc);
+      part[rg * r + k] = acc;
     }
     __syncthreads();
-    for (int k0 = j + 1; k0 < r; k0 += 32) {
-      const int k = k0 + lane;
-      if (k >= r) continue;
-      double tw = 0.0;
-#pragma unroll
-      for (int g = 0; g < NW; ++g) tw += part[g * r + k];
-      tw *= tau;
-      for (int i = j + wid; i < M; i += NW) B[(long long)i * ld + k] -= v[i] * tw;
+    for (int k = j + 1 + cb; k < r; k += CB) {
+      const double tw = tau * ((part[k] + part[r + k]) + (part[2 * r + k] + part[3 * r + k]));
+      for (int i = j + rg; i < M; i += 4) B[(long long)i * ld + k] -= v[i] * tw;
     }
     __syncthreads();
     for (int k = j + 1 + threadIdx.x; k < r; k += blockDim.x) {
