@@ -12,6 +12,7 @@
 // the live bond dimension on the device.  FP32 storage accumulates the Gram's
 // long sums in FP32 runs of 256 terms that a two-float sum takes.
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.h"
 
@@ -299,7 +300,9 @@ cudaError_t launch_leg_contract(const LegItem* items, int n_items, int chimax, v
 // largest tile without a divergent branch.  The 256 / TX^2 groups of threads
 // take different units of a chunk, so a small F keeps the whole block busy;
 // the tile is chosen from the live F (8, 16, 32, 48, 64, 96, 128), not from
-// chi_max.  FP32 storage sums runs of 256 terms in FP32 and the runs in a
+// chi_max.  Their sums are laid side by side and added by one thread per entry: with
+// the groups adding one after another, a warp's FP64 operations (64 clocks each)
+// in 16 turns took longer than the products of a small split.  FP32 storage sums runs of 256 terms in FP32 and the runs in a
 // two-float sum; FP64 sums directly.
 //
 // Bound: FP32 ALU (2 shared 16-byte loads per 4 x MT x MT products at most) or
@@ -317,7 +320,8 @@ struct GlCfg {
   static constexpr int KCU = (U0 / 4) * G > U0 ? (U0 / 4) * G : U0;   // units per row and chunk
   static constexpr int PITCH = (KCU + 1) * U;          // values between rows
   static constexpr size_t kStage = sizeof(T) * (size_t)TL * PITCH;
-  static constexpr size_t kRed = G > 1 ? sizeof(double) * (size_t)TL * TL : 0;
+  using V = std::conditional_t<sizeof(T) == 4, float2, double>;   // a group's sum of an entry
+  static constexpr size_t kRed = G > 1 ? sizeof(V) * (size_t)G * TL * TL : 0;
   static constexpr size_t kSmem = kGlStages * kStage > kRed ? kGlStages * kStage : kRed;
 };
 
@@ -409,30 +413,35 @@ __device__ void gram_tile(const T* __restrict__ X, long long O, long long Q, int
   }
   flush();
   asm volatile("cp.async.wait_group 0;" ::: "memory");
-  auto value = [&](int a, int b) -> double {
-    if constexpr (kF32) return (double)hi[a][b] + (double)lo[a][b];
-    else return acc[a][b];
-  };
   if constexpr (G > 1) {
-    // sum of the groups, one after another, in shared memory
-    double* red = reinterpret_cast<double*>(sh);
-    for (int gg = 0; gg < G; ++gg) {
-      __syncthreads();
-      if (g == gg) {
-#pragma unroll
-        for (int a = 0; a < MT; ++a)
-#pragma unroll
-          for (int b = a; b < MT; ++b) {
-            double* r = red + (ty + TX * a) * TL + tx + TX * b;
-            *r = gg == 0 ? value(a, b) : *r + value(a, b);
-          }
-      }
-    }
+    // sum of the groups' values, one thread per entry of the blocks a <= b, the groups in
+    // order; the other triangle is a mirror
+    using V = typename C::V;
+    V* red = reinterpret_cast<V*>(sh);
     __syncthreads();
-    // entries with row block above the column block were not formed: mirror
-    for (int e = tid; e < F * F; e += 256) {
-      const int i = e / F, j = e - i * F;
-      P[e] = i / TX <= j / TX ? red[i * TL + j] : red[j * TL + i];
+#pragma unroll
+    for (int a = 0; a < MT; ++a)
+#pragma unroll
+      for (int b = a; b < MT; ++b) {
+        V* r = red + (g * TL + ty + TX * a) * TL + tx + TX * b;
+        if constexpr (kF32) *r = make_float2(hi[a][b], lo[a][b]);
+        else *r = acc[a][b];
+      }
+    __syncthreads();
+    for (int e = tid; e < MT * (MT + 1) / 2 * TX * TX; e += 256) {
+      int b = e / (TX * TX), a = 0;
+      while (b >= MT - a) { b -= MT - a; ++a; }        // block (a, a + b)
+      const int in = e % (TX * TX), i = TX * a + in / TX, j = TX * (a + b) + in % TX;
+      if (i >= F || j >= F) continue;
+      double z = 0.0;
+#pragma unroll
+      for (int gg = 0; gg < G; ++gg) {
+        const V v = red[(gg * TL + i) * TL + j];
+        if constexpr (kF32) z += (double)v.x + (double)v.y;
+        else z += v;
+      }
+      P[(long long)i * F + j] = z;
+      if (b > 0) P[(long long)j * F + i] = z;
     }
   } else {
 #pragma unroll
@@ -441,7 +450,9 @@ __device__ void gram_tile(const T* __restrict__ X, long long O, long long Q, int
       for (int b = a; b < MT; ++b) {
         const int i = ty + TX * a, j = tx + TX * b;
         if (i < F && j < F) {
-          const double v = value(a, b);
+          double v;
+          if constexpr (kF32) v = (double)hi[a][b] + (double)lo[a][b];
+          else v = acc[a][b];
           P[(long long)i * F + j] = v;
           if (a != b) P[(long long)j * F + i] = v;
         }
