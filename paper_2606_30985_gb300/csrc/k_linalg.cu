@@ -1628,7 +1628,7 @@ __device__ int jacobi_block64(double* buf, int n, double* nrm, int max_sweeps, i
 // moves no singular value by more than that, and without the cut the columns of
 // tiny singular values (mostly rounding noise from rotations with the large
 // ones) are chased for many sweeps without ever reaching relative
-// orthogonality.  Squared norms are recomputed every round and updated by the
+// orthogonality.  Squared norms are recomputed every round (up to n = 32 every sweep) and updated by the
 // rotations between.  flags: 3 ints, zeroed by the caller; cnorm: n doubles.
 template <typename R>
 __device__ __noinline__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* capped, double abs_rel, const Cta& ct,
@@ -1775,7 +1775,9 @@ __device__ __noinline__ int jacobi_cluster(R* A, int m, int n, R* V, int max_swe
       const int steps = all ? steps0 : bs;
       if (resident) {
         if (ct.rank == 0) {
-          norms(n);
+          // (up to n = 32 no cluster size takes the columns apart: once a sweep, as 15
+          // times cost as much as the rotations)
+          if (round == 0 || n > 32) norms(n);
           for (int k = 0; k < steps; ++k)
             rot |= round_of(npair * bs, [&](int e) {
               const int pi = e / bs, i = e - pi * bs;
