@@ -95,8 +95,10 @@ typedef struct {
   double qr_ratio_thresh;  /* ... and m / n > qr_ratio_thresh (150, 150).  A Cholesky-QR
                               site whose Gram has an accepted pivot keeping less than
                               1e-4 (FP32 storage) / 1e-10 (FP64) of its own column's
-                              diagonal is factored by Householder instead (Sec. 4.2's
-                              fallback; counted by pepo_qr_branch_counts) */
+                              diagonal takes the other branch instead (Sec. 4.2's
+                              fallback; counted by pepo_qr_branch_counts): Householder
+                              in FP64 storage, the exact Gram of its FP32 data and a
+                              pivoted Cholesky in FP32 storage */
   double pinv_rel;         /* rank threshold for message square roots (1e-12) */
   int gates;               /* pepo_gateset */
   int prec;                /* pepo_precision */
@@ -371,9 +373,10 @@ int pepo_num_bonds(const pepo_ctx* ctx, int inst);
  * bracketed by CUDA events on the context's stream and credited with its
  * algorithmic bytes and FLOPs, computed from the live bond dimensions read at
  * the start of each call (exact whenever chi does not change inside the call,
- * e.g. in the saturated regime).  The Householder class ("householder_tsqr")
- * is the exception: which sites take that branch is decided on the device,
- * so its FLOPs (2 m n^2 - 2 n^3 / 3 per factored m x n matrix) and bytes (one
+ * e.g. in the saturated regime).  The Householder class ("householder_tsqr":
+ * FP64 storage the TSQR, FP32 storage the exact Gram) is the exception: which
+ * sites take that branch is decided on the device, so its FLOPs (TSQR: 2 m n^2 -
+ * 2 n^3 / 3 per factored m x n matrix; exact Gram: m n (n + 1)) and bytes (one
  * read of it) are counted there, whether timing is on or not, and reset by
  * pepo_reset_timing.  Classes are numbered 0 .. pepo_timing_classes()-1. */
 pepo_status pepo_set_timing(pepo_ctx* ctx, int enable);

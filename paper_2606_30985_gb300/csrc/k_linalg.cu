@@ -8,14 +8,17 @@
 //                  m / n > ratio_thr, Householder otherwise (Sec. 4.2).
 //   k_hh_level     FP64 storage: Householder QR (TSQR tree, R only) of cv
 //                  (Sec. 4.2 Householder-QR); each tree block factored in panels
-//                  (compact WY).
+//                  (compact WY).  FP32 storage forms the exact Gram of cv instead
+//                  (k_gram_exact) and factors that.
 //   k_form         fold the gate's operator-Schmidt factors into the
 //                  R-factor: X = (F_kappa (x) 1) cv, G = X^T X or B = R-side of X.
-//   k_factor       rank-revealing factor T of X: pivoted Cholesky of G
-//                  (Cholesky-QR branch) or column-pivoted Householder of B.
+//   k_factor       rank-revealing factor T of X: pivoted Cholesky of G (from a
+//                  Gram) or column-pivoted Householder of B (from an R-factor).
 //   k_core         per bond: R1 R2^T, one-sided Jacobi SVD, truncation
 //                  (Eq. 11), lambda (Eq. 12), reconstruct matrices W1, W2
 //                  (Sec. 2.5 steps 5-8 in Q-less form), messages diag(lambda).
+//   k_env_eig      eigenbasis and square roots of a message (BP rotations).
+//   k_rotate_back  a Gram of the rotated tensor back into the bond's basis.
 #include <algorithm>
 #include <cstddef>
 #include <type_traits>
@@ -32,8 +35,8 @@ __device__ inline double warp_sum(double v) {
   return v;
 }
 
-// FP64 here issues one warp instruction per 16 clocks and SM, whatever the number
-// of useful lanes: scalars that the whole block needs (a root, a quotient, the sum
+// An FP64 operation of a warp holds its quarter of the SM's FP64 units for 64
+// clocks, whatever the number of useful lanes: scalars that the whole block needs (a root, a quotient, the sum
 // of the warps' partials) are formed by one warp and read from shared memory, and
 // magnitudes are compared as integers.
 
@@ -985,9 +988,8 @@ __device__ int qrcp(double* B, int ld, int M, int r, double* dg, double* w, doub
 // (directions too small to matter: the factorisation of G cuts them as rank).
 //
 // Measured, factor class of one saturated layer, right-looking Cholesky and one
-// thread per column before -> now: 4x4 chi = 48 212 -> 87 ms, 3x3 chi = 100 357
-// -> 255 ms, 3x5 chi = 27 42 -> 20 ms, results bit-identical (what is left is the
-// Householder branch).
+// thread per column -> left-looking on a cluster, no Householder in FP32 storage: 4x4
+// chi = 48 212 -> 6.3 ms, 3x3 chi = 100 357 -> 19 ms, 3x5 chi = 27 42 -> 2.1 ms.
 __global__ void __launch_bounds__(kFacThreads)
 k_factor(const SiteFacItem* __restrict__ items, int* ival, int only, unsigned long long* qcount, int rmax, int nmax,
          int householder, int csize) {
@@ -1628,8 +1630,9 @@ __device__ int jacobi_block64(double* buf, int n, double* nrm, int max_sweeps, i
 // moves no singular value by more than that, and without the cut the columns of
 // tiny singular values (mostly rounding noise from rotations with the large
 // ones) are chased for many sweeps without ever reaching relative
-// orthogonality.  Squared norms are recomputed every round (up to n = 32 every sweep) and updated by the
-// rotations between.  flags: 3 ints, zeroed by the caller; cnorm: n doubles.
+// orthogonality.  Squared norms are recomputed every round (up to n = 32 every
+// sweep) and updated by the rotations between.  flags: 3 ints, zeroed by the
+// caller; cnorm: n doubles.
 template <typename R>
 __device__ __noinline__ int jacobi_cluster(R* A, int m, int n, R* V, int max_sweeps, int* capped, double abs_rel, const Cta& ct,
                               int* flags, double* cnorm, unsigned char* sh) {

@@ -1,13 +1,15 @@
 // HBM-bound tensor kernels of the bond update and of BP.
 //
-//   k_gram_rows      cv^T cv with FP64 accumulation (Eq. 10, Cholesky-QR Gram)
-//   k_reconstruct    psi_new = psi W written in the next update's layout
+//   k_gram_rows32/64 cv^T cv (Eq. 10, Cholesky-QR Gram)
+//   k_gram_exact     cv^T cv of FP32 data to ~47 bits (FP32 storage: the sites of the
+//                    Householder side of Eq. 10 and those whose Gram fails its test)
+//   k_reconstruct, k_reconstruct32   psi_new = psi W written in the next update's layout
 //                    (Sec. 2.5 steps 6-7 in Q-less form, Alg. 1 lines 9-12)
 //   k_vec_pair, k_vec_contract   vector contractions of single-layer BP (Sec. 2.6)
 //
 // All sizes are read on the device (see common.cuh).  Accumulation: FP32
-// storage accumulates with FP32 FMAs over short runs that are flushed into
-// FP64 registers, so long sums (up to chi^3 terms) keep FP64-level error
+// storage accumulates with FP32 FMAs over short runs that go into two-float or
+// FP64 sums, so long sums (up to chi^3 terms) keep far below the FP32 error
 // (Sec. 4.2 "Gram matrix accumulation error": the paper's FP32 Gram loses
 // m * eps; this does not).
 #include "kernels.h"

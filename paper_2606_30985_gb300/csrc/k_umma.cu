@@ -18,19 +18,21 @@
 // operands are the same tile X, stacked as [Xh; Xl] along N: one MMA gives
 // [Xh Xh^T | Xh Xl^T] and the symmetrisation supplies Xl Xh^T.
 //
-// Pipeline (one persistent CTA per SM, 512 threads):
-//   warp 0        allocates tensor memory; lane 0 issues every MMA and the
-//                 commits that release shared-memory stages and hand finished
-//                 accumulators to the epilogue
+// Pipeline (one persistent CTA per SM; 512 threads, the Gram 768):
+//   warp 0        allocates tensor memory; waits as a whole and elects the lane
+//                 that issues a chunk's MMAs and the commits that release
+//                 shared-memory stages and hand finished accumulators to the
+//                 epilogue
+//   warp 1        reconstruct: bulk copies of the packed W blocks
 //   warps 4-7     epilogue: tcgen05.ld of the accumulator (warp w reads TMEM
 //                 lanes 32 (w % 4) .. +31), store to global memory (leg) or
 //                 add into compensated FP32 sums in shared memory (Gram)
-//   warps 8-15    converters: coalesced global loads (leg, reconstruct:
-//                 a register ring two or one chunks ahead; Gram: per-thread
-//                 cp.async into a ring of raw shared-memory stages four chunks
-//                 ahead), split, and 16-byte conflict-free stores into
-//                 the swizzled K-major layout the MMA descriptors describe
-//                 (below); the reconstruct's W block arrives by bulk copy
+//   warps 8-      converters in groups of 128 threads that take turns with the
+//                 chunks (leg, reconstruct: two groups, the next chunk of each
+//                 in a second set of registers; Gram: up to four groups, one
+//                 set each): coalesced global loads, split, and 16-byte
+//                 conflict-free stores into the swizzled K-major layout the MMA
+//                 descriptors describe (below)
 // Stages and accumulators are handed over with mbarriers.  Every wait is
 // bounded (a few seconds of %globaltimer); on expiry the kernel records bit 0
 // in *err (bit 1 marks a reconstruct item without its packed-W workspace),

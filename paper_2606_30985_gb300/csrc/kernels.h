@@ -65,11 +65,6 @@ __host__ __device__ inline int gram_rows_splits(long long K, int splits_max) {
   if (s < 1) s = 1;
   return (int)(s < splits_max ? s : splits_max);
 }
-// chunks of 32 (o, q) pairs: one o and 32 consecutive q when Q >= 32, else
-// floor(32 / Q) consecutive o with all q (tensor-core Gram)
-__host__ __device__ inline long long gram_leg_chunks(long long O, long long Q) {
-  return Q >= 32 ? O * ((Q + 31) / 32) : (O + (32 / Q) - 1) / (32 / Q);
-}
 // split count of a free-leg Gram from its summed extent K = O * Q, about `rows`
 // terms per split.  Tensor cores: 2048, 64 chunks of their pipeline.  SIMT: 512,
 // so that the Grams of small bonds (K = 2048 at chi = 8) still spread over
