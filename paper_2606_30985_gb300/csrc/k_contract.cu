@@ -299,14 +299,17 @@ cudaError_t launch_leg_contract(const LegItem* items, int n_items, int chimax, v
 // only: the Gram is symmetric, and this drops 44 % of the products for the
 // largest tile without a divergent branch.  The 256 / TX^2 groups of threads
 // take different units of a chunk, so a small F keeps the whole block busy;
-// the tile is chosen from the live F (8, 16, 32, 48, 64, 96, 128), not from
+// the tile is chosen from the live F (8, 16, 24, 32, 48, 64, 96, 128), not from
 // chi_max.  Their sums are laid side by side and added by one thread per entry: with
 // the groups adding one after another, a warp's FP64 operations (64 clocks each)
 // in 16 turns took longer than the products of a small split.  FP32 storage sums runs of 256 terms in FP32 and the runs in a
 // two-float sum; FP64 sums directly.
 //
-// Bound: FP32 ALU (2 shared 16-byte loads per 4 x MT x MT products at most) or
-// the FP64 pipe.  Class of a case, before -> now: chi = 8 FP64 (107 launches)
+// Bound: shared memory (a 16-byte load of a warp takes 4 clocks of the SM, 2 where
+// neighbouring lanes share it, and MT + MT of them feed 2 MT (MT + 1) products), so up
+// to F = 32 the threads of a group are 4 x 4 with as many entries each as that
+// takes: 24 clocks of loads per unit at F = 32 instead of 48 with 8 x 8 threads;
+// or the FP64 pipe.  Class of a case, before -> now: chi = 8 FP64 (107 launches)
 // 143 -> 1.8 ms, 4x4 chi = 12 FP64 154 -> 1.7 ms, 4x4 chi = 48 FP32 82 -> 25 ms.  The 64 x 64 (128 x 128) tile it replaces did 64 x 64 products
 // for an 8 x 8 Gram and stored every chunk with 32-way bank conflicts.
 constexpr int kGlStages = 3;
@@ -434,12 +437,18 @@ __device__ void gram_tile(const T* __restrict__ X, long long O, long long Q, int
       const int in = e % (TX * TX), i = TX * a + in / TX, j = TX * (a + b) + in % TX;
       if (i >= F || j >= F) continue;
       double z = 0.0;
+      TwoFloat t;
 #pragma unroll
       for (int gg = 0; gg < G; ++gg) {
         const V v = red[(gg * TL + i) * TL + j];
-        if constexpr (kF32) z += (double)v.x + (double)v.y;
-        else z += v;
+        if constexpr (kF32) {
+          t.take(v.x);
+          t.c += v.y;
+        } else {
+          z += v;
+        }
       }
+      if constexpr (kF32) z = t.value();
       P[(long long)i * F + j] = z;
       if (b > 0) P[(long long)j * F + i] = z;
     }
@@ -462,10 +471,10 @@ __device__ void gram_tile(const T* __restrict__ X, long long O, long long Q, int
 
 // Bands of F, a launch of its own for each that chi_max can reach, so that the
 // small tiles do not carry the large ones' registers (two blocks per SM up to
-// F = 48): blocks of the other bands return.
-constexpr int kGramBands[] = {32, 48, 64, 128};
+// F = 24 and for 33 .. 48): blocks of the other bands return.
+constexpr int kGramBands[] = {0, 24, 32, 48, 64, 128};
 template <typename T, int BAND>
-__global__ void __launch_bounds__(256, BAND < 2 ? 2 : 1)
+__global__ void __launch_bounds__(256, BAND == 0 || BAND == 2 ? 2 : 1)
 k_gram_leg(const GramLegItem* __restrict__ items, int splits_max, void* const* ptrs, const int* __restrict__ ival) {
   const GramLegItem it = items[blockIdx.y];
   int d[PEPO_MAXLEG];
@@ -479,9 +488,9 @@ k_gram_leg(const GramLegItem* __restrict__ items, int splits_max, void* const* p
     else if (i < k) O *= d[i];
     else Q *= d[i];                                    // legs beyond nlegs have size 1
   }
-  if (F > (BAND == 0 ? 32 : BAND == 1 ? 48 : BAND == 2 ? 64 : 128)) return;
-  if (F <= (BAND == 0 ? 0 : BAND == 1 ? 32 : BAND == 2 ? 48 : 64)) return;
-  const int S = gram_leg_splits_k(O * Q, splits_max, kGramLegRowsSimt);
+  constexpr int kAbove = BAND == 0 ? -1 : kGramBands[BAND], kUpTo = kGramBands[BAND + 1];
+  if (F <= kAbove || F > kUpTo) return;
+  const int S = gram_leg_splits_k(O * Q, splits_max, gram_leg_rows_simt(sizeof(T)));
   extern __shared__ __align__(16) unsigned char gl_sh[];
   const T* X = static_cast<const T*>(ptrs[it.x.ref]);
   for (int s = blockIdx.x; s < S; s += gridDim.x) {
@@ -489,10 +498,12 @@ k_gram_leg(const GramLegItem* __restrict__ items, int splits_max, void* const* p
     if constexpr (BAND == 0) {
       if (F <= 8) gram_tile<T, 2, 4>(X, O, Q, F, s, S, P, gl_sh);
       else if (F <= 16) gram_tile<T, 4, 4>(X, O, Q, F, s, S, P, gl_sh);
-      else gram_tile<T, 4, 8>(X, O, Q, F, s, S, P, gl_sh);
+      else gram_tile<T, 6, 4>(X, O, Q, F, s, S, P, gl_sh);
     } else if constexpr (BAND == 1) {
-      gram_tile<T, 6, 8>(X, O, Q, F, s, S, P, gl_sh);
+      gram_tile<T, 8, 4>(X, O, Q, F, s, S, P, gl_sh);
     } else if constexpr (BAND == 2) {
+      gram_tile<T, 6, 8>(X, O, Q, F, s, S, P, gl_sh);
+    } else if constexpr (BAND == 3) {
       gram_tile<T, 8, 8>(X, O, Q, F, s, S, P, gl_sh);
     } else {
       if (F <= 96) gram_tile<T, 6, 16>(X, O, Q, F, s, S, P, gl_sh);
@@ -504,9 +515,10 @@ k_gram_leg(const GramLegItem* __restrict__ items, int splits_max, void* const* p
 
 template <typename T, int BAND>
 size_t gram_leg_smem() {
-  if (BAND == 0) return std::max(std::max(GlCfg<T, 2, 4>::kSmem, GlCfg<T, 4, 4>::kSmem), GlCfg<T, 4, 8>::kSmem);
-  if (BAND == 1) return GlCfg<T, 6, 8>::kSmem;
-  if (BAND == 2) return GlCfg<T, 8, 8>::kSmem;
+  if (BAND == 0) return std::max(std::max(GlCfg<T, 2, 4>::kSmem, GlCfg<T, 4, 4>::kSmem), GlCfg<T, 6, 4>::kSmem);
+  if (BAND == 1) return GlCfg<T, 8, 4>::kSmem;
+  if (BAND == 2) return GlCfg<T, 6, 8>::kSmem;
+  if (BAND == 3) return GlCfg<T, 8, 8>::kSmem;
   return std::max(GlCfg<T, 6, 16>::kSmem, GlCfg<T, 8, 16>::kSmem);
 }
 
@@ -552,9 +564,10 @@ cudaError_t launch_gram_leg(const GramLegItem* items, int n_items, int splits_ma
                             void* const* ptrs, const int* ival, cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
   cudaError_t e = launch_gram_band<T, 0>(items, n_items, splits_max, ptrs, ival, s);
-  if (e == cudaSuccess && chimax > kGramBands[0]) e = launch_gram_band<T, 1>(items, n_items, splits_max, ptrs, ival, s);
-  if (e == cudaSuccess && chimax > kGramBands[1]) e = launch_gram_band<T, 2>(items, n_items, splits_max, ptrs, ival, s);
-  if (e == cudaSuccess && chimax > kGramBands[2]) e = launch_gram_band<T, 3>(items, n_items, splits_max, ptrs, ival, s);
+  if (e == cudaSuccess && chimax > kGramBands[1]) e = launch_gram_band<T, 1>(items, n_items, splits_max, ptrs, ival, s);
+  if (e == cudaSuccess && chimax > kGramBands[2]) e = launch_gram_band<T, 2>(items, n_items, splits_max, ptrs, ival, s);
+  if (e == cudaSuccess && chimax > kGramBands[3]) e = launch_gram_band<T, 3>(items, n_items, splits_max, ptrs, ival, s);
+  if (e == cudaSuccess && chimax > kGramBands[4]) e = launch_gram_band<T, 4>(items, n_items, splits_max, ptrs, ival, s);
   return e;
 }
 

@@ -66,11 +66,13 @@ __host__ __device__ inline int gram_rows_splits(long long K, int splits_max) {
   return (int)(s < splits_max ? s : splits_max);
 }
 // split count of a free-leg Gram from its summed extent K = O * Q, about `rows`
-// terms per split.  Tensor cores: 2048, 64 chunks of their pipeline.  SIMT: 512,
-// so that the Grams of small bonds (K = 2048 at chi = 8) still spread over
-// several SMs; the FP64 pipe of one SM needs 30 us for such a Gram alone.
+// terms per split.  Tensor cores: 2048, 64 chunks of their pipeline.  SIMT in FP64:
+// 512, so that the Grams of small bonds (K = 2048 at chi = 8) still spread over several
+// SMs (the FP64 pipe of one needs 30 us for such a Gram alone); in FP32 2048, as a
+// split also costs the sums of its groups (20 of 41 thousand clocks at chi = 20 with
+// 512 terms).
 constexpr int kGramLegRowsUmma = 2048;
-constexpr int kGramLegRowsSimt = 512;
+__host__ __device__ constexpr int gram_leg_rows_simt(size_t item_bytes) { return item_bytes == 8 ? 512 : 2048; }
 __host__ __device__ inline int gram_leg_splits_k(long long K, int splits_max, int rows) {
   long long s = K / rows;
   if (s < 1) s = 1;

@@ -1428,7 +1428,7 @@ pepo_status run_bp_waves(pepo_ctx* c, Inst& I, std::vector<BpWave>& waves) {
              gram_leg_dispatch<T>(c, w.gram.d, w.gram.n, chimax));
     LAUNCH_T(K_GRAM_LEG_RED, nullptr, w.gram.n,
              launch_gram_leg_reduce(w.gram.d, w.gram.n, chimax, c->tune.gram_leg_splits,
-                                    use_umma<T>(c, chimax) ? kGramLegRowsUmma : kGramLegRowsSimt,
+                                    use_umma<T>(c, chimax) ? kGramLegRowsUmma : gram_leg_rows_simt(sizeof(T)),
                                     use_umma<T>(c, chimax) ? 1 : 0, c->d_ival, s));
     LAUNCH_T(K_MSG, nullptr, w.rot.n, launch_rotate_back(w.rot.d, w.rot.n, chimax, c->d_ival, s));
     if (w.pw.n > 0) {
