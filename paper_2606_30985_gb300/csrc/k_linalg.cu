@@ -1657,9 +1657,12 @@ __device__ __noinline__ int jacobi_cluster(R* A, int m, int n, R* V, int max_swe
     JacRound jr;                                            // FP64
     float2 hs[32 * 32];                                     // FP32
   } rs;
-  // columns below 1e-30 (FP64) or 1e-13 (FP32) of the total squared norm are
-  // numerically zero in that precision
-  const R negligible = (R)((sizeof(R) == 4 ? 1e-13 : 1e-30) * fro);
+  // columns below 1e-30 (FP64) or 1e-22 (FP32) of the total squared norm are
+  // numerically zero: kept values reach 1e-11 of the largest, and the FP32 pass has
+  // to find their directions too (a rotation keeps a small column's relative
+  // accuracy; with 1e-13 the spectra of a 4x4, chi = 40 run were 3e-4 off after 19
+  // steps, now 4e-7)
+  const R negligible = (R)((sizeof(R) == 4 ? 1e-22 : 1e-30) * fro);
   const R abs_cut = (R)(abs_rel * fro);
   const int longest = max(m, n);                            // of a column: registers per lane
   const int room = (int)((kCoreSmem - 4096) / sizeof(R));
@@ -1858,6 +1861,11 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize
   const long long gw = ct.tid >> 5, ngw = ct.nthr >> 5;   // warps of the cluster
   if (threadIdx.x == 0) sh_capped = 0;
   if (ct.rank == 0 && threadIdx.x < 8) cflag[threadIdx.x] = 0;
+  __shared__ float mold[2][128];                   // square roots of the old messages' diagonals
+  for (int c = threadIdx.x; c < chic; c += blockDim.x) {
+    mold[0][c] = sqrtf((float)fmax(it.msg12[(long long)c * it.chimax + c], 0.0));
+    mold[1][c] = sqrtf((float)fmax(it.msg21[(long long)c * it.chimax + c], 0.0));
+  }
   for (int q = threadIdx.x; q < r; q += blockDim.x) order[it.perm1[q]] = q;   // position in R1's pivot order
   __syncthreads();
   for (long long e = ct.tid; e < (long long)k2 * r; e += ct.nthr) {
@@ -2177,6 +2185,33 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize
     }
   }
   cta_sync(ct);
+  // Sign of a singular pair (mixed path).  Single-layer BP starts from the positive
+  // square roots of the messages' diagonals, so a pair is turned the way in
+  // which the new index carries the old one's positive vector on the identity
+  // component of both sites.
+  __shared__ float turn[128];
+  for (int c = threadIdx.x; c < chi; c += blockDim.x) turn[c] = 0.f;
+  if (it.mixed_svd) {
+    for (int side = 0; side < 2; ++side) {
+      const int ks = side == 0 ? k1 : k2;
+      const int* perms = side == 0 ? it.perm1 : it.perm2;
+      const double* Fs = side == 0 ? it.FA : it.FB;
+      __syncthreads();
+      for (int q = threadIdx.x; q < r; q += blockDim.x) order[perms[q]] = q;
+      __syncthreads();
+      for (int c = threadIdx.x >> 5; c < chi; c += (int)(blockDim.x >> 5)) {
+        float x = 0.f;
+        for (int e = lane; e < r; e += 32) {
+          const int q = order[e];
+          if (q < ks) x = fmaf(mold[side][e / rg] * (float)Fs[(e % rg) * 16], (float)Zs[side][(long long)c * ks + q], x);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) turn[c] += x;
+      }
+    }
+  }
+  __syncthreads();
   // Y[(c,kappa), c'] = Z[q, c'] at original column perm[q] (zero for q >= ks)
   // W[(c,p), (c',p')] = sum_kappa F_kappa[p', p] Y[(c,kappa), c']
   for (int side = 0; side < 2; ++side) {
@@ -2197,7 +2232,7 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize
         const double y = q < ks ? Zs[side][(long long)c2 * ks + q] : 0.0;
         x += Fs[kk * 16 + p2 * 4 + p] * y;
       }
-      W[(long long)row * it.ldw + col] = x;
+      W[(long long)row * it.ldw + col] = turn[c2] < 0.f ? -x : x;
     }
   }
 }
