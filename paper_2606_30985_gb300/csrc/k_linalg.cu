@@ -1825,6 +1825,111 @@ __device__ __noinline__ int jacobi_cluster(R* A, int m, int n, R* V, int max_swe
   return sweep;
 }
 
+// Sign of a singular pair.  It is a gauge of the state that single-layer BP feels: it
+// starts from the positive square roots of the messages' diagonals and stops at a
+// tolerance, so signs left to rounding move C(t) by ~bp_tol^2 and may lead BP into
+// another fixed point.  The sign is therefore a function of the state alone: of
+// g_1 = X_1^T u and g_2 = X_2^T v (u, v the pair's vectors), which do not depend on
+// the order of the pivots or on the signs of reflections.  (Where X_1 has full rank
+// g_2 / sqrt(s) is the new index's column over the old ones, sqrt(s) X_1^+ u; where it
+// has not, that column is not unique, but g_2 is.)
+//
+// A pair is turned the way in which the new index carries the old messages' positive
+// vectors on the identity component: x = cos(m_1, g_2) + cos(m_2, g_1).  An index
+// made by the odd Schmidt factors of the gate alone has no identity component and
+// x is rounding noise; below kSignFloor the first entry of g_1 within 10 % of its
+// largest is made positive instead.
+//
+// Entries are taken to FP32 by integer operations (FP64 conversions hold the FP64 unit
+// for 64 clocks a warp); T is upper trapezoidal in the pivots' order.  A thread owns a
+// column of T and up to eight pairs, so T is read once per eight pairs; the pairs are
+// shared out over the cluster's CTAs.  Core class of a saturated layer, no rule (FP64)
+// or one that read FP32 noise -> this one: 4x4 chi = 12 FP64 4.05 -> 4.11 ms, 4x4
+// chi = 64 24.6 -> 24.5, 3x3 chi = 100 89.0 -> 90.1 (94 with a warp per pair, which reads
+// T once per pair).
+constexpr float kSignFloor = 1e-3f;
+struct FactorSide {
+  const double* T;         // k x r, leading dimension ld
+  const int* perm;         // original column of each position
+  int ld, k;
+};
+// vec(side, c): pair c's vector of that side times 2^(ex(side, c) - 1023) or less; m[side]:
+// r values each.  Signs of this CTA's pairs -> out.  sh: kSignSmem floats.
+constexpr int kSignPairs = 8;
+constexpr int kSignSmem = 3 * kSignPairs * kCoreThreads;
+template <class Vec, class Ex>
+__device__ __noinline__ void pair_signs(const FactorSide s1, const FactorSide s2, int r, int chi, Vec vec, Ex ex,
+                                        const float* m, const Cta& ct, double* out, float* sh) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int r32 = (r + 31) & ~31, ng = kCoreThreads / r32;   // r <= kCoreMaxDim = the threads
+  const int grp = threadIdx.x / r32, q = threadIdx.x - grp * r32;
+  float* us = sh;                                            // [group][row][pair of the group]
+  float* gs = sh + kSignPairs * kCoreThreads;                // [side][pair][r32]
+  const int per = (chi + ct.size - 1) / ct.size;
+  const int end = min(chi, (ct.rank + 1) * per);
+  for (int c0 = ct.rank * per; c0 < end; c0 += kSignPairs * ng) {
+    const int n = min(kSignPairs * ng, end - c0);            // pair c0 + i: group i % ng, slot i / ng
+    for (int side = 0; side < 2; ++side) {
+      const FactorSide s = side == 0 ? s1 : s2;
+      __syncthreads();
+      for (int e = threadIdx.x; e < n * s.k; e += kCoreThreads) {
+        const int i = e / s.k, a = e - i * s.k;
+        us[((i % ng) * s.k + a) * kSignPairs + i / ng] = top_float(vec(side, c0 + i)[a], ex(side, c0 + i));
+      }
+      __syncthreads();
+      if (grp < ng && grp < n) {
+        const int et = s.k > 0 ? (__double2hiint(s.T[0]) >> 20) & 0x7ff : 0;   // the largest column's norm
+        const int rows = min(s.k, (q | 31) + 1);
+        const float4* u = reinterpret_cast<const float4*>(us + (size_t)grp * s.k * kSignPairs);
+        float g[kSignPairs] = {};
+#pragma unroll 8
+        for (int a = 0; a < rows; ++a) {
+          const float t = a <= q && q < r ? top_float(s.T[(long long)a * s.ld + q], et) : 0.f;
+          const float4 x = u[2 * a], y = u[2 * a + 1];
+          g[0] = fmaf(t, x.x, g[0]); g[1] = fmaf(t, x.y, g[1]); g[2] = fmaf(t, x.z, g[2]); g[3] = fmaf(t, x.w, g[3]);
+          g[4] = fmaf(t, y.x, g[4]); g[5] = fmaf(t, y.y, g[5]); g[6] = fmaf(t, y.z, g[6]); g[7] = fmaf(t, y.w, g[7]);
+        }
+#pragma unroll
+        for (int p = 0; p < kSignPairs; ++p)
+          if (p * ng + grp < n) gs[(side * kSignPairs * ng + p * ng + grp) * r32 + q] = g[p];
+      }
+    }
+    __syncthreads();
+    for (int i = wid; i < n; i += kCoreThreads / 32) {
+      float x = 0.f, turn = 1.f;
+      for (int side = 0; side < 2; ++side) {
+        const FactorSide s = side == 0 ? s1 : s2;
+        const float* g = gs + (side * kSignPairs * ng + i) * r32;
+        const float* w = m + (1 - side) * r;                 // m_2 meets g_1, m_1 meets g_2
+        float d = 0.f, gg = 0.f, mm = 0.f, top = 0.f;
+        for (int j = lane; j < r; j += 32) {
+          const float v = g[j], z = w[s.perm[j]];
+          d = fmaf(v, z, d);
+          gg = fmaf(v, v, gg);
+          mm = fmaf(z, z, mm);
+          top = fmaxf(top, fabsf(v));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          d += __shfl_xor_sync(0xffffffffu, d, o);
+          gg += __shfl_xor_sync(0xffffffffu, gg, o);
+          mm += __shfl_xor_sync(0xffffffffu, mm, o);
+          top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+        }
+        if (gg > 0.f && mm > 0.f) x += d * rsqrtf(gg) * rsqrtf(mm);
+        if (side == 0) {
+          int first = 4 * kCoreMaxDim;                       // 2 x column + (negative)
+          for (int j = lane; j < r; j += 32)
+            if (fabsf(g[j]) >= 0.9f * top) first = min(first, 2 * s.perm[j] + (g[j] < 0.f ? 1 : 0));
+          first = __reduce_min_sync(0xffffffffu, first);
+          turn = first & 1 ? -1.f : 1.f;
+        }
+      }
+      if (lane == 0) out[c0 + i] = fabsf(x) > kSignFloor ? x : turn;
+    }
+  }
+}
+
 // Bond core, one cluster per bond.  Bound: the FP64 pipe (T_core = R1 R2^T, T Q
 // and the FP64 Jacobi: 2 multiply-adds per clock and SM) and the shared-memory
 // bandwidth of the FP32 Jacobi, both spread over the cluster's SMs; one CTA
@@ -2112,6 +2217,23 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize
     }
   }
   cta_sync(ct);
+  // Signs of the singular pairs -> cnorm; msh[side][e]: what the side's old positive
+  // vector brings to column e = (c, kappa) of X.
+  {
+    float* msh = reinterpret_cast<float*>(core_sh) + kSignSmem;
+    for (int e = threadIdx.x; e < 2 * r; e += blockDim.x) {
+      const int side = e >= r, col = e - side * r;
+      msh[e] = mold[side][col / rg] * (float)(side == 0 ? it.FA : it.FB)[(col % rg) * 16];
+    }
+    // columns of Tc are s_c times their side's vectors
+    auto vec = [&](int side, int c) -> const double* {
+      if ((side == 0) != tr) return Tc + (long long)order[c] * M;
+      return it.mixed_svd ? Vr + (long long)c * N : V + (long long)order[c] * N;
+    };
+    auto ex = [&](int side, int c) { return (side == 0) != tr ? (__double2hiint(sv[order[c]]) >> 20) & 0x7ff : 1023; };
+    pair_signs({it.T1, it.perm1, it.ldt1, k1}, {it.T2, it.perm2, it.ldt2, k2}, r, chi, vec, ex, msh, ct, cnorm,
+               reinterpret_cast<float*>(core_sh));
+  }
   // For each side: Z_s = T_s11^{-1} (singular vectors of that side) sqrt(s) / sqrt(sum s);
   // side 1 vectors: left vectors of Tcore (rows of R1 space, length k1), side 2
   // vectors: right vectors (length k2).  Both sides at once, the columns
@@ -2185,33 +2307,8 @@ k_core(const CoreItem* __restrict__ items, int* ival, int* flags_base, int csize
     }
   }
   cta_sync(ct);
-  // Sign of a singular pair (mixed path).  Single-layer BP starts from the positive
-  // square roots of the messages' diagonals, so a pair is turned the way in
-  // which the new index carries the old one's positive vector on the identity
-  // component of both sites.
   __shared__ float turn[128];
-  for (int c = threadIdx.x; c < chi; c += blockDim.x) turn[c] = 0.f;
-  if (it.mixed_svd) {
-    for (int side = 0; side < 2; ++side) {
-      const int ks = side == 0 ? k1 : k2;
-      const int* perms = side == 0 ? it.perm1 : it.perm2;
-      const double* Fs = side == 0 ? it.FA : it.FB;
-      __syncthreads();
-      for (int q = threadIdx.x; q < r; q += blockDim.x) order[perms[q]] = q;
-      __syncthreads();
-      for (int c = threadIdx.x >> 5; c < chi; c += (int)(blockDim.x >> 5)) {
-        float x = 0.f;
-        for (int e = lane; e < r; e += 32) {
-          const int q = order[e];
-          if (q < ks) x = fmaf(mold[side][e / rg] * (float)Fs[(e % rg) * 16], (float)Zs[side][(long long)c * ks + q], x);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) turn[c] += x;
-      }
-    }
-  }
-  __syncthreads();
+  for (int c = threadIdx.x; c < chi; c += blockDim.x) turn[c] = (float)cnorm[c];
   // Y[(c,kappa), c'] = Z[q, c'] at original column perm[q] (zero for q >= ks)
   // W[(c,p), (c',p')] = sum_kappa F_kappa[p', p] Y[(c,kappa), c']
   for (int side = 0; side < 2; ++side) {
