@@ -182,6 +182,7 @@ struct SiteFacItem {
   int* perm;               // pivot order (r entries)
   int rank_idx;            // ival: rank of the factor
   double rel;              // rank threshold
+  double rel_exact;        // of a factor from an exact Gram (FP32 storage)
   double rel_safe;         // smallest fraction of its column's Gram diagonal a Cholesky-QR pivot keeps
   int n_thr;               // Eq. 10 branch thresholds of the instance
   double ratio_thr;

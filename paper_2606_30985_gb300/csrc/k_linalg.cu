@@ -1018,23 +1018,23 @@ k_factor(const SiteFacItem* __restrict__ items, int* ival, int only, unsigned lo
   int* pos = reinterpret_cast<int*>(fsh + S.pos);
   int* perm = reinterpret_cast<int*>(fsh + S.perm);
   const size_t room = S.total - S.mat;
-  auto chol = [&](auto* zero, const double* A, int lda, int k, auto* scratch, double safe, auto*& U) -> int {
+  auto chol = [&](auto* zero, const double* A, int lda, int k, auto* scratch, double rel, double safe, auto*& U) -> int {
     using R = std::remove_reference_t<decltype(*zero)>;
     const int w = (k + csize - 1) / csize;
     U = sizeof(R) * (size_t)k * w <= room ? reinterpret_cast<R*>(mat) : scratch + (long long)ct.rank * w * k;
     return chol_cluster<R>(A, lda, k, w, U, ct, offer, reinterpret_cast<R*>(fsh + S.cand), ldo,
                            reinterpret_cast<R*>(fsh + S.uc), reinterpret_cast<R*>(fsh + S.part),
-                           reinterpret_cast<R*>(fsh + S.dq), reinterpret_cast<R*>(fsh + S.oq), pos, perm, it.rel, safe);
+                           reinterpret_cast<R*>(fsh + S.dq), reinterpret_cast<R*>(fsh + S.oq), pos, perm, rel, safe);
   };
   double* scratch = T + (long long)2 * ld * ld;      // behind T and G: 2 ld^2 doubles
   if (branch == 1) {
     int ok;
     if (it.rel_safe >= 1e-6) {
       float* U;
-      ok = chol((float*)nullptr, it.C, it.ldc, n, reinterpret_cast<float*>(scratch), it.rel_safe, U);
+      ok = chol((float*)nullptr, it.C, it.ldc, n, reinterpret_cast<float*>(scratch), it.rel, it.rel_safe, U);
     } else {
       double* U;
-      ok = chol((double*)nullptr, it.C, it.ldc, n, scratch, it.rel_safe, U);
+      ok = chol((double*)nullptr, it.C, it.ldc, n, scratch, it.rel, it.rel_safe, U);
     }
     if (ct.tid == 0 && qcount) atomicAdd(&qcount[ok >= 0 ? 1 : 2], 1ull);
     cta_sync(ct);                                    // the last offers are read, every CTA has its branch
@@ -1045,7 +1045,7 @@ k_factor(const SiteFacItem* __restrict__ items, int* ival, int only, unsigned lo
   }
   if (branch == 1 || !householder) {
     double* U;
-    const int rank = chol((double*)nullptr, T + (long long)ld * ld, ld, r, scratch, -1.0, U);
+    const int rank = chol((double*)nullptr, T + (long long)ld * ld, ld, r, scratch, branch == 1 ? it.rel : it.rel_exact, -1.0, U);
     // columns that never became a pivot follow in their own order
     const int w = (r + csize - 1) / csize, c0 = ct.rank * w;
     const int nl = min(w, r - c0);

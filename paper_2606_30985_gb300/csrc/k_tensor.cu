@@ -1,7 +1,7 @@
 // HBM-bound tensor kernels of the bond update and of BP.
 //
 //   k_gram_rows32/64 cv^T cv (Eq. 10, Cholesky-QR Gram)
-//   k_gram_exact     cv^T cv of FP32 data to ~47 bits (FP32 storage: the sites of the
+//   k_gram_exact     cv^T cv of FP32 data to FP64 accuracy (FP32 storage: the sites of the
 //                    Householder side of Eq. 10 and those whose Gram fails its test)
 //   k_reconstruct, k_reconstruct32   psi_new = psi W written in the next update's layout
 //                    (Sec. 2.5 steps 6-7 in Q-less form, Alg. 1 lines 9-12)
@@ -293,28 +293,32 @@ cudaError_t launch_gram_rows_reduce(const GramRowsItem* items, int n_items, int 
 
 
 // ======================================================= exact Gram (rows)
-// C = cv^T cv of FP32 data to about 47 bits, for the sites the branch rule of
-// Eq. 10 sends to Householder and for those whose FP32-run Gram failed the
-// trust test.  A pivoted Cholesky of this C is as good a factor of cv as a
-// Householder QR in FP32: QR perturbs a column by ~6e-8 of its norm, this
-// Gram's ~1e-14 moves a direction that keeps a share e of it by 1e-14 / e,
-// which is smaller for every direction the rank cut leaves (e > 3e-7).
+// C = cv^T cv of FP32 data to the accuracy of FP64 sums, for the sites the branch
+// rule of Eq. 10 sends to Householder and for those whose FP32-run Gram failed the
+// trust test.  A pivoted Cholesky of this C finds every direction that keeps more
+// than 1e-7 of the largest (1e-14 of the squares; the Gram's entries are within ~5e-16
+// of the paired columns' norms at 64 rows and less above).
 //
-// Sum: an accumulator s starts at the anchor 3 P_i P_j, P the next power of two
-// above the run's column norm, so by Cauchy-Schwarz s stays in one binade and
-// every addition rounds to the same grid: with s' = fma(a, b, s), h = s' - s is
-// exact and fma(a, b, -h) is what the rounding left over.  Four FP32
-// operations a term instead of one FP64 multiply-add, which takes 64 issue
-// slots here; a double-float sum takes ten.  Runs of 64 rows go into a
-// two-float sum (S, C), the splits into FP64.  Columns are scaled to a largest
+// Sum: the product's rounded part p and its rest q = ab - p; p goes into an
+// accumulator s that starts at the anchor 3 P_i P_j, P the next power of two above the
+// run's column norm, so by Cauchy-Schwarz s stays in one binade and what it leaves
+// over, r, is at most 2^-23 P_i P_j.  The r go the same way into a second
+// accumulator c, anchored 2^-17 lower, and what that leaves over (2^-40) and q into
+// a third, d, in plain FP32: ten FP32 operations a term instead of one FP64
+// multiply-add, which takes 64 issue slots here.  (With the r summed in plain FP32,
+// four operations a term, an entry was 1e-12 off at 64 rows and a Cholesky took
+// its noise for directions.)  A run's 64 rows go into (S, U, W), each the rounding of
+// the one before, the splits into FP64.  Columns are scaled to a largest
 // magnitude in [1/2, 1) first (k_col_scale), so tiny tensors do not underflow.
 //
-// 64 x 64 tiles, 4 x 4 entries a thread (64 FP32 operations per two 16-byte
-// shared loads: ALU-bound), 16-byte asynchronous copies one run ahead.
+// 64 x 64 tiles, 4 x 4 entries a thread (160 FP32 operations per two 16-byte
+// shared loads: ALU-bound), 16-byte asynchronous copies one run ahead; U and W lie
+// in shared memory, which leaves two blocks an SM.
 // K splits: rows per split ~512, at most kExactSplits.
 constexpr int GX_T = 64;
 constexpr int GX_RUN = 64;
 constexpr int kExactSplits = 60;
+constexpr float kGxLower = 1.f / 131072.f;   // 64 remainders of 2^-23 P_i P_j stay below 2^-17
 
 __device__ inline float pow2f(int e) { return __int_as_float((min(max(e, -126), 127) + 127) << 23); }
 
@@ -381,7 +385,8 @@ k_gram_exact(const GramRowsItem* __restrict__ items, int pass, void* const* ptrs
   const bool diag = ti == tj;
   const long long k0 = K * sp / S, k1 = K * (sp + 1) / S;
   const float* __restrict__ X = static_cast<const float*>(ptrs[it.x.ref]);
-  extern __shared__ __align__(16) float gx_sh[];      // 2 buffers of [X tile | Y tile], 64 rows x 64 columns each
+  // 2 buffers of [X tile | Y tile], 64 rows x 64 columns each; then U and W, 16 values a thread
+  extern __shared__ __align__(16) float gx_sh[];
   __shared__ float nrm[2][2 * GX_T];                   // half sums of squares per column
   __shared__ float pw[2 * GX_T];                       // P per column
   __shared__ float sc[2 * GX_T];                       // column pre-scale 2^-e
@@ -404,11 +409,15 @@ k_gram_exact(const GramRowsItem* __restrict__ items, int pass, void* const* ptrs
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  float Sh[4][4], Cl[4][4];
+  float S0[4][4];
+  float* UW = gx_sh + 4 * GX_RUN * GX_T + tid;         // U at 512 e, W at 512 e + 256
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) Sh[a][b] = Cl[a][b] = 0.f;
+    for (int b = 0; b < 4; ++b) {
+      S0[a][b] = 0.f;
+      UW[512 * (4 * a + b)] = UW[512 * (4 * a + b) + 256] = 0.f;
+    }
   if (k0 < k1) load(0, k0);
   int buf = 0;
   for (long long kb = k0; kb < k1; kb += GX_RUN, buf ^= 1) {
@@ -444,15 +453,16 @@ k_gram_exact(const GramRowsItem* __restrict__ items, int pass, void* const* ptrs
       pw[tid] = pow2f(max((e + 2) >> 1, -50));                 // P^2 > q
     }
     __syncthreads();
-    float P[4], Q[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) { P[a] = pw[ty * 4 + a]; Q[a] = pw[GX_T + tx * 4 + a]; }
-    float s[4][4], c[4][4];
+    float s[4][4], c[4][4], d[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int b = 0; b < 4; ++b) { s[a][b] = 3.f * (P[a] * Q[b]); c[a][b] = 0.f; }
-#pragma unroll 8
+      for (int b = 0; b < 4; ++b) {
+        s[a][b] = 3.f * (pw[ty * 4 + a] * pw[GX_T + tx * 4 + b]);
+        c[a][b] = kGxLower * s[a][b];
+        d[a][b] = 0.f;
+      }
+#pragma unroll 4
     for (int kk = 0; kk < GX_RUN; ++kk) {
       const float4 xa = *reinterpret_cast<const float4*>(xs + kk * GX_T + ty * 4);
       const float4 yb = *reinterpret_cast<const float4*>(ys + kk * GX_T + tx * 4);
@@ -461,20 +471,33 @@ k_gram_exact(const GramRowsItem* __restrict__ items, int pass, void* const* ptrs
       for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-          const float t = fmaf(a4[a], b4[b], s[a][b]);
-          const float h = t - s[a][b];
-          c[a][b] += fmaf(a4[a], b4[b], -h);
+          const float p = __fmul_rn(a4[a], b4[b]);
+          const float q = fmaf(a4[a], b4[b], -p);
+          const float t = __fadd_rn(s[a][b], p);
+          const float r = __fsub_rn(p, __fsub_rn(t, s[a][b]));
+          const float u = __fadd_rn(c[a][b], r);
+          d[a][b] += __fsub_rn(r, __fsub_rn(u, c[a][b]));
+          d[a][b] += q;
           s[a][b] = t;
+          c[a][b] = u;
         }
     }
+    // the run's sum into (S, U, W)
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
-        const float v = s[a][b] - 3.f * (P[a] * Q[b]);          // exact
-        const float t = Sh[a][b] + v, bb = t - Sh[a][b];
-        Cl[a][b] += ((Sh[a][b] - (t - bb)) + (v - bb)) + c[a][b];
-        Sh[a][b] = t;
+        const float anchor = 3.f * (pw[ty * 4 + a] * pw[GX_T + tx * 4 + b]);
+        float* uw = UW + 512 * (4 * a + b);
+        TwoFloat hi, mid;                                      // c: what the sum leaves over
+        hi.s = S0[a][b];
+        hi.take(s[a][b] - anchor);                             // exact difference
+        mid.s = uw[0];
+        mid.take(c[a][b] - kGxLower * anchor);                 // exact too
+        mid.take(hi.c);
+        S0[a][b] = hi.s;
+        uw[0] = mid.s;
+        uw[256] += mid.c + d[a][b];
       }
     __syncthreads();                                           // the buffer is refilled next
   }
@@ -488,7 +511,8 @@ k_gram_exact(const GramRowsItem* __restrict__ items, int pass, void* const* ptrs
     for (int b = 0; b < 4; ++b) {
       const int fj = tj * GX_T + tx * 4 + b;
       if (fj < F) {
-        const double v = (double)Sh[a][b] + (double)Cl[a][b];
+        const float* uw = UW + 512 * (4 * a + b);
+        const double v = (double)S0[a][b] + ((double)uw[0] + (double)uw[256]);
         Pt[(long long)fi * F + fj] = scalbn(v, ei + col_exp(it.colmax[fj]));
       }
     }
@@ -528,7 +552,7 @@ cudaError_t launch_gram_exact(const GramRowsItem* items, int n_items, int fmax, 
   if (n_items == 0) return cudaSuccess;
   k_col_scale<<<dim3(1, n_items), 256, 0, s>>>(items, pass, 0, ptrs, ival);
   k_col_scale<<<dim3(64, n_items), 256, 0, s>>>(items, pass, 1, ptrs, ival);
-  const size_t smem = sizeof(float) * 4 * GX_RUN * GX_T;
+  const size_t smem = sizeof(float) * (4 * GX_RUN * GX_T + 2 * GX_T * GX_T);
   cudaError_t e = cudaFuncSetAttribute(k_gram_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int nt = ceil_div(fmax, GX_T);

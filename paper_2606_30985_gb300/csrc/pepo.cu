@@ -512,12 +512,17 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
 
   // ---- gate-update waves
   const double rel_fac = (c->prec == PEPO_FP64) ? 1e-15 : 1e-13;
+  // exact Grams of FP32 data (~5e-16 of the paired columns' norms: the pivots of a
+  // rank-deficient one end at 3e-15 of the first): directions above 1e-7 of the
+  // largest.  With 1e-13 the spectra of a 4x4, chi = 20 FP32 evolution of six steps
+  // were 1.5e-7 off 64 bits, with 1e-14 2.2e-8, with a Householder TSQR in FP64 1.9e-8.
+  const double rel_exact = 1e-14;
   // smallest fraction of a column's own Gram diagonal that a Cholesky-QR
   // pivot must keep: far above the Gram's relative rounding (FP32-storage
   // Gram: ~1e-8 of the paired columns' scale; FP64: ~1e-14) and the FP32
   // pivot check's own (~1e-6), where the pivots of columns that depend
-  // linearly on the others land; below it the site takes the Householder
-  // branch
+  // linearly on the others land; below it the site takes the other branch
+  // (Householder in FP64 storage, the exact Gram in FP32 storage)
   const double rel_safe = (c->prec == PEPO_FP64) ? 1e-10 : 1e-4;
   const double rel_env = I.cfg.pinv_rel;
   for (int col = 0; col < 4; ++col) {
@@ -632,6 +637,7 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
           f.perm = sws[v].perm;
           f.rank_idx = sws[v].rankT_idx;
           f.rel = rel_fac;
+          f.rel_exact = rel_exact;
           f.rel_safe = rel_safe;
           f.n_thr = I.cfg.qr_n_thresh;
           f.ratio_thr = I.cfg.qr_ratio_thresh;
@@ -1357,11 +1363,9 @@ pepo_status run_gate_wave(pepo_ctx* c, Inst& I, GateWave& w) {
   // R-factor of the sites with branch value `pass` (0: the Householder branch of
   // Eq. 10; 2: the Cholesky-branch sites whose Gram was too ill-conditioned).
   // FP64 storage: Householder TSQR.  FP32 storage: the exact Gram of the FP32
-  // data, whose Cholesky factor carries no more error than FP32 reflections
-  // (k_gram_exact).  Both sides, TSQR and its column-pivoted factor against exact
-  // Gram and Cholesky, per saturated layer: 4x4 chi = 64 229 -> 34 ms, 4x4 chi = 48
-  // 155 -> 16 ms, 3x5 chi = 27 50 -> 4 ms; 3x3 chi = 100 (two interior and eight
-  // corner factors) 443 -> 86 ms.
+  // data, whose Cholesky factor carries no more error (k_gram_exact).  Both
+  // sides, TSQR and its column-pivoted factor against exact Gram and Cholesky, classes
+  // of a saturated layer: 4x4 chi = 64 544 -> 26 ms, 3x3 chi = 100 545 -> 63 ms.
   const int householder = sizeof(T) == 8 ? 1 : 0;
   auto factor_rows = [&](int pass) -> pepo_status {
     if (!householder) {
