@@ -186,7 +186,8 @@ pepo_status pepo_trotter_colour(pepo_ctx* ctx, int colour);
  * Synchronises the stream.  Errors: PEPO_E_INVALID (NULL context),
  * PEPO_E_CUDA (a launch or read-back failed, or a tensor-core pipeline wait
  * ran out of time: the kernels return instead of hanging and the call fails
- * with that message). */
+ * with that message; pepo_diag.flags keeps what the calls before the one that ran
+ * out had raised). */
 pepo_status pepo_bp_converge(pepo_ctx* ctx, int* sweeps_out, double* delta_out);
 
 /* Single-layer BP on the pinned network and the Bethe value of C(t)

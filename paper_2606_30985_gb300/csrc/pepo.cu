@@ -177,6 +177,7 @@ struct pepo_ctx {
   unsigned long long* d_delta2 = nullptr;
   unsigned long long* d_delta1 = nullptr;
   int* d_flags = nullptr;
+  int* d_flags_kept = nullptr;   // the flags before the first call since the error word was clear
   unsigned long long* d_qr_count = nullptr;   // sites per QR branch (k_factor)
   double* d_hh_acct = nullptr;   // Householder QR FLOPs and bytes (k_hh_extract; timing class K_HH)
   int* d_kerr = nullptr;   // bit 0: a tensor-core pipeline wait expired (bits: launch_leg_umma)
@@ -1160,6 +1161,7 @@ size_t layout_arena(pepo_ctx* c, char* base, Planner* keep) {
   c->d_delta2 = cv.take<unsigned long long>(c->n_inst);
   c->d_delta1 = cv.take<unsigned long long>(c->n_inst);
   c->d_flags = cv.take<int>(c->n_inst);
+  c->d_flags_kept = cv.take<int>(c->n_inst);
   c->d_kerr = cv.take<int>(1);
   c->d_qr_count = cv.take<unsigned long long>(3);
   c->d_hh_acct = cv.take<double>(2);
@@ -1291,15 +1293,30 @@ void timing_harvest(pepo_ctx* c) {
 // A tensor-core kernel's error word was set: report it once and clear it, so
 // that the context stays usable (its state is undefined until restored or
 // re-uploaded).  The flags that the kernels behind the aborted one raised on
-// its unwritten results (a rank-0 bond core, a zero trace) go with it.
+// its unwritten results (a rank-0 bond core, a zero trace) go with it; those of
+// the calls before it stay (keep_flags).
 pepo_status kernel_error(pepo_ctx* c, int kerr) {
   cudaMemsetAsync(c->d_kerr, 0, sizeof(int), c->stream);
-  cudaMemsetAsync(c->d_flags, 0, sizeof(int) * c->n_inst, c->stream);
+  cudaMemcpyAsync(c->d_flags, c->d_flags_kept, sizeof(int) * c->n_inst, cudaMemcpyDeviceToDevice, c->stream);
   cudaStreamSynchronize(c->stream);
   return fail(c, PEPO_E_CUDA,
               "tensor-core kernel error word %d (bit 0: a pipeline wait ran longer than the wait limit, "
               "bit 1: missing packed-W workspace, bit 2: an exit drain ran out of time); the state is "
               "undefined until it is restored or uploaded again", kerr);
+}
+
+// Copy of the flags at the start of a call, unless an earlier call has already set
+// the error word (its flags are not to be trusted, and nobody has been told yet).
+__global__ void k_keep_flags(const int* flags, int* kept, int n, const int* kerr) {
+  if (*kerr != 0) return;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) kept[i] = flags[i];
+}
+pepo_status keep_flags(pepo_ctx* c) {
+  if (c->prec != PEPO_TF32X3) return PEPO_OK;              // no other kernel sets the word
+  k_keep_flags<<<1, 256, 0, c->stream>>>(c->d_flags, c->d_flags_kept, c->n_inst, c->d_kerr);
+  c->launches++;
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? PEPO_OK : fail(c, PEPO_E_CUDA, "flag copy: %s", cudaGetErrorString(e));
 }
 
 // Every launch wrapper returns without launching when its item count is 0;
@@ -1937,6 +1954,7 @@ pepo_status pepo_init(const pepo_config* cfgs, int n_inst, void* dev_arena, size
   ok = ok && cudaMemcpyAsync(c->d_items, P.st.bytes.data(), P.st.bytes.size(), cudaMemcpyHostToDevice,
                              s) == cudaSuccess;
   ok = ok && cudaMemsetAsync(c->d_flags, 0, sizeof(int) * n_inst, s) == cudaSuccess;
+  ok = ok && cudaMemsetAsync(c->d_flags_kept, 0, sizeof(int) * n_inst, s) == cudaSuccess;
   ok = ok && cudaMemsetAsync(c->d_kerr, 0, sizeof(int), s) == cudaSuccess;
   ok = ok && cudaMemsetAsync(c->d_qr_count, 0, 3 * sizeof(unsigned long long), s) == cudaSuccess;
   ok = ok && cudaMemsetAsync(c->d_hh_acct, 0, 2 * sizeof(double), s) == cudaSuccess;
@@ -2015,7 +2033,8 @@ pepo_status pepo_trotter_step(pepo_ctx* c, int n_steps) {
   if (n_steps < 0) return fail(c, PEPO_E_INVALID, "n_steps must be >= 0");
   if (!at_step_boundary(c, "pepo_trotter_step")) return PEPO_E_STATE;
   timing_begin(c);
-  pepo_status st = c->tsize == 8 ? do_steps<double>(c, n_steps) : do_steps<float>(c, n_steps);
+  pepo_status st = keep_flags(c);
+  if (st == PEPO_OK) st = c->tsize == 8 ? do_steps<double>(c, n_steps) : do_steps<float>(c, n_steps);
   return st;
 }
 
@@ -2026,7 +2045,8 @@ pepo_status pepo_trotter_colour(pepo_ctx* c, int colour) {
     return fail(c, PEPO_E_STATE, "colour %d out of order: the current step has colours 0..%d applied, "
                 "the next is %d", colour, c->phase - 1, c->phase);
   timing_begin(c);
-  pepo_status st = c->tsize == 8 ? colour_launches<double>(c, colour) : colour_launches<float>(c, colour);
+  pepo_status st = keep_flags(c);
+  if (st == PEPO_OK) st = c->tsize == 8 ? colour_launches<double>(c, colour) : colour_launches<float>(c, colour);
   if (st != PEPO_OK) return st;
   c->phase = (colour + 1) % 4;
   if (c->phase == 0) {
@@ -2068,7 +2088,8 @@ pepo_status pepo_bp_converge(pepo_ctx* c, int* sweeps_out, double* delta_out) {
     if (ws != PEPO_OK) return ws;
   }
   timing_begin(c);
-  pepo_status st = c->tsize == 8 ? do_bp<double>(c, sweeps_out, delta_out) : do_bp<float>(c, sweeps_out, delta_out);
+  pepo_status st = keep_flags(c);
+  if (st == PEPO_OK) st = c->tsize == 8 ? do_bp<double>(c, sweeps_out, delta_out) : do_bp<float>(c, sweeps_out, delta_out);
   timing_harvest(c);
   return st;
 }
@@ -2077,7 +2098,8 @@ pepo_status pepo_correlator(pepo_ctx* c, double* C_out, pepo_diag* diag_out) {
   if (!c) return PEPO_E_INVALID;
   if (!at_step_boundary(c, "pepo_correlator")) return PEPO_E_STATE;
   timing_begin(c);
-  pepo_status st = c->tsize == 8 ? do_correlator<double>(c, C_out, diag_out) : do_correlator<float>(c, C_out, diag_out);
+  pepo_status st = keep_flags(c);
+  if (st == PEPO_OK) st = c->tsize == 8 ? do_correlator<double>(c, C_out, diag_out) : do_correlator<float>(c, C_out, diag_out);
   timing_harvest(c);
   return st;
 }
