@@ -428,7 +428,8 @@ pepo_status pepo_set_wait_limit(pepo_ctx* ctx, double seconds);
  * read.  Synchronises the stream.  Errors: PEPO_E_INVALID (null), PEPO_E_CUDA. */
 pepo_status pepo_qr_branch_counts(pepo_ctx* ctx, long long* out, int reset);
 
-/* Number of kernel launches enqueued by this context so far. */
+/* Number of kernel launches enqueued by this context so far (a sweep of a BP loop as
+ * many as the direct launches have: the kernel that closes it is not counted). */
 long long pepo_launch_count(const pepo_ctx* ctx);
 
 /* Last error message of the context (static string if ctx is NULL). */

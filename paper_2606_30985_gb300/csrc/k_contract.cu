@@ -46,7 +46,6 @@ __device__ inline void load_dims4(const TView& v, const int* ival, int* d) {
 template <typename T> struct LegBlock;
 template <> struct LegBlock<float> { static constexpr int NT = 256, CTAS = 2; };
 template <> struct LegBlock<double> { static constexpr int NT = 64, CTAS = 8; };
-constexpr int kLegMaxItems = 512;                      // of a launch
 constexpr int kLegRows = 8, kLegStages = 3;
 template <typename T, int MI, int TI>
 struct LegCfg {
@@ -201,7 +200,7 @@ template <typename T>
 __global__ void __launch_bounds__(LegBlock<T>::NT, LegBlock<T>::CTAS)
 k_leg_contract(const LegItem* __restrict__ items, int n_items, void* const* ptrs, const int* __restrict__ ival) {
   extern __shared__ __align__(16) unsigned char lc_sh[];
-  __shared__ unsigned toff[kLegMaxItems + 1];          // tiles before each item
+  __shared__ unsigned toff[kMaxItems + 1];          // tiles before each item
   auto extents = [&](const LegItem& it, int& J, unsigned& O, unsigned& QU) {
     int d[PEPO_MAXLEG];
     load_dims4(it.in, ival, d);
@@ -278,8 +277,8 @@ cudaError_t launch_leg_contract(const LegItem* items, int n_items, int chimax, v
     smem = std::max(smem, sizeof(T) * (size_t)chimax * ti + (size_t)kLegStages * kLegRows * (leg_tu<T>(ti) + 1) * 16);
   cudaError_t e = cudaFuncSetAttribute(k_leg_contract<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  for (int i0 = 0; i0 < n_items; i0 += kLegMaxItems) {
-    const int n = std::min(kLegMaxItems, n_items - i0);
+  for (int i0 = 0; i0 < n_items; i0 += kMaxItems) {
+    const int n = std::min(kMaxItems, n_items - i0);
     // FP64: a row of the grid per item (a small launch is all latency, and the
     // shared sequence has more of it: 8.1 -> 11.4 us at chi = 8)
     const dim3 grid = sizeof(T) == 8 ? dim3(std::max(8, 8 * 152 / n), n) : dim3(152 * LegBlock<T>::CTAS);
@@ -559,15 +558,22 @@ static cudaError_t launch_gram_band(const GramLegItem* items, int n_items, int s
   return cudaGetLastError();
 }
 
+int gram_leg_launches(int chimax) {
+  int n = 1;
+  while (n < 5 && chimax > kGramBands[n]) ++n;
+  return n;
+}
+
 template <typename T>
 cudaError_t launch_gram_leg(const GramLegItem* items, int n_items, int splits_max, int chimax,
                             void* const* ptrs, const int* ival, cudaStream_t s) {
   if (n_items == 0) return cudaSuccess;
   cudaError_t e = launch_gram_band<T, 0>(items, n_items, splits_max, ptrs, ival, s);
-  if (e == cudaSuccess && chimax > kGramBands[1]) e = launch_gram_band<T, 1>(items, n_items, splits_max, ptrs, ival, s);
-  if (e == cudaSuccess && chimax > kGramBands[2]) e = launch_gram_band<T, 2>(items, n_items, splits_max, ptrs, ival, s);
-  if (e == cudaSuccess && chimax > kGramBands[3]) e = launch_gram_band<T, 3>(items, n_items, splits_max, ptrs, ival, s);
-  if (e == cudaSuccess && chimax > kGramBands[4]) e = launch_gram_band<T, 4>(items, n_items, splits_max, ptrs, ival, s);
+  const int bands = gram_leg_launches(chimax);
+  if (e == cudaSuccess && bands > 1) e = launch_gram_band<T, 1>(items, n_items, splits_max, ptrs, ival, s);
+  if (e == cudaSuccess && bands > 2) e = launch_gram_band<T, 2>(items, n_items, splits_max, ptrs, ival, s);
+  if (e == cudaSuccess && bands > 3) e = launch_gram_band<T, 3>(items, n_items, splits_max, ptrs, ival, s);
+  if (e == cudaSuccess && bands > 4) e = launch_gram_band<T, 4>(items, n_items, splits_max, ptrs, ival, s);
   return e;
 }
 

@@ -821,12 +821,10 @@ __device__ __noinline__ unsigned r3_tiles(const R3Plan& pl, float* r3_sh, unsign
   return tiles;
 }
 
-constexpr int kR3MaxItems = 512;                       // of a launch
-
 __global__ void __launch_bounds__(256, 2)
 k_reconstruct32(const ReconItem* __restrict__ items, int n_items, void* const* ptrs, const int* __restrict__ ival) {
   __shared__ R3Plan pl;
-  __shared__ unsigned toff[kR3MaxItems + 1];
+  __shared__ unsigned toff[kMaxItems + 1];
   extern __shared__ __align__(16) float r3_sh[];
   tile_prefix(toff, n_items, [&](int i) {
     const ReconItem& it = items[i];
@@ -858,8 +856,8 @@ cudaError_t launch_reconstruct(const ReconItem* items, int n_items, int chimax, 
     const size_t smem = sizeof(float) * ((size_t)nmax * R3_COLS + (size_t)R3_STAGES * R3_ROWS * R3_PITCH);
     cudaError_t e = cudaFuncSetAttribute(k_reconstruct32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    for (int i0 = 0; i0 < n_items; i0 += kR3MaxItems)
-      k_reconstruct32<<<2 * 152, 256, smem, s>>>(items + i0, std::min(kR3MaxItems, n_items - i0), ptrs, ival);
+    for (int i0 = 0; i0 < n_items; i0 += kMaxItems)
+      k_reconstruct32<<<2 * 152, 256, smem, s>>>(items + i0, std::min(kMaxItems, n_items - i0), ptrs, ival);
   } else {
     const long long rows = (long long)chimax * chimax * chimax;
     const long long tiles = (rows + RC_T - 1) / RC_T * ceil_div(nmax, RC_T);

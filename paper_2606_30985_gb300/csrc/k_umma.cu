@@ -69,7 +69,6 @@ constexpr int kTmemCols = 512;          // two accumulators of 256 columns
 // and the epilogue's pass over the accumulator is paid once per run
 constexpr int kRun = 32;
 constexpr unsigned long long kDrainNs = 2000000000ull;   // bound of the exit drains
-constexpr int kMaxItems = 512;
 
 // ---------------------------------------------------------------- PTX helpers
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -1354,8 +1353,8 @@ cudaError_t launch_leg_umma(const LegItem* items, int n_items, int chimax, void*
   if (P.stages < 2) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(um::k_leg_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.total);
   if (e != cudaSuccess) return e;
-  for (int i0 = 0; i0 < n_items; i0 += um::kMaxItems) {
-    const int n = std::min(um::kMaxItems, n_items - i0);
+  for (int i0 = 0; i0 < n_items; i0 += kMaxItems) {
+    const int n = std::min(kMaxItems, n_items - i0);
     um::k_leg_umma<<<um::sm_count(), um::kThreads, P.total, s>>>(items + i0, n, chimax, ptrs, ival, err, wait_ns);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1385,8 +1384,8 @@ cudaError_t launch_recon_umma(const ReconItem* items, int n_items, int chimax, v
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(um::k_recon_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.total);
   if (e != cudaSuccess) return e;
-  for (int i0 = 0; i0 < n_items; i0 += um::kMaxItems) {
-    const int n = std::min(um::kMaxItems, n_items - i0);
+  for (int i0 = 0; i0 < n_items; i0 += kMaxItems) {
+    const int n = std::min(kMaxItems, n_items - i0);
     um::k_recon_umma<<<um::sm_count(), um::kThreads, P.total, s>>>(items + i0, n, ptrs, ival, err, wait_ns);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1403,8 +1402,8 @@ cudaError_t launch_gram_umma(const GramLegItem* items, int n_items, int splits_m
   if (P.stages < 2) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(um::k_gram_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.total);
   if (e != cudaSuccess) return e;
-  for (int i0 = 0; i0 < n_items; i0 += um::kMaxItems) {
-    const int n = std::min(um::kMaxItems, n_items - i0);
+  for (int i0 = 0; i0 < n_items; i0 += kMaxItems) {
+    const int n = std::min(kMaxItems, n_items - i0);
     um::k_gram_umma<<<um::sm_count(), um::kGramThreads, P.total, s>>>(items + i0, n, splits_max, chimax, ptrs, ival,
                                                                    err, wait_ns);
     e = cudaGetLastError();

@@ -21,6 +21,11 @@ cudaError_t launch_gram_rows_reduce(const GramRowsItem* items, int n_items, int 
 constexpr int kGramExactLaunches = 4;
 cudaError_t launch_gram_exact(const GramRowsItem* items, int n_items, int fmax, int pass, void* const* ptrs,
                               const int* ival, double* acct, cudaStream_t s);
+// kernels that launch_gram_leg enqueues (one per band of F up to chimax), and that the
+// launchers with a limit on the items of a launch do
+int gram_leg_launches(int chimax);
+constexpr int kMaxItems = 512;
+__host__ inline int item_launches(int n_items) { return (n_items + kMaxItems - 1) / kMaxItems; }
 template <typename T>
 cudaError_t launch_gram_leg(const GramLegItem* items, int n_items, int splits_max, int chimax,
                             void* const* ptrs, const int* ival, cudaStream_t s);

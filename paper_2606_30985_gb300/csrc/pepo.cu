@@ -1321,14 +1321,15 @@ pepo_status keep_flags(pepo_ctx* c) {
 
 // Every launch wrapper returns without launching when its item count is 0;
 // LAUNCH_T counts (and, in timing mode, brackets with events) the launches
-// that happen.
-#define LAUNCH_T(cls, hptr, n, expr)                                                    \
+// that happen; LAUNCH_K the `k` kernels of a wrapper that enqueues several.
+#define LAUNCH_T(cls, hptr, n, expr) LAUNCH_K(cls, hptr, n, 1, expr)
+#define LAUNCH_K(cls, hptr, n, k, expr)                                                 \
   do {                                                                                  \
     if ((n) > 0) {                                                                      \
       cudaEvent_t _a = nullptr, _b = nullptr;                                           \
       if (c->timing) { _a = next_event(c); _b = next_event(c); cudaEventRecord(_a, c->stream); } \
       cudaError_t _e = (expr);                                                          \
-      c->launches++;                                                                    \
+      c->launches += (k);                                                               \
       if (_e != cudaSuccess)                                                            \
         return fail(c, PEPO_E_CUDA, "%s: %s", #expr, cudaGetErrorString(_e));           \
       if (c->timing && _a && _b) {                                                      \
@@ -1369,7 +1370,8 @@ pepo_status run_gate_wave(pepo_ctx* c, Inst& I, GateWave& w) {
   LAUNCH_T(K_ENV, nullptr, w.env.n, launch_env_factor(w.env.d, w.env.n, chimax, c->d_ival, s));
   LAUNCH_N(w.copy.n, launch_copy<T>(w.copy.d, w.copy_out.d, w.copy.n, 64, c->d_ptrs, c->d_ival, s));
   for (int r = 0; r < 3; ++r)
-    LAUNCH_T(K_LEG, hitems(c, w.leg[r]), w.leg[r].n, leg_dispatch<T>(c, w.leg[r].d, w.leg[r].n, chimax));
+    LAUNCH_K(K_LEG, hitems(c, w.leg[r]), w.leg[r].n, item_launches(w.leg[r].n),
+             leg_dispatch<T>(c, w.leg[r].d, w.leg[r].n, chimax));
   LAUNCH_N(w.fac.n, launch_branch(w.fac.d, w.fac.n, c->d_ival, s));
   {
     int nt = ceil_div(nmax, 64);
@@ -1386,9 +1388,8 @@ pepo_status run_gate_wave(pepo_ctx* c, Inst& I, GateWave& w) {
   const int householder = sizeof(T) == 8 ? 1 : 0;
   auto factor_rows = [&](int pass) -> pepo_status {
     if (!householder) {
-      LAUNCH_T(K_HH, nullptr, w.gram.n, launch_gram_exact(w.gram.d, w.gram.n, nmax, pass, c->d_ptrs, c->d_ival,
-                                                          c->d_hh_acct, s));
-      if (w.gram.n > 0) c->launches += kGramExactLaunches - 1;
+      LAUNCH_K(K_HH, nullptr, w.gram.n, kGramExactLaunches,
+               launch_gram_exact(w.gram.d, w.gram.n, nmax, pass, c->d_ptrs, c->d_ival, c->d_hh_acct, s));
       return PEPO_OK;
     }
     const long long mmax = (long long)pow_sz(chimax, 3);
@@ -1425,10 +1426,10 @@ pepo_status run_gate_wave_tail(pepo_ctx* c, Inst& I, GateWave& w) {
   const int chimax = I.cfg.chi_max;
   {
     if (use_umma<T>(c, chimax))
-      LAUNCH_T(K_RECON, hitems(c, w.recon), w.recon.n,
+      LAUNCH_K(K_RECON, hitems(c, w.recon), w.recon.n, 1 + item_launches(w.recon.n),
                launch_recon_umma(w.recon.d, w.recon.n, chimax, c->d_ptrs, c->d_ival, c->d_kerr, c->wait_ns, s));
     else
-      LAUNCH_T(K_RECON, hitems(c, w.recon), w.recon.n,
+      LAUNCH_K(K_RECON, hitems(c, w.recon), w.recon.n, sizeof(T) == 4 ? item_launches(w.recon.n) : 1,
                launch_reconstruct<T>(w.recon.d, w.recon.n, chimax, c->d_ptrs, c->d_ival, s));
   }
   LAUNCH_N(w.npairs, launch_commit(w.pairs.d, w.npairs, w.moves.d, w.nmoves, c->d_ptrs, c->d_ival, s));
@@ -1442,10 +1443,11 @@ pepo_status run_bp_waves(pepo_ctx* c, Inst& I, std::vector<BpWave>& waves) {
   for (auto& w : waves) {
     LAUNCH_T(K_BP_EIG, nullptr, w.eig.n, launch_env_eig(w.eig.d, w.eig.n, chimax, c->tsize == 4 ? 1 : 0, c->d_ival, s));
     for (int a = 0; a < 4; ++a) {
-      LAUNCH_T(K_BP_LEG, hitems(c, w.leg[a]), w.leg[a].n,
+      LAUNCH_K(K_BP_LEG, hitems(c, w.leg[a]), w.leg[a].n, item_launches(w.leg[a].n),
                leg_dispatch<T>(c, w.leg[a].d, w.leg[a].n, chimax));
     }
-    LAUNCH_T(K_GRAM_LEG, hitems(c, w.gram), w.gram.n,
+    LAUNCH_K(K_GRAM_LEG, hitems(c, w.gram), w.gram.n,
+             use_umma<T>(c, chimax) ? item_launches(w.gram.n) : gram_leg_launches(chimax),
              gram_leg_dispatch<T>(c, w.gram.d, w.gram.n, chimax));
     LAUNCH_T(K_GRAM_LEG_RED, nullptr, w.gram.n,
              launch_gram_leg_reduce(w.gram.d, w.gram.n, chimax, c->tune.gram_leg_splits,
@@ -1453,8 +1455,7 @@ pepo_status run_bp_waves(pepo_ctx* c, Inst& I, std::vector<BpWave>& waves) {
                                     use_umma<T>(c, chimax) ? 1 : 0, c->d_ival, s));
     LAUNCH_T(K_MSG, nullptr, w.rot.n, launch_rotate_back(w.rot.d, w.rot.n, chimax, c->d_ival, s));
     if (w.pw.n > 0) {
-      LAUNCH_T(K_OTHER, nullptr, w.pw.n, launch_pauli_weights<T>(w.pw.d, w.pw.n, c->d_ptrs, c->d_ival, s));
-      c->launches++;   // the zeroing kernel
+      LAUNCH_K(K_OTHER, nullptr, w.pw.n, 2, launch_pauli_weights<T>(w.pw.d, w.pw.n, c->d_ptrs, c->d_ival, s));
     }
   }
   return PEPO_OK;
