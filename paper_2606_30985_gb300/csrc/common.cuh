@@ -58,17 +58,15 @@ struct LegItem {
   int out_ref;
   int leg;
   int out_dim;             // ival index of the output size of that leg
-  int a_rows;              // ival index of A's row count (== out size)
   const double* A;         // row-major, leading dimension lda
   int lda;
 };
 
-// Gram over rows: C[f, f'] = sum_k X[k, f] Y[k, f'], X, Y row-major K x F with
+// Gram over rows: C[f, f'] = sum_k X[k, f] X[k, f'], X row-major K x F with
 // F = 4 * (size of the innermost leg): the cv^T cv of Eq. 10 (Cholesky-QR).
 struct GramRowsItem {
   TView x;
-  int y_ref;
-  int active;              // ival index of a 0/1 flag (-1: always active)
+  int active;              // ival index of the site's branch value (-1: always active)
   double* partial;         // [splits][Fmax * Fmax]
   double* out;             // F x F, leading dimension ldo
   int ldo;
@@ -120,7 +118,6 @@ struct ReconItem {
   int out_perm[PEPO_MAXLEG];
   const double* W;         // n x n', row-major, leading dimension ldw
   int ldw;
-  double* scale_sq;        // optional: sum of squares of the output (may be null)
   float* Wp;               // tensor-core path: W packed into swizzled B blocks (recon_packed_floats(nmax))
 };
 

@@ -198,7 +198,7 @@ struct PlainSum {
 };
 template <typename T> struct PauliAcc;
 template <> struct PauliAcc<float> { using Sum = TwoFloat; using Quad = float4; };
-template <> struct PauliAcc<double> { using Sum = PlainSum; using Quad = double4; };
+template <> struct PauliAcc<double> { using Sum = PlainSum; using Quad = double4_16a; };
 
 template <typename T>
 __global__ void __launch_bounds__(256)

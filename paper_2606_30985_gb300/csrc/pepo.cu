@@ -127,7 +127,6 @@ struct Inst {
   int chi0 = 0, pend0 = 0, grank0 = 0;
   int site_ref0 = 0;
   // device arrays
-  void* slab[1];       // unused
   std::vector<void*> site_slab;
   double *lam = nullptr, *msg = nullptr, *hat = nullptr, *vec = nullptr, *vhat = nullptr;
   WsGeom* ws_geom = nullptr;          // 2 nb directed-bond descriptors of the warm-start features
@@ -205,7 +204,6 @@ struct pepo_ctx {
   size_t pool_next = 0;
   struct Tot { long long n = 0; double ms = 0, bytes = 0, flops = 0; };
   std::vector<Tot> tot;
-  int max_levels = 1;      // TSQR levels
   int rmax = 4, nmax = 4;
   // grouped execution: every instance's items of one wave / colour / level
   // concatenated into one launch (plan fields of grp only; grp.cfg.chi_max =
@@ -525,7 +523,6 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
   // linearly on the others land; below it the site takes the other branch
   // (Householder in FP64 storage, the exact Gram in FP32 storage)
   const double rel_safe = (c->prec == PEPO_FP64) ? 1e-10 : 1e-4;
-  const double rel_env = I.cfg.pinv_rel;
   for (int col = 0; col < 4; ++col) {
     const auto& bl = I.colours[col];
     std::vector<CoreItem> core_all;
@@ -613,7 +610,6 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
               li.out_ref = (r % 2 == 0) ? sref0 : sref1;
               li.leg = r;
               li.out_dim = W.rank_idx[r];
-              li.a_rows = W.rank_idx[r];
               li.A = W.L[r];
               li.lda = chimax;
               leg[r].push_back(li);
@@ -646,7 +642,6 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
           fac.push_back(f);
           GramRowsItem g;
           g.x = cvv;
-          g.y_ref = cv_ref;
           g.active = sws[v].branch_idx;
           g.partial = W.partial;
           g.out = sws[v].C;
@@ -668,7 +663,6 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
           rc.W = sws[v].W;
           rc.Wp = sws[v].Wp;
           rc.ldw = nmax;
-          rc.scale_sq = nullptr;
           recon.push_back(rc);
           pairs.push_back(I.site_ref0 + v);
           pairs.push_back(out_ref);
@@ -789,7 +783,6 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
           li.out_ref = refs[1 + (j % 2)];
           li.leg = j;
           li.out_dim = view.dim[j];
-          li.a_rows = view.dim[j];
           // the rotated leg carries the square roots of the message's
           // eigenvalues: the Grams below then need no weights
           li.A = W.Ls[j];
@@ -981,7 +974,6 @@ bool plan_instance(Planner& P, Inst& I, int inst_id) {
     bi[0].out = I.bethe_out;
     I.bethe = stage(P, bi);
   }
-  (void)rel_env;
   return true;
 }
 
