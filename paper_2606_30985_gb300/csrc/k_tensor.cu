@@ -390,7 +390,12 @@ k_gram_exact(const GramRowsItem* __restrict__ items, int pass, void* const* ptrs
   __shared__ float nrm[2][2 * GX_T];                   // half sums of squares per column
   __shared__ float pw[2 * GX_T];                       // P per column
   __shared__ float sc[2 * GX_T];                       // column pre-scale 2^-e
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  // A warp takes 32 x 16 entries, 8 x 4 threads; it has none outside the matrix or below
+  // the diagonal.  Which of the four column strips it takes turns with the block, so that
+  // the warps without entries are not all on one scheduler.
+  const int tid = threadIdx.x, wr = tid >> 7, wc = ((tid >> 5) + 2 * wr + blockIdx.x) & 3;
+  const int ty = 8 * wr + ((tid & 31) >> 2), tx = 4 * wc + (tid & 3);
+  const bool live = ti * GX_T + 32 * wr < F && tj * GX_T + 16 * wc < F && (!diag || 32 * wr < 16 * wc + 16);
   if (tid < 2 * GX_T) {
     const int c = (tid < GX_T ? ti : tj) * GX_T + (tid & (GX_T - 1));
     sc[tid] = c < F ? pow2f(-col_exp(it.colmax[c])) : 0.f;
@@ -453,54 +458,57 @@ k_gram_exact(const GramRowsItem* __restrict__ items, int pass, void* const* ptrs
       pw[tid] = pow2f(max((e + 2) >> 1, -50));                 // P^2 > q
     }
     __syncthreads();
-    float s[4][4], c[4][4], d[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        s[a][b] = 3.f * (pw[ty * 4 + a] * pw[GX_T + tx * 4 + b]);
-        c[a][b] = kGxLower * s[a][b];
-        d[a][b] = 0.f;
-      }
-#pragma unroll 4
-    for (int kk = 0; kk < GX_RUN; ++kk) {
-      const float4 xa = *reinterpret_cast<const float4*>(xs + kk * GX_T + ty * 4);
-      const float4 yb = *reinterpret_cast<const float4*>(ys + kk * GX_T + tx * 4);
-      const float a4[4] = {xa.x, xa.y, xa.z, xa.w}, b4[4] = {yb.x, yb.y, yb.z, yb.w};
+    if (live) {
+      float s[4][4], c[4][4], d[4][4];
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-          const float p = __fmul_rn(a4[a], b4[b]);
-          const float q = fmaf(a4[a], b4[b], -p);
-          const float t = __fadd_rn(s[a][b], p);
-          const float r = __fsub_rn(p, __fsub_rn(t, s[a][b]));
-          const float u = __fadd_rn(c[a][b], r);
-          d[a][b] += __fsub_rn(r, __fsub_rn(u, c[a][b]));
-          d[a][b] += q;
-          s[a][b] = t;
-          c[a][b] = u;
+          s[a][b] = 3.f * (pw[ty * 4 + a] * pw[GX_T + tx * 4 + b]);
+          c[a][b] = kGxLower * s[a][b];
+          d[a][b] = 0.f;
+        }
+#pragma unroll 4
+      for (int kk = 0; kk < GX_RUN; ++kk) {
+        const float4 xa = *reinterpret_cast<const float4*>(xs + kk * GX_T + ty * 4);
+        const float4 yb = *reinterpret_cast<const float4*>(ys + kk * GX_T + tx * 4);
+        const float a4[4] = {xa.x, xa.y, xa.z, xa.w}, b4[4] = {yb.x, yb.y, yb.z, yb.w};
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            const float p = __fmul_rn(a4[a], b4[b]);
+            const float q = fmaf(a4[a], b4[b], -p);
+            const float t = __fadd_rn(s[a][b], p);
+            const float r = __fsub_rn(p, __fsub_rn(t, s[a][b]));
+            const float u = __fadd_rn(c[a][b], r);
+            d[a][b] += __fsub_rn(r, __fsub_rn(u, c[a][b]));
+            d[a][b] += q;
+            s[a][b] = t;
+            c[a][b] = u;
+          }
+      }
+      // the run's sum into (S, U, W)
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const float anchor = 3.f * (pw[ty * 4 + a] * pw[GX_T + tx * 4 + b]);
+          float* uw = UW + 512 * (4 * a + b);
+          TwoFloat hi, mid;                                      // c: what the sum leaves over
+          hi.s = S0[a][b];
+          hi.take(s[a][b] - anchor);                             // exact difference
+          mid.s = uw[0];
+          mid.take(c[a][b] - kGxLower * anchor);                 // exact too
+          mid.take(hi.c);
+          S0[a][b] = hi.s;
+          uw[0] = mid.s;
+          uw[256] += mid.c + d[a][b];
         }
     }
-    // the run's sum into (S, U, W)
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const float anchor = 3.f * (pw[ty * 4 + a] * pw[GX_T + tx * 4 + b]);
-        float* uw = UW + 512 * (4 * a + b);
-        TwoFloat hi, mid;                                      // c: what the sum leaves over
-        hi.s = S0[a][b];
-        hi.take(s[a][b] - anchor);                             // exact difference
-        mid.s = uw[0];
-        mid.take(c[a][b] - kGxLower * anchor);                 // exact too
-        mid.take(hi.c);
-        S0[a][b] = hi.s;
-        uw[0] = mid.s;
-        uw[256] += mid.c + d[a][b];
-      }
     __syncthreads();                                           // the buffer is refilled next
   }
+  if (!live) return;
   double* Pt = it.partial + (long long)sp * F * F;
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
