@@ -162,13 +162,13 @@ struct EnvFactorItem {
   double rel;              // relative pivot threshold of the instance
 };
 
-// Per-site factor of the bond update: either Cholesky-QR (Gram) or
-// Householder (TSQR) produces an R-factor of cv (Eq. 10); the gate's
+// Per-site factor of the bond update: Cholesky-QR (Gram), Householder (TSQR, FP64
+// storage) or an exact Gram (FP32 storage) produces an R-factor of cv (Eq. 10); the gate's
 // operator-Schmidt factors turn it into the factor T of X = (gate half) cv.
 struct SiteFacItem {
   TView cv;                // absorbed tensor, cut leg innermost (env dims = factor ranks)
-  int branch_idx;          // ival: 1 Cholesky-QR, 0 Householder, 2 Householder after a
-                           // Gram too ill-conditioned for Cholesky-QR
+  int branch_idx;          // ival: 1 Cholesky-QR, 0 the other branch (Householder or exact
+                           // Gram), 2 the same after a Gram too ill-conditioned for Cholesky-QR
   int kfac_idx;            // ival: rows of the R-factor (Householder branch)
   int rg_idx;              // ival: operator-Schmidt rank of the bond gate
   const double* F;         // gate factors [kappa][4][4] of this side

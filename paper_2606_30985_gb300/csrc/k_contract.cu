@@ -301,16 +301,18 @@ cudaError_t launch_leg_contract(const LegItem* items, int n_items, int chimax, v
 // the tile is chosen from the live F (8, 16, 24, 32, 48, 64, 96, 128), not from
 // chi_max.  Their sums are laid side by side and added by one thread per entry: with
 // the groups adding one after another, a warp's FP64 operations (64 clocks each)
-// in 16 turns took longer than the products of a small split.  FP32 storage sums runs of 256 terms in FP32 and the runs in a
-// two-float sum; FP64 sums directly.
+// in 16 turns took longer than the products of a small split.  FP32 storage sums runs
+// of 256 terms in FP32 and the runs in a two-float sum (which is within 1e-16 of the
+// rows' norms of an FP64 sum of them); FP64 sums directly.
 //
 // Bound: shared memory (a 16-byte load of a warp takes 4 clocks of the SM, 2 where
 // neighbouring lanes share it, and MT + MT of them feed 2 MT (MT + 1) products), so up
 // to F = 32 the threads of a group are 4 x 4 with as many entries each as that
 // takes: 24 clocks of loads per unit at F = 32 instead of 48 with 8 x 8 threads;
 // or the FP64 pipe.  Class of a case, before -> now: chi = 8 FP64 (107 launches)
-// 143 -> 1.8 ms, 4x4 chi = 12 FP64 154 -> 1.7 ms, 4x4 chi = 48 FP32 82 -> 25 ms.  The 64 x 64 (128 x 128) tile it replaces did 64 x 64 products
-// for an 8 x 8 Gram and stored every chunk with 32-way bank conflicts.
+// 143 -> 1.8 ms, 4x4 chi = 12 FP64 154 -> 1.7 ms, 4x4 chi = 48 FP32 82 -> 25 ms.  The
+// 64 x 64 (128 x 128) tile it replaces did 64 x 64 products for an 8 x 8 Gram and
+// stored every chunk with 32-way bank conflicts.
 constexpr int kGlStages = 3;
 
 template <typename T, int MT, int TX>

@@ -5,7 +5,7 @@
 //                  "pseudo_sqrt"); any factor with L^T L = M gives the same cv
 //                  Gram, so no eigensolver is needed.
 //   k_branch       Eq. 10 branch rule: Cholesky-QR when n > n_thr and
-//                  m / n > ratio_thr, Householder otherwise (Sec. 4.2).
+//                  m / n > ratio_thr, the other branch otherwise (Sec. 4.2).
 //   k_hh_level     FP64 storage: Householder QR (TSQR tree, R only) of cv
 //                  (Sec. 4.2 Householder-QR); each tree block factored in panels
 //                  (compact WY).  FP32 storage forms the exact Gram of cv instead
@@ -976,8 +976,8 @@ __device__ int qrcp(double* B, int ld, int M, int r, double* dg, double* w, doub
 //
 // Whether the Cholesky-QR branch can be trusted with its Gram C = cv^T cv
 // (n x n): its factor is only as accurate as C.  The Gram's rounding is
-// relative to the norms of the columns it pairs (FP32 runs flushed into
-// FP64: ~1e-8 of that scale; FP64: ~1e-14), so a column that is a linear
+// relative to the norms of the columns it pairs (runs of 256 terms in FP32:
+// ~1e-8 of that scale; FP64: ~1e-14), so a column that is a linear
 // combination of the others in exact arithmetic keeps a Schur complement of
 // that relative size, and the Q-less update would take the noise for a
 // direction (Q = cv R^-1 is then far from orthonormal).  The pivoted Cholesky
@@ -985,7 +985,8 @@ __device__ int qrcp(double* B, int ld, int M, int r, double* dg, double* w, doub
 // against the column's own diagonal; when one keeps less than rel_safe of it
 // the site is marked branch 2 and left for the pass that follows (only = 2
 // runs that pass only).  Pivots below rel of the first end the check
-// (directions too small to matter: the factorisation of G cuts them as rank).
+// (directions too small to matter: the factorisation of G cuts them as rank;
+// rel_exact where G comes from an exact Gram).
 //
 // Measured, factor class of one saturated layer, right-looking Cholesky and one
 // thread per column -> left-looking on a cluster, no Householder in FP32 storage: 4x4

@@ -6,7 +6,8 @@
 // device.  Per colour the bonds are cut into waves that fit the scratch slabs;
 // per wave the launch sequence is (Alg. 1 / Fig. 1, Q-less form):
 //   env factors -> absorb (leg contractions) -> Eq. 10 branch ->
-//   [Cholesky-QR: Gram -> reduce] | [Householder: TSQR levels -> extract] ->
+//   [Cholesky-QR: Gram -> reduce] | [Householder: TSQR levels -> extract, or in FP32
+//   storage the exact Gram] ->
 //   gate fold (formG / formB) -> rank-revealing factor -> bond core (SVD,
 //   truncation, lambda, W, messages) -> reconstruct into the next layout ->
 //   commit (pointer swap, chi_new).
@@ -1376,7 +1377,7 @@ pepo_status run_gate_wave(pepo_ctx* c, Inst& I, GateWave& w) {
   // FP64 storage: Householder TSQR.  FP32 storage: the exact Gram of the FP32
   // data, whose Cholesky factor carries no more error (k_gram_exact).  Both
   // sides, TSQR and its column-pivoted factor against exact Gram and Cholesky, classes
-  // of a saturated layer: 4x4 chi = 64 544 -> 26 ms, 3x3 chi = 100 545 -> 63 ms.
+  // of a saturated layer: 4x4 chi = 64 544 -> 26 ms, 3x3 chi = 100 545 -> 58 ms.
   const int householder = sizeof(T) == 8 ? 1 : 0;
   auto factor_rows = [&](int pass) -> pepo_status {
     if (!householder) {
@@ -2750,8 +2751,8 @@ pepo_status pepo_get_timing(pepo_ctx* c, int k, long long* launches, double* ms,
   const auto& t = c->tot[k];
   double dev[2] = {0.0, 0.0};
   if (k == K_HH) {
-    // which sites take the Householder branch is decided on the device, so
-    // this class's work is counted there (k_hh_extract)
+    // which sites take this branch is decided on the device, so this class's
+    // work is counted there (k_hh_extract, k_gram_exact_reduce)
     if (cudaMemcpyAsync(dev, c->d_hh_acct, sizeof(dev), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
         cudaStreamSynchronize(c->stream) != cudaSuccess)
       return fail(c, PEPO_E_CUDA, "pepo_get_timing: %s", cudaGetErrorString(cudaGetLastError()));
